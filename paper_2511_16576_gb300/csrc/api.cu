@@ -332,6 +332,8 @@ extern "C" int pmh_poly_reload(pmh_polys polys, const int32_t* xy, const int64_t
                              (long long)n_polys, (long long)n_vertices);
     cudaStream_t s = (cudaStream_t)stream;
     PMH_CUDA_TRY(cudaStreamSynchronize(s));  // no kernel of this stream may still read the old data
+    // (a reload that fails leaves no slab index behind)
+    if (polys->d_slabs) PMH_CUDA_TRY(cudaMemsetAsync(polys->d_slabs, 0, sizeof(SlabPtrs), s));
     free_derived(polys);
     return upload_fill(polys, xy, offsets, host_memory != 0, s);
 }
@@ -376,7 +378,7 @@ extern "C" int pmh_polys_destroy(pmh_polys p)
     cudaSetDevice(p->device);
     if (p->xy || p->offsets || p->bbox || p->area2) cudaDeviceSynchronize();
     void* bufs[] = {p->xy, p->offsets, p->bbox, p->area2, p->feat, p->slab_info, p->slab_ptr,
-                    p->slab_edges, p->order, p->order_cls, p->mask};
+                    p->slab_edges, p->d_slabs, p->order, p->order_cls, p->mask};
     for (void* b : bufs)
         if (b) cudaFree(b);
     delete p;

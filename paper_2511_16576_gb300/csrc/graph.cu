@@ -40,6 +40,8 @@ struct pmh_qgraph_s {
     int32_t* slab_ptr = nullptr;
     int32_t* slab_cursor = nullptr;
     int32_t* slab_edges = nullptr;
+    SlabPtrs* d_slabs = nullptr;
+    int32_t* ref_queue = nullptr;     // pairs of large rings (nullable)
     int64_t cap_ptr = 0, cap_edges = 0;
     int64_t* counts = nullptr;
     void* join_stage = nullptr;       // join rows sorted by the count pass (nullable): a pool of cap ids
@@ -66,7 +68,7 @@ struct pmh_qgraph_s {
     double* ref_j = nullptr;
     int* flags = nullptr;
     int64_t* d_n = nullptr;
-    unsigned long long* ticket = nullptr;  // [2]: signing grid, refinement grid
+    unsigned long long* ticket = nullptr;  // [4]: signing grid, refinement grids
     int64_t* scan_sums = nullptr;
     const uint2* sidx_cell = nullptr;  // the stream index the graph captured (nullptr: none)
     int64_t kernels = 0;               // kernel launches per replay
@@ -93,7 +95,8 @@ extern "C" int pmh_qgraph_destroy(pmh_qgraph g)
                     g->top_ids,   g->top_n,      g->jv,         g->ref_ids,   g->ref_j,
                     g->flags,     g->d_n,        g->ticket,     g->scan_sums, g->sl_ids,
                     g->sl_n,      g->sl_counts,  g->sl_sums,    g->sl_row_ptr, g->sl_cand,
-                    g->qfeat,     g->feat,       g->score,     g->join_stage};
+                    g->qfeat,     g->feat,       g->score,     g->join_stage,
+                    g->d_slabs,   g->ref_queue};
     for (void* b : bufs)
         if (b) cudaFree(b);
     delete g;
@@ -186,7 +189,12 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
                           cudaMalloc(&g->ref_j, sizeof(double) * Q * k) == cudaSuccess)) &&
               cudaMalloc(&g->flags, sizeof(int) * 4) == cudaSuccess &&
               cudaMalloc(&g->d_n, sizeof(int64_t)) == cudaSuccess &&
-              cudaMalloc(&g->ticket, 2 * sizeof(unsigned long long)) == cudaSuccess &&
+              cudaMalloc(&g->ticket, 4 * sizeof(unsigned long long)) == cudaSuccess &&
+              cudaMalloc(&g->d_slabs, sizeof(SlabPtrs)) == cudaSuccess &&
+              // (a batch of a few small queries against small polygons has no large ring; a set
+              // reloaded with larger ones is still refined, by the two-warp form)
+              (k == 0 || std::max<int64_t>(max_vertices, db->max_n) <= kRefineBigVerts ||
+               cudaMalloc(&g->ref_queue, pmh_refine_queue_bytes(Q * m)) == cudaSuccess) &&
               cudaMalloc(&g->scan_sums, sizeof(int64_t) * pmh_scan_sums_size(Q)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -195,6 +203,8 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
     }
     cudaMemset(g->d_n, 0, sizeof(int64_t));
     cudaMemset(g->off, 0, sizeof(int64_t) * (Q + 1));
+    const SlabPtrs slabs{g->slab_info, g->slab_ptr, g->slab_edges};
+    cudaMemcpy(g->d_slabs, &slabs, sizeof(slabs), cudaMemcpyHostToDevice);
     cudaStream_t cs;
     PMH_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     const int U = 4;  // points per lane per round of the walk form
@@ -258,8 +268,9 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
         }
     }
     if (rc == PMH_OK && k > 0)
-        rc = pmh_launch_refine_topk(ctx, g->xy, g->off, g->area2, g->bbox, db, g->top_ids, g->top_n, Q, g->d_n, m,
-                                    k, g->jv, g->ticket + 1, g->ref_ids, g->ref_j, cs);
+        rc = pmh_launch_refine_topk(ctx, RefineQueries{g->xy, g->off, g->area2, g->bbox, g->d_slabs}, db,
+                                    g->top_ids, g->top_n, Q, g->d_n, m, k, g->jv, g->ticket + 1, g->ref_queue,
+                                    g->ref_ids, g->ref_j, cs);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(cs, &graph);
     if (rc == PMH_OK && e != cudaSuccess)

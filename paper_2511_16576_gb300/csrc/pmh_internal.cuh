@@ -232,6 +232,19 @@ struct SlabInfo {
     int32_t ymin;       // lowest vertex y
 };
 constexpr int kSlabMinVerts = 256;  // polygons above this size get a slab index
+// a set's slab index as kernels find it through a device-resident word: a reload rebuilds
+// the arrays, and a captured graph that refines against the set reads the current ones
+struct SlabPtrs {
+    const SlabInfo* info;
+    const int32_t* ptr;
+    const int32_t* edges;
+};
+// floor(x / h) by a multiply: with m = floor(2^40 / h) + 1 (slab_div_magic), x * m / 2^40
+// exceeds x / h by less than x / 2^40 < 2^-18 for x < 2^22, which is below the gap 1/h
+// between x / h and the next integer for every h < 2^18 (slab heights here are at most
+// 2^21 / 64 for polygons above 256 vertices, or 1), so the floor is exact
+__host__ __device__ __forceinline__ uint64_t slab_div_magic(int h) { return (1ull << 40) / (uint64_t)h + 1ull; }
+__host__ __device__ __forceinline__ int slab_div(int x, uint64_t m) { return (int)(((uint64_t)x * m) >> 40); }
 
 // Handles record their device so that they can be released after their context.
 struct pmh_polys_s {
@@ -247,6 +260,7 @@ struct pmh_polys_s {
     SlabInfo* slab_info = nullptr;  // [n]
     int32_t* slab_ptr = nullptr;
     int32_t* slab_edges = nullptr;
+    SlabPtrs* d_slabs = nullptr;    // the three above, device-resident (rewritten by a reload)
     int32_t* order = nullptr;       // polygons by expected signing cost, largest first (built
                                     // on the first signing call without the stream index)
     int32_t* order_cls = nullptr;   // class order: polygons above kChunkMinVerts vertices, then
@@ -449,13 +463,23 @@ int pmh_launch_agree_features(pmh_ctx ctx, const uint32_t* qh, const uint32_t* p
                               uint16_t* feat, FeatSrc qf, FeatSrc pf, const int* d_flags,
                               cudaStream_t s);
 // exact refinement of fixed-width top-m lists (ids [Q][m], nlist [Q]) to the top-k by
-// (J desc, id asc) (refine.cu); jv: Q * m doubles of scratch; ticket: the grid's counter;
-// d_n (optional) caps Q on the device
-int pmh_launch_refine_topk(pmh_ctx ctx, const int2* qxy, const int64_t* qoff, const int64_t* qarea2,
-                           const int4* qbox, pmh_polys db, const int32_t* ids, const int32_t* nlist, int64_t Q,
-                           const int64_t* d_n, int32_t m, int32_t k, double* jv,
-                           unsigned long long* ticket, int32_t* top_ids, double* top_j,
-                           cudaStream_t s);
+// (J desc, id asc) (refine.cu); jv: Q * m doubles of scratch; tickets: the grids' three
+// counters; d_n (optional) caps Q on the device.  big (pmh_refine_queue_bytes(Q * m);
+// nullable) is the queue of the pairs with a ring above kRefineBigVerts vertices, which
+// then go to a block each; without it every pair takes the two-warp form.
+struct RefineQueries {
+    const int2* xy;
+    const int64_t* off;
+    const int64_t* area2;
+    const int4* box;
+    const SlabPtrs* slabs;  // nullptr: no slab lists
+};
+constexpr int kRefineBigVerts = 1024;
+size_t pmh_refine_queue_bytes(int64_t n_pairs);
+int pmh_launch_refine_topk(pmh_ctx ctx, const RefineQueries& qs, pmh_polys db, const int32_t* ids,
+                           const int32_t* nlist, int64_t Q, const int64_t* d_n, int32_t m, int32_t k,
+                           double* jv, unsigned long long* tickets, int32_t* big, int32_t* top_ids,
+                           double* top_j, cudaStream_t s);
 // fixed-width lists ids [Q][m] with counts n [Q] to compact CSR (row_ptr [Q + 1], cand);
 // rows at or past *d_q (optional) are empty; counts: Q entries of scratch; sums: the
 // scan's partial sums (pmh_scan_sums_size(Q) entries; nullptr: context scratch)

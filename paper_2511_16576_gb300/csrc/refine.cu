@@ -496,20 +496,22 @@ refine_pairs_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qo
                     const int2* __restrict__ pxy, const int64_t* __restrict__ poff,
                     const int64_t* __restrict__ parea2, const int4* __restrict__ pbox,
                     const int32_t* __restrict__ ids, const int32_t* __restrict__ nlist, int m,
-                    const int32_t* __restrict__ qid_list, int64_t n_pairs, double* __restrict__ out,
-                    unsigned long long* __restrict__ ticket, const int64_t* __restrict__ d_n)
+                    const int32_t* __restrict__ qid_list, int64_t e0, int64_t n_pairs, double* __restrict__ out,
+                    unsigned long long* __restrict__ ticket /* [0]: pairs, [1]: queued pairs */,
+                    int32_t* __restrict__ big, const int64_t* __restrict__ d_n)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int g = wid >> 1, wip = wid & 1;
     RefPair& P = reinterpret_cast<RefPair*>(smem_raw)[g];
-    if (d_n && !qid_list) n_pairs = min(n_pairs, *d_n * (int64_t)m);  // lists of the live queries
+    // pairs [e0, n_pairs) of the call, those of the live queries
+    if (d_n && !qid_list) n_pairs = min(n_pairs, *d_n * (int64_t)m);
     // persistent warp pairs pull pairs from a ticket: pair costs differ by orders of
     // magnitude (a query against its own source vs a neighbour it barely touches)
     for (;;) {
         if (wip == 0 && lane == 0) P.e = (long long)atomicAdd(ticket, 1ull);
         pair_sync(g);
-        const int64_t e = P.e;
+        const int64_t e = e0 + P.e;
         if (e >= n_pairs) break;  // the same for both warps
         int64_t q;
         int32_t p;
@@ -529,11 +531,384 @@ refine_pairs_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qo
             // an empty intersection, J = 0 exactly, as the full computation gives
             const int4 qa = qbox[q], pb = pbox[p];
             const bool apart = !(qa.x < pb.z && pb.x < qa.z && qa.y < pb.w && pb.y < qa.w);
-            j = apart ? 0.0
-                      : pair_jaccard(view(qxy, qoff, qarea2, q), view(pxy, poff, parea2, p), P, wip, lane, g);
+            const PairView A = view(qxy, qoff, qarea2, q), B = view(pxy, poff, parea2, p);
+            if (!apart && big && max(A.n, B.n) > kRefineBigVerts) {
+                if (wip == 0 && lane == 0) big[atomicAdd(ticket + 1, 1ull)] = (int32_t)(e - e0);
+                pair_sync(g);
+                continue;  // refine_big_kernel takes the pair
+            }
+            j = apart ? 0.0 : pair_jaccard(A, B, P, wip, lane, g);
         }
         if (wip == 0 && lane == 0) out[e] = j;
         pair_sync(g);  // the slice is free for the next pair
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Pairs with a ring above kRefineBigVerts vertices: a block each.  The two-warp form
+// keeps both rings' slab lists in 2,048 shared references; above ~1,700 vertices they
+// overflow and every edge pair was tested (n * m predicates by 64 threads).  Here a
+// ring's lists are the y-slab index of its set (slabs.cu: about n / 4 slabs, read from
+// L2), or lists built in shared memory for a ring without one, so that a vertex or an
+// edge meets only the few edges of its own rows.  The index lists an edge in the slabs
+// of its rows [min y, max y) and leaves horizontal edges out, so
+//  * a vertex a of A (+e) sees B's edges straddling the row of a.y: slab of a.y;
+//  * a vertex c of B sees the shifted A's edges with min < c.y <= max: slab of c.y - 1;
+//  * an A edge meets B's non-horizontal edges in the slabs from its lowest to its
+//    highest row (a crossing of the shifted edge lies strictly inside B's rows, or just
+//    below B's top vertex), each pair in the first slab that lists both;
+//  * a horizontal edge of B meets the A edges with min < y <= max: slab of y - 1.
+// The end terms are integers (twice dy (x0 + dx / 2)), the crossings' fp64 terms are
+// added as two integers (multiples of 2^-18, and the remainder's of 2^-56, modulo 2^64):
+// sums of integers do not depend on their order, so neither the list order (atomics)
+// nor the split over the threads shows in the result.
+// Bound by the latency of list entry -> two vertices, from L1/L2; 512 threads a pair.
+// 512 pairs of coastlines of 4 to 16,384 vertices: 0.94 ms, 153 ms before.
+// ---------------------------------------------------------------------------
+constexpr int kBigThreads = 512;
+constexpr int kBigWarps = kBigThreads / 32;
+constexpr int kBigCap = 2048;     // shared references of a ring without a slab index
+constexpr int kBigSlabs = 256;
+
+// a ring and its edge lists: sp / se in global memory (slab index) or shared memory;
+// sp == nullptr: one list of every edge
+struct ListRing {
+    const int2* v;
+    int n;
+    const int32_t* sp;
+    const int32_t* se;
+    int S, y0;
+    uint64_t magic;
+    int x0, x1;  // the ring's x-range
+    __device__ __forceinline__ int2 vert(int e) const { return v[e == n ? 0 : e]; }
+    // list positions of the edges whose rows [min y, max y) can hold row y
+    __device__ __forceinline__ void row(int y, int& lo, int& hi) const
+    {
+        lo = hi = 0;
+        if (!sp) {
+            hi = n;
+            return;
+        }
+        if (y < y0) return;
+        const int q = slab_div(y - y0, magic);
+        if (q >= S) return;
+        lo = sp[q];
+        hi = sp[q + 1];
+    }
+    __device__ __forceinline__ int edge(int t) const { return sp ? se[t] : t; }
+};
+
+struct BigSmem {
+    uint2 cq[kBigWarps][64];
+    int32_t ids[2][kBigCap];
+    int32_t beg[2][kBigSlabs + 1];
+    int cnt[2][kBigSlabs];
+    int range[2][4];  // min x, max x, min y, max y of each ring
+    int listed[2], sh[2];
+    unsigned long long ends, q18, r56;
+    long long e;
+};
+
+// the lists of a ring without a slab index (of at most kBigCap references), by one
+// warp: slabs of 2^sh rows from the ring's lowest vertex
+__device__ bool build_big_lists(const int2* v, int n, int y0, int y1, int32_t* ids, int32_t* beg, int* cnt,
+                                int& sh_out, int lane)
+{
+    int sh = 0;
+    while (((y1 - y0) >> sh) >= kBigSlabs) ++sh;
+    for (int s = lane; s < kBigSlabs; s += 32) cnt[s] = 0;
+    __syncwarp();
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int e = lane; e < n; e += 32) {
+            const int2 a = v[e], b = v[e + 1 == n ? 0 : e + 1];
+            if (a.y == b.y) continue;
+            const int s0 = (min(a.y, b.y) - y0) >> sh, s1 = (max(a.y, b.y) - 1 - y0) >> sh;
+            for (int s = s0; s <= s1; ++s) {
+                const int t = atomicAdd(&cnt[s], 1);
+                if (pass) ids[t] = e;
+            }
+        }
+        __syncwarp();
+        if (pass) break;
+        int carry = 0;
+        for (int s0 = 0; s0 < kBigSlabs; s0 += 32) {
+            const int c = cnt[s0 + lane];
+            int x = c;
+            for (int d = 1; d < 32; d <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, x, d);
+                if (lane >= d) x += t;
+            }
+            beg[s0 + lane] = cnt[s0 + lane] = carry + x - c;
+            carry += __shfl_sync(0xffffffffu, x, 31);
+        }
+        if (carry > kBigCap) return false;
+        if (lane == 0) beg[kBigSlabs] = carry;
+        __syncwarp();
+    }
+    sh_out = sh;
+    return true;
+}
+
+// exact running sum of fp64 terms |x| < 2^44: multiples of 2^-18 and of 2^-56, modulo 2^64
+struct ExactSum {
+    unsigned long long q18 = 0, r56 = 0;
+    __device__ __forceinline__ void add(double x)
+    {
+        const long long q = __double2ll_rn(x * 262144.0);
+        const double r = fma((double)q, -1.0 / 262144.0, x);  // exact: |r| <= 2^-19
+        q18 += (unsigned long long)q;
+        r56 += (unsigned long long)__double2ll_rn(r * 72057594037927936.0);
+    }
+};
+
+__device__ __forceinline__ bool edges_cross(int2 a, int2 b, int2 c, int2 d)
+{
+    if (max(min(a.x, b.x), min(c.x, d.x)) > min(max(a.x, b.x), max(c.x, d.x)) ||
+        max(min(a.y, b.y), min(c.y, d.y)) > min(max(a.y, b.y), max(c.y, d.y)))
+        return false;
+    return side_of_shifted_point(c, d, a) != side_of_shifted_point(c, d, b) &&
+           side_of_point_to_shifted(a, b, c) != side_of_point_to_shifted(a, b, d);
+}
+
+// queue the lanes' hits (edge of A, edge of B); evaluate 32 at a time
+__device__ __forceinline__ void push_crossings(bool hit, int i, int j, uint2* cq, int& nq, const ListRing& A,
+                                               int sA, const ListRing& B, int sB, int2 org, ExactSum& sum,
+                                               int lane)
+{
+    const unsigned bal = __ballot_sync(0xffffffffu, hit);
+    if (!bal) return;
+    if (hit) cq[nq + __popc(bal & pmh_lanemask_lt())] = make_uint2((uint32_t)i, (uint32_t)j);
+    nq += __popc(bal);
+    __syncwarp();
+    if (nq >= 32) {
+        sum.add(crossing_terms(A.v, A.n, sA, B.v, B.n, sB, org, cq[lane]));
+        nq -= 32;
+        const uint2 rest = lane < nq ? cq[32 + lane] : make_uint2(0u, 0u);
+        __syncwarp();
+        if (lane < nq) cq[lane] = rest;
+        __syncwarp();
+    }
+}
+
+__global__ void __launch_bounds__(kBigThreads, 2)
+refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff,
+                  const int64_t* __restrict__ qarea2, const SlabPtrs* __restrict__ qslabs,
+                  const int2* __restrict__ pxy, const int64_t* __restrict__ poff,
+                  const int64_t* __restrict__ parea2, const SlabPtrs* __restrict__ pslabs,
+                  const int32_t* __restrict__ ids, int m, const int32_t* __restrict__ qid_list, int64_t e0,
+                  double* __restrict__ out, unsigned long long* __restrict__ ticket /* [1], [2] */,
+                  const int32_t* __restrict__ big)
+{
+    __shared__ BigSmem s;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const long long queued = (long long)ticket[1];
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) s.e = (long long)atomicAdd(ticket + 2, 1ull);
+        if (tid < 2) {
+            s.range[tid][0] = s.range[tid][2] = INT_MAX;
+            s.range[tid][1] = s.range[tid][3] = INT_MIN;
+        }
+        if (tid == 0) s.ends = s.q18 = s.r56 = 0;
+        __syncthreads();
+        if (s.e >= queued) break;
+        const int64_t e = e0 + big[s.e];
+        const int64_t q = qid_list ? (int64_t)qid_list[e] : e / m;
+        const int64_t p = ids[e];
+        const PairView va = view(qxy, qoff, qarea2, q), vb = view(pxy, poff, parea2, p);
+        if (va.sgn == 0 || vb.sgn == 0) {  // (uniform over the block)
+            if (tid == 0) out[e] = 0.0;
+            continue;
+        }
+        // both rings' ranges
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int2* v = r ? vb.v : va.v;
+            const int n = r ? vb.n : va.n;
+            int x0 = INT_MAX, x1 = INT_MIN, y0 = INT_MAX, y1 = INT_MIN;
+#pragma unroll 4
+            for (int i = tid; i < n; i += kBigThreads) {
+                const int2 u = v[i];
+                x0 = min(x0, u.x);
+                x1 = max(x1, u.x);
+                y0 = min(y0, u.y);
+                y1 = max(y1, u.y);
+            }
+            x0 = __reduce_min_sync(0xffffffffu, x0);
+            x1 = __reduce_max_sync(0xffffffffu, x1);
+            y0 = __reduce_min_sync(0xffffffffu, y0);
+            y1 = __reduce_max_sync(0xffffffffu, y1);
+            if (lane == 0) {
+                atomicMin(&s.range[r][0], x0);
+                atomicMax(&s.range[r][1], x1);
+                atomicMin(&s.range[r][2], y0);
+                atomicMax(&s.range[r][3], y1);
+            }
+        }
+        __syncthreads();
+        ListRing A{va.v, va.n, nullptr, nullptr, 0, 0, 0, s.range[0][0], s.range[0][1]};
+        ListRing B{vb.v, vb.n, nullptr, nullptr, 0, 0, 0, s.range[1][0], s.range[1][1]};
+        // lists: the set's slab index, else shared lists (warp r builds ring r's), else
+        // every edge
+        const SlabInfo sia = qslabs && qslabs->info ? qslabs->info[q] : SlabInfo{0, 0, 0, 1, 0};
+        const SlabInfo sib = pslabs && pslabs->info ? pslabs->info[p] : SlabInfo{0, 0, 0, 1, 0};
+        if (wid < 2 && (wid ? sib.S : sia.S) == 0) {
+            int sh = 0;
+            const bool ok = build_big_lists(wid ? B.v : A.v, wid ? B.n : A.n, s.range[wid][2], s.range[wid][3],
+                                            s.ids[wid], s.beg[wid], s.cnt[wid], sh, lane);
+            if (lane == 0) {
+                s.listed[wid] = ok;
+                s.sh[wid] = sh;
+            }
+        }
+        __syncthreads();
+        auto lists = [&](ListRing& R, const SlabInfo& si, const SlabPtrs* sl, int r) {
+            if (si.S > 0) {
+                R.sp = sl->ptr + si.slab_base;
+                R.se = sl->edges + si.edge_base;
+                R.S = si.S;
+                R.y0 = si.ymin;
+                R.magic = slab_div_magic(si.slab_h);
+            } else if (s.listed[r]) {
+                R.sp = s.beg[r];
+                R.se = s.ids[r];
+                R.S = kBigSlabs;
+                R.y0 = s.range[r][2];
+                R.magic = slab_div_magic(1 << s.sh[r]);
+            }
+        };
+        lists(A, sia, qslabs, 0);
+        lists(B, sib, pslabs, 1);
+        const int ya0 = s.range[0][2], ya1 = s.range[0][3], yb0 = s.range[1][2], yb1 = s.range[1][3];
+        const int2 org = B.v[0];
+        long long ends = 0;  // twice the end terms
+        ExactSum sum;
+        // end terms of A's edges: vertex a_i + e inside B closes edge i - 1
+        for (int i = tid; i < A.n; i += kBigThreads) {
+            const int2 a = A.v[i];
+            if (a.y < yb0 || a.y > yb1 || a.x < B.x0 || a.x > B.x1) continue;
+            int lo, hi;
+            B.row(a.y, lo, hi);
+            unsigned in = 0;
+#pragma unroll 2
+            for (int t = lo; t < hi; ++t) {
+                const int j = B.edge(t);
+                const int2 c = B.v[j], d = B.vert(j + 1);
+                if ((c.y > a.y) != (d.y > a.y)) {
+                    const long long cr = cross3(c, d, a);
+                    in ^= (cr != 0) & ((cr > 0) == (d.y > c.y));
+                }
+            }
+            if (in) {
+                const int2 u = A.v[i == 0 ? A.n - 1 : i - 1];
+                ends += va.sgn * (long long)(a.y - u.y) * (2 * (u.x - org.x) + (a.x - u.x));
+            }
+        }
+        // end terms of B's edges: vertex c_j - e inside A closes edge j - 1
+        for (int j = tid; j < B.n; j += kBigThreads) {
+            const int2 c = B.v[j];
+            if (c.y < ya0 || c.y > ya1 || c.x < A.x0 || c.x > A.x1) continue;
+            int lo, hi;
+            A.row(c.y - 1, lo, hi);
+            unsigned in = 0;
+#pragma unroll 2
+            for (int t = lo; t < hi; ++t) {
+                const int i = A.edge(t);
+                const int2 a = A.v[i], b = A.vert(i + 1);
+                if ((a.y >= c.y) != (b.y >= c.y)) {
+                    const long long cr = cross3(a, b, c);
+                    in ^= (cr == 0) | ((cr > 0) == (b.y > a.y));
+                }
+            }
+            if (in) {
+                const int2 u = B.v[j == 0 ? B.n - 1 : j - 1];
+                ends += vb.sgn * (long long)(c.y - u.y) * (2 * (u.x - org.x) + (c.x - u.x));
+            }
+        }
+        // crossings of A's edges with B's non-horizontal edges
+        int nq = 0;  // warp-uniform queue length
+        for (int i0 = 32 * wid; i0 < A.n; i0 += kBigThreads) {
+            const int i = i0 + lane;
+            int2 a = make_int2(0, 0), b = make_int2(0, 0);
+            int k0 = 0, cntk = 0, q0 = 0;
+            if (i < A.n) {
+                a = A.v[i];
+                b = A.vert(i + 1);
+                const int lo = max(min(a.y, b.y), yb0), hi = min(max(a.y, b.y), yb1);
+                if ((a.x != b.x || a.y != b.y) && hi >= lo && max(a.x, b.x) >= B.x0 && min(a.x, b.x) <= B.x1) {
+                    if (B.sp) {
+                        q0 = slab_div(lo - B.y0, B.magic);
+                        const int q1 = min(slab_div(hi - B.y0, B.magic), B.S - 1);
+                        if (q0 <= q1) {
+                            k0 = B.sp[q0];
+                            cntk = B.sp[q1 + 1] - k0;
+                        }
+                    } else {
+                        cntk = B.n;
+                    }
+                }
+            }
+            const int steps = __reduce_max_sync(0xffffffffu, cntk);
+            int qs = q0;  // slab of list position k0 + t
+            for (int t = 0; t < steps; ++t) {
+                bool hit = false;
+                int j = 0;
+                if (t < cntk) {
+                    const int k = k0 + t;
+                    j = B.edge(k);
+                    const int2 c = B.v[j], d = B.vert(j + 1);
+                    bool once = c.y != d.y;
+                    if (B.sp) {
+                        while (k >= B.sp[qs + 1]) ++qs;
+                        once = once && qs == max(q0, slab_div(min(c.y, d.y) - B.y0, B.magic));
+                    }
+                    hit = once && edges_cross(a, b, c, d);
+                }
+                push_crossings(hit, i, j, s.cq[wid], nq, A, va.sgn, B, vb.sgn, org, sum, lane);
+            }
+        }
+        // crossings of B's horizontal edges with A's edges
+        for (int j0 = 32 * wid; j0 < B.n; j0 += kBigThreads) {
+            const int j = j0 + lane;
+            int2 c = make_int2(0, 0), d = make_int2(0, 0);
+            int lo = 0, hi = 0;
+            if (j < B.n) {
+                c = B.v[j];
+                d = B.vert(j + 1);
+                if (c.y == d.y && c.x != d.x && c.y >= ya0 && c.y <= ya1) A.row(c.y - 1, lo, hi);
+            }
+            const int steps = __reduce_max_sync(0xffffffffu, hi - lo);
+            for (int t = 0; t < steps; ++t) {
+                bool hit = false;
+                int i = 0;
+                if (t < hi - lo) {
+                    i = A.edge(lo + t);
+                    const int2 a = A.v[i], b = A.vert(i + 1);
+                    hit = (a.x != b.x || a.y != b.y) && edges_cross(a, b, c, d);
+                }
+                push_crossings(hit, i, j, s.cq[wid], nq, A, va.sgn, B, vb.sgn, org, sum, lane);
+            }
+        }
+        if (lane < nq) sum.add(crossing_terms(A.v, A.n, va.sgn, B.v, B.n, vb.sgn, org, s.cq[wid][lane]));
+        unsigned long long en = (unsigned long long)ends;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            en += __shfl_xor_sync(0xffffffffu, en, o);
+            sum.q18 += __shfl_xor_sync(0xffffffffu, sum.q18, o);
+            sum.r56 += __shfl_xor_sync(0xffffffffu, sum.r56, o);
+        }
+        if (lane == 0) {
+            atomicAdd(&s.ends, en);
+            atomicAdd(&s.q18, sum.q18);
+            atomicAdd(&s.r56, sum.r56);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            const long long q18 = (long long)(s.q18 + (s.ends << 17));
+            const double inter = (double)q18 * (1.0 / 262144.0) + (double)(long long)s.r56 * (1.0 / 72057594037927936.0);
+            const double uni = va.area + vb.area - inter;
+            out[e] = uni > 0 ? fmin(fmax(inter / uni, 0.0), 1.0) : 0.0;
+        }
     }
 }
 
@@ -592,11 +967,19 @@ __global__ void topk_by_j_kernel(const int32_t* __restrict__ ids, const int32_t*
 
 }  // namespace
 
-// persistent grid (SM count x resident blocks) over the pairs
-static int launch_refine(pmh_ctx ctx, const int2* qxy, const int64_t* qoff, const int64_t* qarea2,
-                         const int4* qbox, pmh_polys db, const int32_t* ids, const int32_t* nlist, int m,
-                         const int32_t* qid_list, int64_t n_pairs, double* out,
-                         unsigned long long* ticket, const int64_t* d_n, cudaStream_t s)
+// pairs of one launch: the queue of large rings holds a launch's pairs
+constexpr int64_t kRefineSlice = 1 << 20;
+
+size_t pmh_refine_queue_bytes(int64_t n_pairs)
+{
+    return sizeof(int32_t) * (size_t)std::min(std::max<int64_t>(n_pairs, 1), kRefineSlice);
+}
+
+// persistent grids (SM count x resident blocks) over the pairs, kRefineSlice at a time; with
+// a queue, the pairs of large rings are left to refine_big_kernel
+static int launch_refine(pmh_ctx ctx, const RefineQueries& qs, pmh_polys db, const int32_t* ids,
+                         const int32_t* nlist, int m, const int32_t* qid_list, int64_t n_pairs, double* out,
+                         unsigned long long* tickets, int32_t* big, const int64_t* d_n, cudaStream_t s)
 {
     const size_t smem = sizeof(RefPair) * (kRefineWarps / 2);
     PMH_CUDA_TRY(cudaFuncSetAttribute(refine_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -604,34 +987,60 @@ static int launch_refine(pmh_ctx ctx, const int2* qxy, const int64_t* qoff, cons
     int per_sm = 0;
     PMH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, refine_pairs_kernel,
                                                                kRefineWarps * 32, smem));
-    const int blocks = (int)std::min<int64_t>((n_pairs + 1) / 2,
-                                              (int64_t)ctx->sm_count * std::max(per_sm, 1));
-    PMH_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned long long), s));
-    refine_pairs_kernel<<<blocks, kRefineWarps * 32, smem, s>>>(
-        qxy, qoff, qarea2, qbox, db->xy, db->offsets, db->area2, db->bbox, ids, nlist, m, qid_list,
-        n_pairs, out, ticket, d_n);
-    PMH_LAUNCHED("refine_pairs_kernel");
+    for (int64_t e0 = 0; e0 < n_pairs; e0 += kRefineSlice) {
+        const int64_t e1 = std::min(n_pairs, e0 + kRefineSlice);
+        const int blocks = (int)std::min<int64_t>((e1 - e0 + 1) / 2,
+                                                  (int64_t)ctx->sm_count * std::max(per_sm, 1));
+        PMH_CUDA_TRY(cudaMemsetAsync(tickets, 0, 3 * sizeof(unsigned long long), s));
+        refine_pairs_kernel<<<blocks, kRefineWarps * 32, smem, s>>>(
+            qs.xy, qs.off, qs.area2, qs.box, db->xy, db->offsets, db->area2, db->bbox, ids, nlist, m, qid_list,
+            e0, e1, out, tickets, big, d_n);
+        PMH_LAUNCHED("refine_pairs_kernel");
+        if (!big) continue;
+        const int bblocks = (int)std::min<int64_t>(e1 - e0, (int64_t)ctx->sm_count * 2);
+        refine_big_kernel<<<bblocks, kBigThreads, 0, s>>>(qs.xy, qs.off, qs.area2, qs.slabs, db->xy, db->offsets,
+                                                          db->area2, db->d_slabs, ids, m, qid_list, e0, out,
+                                                          tickets, big);
+        PMH_LAUNCHED("refine_big_kernel");
+    }
     return PMH_OK;
 }
 
-// context ticket slot of the refinement grid
-constexpr int kRefineTicket = 6;
+// first of the three context ticket slots of the refinement grids
+constexpr int kRefineTicket = 40;
 
-int pmh_launch_refine_topk(pmh_ctx ctx, const int2* qxy, const int64_t* qoff, const int64_t* qarea2,
-                           const int4* qbox, pmh_polys db, const int32_t* ids, const int32_t* nlist, int64_t Q,
-                           const int64_t* d_n, int32_t m, int32_t k, double* jv,
-                           unsigned long long* ticket, int32_t* top_ids, double* top_j,
-                           cudaStream_t s)
+int pmh_launch_refine_topk(pmh_ctx ctx, const RefineQueries& qs, pmh_polys db, const int32_t* ids,
+                           const int32_t* nlist, int64_t Q, const int64_t* d_n, int32_t m, int32_t k,
+                           double* jv, unsigned long long* tickets, int32_t* big, int32_t* top_ids,
+                           double* top_j, cudaStream_t s)
 {
     if (Q <= 0) return PMH_OK;
-    PMH_TRY(launch_refine(ctx, qxy, qoff, qarea2, qbox, db, ids, nlist, m, nullptr, Q * m, jv, ticket, d_n,
-                          s));
+    PMH_TRY(launch_refine(ctx, qs, db, ids, nlist, m, nullptr, Q * m, jv, tickets, big, d_n, s));
     int cap = 1;
     while (cap < m) cap <<= 1;
     const size_t smem = sizeof(JKey) * cap;
     topk_by_j_kernel<<<(unsigned)Q, 256, smem, s>>>(ids, nlist, jv, m, cap, k, top_ids, top_j, d_n);
     PMH_LAUNCHED("topk_by_j_kernel");
     return PMH_OK;
+}
+
+// scratch of a library call: `doubles` exact Jaccards, then the queue of large rings when
+// either set has one
+static int refine_scratch(pmh_ctx ctx, pmh_polys queries, pmh_polys db, int64_t doubles, int64_t n_pairs,
+                          double** jv, int32_t** big)
+{
+    const bool large = std::max(queries->max_n, db->max_n) > kRefineBigVerts;
+    void* buf = nullptr;
+    PMH_TRY(pmh_scratch(ctx, SCR_REFINE, sizeof(double) * (size_t)doubles +
+                                             (large ? pmh_refine_queue_bytes(n_pairs) : 0), &buf));
+    *jv = static_cast<double*>(buf);
+    *big = large ? reinterpret_cast<int32_t*>(*jv + doubles) : nullptr;
+    return PMH_OK;
+}
+
+static RefineQueries refine_queries(pmh_polys q)
+{
+    return RefineQueries{q->xy, q->offsets, q->area2, q->bbox, q->d_slabs};
 }
 
 extern "C" int pmh_refine_topk(pmh_ctx ctx, pmh_polys queries, pmh_polys db, const int32_t* d_ids,
@@ -644,10 +1053,10 @@ extern "C" int pmh_refine_topk(pmh_ctx ctx, pmh_polys queries, pmh_polys db, con
         return pmh_set_error(PMH_ERR_ARG, "bad arguments (1 <= k <= m <= 1024)");
     if (Q == 0) return PMH_OK;
     double* jv = nullptr;
-    PMH_TRY(pmh_scratch(ctx, SCR_REFINE, sizeof(double) * (size_t)(Q * m), (void**)&jv));
-    return pmh_launch_refine_topk(ctx, queries->xy, queries->offsets, queries->area2, queries->bbox, db,
-                                  d_ids, d_n, Q,
-                                  nullptr, m, k, jv, ctx->d_tickets + kRefineTicket, d_top_ids, d_top_j,
+    int32_t* big = nullptr;
+    PMH_TRY(refine_scratch(ctx, queries, db, Q * m, Q * m, &jv, &big));
+    return pmh_launch_refine_topk(ctx, refine_queries(queries), db, d_ids, d_n, Q, nullptr, m, k, jv,
+                                  ctx->d_tickets + kRefineTicket, big, d_top_ids, d_top_j,
                                   (cudaStream_t)stream);
 }
 
@@ -658,9 +1067,11 @@ extern "C" int pmh_pair_jaccard(pmh_ctx ctx, pmh_polys queries, pmh_polys db, co
     if (!queries || !db || n_pairs < 0 || (n_pairs > 0 && (!d_qid || !d_pid || !d_j)))
         return pmh_set_error(PMH_ERR_ARG, "bad arguments");
     if (n_pairs == 0) return PMH_OK;
-    return launch_refine(ctx, queries->xy, queries->offsets, queries->area2, queries->bbox, db, d_pid,
-                         nullptr, 1, d_qid, n_pairs, d_j, ctx->d_tickets + kRefineTicket, nullptr,
-                         (cudaStream_t)stream);
+    double* none = nullptr;
+    int32_t* big = nullptr;
+    PMH_TRY(refine_scratch(ctx, queries, db, 0, n_pairs, &none, &big));
+    return launch_refine(ctx, refine_queries(queries), db, d_pid, nullptr, 1, d_qid, n_pairs, d_j,
+                         ctx->d_tickets + kRefineTicket, big, nullptr, (cudaStream_t)stream);
 }
 
 // ---------------------------------------------------------------------------

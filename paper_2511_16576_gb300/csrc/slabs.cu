@@ -31,13 +31,6 @@ __device__ __forceinline__ int slab_count_for(int n, int height)
     return min(s, 1 << 16);
 }
 
-// floor(x / h) by a multiply: with m = floor(2^40 / h) + 1 (slab_div_magic), x * m / 2^40
-// exceeds x / h by less than x / 2^40 < 2^-18 for x < 2^22, which is below the gap 1/h
-// between x / h and the next integer for every h < 2^18 (slab heights here are at most
-// 2^21 / 64 for polygons above 256 vertices, or 1), so the floor is exact
-__device__ __forceinline__ uint64_t slab_div_magic(int h) { return (1ull << 40) / (uint64_t)h + 1ull; }
-__device__ __forceinline__ int slab_div(int x, uint64_t m) { return (int)(((uint64_t)x * m) >> 40); }
-
 // y of the two end points of edges e0 + 32u + lane (u < 4) of the ring of n vertices at
 // xy + b, four loads in flight per lane: an edge's end vertex is the next lane's start
 // vertex (a shuffle); lane 31 and the closing edge read theirs
@@ -277,10 +270,24 @@ __global__ void class_key_kernel(const int4* __restrict__ bbox, const int64_t* _
 
 }  // namespace
 
+static int build_slab_lists(pmh_polys P, cudaStream_t s);
+
 int pmh_build_slabs(pmh_polys P, cudaStream_t s)
 {
-    pmh_ctx ctx = P->ctx;
     if (P->n == 0) return PMH_OK;
+    PMH_TRY(build_slab_lists(P, s));
+    if (!P->d_slabs && cudaMalloc(&P->d_slabs, sizeof(SlabPtrs)) != cudaSuccess) {
+        cudaGetLastError();
+        return pmh_set_error(PMH_ERR_NOMEM, "slab pointer allocation failed");
+    }
+    const SlabPtrs v{P->slab_info, P->slab_ptr, P->slab_edges};
+    PMH_CUDA_TRY(cudaMemcpyAsync(P->d_slabs, &v, sizeof(v), cudaMemcpyHostToDevice, s));
+    return PMH_OK;
+}
+
+static int build_slab_lists(pmh_polys P, cudaStream_t s)
+{
+    pmh_ctx ctx = P->ctx;
     const int64_t n = P->n;
     if (cudaMalloc(&P->slab_info, sizeof(SlabInfo) * n) != cudaSuccess) {
         cudaGetLastError();
