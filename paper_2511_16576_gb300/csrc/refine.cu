@@ -1077,33 +1077,79 @@ extern "C" int pmh_pair_jaccard(pmh_ctx ctx, pmh_polys queries, pmh_polys db, co
 // ---------------------------------------------------------------------------
 // Brute-force candidate set of the exact search (the paper's BF baseline,
 // Sec. 5.2): every database polygon whose bounding box overlaps the query's
-// with positive area -- the only ones with J > 0.  One warp per query scans
-// the database 32 polygons at a time; ballots keep ids ascending.
+// with positive area -- the only ones with J > 0.  The database is cut into
+// segments; a warp takes kBoxQueries queries over one segment, 64 boxes at a
+// time, one read of a box serving all of its queries; ballots keep ids
+// ascending.  The counting pass leaves every (query, segment)'s hits in seg;
+// the filling pass starts behind the sum of the segments before.  (A warp per
+// query over the whole set left a batch of 96 queries to 96 warps: 1.27 ms a
+// pass over 100,000 boxes, bound by the latency of one load at a time;
+// 22 us now.)
 // ---------------------------------------------------------------------------
 namespace {
 
+constexpr int kBoxQueries = 4;
+constexpr int kBoxWarps = 8;
+
 template <bool kWrite>
-__global__ void bbox_join_kernel(const int4* __restrict__ qbox, int64_t Q, const int4* __restrict__ pbox,
-                                 int64_t N, int64_t* __restrict__ counts,
-                                 const int64_t* __restrict__ row_ptr, int32_t* __restrict__ cand)
+__global__ void __launch_bounds__(kBoxWarps * 32)
+bbox_join_kernel(const int4* __restrict__ qbox, int64_t Q, const int4* __restrict__ pbox, int64_t N, int segs,
+                 int32_t* __restrict__ seg, int64_t* __restrict__ counts,
+                 const int64_t* __restrict__ row_ptr, int32_t* __restrict__ cand)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (q >= Q) return;
-    const int4 a = qbox[q];
-    int64_t cnt = 0, out = kWrite ? row_ptr[q] : 0;
-    for (int64_t base = 0; base < N; base += 32) {
-        const int64_t p = base + lane;
-        bool hit = false;
-        if (p < N) {
-            const int4 b = pbox[p];
-            hit = a.x < b.z && b.x < a.z && a.y < b.w && b.y < a.w;
+    const int64_t groups = (Q + kBoxQueries - 1) / kBoxQueries;
+    const int64_t nwarps = (int64_t)gridDim.x * kBoxWarps;
+    for (int64_t w = (int64_t)blockIdx.x * kBoxWarps + (threadIdx.x >> 5); w < groups * segs; w += nwarps) {
+        const int64_t g = w / segs;
+        const int i = (int)(w - g * segs);
+        const int64_t q0 = g * kBoxQueries;
+        const int nq = (int)min((int64_t)kBoxQueries, Q - q0);
+        int4 a[kBoxQueries];
+        int64_t out[kBoxQueries];
+        int cnt[kBoxQueries];
+#pragma unroll
+        for (int t = 0; t < kBoxQueries; ++t) {
+            a[t] = t < nq ? qbox[q0 + t] : make_int4(0, 0, 0, 0);
+            out[t] = cnt[t] = 0;
+            if (kWrite && t < nq) {
+                int64_t before = 0;
+                for (int u = lane; u < i; u += 32) before += seg[(q0 + t) * segs + u];
+                for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+                out[t] = row_ptr[q0 + t] + before;
+            }
         }
-        const unsigned m = __ballot_sync(0xffffffffu, hit);
-        if (kWrite && hit) cand[out + cnt + __popc(m & pmh_lanemask_lt())] = (int32_t)p;
-        cnt += __popc(m);
+        const int64_t b = N * i / segs, e = N * (i + 1) / segs;
+        for (int64_t x0 = b; x0 < e; x0 += 64) {
+            int4 box[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int64_t x = x0 + 32 * u + lane;
+                // (an empty box at the far corner overlaps nothing)
+                box[u] = x < e ? pbox[x] : make_int4(INT_MAX, INT_MAX, INT_MIN, INT_MIN);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int4 p = box[u];
+#pragma unroll
+                for (int t = 0; t < kBoxQueries; ++t) {
+                    const bool hit = t < nq && a[t].x < p.z && p.x < a[t].z && a[t].y < p.w && p.y < a[t].w;
+                    const unsigned m = __ballot_sync(0xffffffffu, hit);
+                    if (kWrite && hit)
+                        cand[out[t] + cnt[t] + __popc(m & pmh_lanemask_lt())] = (int32_t)(x0 + 32 * u + lane);
+                    cnt[t] += __popc(m);
+                }
+            }
+        }
+        if (!kWrite && lane == 0) {
+#pragma unroll
+            for (int t = 0; t < kBoxQueries; ++t)
+                if (t < nq) {
+                    seg[(q0 + t) * segs + i] = cnt[t];
+                    atomicAdd(reinterpret_cast<unsigned long long*>(&counts[q0 + t]), (unsigned long long)cnt[t]);
+                }
+        }
     }
-    if (!kWrite && lane == 0) counts[q] = cnt;
 }
 
 }  // namespace
@@ -1121,11 +1167,18 @@ extern "C" int pmh_bbox_join(pmh_ctx ctx, pmh_polys queries, pmh_polys db, int64
         PMH_CUDA_TRY(cudaMemsetAsync(d_row_ptr, 0, sizeof(int64_t), s));
         return PMH_OK;
     }
+    // segments of the database: enough (query group, segment) items for the device, at least
+    // 64 boxes and at most 1,024 segments each
+    const int64_t groups = (Q + kBoxQueries - 1) / kBoxQueries;
+    const int64_t full = (int64_t)ctx->sm_count * 8, want = (full * kBoxWarps + groups - 1) / groups;
+    const int segs = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(want, 1024), db->n / 64));
     int64_t* counts = nullptr;
-    PMH_TRY(pmh_scratch(ctx, SCR_QUERY, sizeof(int64_t) * (size_t)Q, (void**)&counts));
-    const unsigned blocks = (unsigned)((Q + 7) / 8);
-    bbox_join_kernel<false><<<blocks, 256, 0, s>>>(queries->bbox, Q, db->bbox, db->n, counts, nullptr,
-                                                   nullptr);
+    PMH_TRY(pmh_scratch(ctx, SCR_QUERY, (sizeof(int64_t) + sizeof(int32_t) * segs) * (size_t)Q, (void**)&counts));
+    int32_t* seg = reinterpret_cast<int32_t*>(counts + Q);
+    const unsigned blocks = (unsigned)std::min<int64_t>((groups * segs + kBoxWarps - 1) / kBoxWarps, full);
+    PMH_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(int64_t) * (size_t)Q, s));
+    bbox_join_kernel<false><<<blocks, kBoxWarps * 32, 0, s>>>(queries->bbox, Q, db->bbox, db->n, segs, seg,
+                                                              counts, nullptr, nullptr);
     PMH_LAUNCHED("bbox_join_kernel<count>");
     PMH_TRY(pmh_exclusive_scan_i64(ctx, counts, d_row_ptr, Q, s));
     PMH_CUDA_TRY(cudaMemcpyAsync(ctx->h_pinned, d_row_ptr + Q, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -1137,8 +1190,8 @@ extern "C" int pmh_bbox_join(pmh_ctx ctx, pmh_polys queries, pmh_polys db, int64
                              (long long)cand_capacity);
     if (total == 0) return PMH_OK;
     if (!d_cand) return pmh_set_error(PMH_ERR_ARG, "null candidate buffer");
-    bbox_join_kernel<true><<<blocks, 256, 0, s>>>(queries->bbox, Q, db->bbox, db->n, nullptr, d_row_ptr,
-                                                  d_cand);
+    bbox_join_kernel<true><<<blocks, kBoxWarps * 32, 0, s>>>(queries->bbox, Q, db->bbox, db->n, segs, seg,
+                                                             nullptr, d_row_ptr, d_cand);
     PMH_LAUNCHED("bbox_join_kernel<fill>");
     return PMH_OK;
 }

@@ -95,3 +95,29 @@ def test_one_hashmap_in_the_query_graph(B, ctx):
         assert cap < total or torch.equal(g.cand, cand)
         g.close()
     index.close()
+
+
+@pytest.mark.parametrize("n,Q", [(1, 1), (63, 5), (64, 4), (129, 1), (4097, 9), (70_001, 3), (5000, 400)])
+def test_bbox_join_segments(B, ctx, n, Q):
+    """Box overlaps with positive area, ids ascending, for sets and batches around the edges of a
+    segment (64 boxes), a query group (4) and a warp; empty boxes (beyond the domain) overlap nothing."""
+    rng = np.random.default_rng(n + Q)
+
+    def rects(k):
+        c = rng.integers(-2000, 66_000, size=(k, 2))
+        s = rng.integers(1, 6000, size=(k, 2))
+        c[::50] += 100_000
+        x0, y0, x1, y1 = c[:, 0], c[:, 1], c[:, 0] + s[:, 0], c[:, 1] + s[:, 1]
+        xy = np.stack([x0, y0, x1, y0, x1, y1, x0, y1], 1).reshape(-1, 2).astype(np.int32)
+        box = np.clip(np.stack([x0, y0, x1, y1], 1), 0, 65536)
+        return B.poly_upload(ctx, torch.from_numpy(xy).to(DEV),
+                             torch.arange(0, 4 * k + 1, 4, dtype=torch.int64, device=DEV)), box
+    qp, qb = rects(Q)
+    dbp, pb = rects(n)
+    row_ptr, cand = B.bbox_join(ctx, qp, dbp)
+    rp, cd = row_ptr.cpu().numpy(), cand.cpu().numpy()
+    for q in range(Q):
+        a = qb[q]
+        exp = np.nonzero((a[0] < pb[:, 2]) & (pb[:, 0] < a[2]) & (a[1] < pb[:, 3]) & (pb[:, 1] < a[3]) &
+                         (pb[:, 0] < pb[:, 2]) & (pb[:, 1] < pb[:, 3]))[0]
+        assert np.array_equal(cd[rp[q]:rp[q + 1]], exp)
