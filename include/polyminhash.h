@@ -233,10 +233,11 @@ int pmh_index_destroy(pmh_index index);
  *   h_total   (host) receives the number of candidates over all queries.
  * Synchronises `stream` once (to learn the total).  With cand_capacity <
  * total, d_cand is left unwritten, d_row_ptr is still written, and the call
- * returns PMH_ERR_CAPACITY: call again with a larger buffer.  From 16 bands the
- * counting pass keeps its sorted rows in context scratch (8 bytes per query and
- * up to 4,096 ids per query, at most 64M ids) and the filling pass copies them;
- * rows past that pool are joined again.  Errors also: PMH_ERR_NOMEM (scratch). */
+ * returns PMH_ERR_CAPACITY: call again with a larger buffer.  With two bands or
+ * more and a capacity, the counting pass keeps its sorted rows in context scratch (8
+ * bytes per query and up to 4,096 ids per query, at most 64M ids) and the filling pass
+ * copies them; rows past that pool (all of them without a capacity or without room
+ * for it) are joined again.  Errors also: PMH_ERR_NOMEM (scratch). */
 int pmh_lsh_query(pmh_ctx ctx, pmh_index index, const uint32_t* d_qhashes, int64_t Q,
                   int64_t* d_row_ptr, int32_t* d_cand, int64_t cand_capacity, int64_t* h_total,
                   void* stream);

@@ -168,8 +168,7 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
               cudaMalloc(&g->slab_cursor, sizeof(int32_t) * g->cap_ptr) == cudaSuccess &&
               cudaMalloc(&g->slab_edges, sizeof(int32_t) * g->cap_edges) == cudaSuccess &&
               cudaMalloc(&g->counts, sizeof(int64_t) * Q) == cudaSuccess &&
-              ((index->params.bands < 16 && index->params.bands != 1) ||
-               cudaMalloc(&g->join_stage, pmh_join_stage_bytes(index, Q, g->cap)) == cudaSuccess) &&
+              cudaMalloc(&g->join_stage, pmh_join_stage_bytes(index, Q, g->cap)) == cudaSuccess &&
               cudaMalloc(&g->row_ptr, sizeof(int64_t) * (Q + 1)) == cudaSuccess &&
               cudaMalloc(&g->cand, sizeof(int32_t) * cand_capacity) == cudaSuccess &&
               cudaMalloc(&g->count16, sizeof(uint16_t) * cand_capacity) == cudaSuccess &&

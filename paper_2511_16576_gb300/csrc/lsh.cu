@@ -7,12 +7,15 @@
 // (j in the top band_bits bits, the top bits of the 64-bit band key below),
 // stable-radix-sorted so that equal composites keep ascending ids.  A
 // directory over the composites' top bits (about eight entries per slot)
-// bounds each lookup to one short range.  A query
-// binary-searches its composite there per band and walks the equal range, keeping
-// the entries whose r-tuple equals its own (exact bucket membership; an entry of
-// another key shares the composite with probability ~n / 2^(32 - band_bits) per
-// lookup and costs one tuple read).  The per-band id lists are ascending, so a
-// warp merges them (min over lanes) into the sorted, duplicate-free candidate row.
+// bounds each lookup to one short range.  A query looks its composite up there per
+// band and walks the equal range, keeping the entries whose r-tuple equals its own
+// (exact bucket membership; an entry of another key shares the composite with
+// probability ~n / 2^(32 - band_bits) per lookup and costs one tuple read).  The
+// sorted, duplicate-free candidate row is made of the bands' matches by one of five
+// joins, chosen by the bands, the tuple length, the set and the batch
+// (pmh_launch_query): the bucket's range itself (one band), a warp's sorted list
+// (sparse rows), a bitmap of the set in shared memory, an open-addressing set in shared
+// memory (sets above the bitmap's), or a warp's merge of the ascending lists.
 #include <algorithm>
 
 #include "pmh_internal.cuh"
@@ -140,7 +143,8 @@ __device__ __forceinline__ void advance(BandCursor& c, const uint32_t* __restric
     }
 }
 
-// One warp per query.  The count pass writes the row length (0 for rows past the
+// Warp merge (fewer than 16 bands, sets above the bitmap's): one warp per query, each
+// lane walking its bands' ascending lists.  The count pass writes the row length (0 for rows past the
 // device-side batch size d_n or after a failed validation, flag bits 0-2); the
 // fill pass writes the row, unless the total exceeds the capacity (then it
 // raises flag bit 3).
@@ -331,7 +335,7 @@ __device__ int join_walk(const uint32_t* __restrict__ qh, int K, int bands, int 
     constexpr int kJoinTable = S::kTable, kJoinMaxUnique = S::kMaxUnique;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     volatile int* nu_v = n_unique;
-    const bool vec = (K & 3) == 0;
+    const bool vec = (K & 3) == 0 && (reinterpret_cast<uintptr_t>(qh) & 15) == 0;
     __syncthreads();
     for (int i = threadIdx.x; i < kJoinTable; i += blockDim.x) table[i] = kNone;
     if (threadIdx.x == 0) *n_unique = 0;
@@ -462,7 +466,7 @@ join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int bands, i
             const int32_t* __restrict__ ids, const uint32_t* __restrict__ dbh,
             const int64_t* __restrict__ dir, int dsh, int64_t m, int64_t n_db, int64_t* __restrict__ counts,
             const int64_t* __restrict__ row_ptr, int32_t* __restrict__ cand, int64_t cap,
-            JoinStage st, const int64_t* __restrict__ d_n, int* __restrict__ d_flags)
+            JoinStage st, bool deferred, const int64_t* __restrict__ d_n, int* __restrict__ d_flags)
 {
     using S = JoinShape<kBig>;
     constexpr int kJoinMaxUnique = S::kMaxUnique;
@@ -496,10 +500,11 @@ join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int bands, i
             if (threadIdx.x == 0 && d_flags) atomicOr(d_flags, 8);
             return;
         }
-        // rows by size: the small set counts every row and fills the short ones; the
+        // rows by size: the small set counts every row (every row that the warp join left it,
+        // after one: `deferred`, those of count -1) and fills the short ones; the
         // large set counts the rows that overflowed the small one and fills the long ones;
         // staged rows are copied instead
-        if (!kWrite && kBig && counts[q] >= 0) continue;
+        if (!kWrite && (kBig || deferred) && counts[q] >= 0) continue;
         if (kWrite && ((row_ptr[q + 1] - row_ptr[q] > kSmallRowMax) != kBig)) continue;
         int passes = 1;
         if (kWrite && st.where) {
@@ -605,6 +610,334 @@ copy_rows_kernel(JoinStage st, int64_t Q, const int64_t* __restrict__ row_ptr, i
                 if (k < len) dst[k] = v[u];
             }
         }
+    }
+}
+
+// Warp join (two bands or more, before one of the block joins): a warp per query takes the
+// sparse rows, of at most kWarpList entries in all of their bands' equal ranges: the
+// matches are listed, sorted and freed of duplicates in the warp's shared slice -- a
+// block with its set or bitmap to clear, read and synchronise over costs several times
+// that for a handful of candidates.  All entries are read at once (four per lane).  A row
+// of more entries is left to the block join: count -1 in the counting pass and where -1
+// in both.
+constexpr int kWarpJoinWarps = 8;
+constexpr int kWarpU = 4;
+constexpr int kWarpList = 32 * kWarpU;
+
+struct WarpJoin {
+    int64_t lo[kMaxBandsPerLane * 32];
+    int off[kMaxBandsPerLane * 32 + 1];
+    int32_t list[kWarpList];
+};
+
+template <bool kWrite>
+__global__ void __launch_bounds__(kWarpJoinWarps * 32)
+warp_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int bands, int rows, uint32_t T,
+                 uint64_t lsh_seed, int band_bits, const uint32_t* __restrict__ comp,
+                 const int32_t* __restrict__ ids, const uint32_t* __restrict__ dbh,
+                 const int64_t* __restrict__ dir, int dsh, int64_t* __restrict__ counts,
+                 const int64_t* __restrict__ row_ptr, int32_t* __restrict__ cand, int64_t cap, JoinStage st,
+                 const int64_t* __restrict__ d_n, int* __restrict__ d_flags)
+{
+    __shared__ WarpJoin smem[kWarpJoinWarps];
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    WarpJoin& m = smem[threadIdx.x >> 5];
+    const int64_t q = (int64_t)blockIdx.x * kWarpJoinWarps + (threadIdx.x >> 5);
+    if (q >= Q) return;
+    if ((d_n && q >= *d_n) || (d_flags && (*d_flags & 7))) {
+        if (lane == 0) {
+            if (!kWrite) counts[q] = 0;
+            if (st.where) st.where[q] = kWrite ? 0 : -1;
+        }
+        return;
+    }
+    if (kWrite && row_ptr[Q] > cap) {
+        if (lane == 0 && d_flags) atomicOr(d_flags, 8);
+        return;
+    }
+    // (16-byte tuple loads: the index's rows are aligned when K % 4 == 0, the caller's may not be)
+    const bool vec = (K & 3) == 0 && (reinterpret_cast<uintptr_t>(qhashes) & 15) == 0;
+    const uint32_t* qh = qhashes + q * K;
+    int entries = 0;
+    for (int j0 = 0; j0 < bands; j0 += 32) {
+        const int j = j0 + lane;
+        int64_t lo = 0, n = 0;
+        if (j < bands) {
+            const uint64_t key = band_key(qh, j, rows, T, lsh_seed);
+            if (key != PMH_INVALID_KEY) {
+                const uint32_t c = composite(key, j, band_bits);
+                lo = comp_lower_bound(comp, dir, dsh, c);
+                n = comp_lower_bound(comp, dir, dsh, c + 1) - lo;  // (c is never all ones)
+            }
+        }
+        int x = (int)min(n, (int64_t)(kWarpList + 1));
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(full, x, o);
+            if (lane >= o) x += y;
+        }
+        if (j < bands) {
+            m.lo[j] = lo;
+            m.off[j + 1] = entries + x;
+        }
+        entries += __shfl_sync(full, x, 31);
+    }
+    if (lane == 0) m.off[0] = 0;
+    __syncwarp();
+    if (entries > kWarpList) {
+        if (lane == 0) {
+            if (!kWrite) counts[q] = -1;
+            if (st.where) st.where[q] = -1;
+        }
+        return;
+    }
+    int jj[kWarpU];
+    int32_t pp[kWarpU];
+    bool in[kWarpU];
+#pragma unroll
+    for (int u = 0; u < kWarpU; ++u) {
+        const int g = 32 * u + lane;
+        in[u] = g < entries;
+        int lo = 0, hi = bands;  // the band holding entry g: the last j with off[j] <= g
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (m.off[mid] <= g) lo = mid;
+            else hi = mid;
+        }
+        jj[u] = lo;
+        pp[u] = in[u] ? ids[m.lo[lo] + (g - m.off[lo])] : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < kWarpU; ++u)
+        if (in[u]) in[u] = tuple_match2(qh, dbh + (int64_t)pp[u] * K, jj[u], rows, vec);
+    int nm = 0;  // matches listed
+#pragma unroll
+    for (int u = 0; u < kWarpU; ++u) {
+        const unsigned bal = __ballot_sync(full, in[u]);
+        if (in[u]) m.list[nm + __popc(bal & pmh_lanemask_lt())] = pp[u];
+        nm += __popc(bal);
+    }
+    int n2 = 1;
+    while (n2 < nm) n2 <<= 1;
+    for (int i = nm + lane; i < n2; i += 32) m.list[i] = kNone;
+    __syncwarp();
+    for (int k = 2; k <= n2; k <<= 1)
+        for (int d = k >> 1; d > 0; d >>= 1) {
+            for (int i = lane; i < n2 / 2; i += 32) {
+                const int l = 2 * d * (i / d) + i % d, r = l + d;  // the pair of step d
+                const int32_t a = m.list[l], b = m.list[r];
+                if ((a > b) == ((l & k) == 0)) {
+                    m.list[l] = b;
+                    m.list[r] = a;
+                }
+            }
+            __syncwarp();
+        }
+    int nu = 0;
+    for (int i0 = 0; i0 < nm; i0 += 32) {
+        const int i = i0 + lane;
+        nu += __popc(__ballot_sync(full, i < nm && (i == 0 || m.list[i] != m.list[i - 1])));
+    }
+    int32_t* out = kWrite ? cand + row_ptr[q] : nullptr;
+    if (kWrite) {
+        if (lane == 0) st.where[q] = 0;
+    } else {
+        long long off = -1;
+        if (lane == 0) {
+            if (st.pool) {
+                const unsigned long long o = atomicAdd(st.cursor, (unsigned long long)nu);
+                if ((long long)(o + (unsigned long long)nu) <= st.pool_ints) off = (long long)o;
+            }
+            counts[q] = nu;
+            if (st.where) st.where[q] = off;
+        }
+        off = __shfl_sync(full, off, 0);
+        if (off >= 0) out = st.pool + off;
+    }
+    if (!out) return;
+    int pos = 0;
+    for (int i0 = 0; i0 < nm; i0 += 32) {
+        const int i = i0 + lane;
+        const bool keep = i < nm && (i == 0 || m.list[i] != m.list[i - 1]);
+        const unsigned bal = __ballot_sync(full, keep);
+        if (keep) out[pos + __popc(bal & pmh_lanemask_lt())] = m.list[i];
+        pos += __popc(bal);
+    }
+}
+
+// Bitmap join (two bands or more, sets of at most kBitmapMaxIds): one block per query.
+// The set of a row's candidates is a bit per database polygon in shared memory, so that
+// inserting is one atomicOr, duplicates (a candidate found in several bands) vanish, and
+// the row in ascending order of ids is the bitmap read from front to back: no probing,
+// no sort.  The bands' entries are the directory slots of their composites (two adjacent
+// directory reads per band; the few entries of other composites in a slot are dropped
+// by the composite read beside the id, instead of a bisection of dependent reads),
+// concatenated and split evenly over the warps, four entries per lane in flight.
+// Clearing and reading the bitmap costs n / 128 shared vectors per row, about what
+// sorting a row of a few hundred costs; the block grows with the bitmap (256 threads
+// while four blocks fit an SM) so that its time per row stays the same.  Bound by the
+// latency of hashes -> directory -> entries -> tuples, and by the tuples' sectors.
+// 4,096 queries of 64 x 2 bands against 300,000 polygons (880 candidates a query): 0.51 ms
+// a pass, 1.12 with the open-addressing set.
+//
+// Which sets: with tuples of one or two hashes (rows of hundreds to thousands) up to
+// 2^20 ids, where one bitmap still fits an SM (4,096 queries of 64 x 2 bands, 520,000
+// and 1,040,000 polygons: 0.73 and 1.37 ms a call against 1.87 and 3.24 with the set);
+// with longer tuples up to 409,600, where four do: the rows that reach the block are
+// then fewer than the blocks an SM needs to hide their latency (16 x 8 bands: 69 against
+// 88 us at 260,000 polygons, 116 against 88 at 520,000).
+constexpr int64_t kBitmapMaxIds = 409600;
+constexpr int64_t kBitmapMaxIdsShort = 1 << 20;
+constexpr int kBitmapU = 4;
+
+template <bool kWrite>
+__global__ void __launch_bounds__(1024)
+bitmap_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int bands, int rows, uint32_t T,
+                   uint64_t lsh_seed, int band_bits, const uint32_t* __restrict__ comp,
+                   const int32_t* __restrict__ ids, const uint32_t* __restrict__ dbh,
+                   const int64_t* __restrict__ dir, int dsh, int words4 /* 128-id vectors */,
+                   int64_t* __restrict__ counts, const int64_t* __restrict__ row_ptr,
+                   int32_t* __restrict__ cand, int64_t cap, JoinStage st, bool deferred,
+                   const int64_t* __restrict__ d_n, int* __restrict__ d_flags)
+{
+    extern __shared__ uint4 bits[];
+    __shared__ JoinBands jb;
+    __shared__ uint32_t bcomp[kMaxBandsPerLane * 32];
+    __shared__ int wsum[32];
+    __shared__ long long stage_off;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const bool failed = d_flags && (*d_flags & 7);
+    if (kWrite && failed) return;
+    if (kWrite && row_ptr[Q] > cap) {
+        if (blockIdx.x == 0 && threadIdx.x == 0 && d_flags) atomicOr(d_flags, 8);
+        return;
+    }
+    // (16-byte tuple loads: the index's rows are aligned when K % 4 == 0, the caller's may not be)
+    const bool vec = (K & 3) == 0 && (reinterpret_cast<uintptr_t>(qhashes) & 15) == 0;
+    uint32_t* word = reinterpret_cast<uint32_t*>(bits);
+    for (int64_t q = blockIdx.x; q < Q; q += gridDim.x) {
+        if (failed || (d_n && q >= *d_n)) {
+            if (!kWrite && threadIdx.x == 0) {
+                counts[q] = 0;
+                if (st.where) st.where[q] = -1;
+            }
+            continue;
+        }
+        if (kWrite && st.where && st.where[q] >= 0) continue;  // staged, or the warp join's
+        if (!kWrite && deferred && counts[q] >= 0) continue;   // the warp join's
+        const uint32_t* qh = qhashes + q * K;
+        // the bands' directory slots, the bitmap cleared meanwhile
+        for (int j = threadIdx.x; j < bands; j += blockDim.x) {
+            const uint64_t key = band_key(qh, j, rows, T, lsh_seed);
+            int64_t lo = 0, n = 0;
+            uint32_t c = 0;
+            if (key != PMH_INVALID_KEY) {
+                c = composite(key, j, band_bits);
+                lo = dir[c >> dsh];
+                n = dir[(c >> dsh) + 1] - lo;
+            }
+            bcomp[j] = c;
+            jb.lo[j] = lo;
+            jb.off[j + 1] = n;
+        }
+        for (int i = threadIdx.x; i < words4; i += blockDim.x) bits[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        if (wid == 0) {  // prefix of the bands' entry counts
+            int64_t carry = 0;
+            for (int j0 = 0; j0 < bands; j0 += 32) {
+                const int j = j0 + lane;
+                int64_t x = j < bands ? jb.off[j + 1] : 0;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+                    if (lane >= o) x += y;
+                }
+                if (j < bands) jb.off[j + 1] = carry + x;
+                carry += __shfl_sync(0xffffffffu, x, 31);
+            }
+            if (lane == 0) jb.off[0] = 0;
+        }
+        __syncthreads();
+        const int64_t total = jb.off[bands];
+        for (int64_t g0 = (int64_t)wid * (32 * kBitmapU); g0 < total; g0 += (int64_t)nw * (32 * kBitmapU)) {
+            int jj[kBitmapU];
+            int32_t pp[kBitmapU];
+            bool in[kBitmapU];
+#pragma unroll
+            for (int u = 0; u < kBitmapU; ++u) {
+                const int64_t g = g0 + 32 * u + lane;
+                in[u] = g < total;
+                int lo = 0, hi = bands;  // the band holding entry g: the last j with off[j] <= g
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (jb.off[mid] <= g) lo = mid;
+                    else hi = mid;
+                }
+                jj[u] = lo;
+                pp[u] = 0;
+                if (in[u]) {
+                    const int64_t x = jb.lo[lo] + (g - jb.off[lo]);
+                    pp[u] = ids[x];
+                    in[u] = comp[x] == bcomp[lo];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kBitmapU; ++u)
+                if (in[u] && tuple_match2(qh, dbh + (int64_t)pp[u] * K, jj[u], rows, vec))
+                    atomicOr(&word[pp[u] >> 5], 1u << (pp[u] & 31));
+        }
+        __syncthreads();
+        // the row's length: every warp counts a stretch of the bitmap
+        const int per = (words4 + nw - 1) / nw, w0 = min(words4, wid * per), w1 = min(words4, w0 + per);
+        int mine = 0;
+        for (int i = w0 + lane; i < w1; i += 32) {
+            const uint4 v = bits[i];
+            mine += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+        }
+        mine = __reduce_add_sync(0xffffffffu, mine);
+        if (lane == 0) wsum[wid] = mine;
+        __syncthreads();
+        const int ws = lane < nw ? wsum[lane] : 0;
+        const int nu = __reduce_add_sync(0xffffffffu, ws);
+        int32_t* out = kWrite ? cand + row_ptr[q] : nullptr;
+        if (!kWrite) {
+            if (threadIdx.x == 0) {
+                long long off = -1;
+                if (st.pool) {
+                    const unsigned long long o = atomicAdd(st.cursor, (unsigned long long)nu);
+                    if ((long long)(o + (unsigned long long)nu) <= st.pool_ints) off = (long long)o;
+                }
+                stage_off = off;
+                counts[q] = nu;
+                if (st.where) st.where[q] = off;
+            }
+            if (st.pool) {
+                __syncthreads();
+                if (stage_off >= 0) out = st.pool + stage_off;
+            }
+        }
+        if (out) {  // the ids in order: each lane writes the ids of one vector
+            int pos = __reduce_add_sync(0xffffffffu, lane < wid ? ws : 0);
+            for (int i0 = w0; i0 < w1; i0 += 32) {
+                const int i = i0 + lane;
+                const uint4 v = i < w1 ? bits[i] : make_uint4(0u, 0u, 0u, 0u);
+                const int c = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+                if (!__any_sync(0xffffffffu, c)) continue;
+                int x = c;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, x, o);
+                    if (lane >= o) x += y;
+                }
+                int32_t* dst = out + pos + (x - c);
+                const uint32_t part[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    for (uint32_t b = part[k]; b; b &= b - 1) *dst++ = i * 128 + k * 32 + __ffs(b) - 1;
+                pos += __shfl_sync(0xffffffffu, x, 31);
+            }
+        }
+        __syncthreads();  // the bitmap is free for the next row
     }
 }
 
@@ -819,7 +1152,7 @@ extern "C" int pmh_index_destroy(pmh_index X)
 template <bool kBig>
 static int launch_join(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* d_n,
                        int64_t* counts, const int64_t* row_ptr, int32_t* cand, int64_t cap,
-                       const JoinStage& st, int* d_flags, bool write, cudaStream_t s)
+                       const JoinStage& st, bool deferred, int* d_flags, bool write, cudaStream_t s)
 {
     using S = JoinShape<kBig>;
     const pmh_params& P = X->params;
@@ -834,7 +1167,7 @@ static int launch_join(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t
                                             P.lsh_seed, X->band_bits, X->sorted_comp, X->sorted_id,
                                             X->hashes, X->dir, X->dir_shift, m, X->n,
                                             write ? nullptr : counts, write ? row_ptr : nullptr,
-                                            write ? cand : nullptr, write ? cap : 0, st, d_n, d_flags);
+                                            write ? cand : nullptr, write ? cap : 0, st, deferred, d_n, d_flags);
     PMH_LAUNCHED(write ? (kBig ? "join_kernel<fill,large>" : "join_kernel<fill,small>")
                        : (kBig ? "join_kernel<count,large>" : "join_kernel<count,small>"));
     return PMH_OK;
@@ -880,9 +1213,30 @@ static JoinStage stage_view(void* buf, int64_t Q, int64_t pool_ints)
     char* c = static_cast<char*>(buf);
     st.cursor = reinterpret_cast<unsigned long long*>(c);
     st.where = reinterpret_cast<int64_t*>(c + 16);
-    st.pool = reinterpret_cast<int32_t*>(c + 16 + sizeof(int64_t) * (size_t)Q);
+    if (pool_ints > 0) st.pool = reinterpret_cast<int32_t*>(c + 16 + sizeof(int64_t) * (size_t)Q);
     st.pool_ints = pool_ints;
     return st;
+}
+
+// the bitmap join's pass: 256 threads while four bitmaps fit an SM, more as they grow
+static int launch_bitmap(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* d_n, int64_t* counts,
+                         const int64_t* row_ptr, int32_t* cand, int64_t cap, const JoinStage& st,
+                         bool deferred, int* d_flags, bool write, cudaStream_t s)
+{
+    const pmh_params& P = X->params;
+    const int words4 = (int)((X->n + 127) / 128);
+    const size_t smem = sizeof(uint4) * (size_t)std::max(words4, 1);
+    const int threads = smem <= 50 * 1024 ? 256 : smem <= 104 * 1024 ? 512 : 1024;
+    auto fn = write ? bitmap_join_kernel<true> : bitmap_join_kernel<false>;
+    PMH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 1;
+    PMH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem));
+    const unsigned blocks = (unsigned)std::min<int64_t>(Q, (int64_t)X->ctx->sm_count * std::max(per_sm, 1));
+    fn<<<blocks, threads, smem, s>>>(qh, Q, (int)P.K, (int)P.bands, (int)P.rows, P.T, P.lsh_seed, X->band_bits,
+                                     X->sorted_comp, X->sorted_id, X->hashes, X->dir, X->dir_shift, words4,
+                                     counts, row_ptr, cand, cap, st, deferred, d_n, d_flags);
+    PMH_LAUNCHED(write ? "bitmap_join_kernel<fill>" : "bitmap_join_kernel<count>");
+    return PMH_OK;
 }
 
 int pmh_launch_query(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* d_n,
@@ -891,47 +1245,56 @@ int pmh_launch_query(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* 
 {
     if (Q <= 0) return PMH_OK;
     const pmh_params& P = X->params;
-    const int64_t m = X->n * P.bands;
     if (P.bands == 1) {  // one hashmap: the bucket's range, no merge
         int32_t* seg = static_cast<int32_t*>(stage);
         if (!write) PMH_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(int64_t) * (size_t)Q, s));
         return launch_range(X, qh, Q, d_n, seg, counts, row_ptr, cand, cap, d_flags, write, s);
     }
-    // sixteen bands or more: block per query, parallel bucket walks and a shared-memory
-    // set (rows of thousands of candidates occur on dense sets; the warp merge below
-    // would walk them one candidate at a time)
-    if (P.bands >= 16) {
-        const JoinStage st = stage_view(stage, Q, pool_ints);
-        if (write) {
-            if (st.where) {  // the staged rows: a copy into place
-                const unsigned cblocks = (unsigned)std::min<int64_t>(Q, (int64_t)X->ctx->sm_count * 8);
-                copy_rows_kernel<<<cblocks, 256, 0, s>>>(st, Q, row_ptr, cand, cap, d_n, d_flags);
-                PMH_LAUNCHED("copy_rows_kernel");
-            }
-        } else if (st.cursor) {  // the pool cursor and the large set's row ticket
-            PMH_CUDA_TRY(cudaMemsetAsync(st.cursor, 0, 2 * sizeof(unsigned long long), s));
-        }
-        PMH_TRY(launch_join<false>(X, qh, Q, d_n, counts, row_ptr, cand, cap, st, d_flags, write, s));
-        return launch_join<true>(X, qh, Q, d_n, counts, row_ptr, cand, cap, st, d_flags, write, s);
+    const bool bitmap = X->n <= (P.rows <= 2 ? kBitmapMaxIdsShort : kBitmapMaxIds);
+    if (!bitmap && P.bands < 16) {
+        // a large set under few bands: rows are mostly empty or short, and the warp merge's one
+        // launch a pass beats the sets' two (8 x 16 bands of 520,000: 73 against 110 us)
+        const int wpb = 8;
+        auto fn = write ? query_kernel<true> : query_kernel<false>;
+        fn<<<(unsigned)((Q + wpb - 1) / wpb), wpb * 32, 0, s>>>(
+            qh, Q, (int)P.K, (int)P.bands, (int)P.rows, P.T, P.lsh_seed, X->band_bits, X->sorted_comp,
+            X->sorted_id, X->hashes, X->dir, X->dir_shift, X->n * P.bands, counts, row_ptr, cand, cap, d_n,
+            d_flags);
+        PMH_LAUNCHED(write ? "query_kernel<fill>" : "query_kernel<count>");
+        return PMH_OK;
     }
-    const int wpb = 8;
-    unsigned blocks = (unsigned)((Q + wpb - 1) / wpb);
+    const JoinStage st = stage_view(stage, Q, pool_ints);
+    // the warp join first where rows are mostly short (tuples of more than four hashes) and the
+    // batch is large enough for its throughput to outweigh a launch (4,096 queries of 16 x 8
+    // bands, 260,000 polygons: 64-77 against 86-91 us a call; 64 queries: 59 against 49); the
+    // fill pass runs it only without a staging pool, and needs `where` to mark its rows
+    const bool staged = st.where && st.pool;
+    const bool warp = P.rows > 4 && Q >= 1024 && (write ? st.where && !staged : true);
     if (write) {
-        query_kernel<true><<<blocks, wpb * 32, 0, s>>>(
-            qh, Q, (int)P.K, (int)P.bands, (int)P.rows, P.T, P.lsh_seed, X->band_bits,
-            X->sorted_comp, X->sorted_id, X->hashes, X->dir, X->dir_shift, m, nullptr,
-                row_ptr, cand, cap, d_n,
-            d_flags);
-        PMH_LAUNCHED("query_kernel<fill>");
-    } else {
-        query_kernel<false><<<blocks, wpb * 32, 0, s>>>(
-            qh, Q, (int)P.K, (int)P.bands, (int)P.rows, P.T, P.lsh_seed, X->band_bits,
-            X->sorted_comp, X->sorted_id, X->hashes, X->dir, X->dir_shift, m, counts,
-                nullptr, nullptr, 0, d_n,
-            d_flags);
-        PMH_LAUNCHED("query_kernel<count>");
+        if (staged) {  // the staged rows: a copy into place
+            const unsigned cblocks = (unsigned)std::min<int64_t>(Q, (int64_t)X->ctx->sm_count * 8);
+            copy_rows_kernel<<<cblocks, 256, 0, s>>>(st, Q, row_ptr, cand, cap, d_n, d_flags);
+            PMH_LAUNCHED("copy_rows_kernel");
+        }
+    } else if (st.cursor) {  // the pool cursor and the large set's row ticket
+        PMH_CUDA_TRY(cudaMemsetAsync(st.cursor, 0, 2 * sizeof(unsigned long long), s));
     }
-    return PMH_OK;
+    if (warp) {
+        auto fn = write ? warp_join_kernel<true> : warp_join_kernel<false>;
+        fn<<<(unsigned)((Q + kWarpJoinWarps - 1) / kWarpJoinWarps), kWarpJoinWarps * 32, 0, s>>>(
+            qh, Q, (int)P.K, (int)P.bands, (int)P.rows, P.T, P.lsh_seed, X->band_bits, X->sorted_comp,
+            X->sorted_id, X->hashes, X->dir, X->dir_shift, counts, row_ptr, cand, cap, st, d_n, d_flags);
+        PMH_LAUNCHED(write ? "warp_join_kernel<fill>" : "warp_join_kernel<count>");
+    }
+    // (without a pool and without the warp join's marks every row is the block join's)
+    const JoinStage sb = write && !staged && !warp ? JoinStage{} : st;
+    if (bitmap) {
+        // (a pool of the whole capacity holds every row of a total that may be written)
+        if (write && staged && pool_ints >= cap) return PMH_OK;
+        return launch_bitmap(X, qh, Q, d_n, counts, row_ptr, cand, cap, sb, warp, d_flags, write, s);
+    }
+    PMH_TRY(launch_join<false>(X, qh, Q, d_n, counts, row_ptr, cand, cap, sb, warp, d_flags, write, s));
+    return launch_join<true>(X, qh, Q, d_n, counts, row_ptr, cand, cap, sb, warp, d_flags, write, s);
 }
 
 extern "C" int pmh_lsh_query(pmh_ctx ctx, pmh_index X, const uint32_t* d_qhashes, int64_t Q,
@@ -950,12 +1313,19 @@ extern "C" int pmh_lsh_query(pmh_ctx ctx, pmh_index X, const uint32_t* d_qhashes
     int64_t* counts = nullptr;
     PMH_TRY(pmh_scratch(ctx, SCR_QUERY, sizeof(int64_t) * (size_t)Q, (void**)&counts));
     // the count pass stages its sorted rows in a pool of up to 4,096 ids per query
-    // (at most 64M ids); rows past the pool are joined again by the fill pass
+    // (at most 64M ids); rows past the pool are joined again by the fill pass.  A call
+    // that cannot fill (no capacity) stages nothing
     void* stage = nullptr;
     int64_t pool_ints = 0;
-    if (X->params.bands >= 16 || X->params.bands == 1) {
+    if (X->params.bands == 1) {
+        PMH_TRY(pmh_scratch(ctx, SCR_JOIN, pmh_join_stage_bytes(X, Q, 0), &stage));
+    } else if (cand_capacity > 0) {
         pool_ints = std::min<int64_t>(Q * 4096, 64ll << 20);
-        PMH_TRY(pmh_scratch(ctx, SCR_JOIN, pmh_join_stage_bytes(X, Q, pool_ints), &stage));
+        // (without room for a pool the fill pass joins every row again)
+        if (pmh_scratch(ctx, SCR_JOIN, pmh_join_stage_bytes(X, Q, pool_ints), &stage) != PMH_OK) {
+            stage = nullptr;
+            pool_ints = 0;
+        }
     }
     PMH_TRY(pmh_launch_query(X, d_qhashes, Q, nullptr, counts, nullptr, nullptr, 0, stage, pool_ints,
                              nullptr, false, s));
@@ -988,6 +1358,8 @@ extern "C" int pmh_lsh_query_fill(pmh_ctx ctx, pmh_index X, const uint32_t* d_qh
         PMH_TRY(pmh_scratch(ctx, SCR_JOIN, pmh_join_stage_bytes(X, Q, 0), &stage));
         PMH_TRY(launch_range(X, d_qhashes, Q, nullptr, static_cast<int32_t*>(stage), nullptr, nullptr, nullptr,
                              0, nullptr, false, s));
+    } else if (pmh_scratch(ctx, SCR_JOIN, pmh_join_stage_bytes(X, Q, 0), &stage) != PMH_OK) {
+        stage = nullptr;  // no marks for the warp join: the block joins take every row
     }
     return pmh_launch_query(X, d_qhashes, Q, nullptr, nullptr, d_row_ptr, d_cand, cand_capacity,
                             stage, 0, nullptr, true, s);

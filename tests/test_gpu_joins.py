@@ -121,3 +121,64 @@ def test_bbox_join_segments(B, ctx, n, Q):
         exp = np.nonzero((a[0] < pb[:, 2]) & (pb[:, 0] < a[2]) & (a[1] < pb[:, 3]) & (pb[:, 1] < a[3]) &
                          (pb[:, 0] < pb[:, 2]) & (pb[:, 1] < pb[:, 3]))[0]
         assert np.array_equal(cd[rp[q]:rp[q + 1]], exp)
+
+
+@pytest.mark.parametrize("K,bands,values,n,Q", [
+    (4, 2, 2, 1, 1),            # one polygon: a single bit
+    (4, 4, 3, 127, 9),          # around one 128-id vector, 16-byte rows
+    (8, 2, 2, 128, 3),
+    (6, 3, 2, 129, 700),        # more rows than resident blocks
+    (16, 2, 1, 300, 5),         # 8-hash tuples
+    (36, 2, 1, 200, 4),         # tuples longer than the register form
+    (32, 32, 40, 70_001, 20),   # one-hash bands: long rows with many duplicates
+    (128, 64, 60, 5000, 33),
+    (128, 128, 400, 30_000, 7), # every band slot in use
+    (32, 8, 3, 403_000, 6),     # the last size of 256 threads, and the next two block sizes
+    (32, 8, 3, 409_700, 6),
+    (32, 8, 3, 852_100, 6),
+    (16, 4, 5, 1 << 20, 5),     # the largest bitmap
+    (16, 4, 5, (1 << 20) + 1, 5),    # the shared-memory set, few bands
+    (16, 16, 90, (1 << 20) + 7, 5),  # its rows beyond 16,384 candidates (id-range passes)
+])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_banded_join(B, ctx, orc, K, bands, values, n, Q, shift):
+    rng = np.random.default_rng(K * 1000 + n)
+    ph, qh = hashes(rng, n, K, values), hashes(rng, Q, K, values)
+    qh[0] = T
+    qh[-1] = ph[n // 2]
+    if Q > 2:
+        ph[n // 3:n // 3 + min(n, 50)] = qh[1]
+    rp = check(B, ctx, orc, ph, qh, bands, shift)
+    assert rp[-1] > 0
+
+
+@pytest.mark.parametrize("n,values", [(30_000, 3), (30_000, 9), (409_601, 3), (409_601, 9)])
+def test_warp_join_and_what_it_leaves(B, ctx, orc, n, values):
+    """Batches large enough for the warp join (1,024 queries, tuples of six): rows of no, a few, 128,
+    129 and thousands of entries, the longer ones left to the bitmap or to the shared-memory set."""
+    rng = np.random.default_rng(n + values)
+    K, bands, Q = 96, 16, 1100
+    ph, qh = hashes(rng, n, K, values), hashes(rng, Q, K, 1000)
+    qh[:500:2] = ph[rng.integers(0, n, 250)]
+    for q, copies in ((1, 8), (3, 9), (5, 300)):  # 128, 144 and 4,800 entries of one row
+        qh[q] = 10_000 + q
+        ph[rng.choice(n, copies, replace=False)] = qh[q]
+    P = B.make_params(K, bands)
+    index = B.lsh_build(ctx, on_device(ph), P)
+    pick = np.concatenate([np.arange(8), rng.choice(Q, 24, replace=False)])
+    rp_ref, cand_ref = orc.candidates(np.ascontiguousarray(qh[pick]), ph, bands, K // bands, T)
+    full = None
+    for capacity in (None, 1 << 22):
+        row_ptr, cand = B.lsh_query(ctx, index, on_device(qh), capacity=capacity)
+        rp, cd = row_ptr.cpu().numpy(), cand.cpu().numpy()
+        for i, q in enumerate(pick):
+            assert np.array_equal(cd[rp[q]:rp[q + 1]], cand_ref[rp_ref[i]:rp_ref[i + 1]]), q
+        assert full is None or (np.array_equal(rp, full[0]) and np.array_equal(cd, full[1]))
+        full = (rp, cd)
+    # the fill alone, from the counted rows
+    cand = torch.empty(len(full[1]), dtype=torch.int32, device=DEV)
+    q = on_device(qh)
+    B._check(B.load().pmh_lsh_query_fill(ctx.handle, index.handle, q.data_ptr(), Q, row_ptr.data_ptr(),
+                                         cand.data_ptr(), cand.numel(), None))
+    assert np.array_equal(cand.cpu().numpy(), full[1])
+    index.close()
