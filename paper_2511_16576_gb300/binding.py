@@ -403,9 +403,19 @@ def lsh_query(ctx: Context, index: Index, qhashes: torch.Tensor, capacity: int |
     dev = qhashes.device
     row_ptr = torch.empty(Q + 1, dtype=torch.int64, device=dev)
     total = _i64()
-    cap = 0 if capacity is None else capacity
-    cand = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
     lib = load()
+    if capacity is not None:
+        cap = capacity
+        cand = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
+    else:
+        # room for rows of 1,024 on average (8 to 128 MB): most batches are then joined once and
+        # their rows copied into place, instead of counted and joined again
+        cap = min(max(Q * 1024, 1 << 21), 1 << 25)
+        try:
+            cand = torch.empty(cap, dtype=torch.int32, device=dev)
+        except torch.cuda.OutOfMemoryError:
+            cap = 0
+            cand = torch.empty(1, dtype=torch.int32, device=dev)
     rc = lib.pmh_lsh_query(ctx.handle, index.handle, _ptr(qhashes), Q, _ptr(row_ptr), _ptr(cand),
                            cap, ctypes.byref(total), _stream(stream))
     if rc == PMH_ERR_CAPACITY and capacity is None:
@@ -414,6 +424,16 @@ def lsh_query(ctx: Context, index: Index, qhashes: torch.Tensor, capacity: int |
         rc = lib.pmh_lsh_query_fill(ctx.handle, index.handle, _ptr(qhashes), Q, _ptr(row_ptr),
                                     _ptr(cand), total.value, _stream(stream))
     _check(rc)
+    if capacity is None and total.value < cap // 2 and (stream is None or isinstance(stream, torch.cuda.Stream)):
+        # do not hold the whole buffer for a short result
+        short = torch.empty(max(total.value, 1), dtype=torch.int32, device=dev)
+        if stream is None:
+            short.copy_(cand[:short.numel()])
+        else:
+            with torch.cuda.stream(stream):
+                short.copy_(cand[:short.numel()])
+            cand.record_stream(stream)
+        cand = short
     return row_ptr, cand[:total.value]
 
 

@@ -56,6 +56,7 @@ def check(B, ctx, orc, ph, qh, bands, shift=0):
 @pytest.mark.parametrize("K,values,n,Q", [
     (1, 3, 5000, 3),       # a third of the set per bucket, 512 segments a query
     (1, 1, 129, 2),        # every polygon in one bucket: 128 + 1 entries, one segment's tail
+    (1, 1, 30_000, 100),   # more candidates than a call without a capacity makes room for
     (2, 4, 4097, 100),
     (3, 3, 20000, 37),
     (4, 2, 3000, 5000),    # 16-byte tuples, two segments per query
@@ -128,6 +129,7 @@ def test_bbox_join_segments(B, ctx, n, Q):
     (4, 4, 3, 127, 9),          # around one 128-id vector, 16-byte rows
     (8, 2, 2, 128, 3),
     (6, 3, 2, 129, 700),        # more rows than resident blocks
+    (8, 4, 1, 30_000, 100),     # more candidates than a call without a capacity makes room for
     (16, 2, 1, 300, 5),         # 8-hash tuples
     (36, 2, 1, 200, 4),         # tuples longer than the register form
     (32, 32, 40, 70_001, 20),   # one-hash bands: long rows with many duplicates
