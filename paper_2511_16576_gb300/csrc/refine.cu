@@ -194,213 +194,6 @@ __device__ double warp_intersection_area(const int2* __restrict__ A, int na, int
     return acc;
 }
 
-// y-slab lists of a ring v[0..n) (staged in shared memory or read from global
-// memory; edge e = v[e] -> v[e+1 mod n]): edge e is listed in every slab of
-// [y0 + s*2^sh, y0 + (s+1)*2^sh) that its closed y-range meets, 128 slabs (four
-// per lane).  Returns false (warp-uniform) if more than kRefSlabCap references
-// would be needed.
-constexpr int kRefSlabs = 128;
-constexpr int kSlabsPerLane = kRefSlabs / 32;
-constexpr int kRefSlabCap = 2048;
-struct RefSlabs {
-    uint16_t ids[kRefSlabCap];
-    uint16_t beg[kRefSlabs + 2];
-    int cnt[kRefSlabs];
-    int y0, sh;
-    int x0, x1;  // the ring's x-range
-};
-
-__device__ __forceinline__ bool build_ref_slabs(const int2* v, int n, RefSlabs& L, int lane)
-{
-    int y0 = INT_MAX, y1 = INT_MIN, x0 = INT_MAX, x1 = INT_MIN;
-    for (int e = lane; e < n; e += 32) {
-        const int2 u = v[e];
-        y0 = min(y0, u.y);
-        y1 = max(y1, u.y);
-        x0 = min(x0, u.x);
-        x1 = max(x1, u.x);
-    }
-    y0 = __reduce_min_sync(0xffffffffu, y0);
-    y1 = __reduce_max_sync(0xffffffffu, y1);
-    x0 = __reduce_min_sync(0xffffffffu, x0);
-    x1 = __reduce_max_sync(0xffffffffu, x1);
-    int sh = 0;
-    while (((y1 - y0) >> sh) >= kRefSlabs) ++sh;
-#pragma unroll
-    for (int u = 0; u < kSlabsPerLane; ++u) L.cnt[kSlabsPerLane * lane + u] = 0;
-    __syncwarp();
-    for (int e = lane; e < n; e += 32) {
-        const int2 a = v[e], b = v[e + 1 == n ? 0 : e + 1];
-        const int s0 = (min(a.y, b.y) - y0) >> sh, s1 = (max(a.y, b.y) - y0) >> sh;
-        for (int q = s0; q <= s1; ++q) atomicAdd(&L.cnt[q], 1);
-    }
-    __syncwarp();
-    int c[kSlabsPerLane], mine = 0;
-#pragma unroll
-    for (int u = 0; u < kSlabsPerLane; ++u) {
-        c[u] = L.cnt[kSlabsPerLane * lane + u];
-        mine += c[u];
-    }
-    int incl = mine;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += t;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    if (total > kRefSlabCap) return false;
-    const int excl = incl - mine;
-    {
-        int run = excl;
-#pragma unroll
-        for (int u = 0; u < kSlabsPerLane; ++u) {
-            L.beg[kSlabsPerLane * lane + u] = (uint16_t)run;
-            run += c[u];
-        }
-    }
-    if (lane == 31) L.beg[kRefSlabs] = (uint16_t)total;
-    if (lane == 0) {
-        L.y0 = y0;
-        L.sh = sh;
-        L.x0 = x0;
-        L.x1 = x1;
-    }
-    __syncwarp();
-    {
-        int run = excl;
-#pragma unroll
-        for (int u = 0; u < kSlabsPerLane; ++u) {
-            L.cnt[kSlabsPerLane * lane + u] = run;
-            run += c[u];
-        }
-    }
-    __syncwarp();
-    for (int e = lane; e < n; e += 32) {
-        const int2 a = v[e], b = v[e + 1 == n ? 0 : e + 1];
-        const int s0 = (min(a.y, b.y) - y0) >> sh, s1 = (max(a.y, b.y) - y0) >> sh;
-        for (int q = s0; q <= s1; ++q) L.ids[atomicAdd(&L.cnt[q], 1)] = (uint16_t)e;
-    }
-    __syncwarp();
-    return true;
-}
-
-// area(A n B) as warp_intersection_area, for staged rings with slab lists: a
-// vertex test reads only the other ring's slab of the vertex's y, and an A edge
-// meets only the B edges listed in the slabs its y-range spans (each pair once:
-// in the first of those slabs that also lists the B edge).
-__device__ double warp_intersection_area_slabs(const int2* __restrict__ A, int na, int sA,
-                                               const RefSlabs& LA, const int2* __restrict__ B, int nb,
-                                               int sB, const RefSlabs& LB, uint2* cq, int lane, int wip)
-{
-    const int2 org = B[0];
-    const unsigned full = 0xffffffffu;
-    double acc = 0;
-    const int ya0 = LA.y0, ya1 = LA.y0 + (kRefSlabs << LA.sh) - 1;
-    const int yb0 = LB.y0, yb1 = LB.y0 + (kRefSlabs << LB.sh) - 1;
-    // end terms of A's edges: vertex a_i + e inside B closes edge i-1 (a vertex strictly
-    // left or right of B's x-range sees an even number of B's crossings: outside)
-    for (int i = wip == 0 ? lane : na; i < na; i += 32) {
-        const int2 a = A[i];
-        unsigned in = 0;
-        if (a.y >= yb0 && a.y <= yb1 && a.x >= LB.x0 && a.x <= LB.x1) {
-            const int q = (a.y - yb0) >> LB.sh;
-            for (int k = LB.beg[q]; k < LB.beg[q + 1]; ++k) {
-                const int j = LB.ids[k];
-                const int2 c = B[j], d = B[j + 1 == nb ? 0 : j + 1];
-                if ((c.y > a.y) != (d.y > a.y)) {
-                    const long long cr = cross3(c, d, a);
-                    in ^= (cr != 0) & ((cr > 0) == (d.y > c.y));
-                }
-            }
-        }
-        if (in) {
-            const int2 p = A[i == 0 ? na - 1 : i - 1];
-            const double x0 = (double)(p.x - org.x), dx = (double)(a.x - p.x), dy = (double)(a.y - p.y);
-            acc += (sA > 0 ? 1.0 : -1.0) * dy * (x0 + 0.5 * dx);
-        }
-    }
-    // end terms of B's edges: vertex c_j - e inside A closes edge j-1
-    for (int j = wip == 1 ? lane : nb; j < nb; j += 32) {
-        const int2 c = B[j];
-        unsigned in = 0;
-        if (c.y >= ya0 && c.y <= ya1 && c.x >= LA.x0 && c.x <= LA.x1) {
-            const int q = (c.y - ya0) >> LA.sh;
-            for (int k = LA.beg[q]; k < LA.beg[q + 1]; ++k) {
-                const int i = LA.ids[k];
-                const int2 a = A[i], b = A[i + 1 == na ? 0 : i + 1];
-                if ((a.y >= c.y) != (b.y >= c.y)) {
-                    const long long cr = cross3(a, b, c);
-                    in ^= (cr == 0) | ((cr > 0) == (b.y > a.y));
-                }
-            }
-        }
-        if (in) {
-            const int2 p = B[j == 0 ? nb - 1 : j - 1];
-            const double x0 = (double)(p.x - org.x), ex = (double)(c.x - p.x), ey = (double)(c.y - p.y);
-            acc += (sB > 0 ? 1.0 : -1.0) * ey * (x0 + 0.5 * ex);
-        }
-    }
-    // crossings, queued and evaluated 32 at a time as in warp_intersection_area
-    int nq = 0;
-    for (int i0 = 32 * wip; i0 < na; i0 += 64) {
-        const int i = i0 + lane;
-        int2 a = make_int2(0, 0), b = make_int2(0, 0);
-        int k0 = 0, cntk = 0, q0 = 0;
-        if (i < na) {
-            a = A[i];
-            b = A[i + 1 == na ? 0 : i + 1];
-            const int lo = min(a.y, b.y), hi = max(a.y, b.y);
-            // (an edge outside B's x-range meets no B edge)
-            if ((a.x != b.x || a.y != b.y) && hi >= yb0 && lo <= yb1 && max(a.x, b.x) >= LB.x0 &&
-                min(a.x, b.x) <= LB.x1) {
-                q0 = (max(lo, yb0) - yb0) >> LB.sh;
-                const int q1 = (min(hi, yb1) - yb0) >> LB.sh;
-                k0 = LB.beg[q0];
-                cntk = LB.beg[q1 + 1] - k0;
-            }
-        }
-        const int ax0 = min(a.x, b.x), ax1 = max(a.x, b.x), ay0 = min(a.y, b.y), ay1 = max(a.y, b.y);
-        const int steps = __reduce_max_sync(full, cntk);
-        int q = q0;  // slab of list position k0 + t
-        for (int t = 0; t < steps; ++t) {
-            bool hit = false;
-            int j = 0;
-            if (t < cntk) {
-                const int k = k0 + t;
-                while (k >= LB.beg[q + 1]) ++q;
-                j = LB.ids[k];
-                const int2 c = B[j], d = B[j + 1 == nb ? 0 : j + 1];
-                // this pair is visited once: in the first listed slab of both
-                const int first = max(q0, (min(c.y, d.y) - yb0) >> LB.sh);
-                if (q == first &&
-                    !(max(ax0, min(c.x, d.x)) > min(ax1, max(c.x, d.x)) ||
-                      max(ay0, min(c.y, d.y)) > min(ay1, max(c.y, d.y)) || (c.x == d.x && c.y == d.y))) {
-                    hit = side_of_shifted_point(c, d, a) != side_of_shifted_point(c, d, b) &&
-                          side_of_point_to_shifted(a, b, c) != side_of_point_to_shifted(a, b, d);
-                }
-            }
-            const unsigned bal = __ballot_sync(full, hit);
-            if (bal) {
-                if (hit) cq[nq + __popc(bal & pmh_lanemask_lt())] = make_uint2((uint32_t)i, (uint32_t)j);
-                nq += __popc(bal);
-                __syncwarp();
-                if (nq >= 32) {
-                    acc += crossing_terms(A, na, sA, B, nb, sB, org, cq[lane]);
-                    nq -= 32;
-                    const uint2 rest = lane < nq ? cq[32 + lane] : make_uint2(0u, 0u);
-                    __syncwarp();
-                    if (lane < nq) cq[lane] = rest;
-                    __syncwarp();
-                }
-            }
-        }
-    }
-    if (lane < nq) acc += crossing_terms(A, na, sA, B, nb, sB, org, cq[lane]);
-    __syncwarp();
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(full, acc, o);
-    return acc;
-}
-
 struct PairView {
     const int2* v;
     int n;
@@ -421,18 +214,34 @@ __device__ __forceinline__ PairView view(const int2* xy, const int64_t* off, con
     return r;
 }
 
+// y-slabs of the two-warp form: B's edges that meet the two rings' common box, listed in
+// every slab of 2^sh rows that their closed y-range meets (kRefSlabs slabs over the common
+// rows, four per lane; taller slabs until the references fit kRefSlabCap)
+constexpr int kRefSlabs = 128;
+constexpr int kSlabsPerLane = kRefSlabs / 32;
+constexpr int kRefSlabCap = 2048;
+static_assert(kRefineBigVerts <= kRefSlabCap && kRefineBigVerts <= 32 * 32, "one slab holds every edge");
+
 constexpr int kRefineWarps = 4;  // two pairs per block, two warps per pair
 constexpr int kWarpVerts = 960;   // vertices of a pair's staging slice
 
-// one pair's shared slice: the staged rings, a crossing queue per warp, both rings'
-// slab lists, and the two warps' partial sums
+// one pair's shared slice: the staged rings, a crossing queue per warp, B's slab lists,
+// each ring's crossing parities by edge, and the two warps' partial sums
 struct RefPair {
     int2 sv[kWarpVerts];
-    uint2 cq[2][64];
-    RefSlabs sl[2];
+    union {
+        uint2 cq[2][64];
+        int cnt[kRefSlabs];  // list cursors, before the queues are in use
+    };
+    uint16_t ids[kRefSlabCap];
+    uint16_t beg[kRefSlabs + 2];
+    uint32_t par_a[32], par_b[32];  // bit i % 32 of word i / 32: edge i is crossed an odd number of times
+    int range[2][4];                // min x, max x, min y, max y of A and of B
     double part[2];
+    long long ends[2];
     long long e;
-    int ok[2];
+    int sh;
+    int in0[2];  // first vertex of A inside B, of B inside A
 };
 
 // the named barrier of pair slot g (0 or 1) of the block (barrier 0 is __syncthreads;
@@ -453,44 +262,255 @@ __device__ __forceinline__ void stage_ring(int2* dst, const int2* __restrict__ s
     }
 }
 
+// B's slab lists over the common box (rows [ry0, ry1], columns [rx0, rx1]), by one warp
+__device__ __forceinline__ void build_pair_slabs(const int2* v, int n, int rx0, int rx1, int ry0, int ry1,
+                                                 RefPair& P, int lane)
+{
+    int sh = 0;
+    while (((ry1 - ry0) >> sh) >= kRefSlabs) ++sh;
+    for (;; ++sh) {
+#pragma unroll
+        for (int u = 0; u < kSlabsPerLane; ++u) P.cnt[kSlabsPerLane * lane + u] = 0;
+        __syncwarp();
+        for (int e = lane; e < n; e += 32) {
+            const int2 a = v[e], b = v[e + 1 == n ? 0 : e + 1];
+            const int lo = max(min(a.y, b.y), ry0), hi = min(max(a.y, b.y), ry1);
+            if (lo > hi || max(a.x, b.x) < rx0 || min(a.x, b.x) > rx1) continue;
+            const int s0 = (lo - ry0) >> sh, s1 = (hi - ry0) >> sh;
+            for (int q = s0; q <= s1; ++q) atomicAdd(&P.cnt[q], 1);
+        }
+        __syncwarp();
+        int c[kSlabsPerLane], mine = 0;
+#pragma unroll
+        for (int u = 0; u < kSlabsPerLane; ++u) {
+            c[u] = P.cnt[kSlabsPerLane * lane + u];
+            mine += c[u];
+        }
+        int incl = mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += t;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        if (total > kRefSlabCap) {  // (one slab holds at most n <= kRefineBigVerts)
+            __syncwarp();
+            continue;
+        }
+        int run = incl - mine;
+#pragma unroll
+        for (int u = 0; u < kSlabsPerLane; ++u) {
+            P.beg[kSlabsPerLane * lane + u] = (uint16_t)run;
+            P.cnt[kSlabsPerLane * lane + u] = run;
+            run += c[u];
+        }
+        if (lane == 31) P.beg[kRefSlabs] = (uint16_t)total;
+        if (lane == 0) P.sh = sh;
+        __syncwarp();
+        break;
+    }
+    for (int e = lane; e < n; e += 32) {
+        const int2 a = v[e], b = v[e + 1 == n ? 0 : e + 1];
+        const int lo = max(min(a.y, b.y), ry0), hi = min(max(a.y, b.y), ry1);
+        if (lo > hi || max(a.x, b.x) < rx0 || min(a.x, b.x) > rx1) continue;
+        const int s0 = (lo - ry0) >> sh, s1 = (hi - ry0) >> sh;
+        for (int q = s0; q <= s1; ++q) P.ids[atomicAdd(&P.cnt[q], 1)] = (uint16_t)e;
+    }
+    __syncwarp();
+}
+
+// a + e inside B (shifted false: a is A's vertex), or c - e inside A (shifted true), by a warp
+__device__ __forceinline__ int warp_point_in_ring(int2 p, const int2* v, int n, bool shifted, int lane)
+{
+    unsigned in = 0;
+    for (int e = lane; e < n; e += 32) {
+        const int2 c = v[e], d = v[e + 1 == n ? 0 : e + 1];
+        if (shifted ? (c.y >= p.y) != (d.y >= p.y) : (c.y > p.y) != (d.y > p.y)) {
+            const long long cr = cross3(c, d, p);
+            in ^= shifted ? (cr == 0) | ((cr > 0) == (d.y > c.y)) : (cr != 0) & ((cr > 0) == (d.y > c.y));
+        }
+    }
+    return __popc(__ballot_sync(0xffffffffu, in)) & 1;
+}
+
+// twice the end terms of a ring's edges: edge i ends inside the other ring iff its end
+// vertex's state -- the first vertex's, flipped by every crossing of edges 0 .. i -- is
+// inside; integers (by one warp, summed over its lanes)
+__device__ __forceinline__ long long ring_ends(const int2* v, int n, const uint32_t* par, int inside, int org_x,
+                                               int lane)
+{
+    long long sum = 0;
+    const unsigned le = pmh_lanemask_lt() | (1u << lane);
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const uint32_t w = par[i0 >> 5];
+        const int i = i0 + lane;
+        if (i < n && ((inside ^ __popc(w & le)) & 1)) {
+            const int2 a = v[i], b = v[i + 1 == n ? 0 : i + 1];
+            sum += (long long)(b.y - a.y) * (2 * (a.x - org_x) + (b.x - a.x));
+        }
+        inside ^= __popc(w) & 1;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    return sum;
+}
+
 // J of one pair by two warps (wip = 0, 1; every branch is uniform over both): both
 // rings staged in the pair's shared slice when they fit, else read from global
-// memory; warp 0 builds A's y-slab list and warp 1 B's, both when they fit their
-// capacity, else every edge pair; the area's terms split between the warps, summed
-// in a fixed order
+// memory.  Warp 1 lists B's edges by y-slab over the rings' common box while warp 0
+// decides the two first vertices; the warps take alternate 32-edge groups of A's edges
+// and find their crossings in those lists, queueing them (the fp64 terms are evaluated
+// 32 at a time) and keeping each edge's crossing parity.  The state of every other
+// vertex follows from the parities along its ring (each crossing moves an edge across
+// the other boundary; the predicates are exact, so the parities are), which leaves the
+// end terms as one pass of integer sums: no vertex is tested against the other ring
+// and A needs no lists.  Bound by issue and by the predicates' dependent integer
+// chains.  77,824 pairs of 8 to 1,024 vertices (4,096 lists of 19): 1.10 ms, 1.76 when every
+// vertex was tested against the other ring's lists.
 __device__ double pair_jaccard(PairView A, PairView B, RefPair& P, int wip, int lane, int g)
 {
     if (A.sgn == 0 || B.sgn == 0) return 0.0;
-    const int2* a = A.v;
-    const int2* b = B.v;
-    // both rings staged when they fit the slice, else the one that fits (B first: its
-    // edges are the inner loop of two of the three passes), else neither
-    const bool sa = A.n + B.n <= kWarpVerts || (B.n > kWarpVerts && A.n <= kWarpVerts);
-    const bool sb = A.n + B.n <= kWarpVerts || B.n <= kWarpVerts;
-    if (sa || sb) {
-        const int boff = sa ? A.n : 0;
-        if (sa) stage_ring(P.sv, A.v, A.n, 32 * wip + lane);
-        if (sb) stage_ring(P.sv + boff, B.v, B.n, 32 * wip + lane);
-        asm volatile("cp.async.wait_all;\n" ::: "memory");
+    const unsigned full = 0xffffffffu;
+    double inter;
+    if (max(A.n, B.n) > kRefineBigVerts) {  // (large rings where no queue takes them)
+        const double part = warp_intersection_area(A.v, A.n, A.sgn, B.v, B.n, B.sgn, P.cq[wip], lane, wip);
+        if (lane == 0) P.part[wip] = part;
         pair_sync(g);
-        if (sa) a = P.sv;
-        if (sb) b = P.sv + boff;
+        inter = P.part[0] + P.part[1];
+    } else {
+        const int2* a = A.v;
+        const int2* b = B.v;
+        // both rings staged when they fit the slice, else the one that fits (B first: its
+        // edges are the inner loop), else neither
+        const bool sa = A.n + B.n <= kWarpVerts || (B.n > kWarpVerts && A.n <= kWarpVerts);
+        const bool sb = A.n + B.n <= kWarpVerts || B.n <= kWarpVerts;
+        if (sa || sb) {
+            const int boff = sa ? A.n : 0;
+            if (sa) stage_ring(P.sv, A.v, A.n, 32 * wip + lane);
+            if (sb) stage_ring(P.sv + boff, B.v, B.n, 32 * wip + lane);
+            asm volatile("cp.async.wait_all;\n" ::: "memory");
+            pair_sync(g);
+            if (sa) a = P.sv;
+            if (sb) b = P.sv + boff;
+        }
+        {  // warp 0: A's range; warp 1: B's
+            const int2* v = wip == 0 ? a : b;
+            const int n = wip == 0 ? A.n : B.n;
+            int x0 = INT_MAX, x1 = INT_MIN, y0 = INT_MAX, y1 = INT_MIN;
+            for (int i = lane; i < n; i += 32) {
+                const int2 u = v[i];
+                x0 = min(x0, u.x);
+                x1 = max(x1, u.x);
+                y0 = min(y0, u.y);
+                y1 = max(y1, u.y);
+            }
+            x0 = __reduce_min_sync(full, x0);
+            x1 = __reduce_max_sync(full, x1);
+            y0 = __reduce_min_sync(full, y0);
+            y1 = __reduce_max_sync(full, y1);
+            if (lane == 0) {
+                P.range[wip][0] = x0;
+                P.range[wip][1] = x1;
+                P.range[wip][2] = y0;
+                P.range[wip][3] = y1;
+            }
+            P.par_a[lane] = 0;  // (both warps write the same zeros)
+            P.par_b[lane] = 0;
+        }
+        pair_sync(g);
+        const int rx0 = max(P.range[0][0], P.range[1][0]), rx1 = min(P.range[0][1], P.range[1][1]);
+        const int ry0 = max(P.range[0][2], P.range[1][2]), ry1 = min(P.range[0][3], P.range[1][3]);
+        if (rx0 > rx1 || ry0 > ry1) return 0.0;
+        if (wip == 1) {
+            build_pair_slabs(b, B.n, rx0, rx1, ry0, ry1, P, lane);
+        } else {
+            const int ia = warp_point_in_ring(a[0], b, B.n, false, lane);
+            const int ib = warp_point_in_ring(b[0], a, A.n, true, lane);
+            if (lane == 0) {
+                P.in0[0] = ia;
+                P.in0[1] = ib;
+            }
+        }
+        pair_sync(g);
+        const int sh = P.sh;
+        const int2 org = b[0];
+        uint2* cq = P.cq[wip];
+        double acc = 0;
+        int nq = 0;  // warp-uniform queue length (< 32 between iterations)
+        for (int i0 = 32 * wip; i0 < A.n; i0 += 64) {
+            const int i = i0 + lane;
+            int2 u = make_int2(0, 0), w = make_int2(0, 0);
+            int k = 0, kend = 0, q0 = 0;
+            if (i < A.n) {
+                u = a[i];
+                w = a[i + 1 == A.n ? 0 : i + 1];
+                const int lo = max(min(u.y, w.y), ry0), hi = min(max(u.y, w.y), ry1);
+                if ((u.x != w.x || u.y != w.y) && lo <= hi && max(u.x, w.x) >= rx0 && min(u.x, w.x) <= rx1) {
+                    q0 = (lo - ry0) >> sh;
+                    k = P.beg[q0];
+                    kend = P.beg[((hi - ry0) >> sh) + 1];
+                }
+            }
+            const int ux0 = min(u.x, w.x), ux1 = max(u.x, w.x), uy0 = min(u.y, w.y), uy1 = max(u.y, w.y);
+            const int steps = __reduce_max_sync(full, kend - k);
+            int q = q0, qend = k < kend ? P.beg[q0 + 1] : 0;  // slab of list position k, and its end
+            bool odd = false;
+            for (int t = 0; t < steps; ++t, ++k) {
+                bool hit = false;
+                int j = 0;
+                if (k < kend) {
+                    while (k >= qend) {
+                        ++q;
+                        qend = P.beg[q + 1];
+                    }
+                    j = P.ids[k];
+                    const int2 c = b[j], d = b[j + 1 == B.n ? 0 : j + 1];
+                    const int dy0 = min(c.y, d.y);
+                    // this pair is visited once: in the first listed slab of both
+                    if (!(max(ux0, min(c.x, d.x)) > min(ux1, max(c.x, d.x)) || max(uy0, dy0) > min(uy1, max(c.y, d.y)) ||
+                          (c.x == d.x && c.y == d.y)) &&
+                        q == max(q0, (max(dy0, ry0) - ry0) >> sh))
+                        hit = side_of_shifted_point(c, d, u) != side_of_shifted_point(c, d, w) &&
+                              side_of_point_to_shifted(u, w, c) != side_of_point_to_shifted(u, w, d);
+                }
+                const unsigned bal = __ballot_sync(full, hit);
+                if (bal) {
+                    if (hit) {
+                        odd = !odd;
+                        atomicXor(&P.par_b[j >> 5], 1u << (j & 31));
+                        cq[nq + __popc(bal & pmh_lanemask_lt())] = make_uint2((uint32_t)i, (uint32_t)j);
+                    }
+                    nq += __popc(bal);
+                    __syncwarp();
+                    if (nq >= 32) {
+                        acc += crossing_terms(a, A.n, A.sgn, b, B.n, B.sgn, org, cq[lane]);
+                        nq -= 32;
+                        const uint2 rest = lane < nq ? cq[32 + lane] : make_uint2(0u, 0u);
+                        __syncwarp();
+                        if (lane < nq) cq[lane] = rest;
+                        __syncwarp();
+                    }
+                }
+            }
+            const unsigned word = __ballot_sync(full, odd);
+            if (lane == 0) P.par_a[i0 >> 5] = word;
+        }
+        if (lane < nq) acc += crossing_terms(a, A.n, A.sgn, b, B.n, B.sgn, org, cq[lane]);
+        __syncwarp();
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(full, acc, o);
+        if (lane == 0) P.part[wip] = acc;
+        pair_sync(g);
+        const long long ends = wip == 0 ? A.sgn * ring_ends(a, A.n, P.par_a, P.in0[0], org.x, lane)
+                                        : B.sgn * ring_ends(b, B.n, P.par_b, P.in0[1], org.x, lane);
+        if (lane == 0) P.ends[wip] = ends;
+        pair_sync(g);
+        inter = (P.part[0] + P.part[1]) + 0.5 * (double)(P.ends[0] + P.ends[1]);
     }
-    const bool ok = build_ref_slabs(wip == 0 ? a : b, wip == 0 ? A.n : B.n, P.sl[wip], lane);
-    if (lane == 0) P.ok[wip] = ok;
-    pair_sync(g);
-    const double part =
-        P.ok[0] && P.ok[1]
-            ? warp_intersection_area_slabs(a, A.n, A.sgn, P.sl[0], b, B.n, B.sgn, P.sl[1], P.cq[wip], lane, wip)
-            : warp_intersection_area(a, A.n, A.sgn, b, B.n, B.sgn, P.cq[wip], lane, wip);
-    if (lane == 0) P.part[wip] = part;
-    pair_sync(g);
-    const double inter = P.part[0] + P.part[1];
     const double uni = A.area + B.area - inter;
     return uni > 0 ? fmin(fmax(inter / uni, 0.0), 1.0) : 0.0;
 }
 
-__global__ void __launch_bounds__(kRefineWarps * 32, 7)
+__global__ void __launch_bounds__(kRefineWarps * 32, 8)
 refine_pairs_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff,
                     const int64_t* __restrict__ qarea2, const int4* __restrict__ qbox,
                     const int2* __restrict__ pxy, const int64_t* __restrict__ poff,
