@@ -17,7 +17,7 @@
 // shifted by (e1, e2), 0 < e2 << e1 infinitesimal.  Every predicate is then
 // decided exactly with int64 cross products (coordinates <= 2^20), and the
 // area of the shifted configuration tends to the exact one.  The terms are
-// fp64 in coordinates relative to B's first vertex.  GB300's fp64 rate is low,
+// fp64 in coordinates relative to B's first vertex, summed exactly.  GB300's fp64 rate is low,
 // so the fp64 work is kept to the crossings (a few per edge) and one Newton
 // reciprocal each.
 #include <algorithm>
@@ -68,6 +68,33 @@ __device__ __forceinline__ double recip(long long D)
     e = fma(-d, y, 1.0);
     return fma(y, e, y);
 }
+
+// exact running sum of fp64 terms |x| < 2^44: multiples of 2^-18 and of 2^-56, modulo 2^64
+// (sums of integers: the order of the terms does not show)
+struct ExactSum {
+    unsigned long long q18 = 0, r56 = 0;
+    __device__ __forceinline__ void add(double x)
+    {
+        const long long q = __double2ll_rn(x * 262144.0);
+        const double r = fma((double)q, -1.0 / 262144.0, x);  // exact: |r| <= 2^-19
+        q18 += (unsigned long long)q;
+        r56 += (unsigned long long)__double2ll_rn(r * 72057594037927936.0);
+    }
+    __device__ __forceinline__ void reduce()  // over the warp, in every lane
+    {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            q18 += __shfl_xor_sync(0xffffffffu, q18, o);
+            r56 += __shfl_xor_sync(0xffffffffu, r56, o);
+        }
+    }
+    // the sum plus twice_ends / 2
+    __device__ __forceinline__ double total(long long twice_ends) const
+    {
+        return (double)(long long)(q18 + ((unsigned long long)twice_ends << 17)) * (1.0 / 262144.0) +
+               (double)(long long)r56 * (1.0 / 72057594037927936.0);
+    }
+};
 
 // area(A n B) for one pair, by one warp; returned in every lane.
 //  * end terms: edge e_i of the shifted A ends inside B iff its end vertex
@@ -214,34 +241,38 @@ __device__ __forceinline__ PairView view(const int2* xy, const int64_t* off, con
     return r;
 }
 
-// y-slabs of the two-warp form: B's edges that meet the two rings' common box, listed in
-// every slab of 2^sh rows that their closed y-range meets (kRefSlabs slabs over the common
-// rows, four per lane; taller slabs until the references fit kRefSlabCap)
-constexpr int kRefSlabs = 128;
-constexpr int kSlabsPerLane = kRefSlabs / 32;
-constexpr int kRefSlabCap = 2048;
-static_assert(kRefineBigVerts <= kRefSlabCap && kRefineBigVerts <= 32 * 32, "one slab holds every edge");
+// Cells of the two-warp form: B's edges that meet the two rings' common box, listed in
+// every cell of a grid over it that their bounding box meets.  A row of cells is one
+// stretch of the lists.  With cells about twice as long as an edge, an A edge meets ~2
+// listed edges; y-slabs of any height leave it ~16 (a slab crosses the far side of the
+// ring too).  The grid has up to 32 x 32 cells, fewer for few edges (their clearing and
+// their prefix sum are paid per pair), and larger cells until the references fit
+// kRefCellCap.
+constexpr int kGridLog2 = 5;
+constexpr int kRefCellCap = 2048;
+static_assert(kRefineBigVerts <= kRefCellCap && kRefineBigVerts <= 32 * 32, "one cell holds every edge");
+__device__ __forceinline__ int pair_grid_log2(int n) { return n >= 192 ? 5 : n >= 40 ? 4 : 3; }
 
 constexpr int kRefineWarps = 4;  // two pairs per block, two warps per pair
-constexpr int kWarpVerts = 960;   // vertices of a pair's staging slice
+constexpr int kWarpVerts = 1024;  // vertices of a pair's staging slice (seven blocks per SM)
+static_assert(kRefineBigVerts <= kWarpVerts, "B is always staged");
 
-// one pair's shared slice: the staged rings, a crossing queue per warp, B's slab lists,
+// one pair's shared slice: the staged rings, a crossing queue per warp, B's cell lists,
 // each ring's crossing parities by edge, and the two warps' partial sums
 struct RefPair {
     int2 sv[kWarpVerts];
-    union {
-        uint2 cq[2][64];
-        int cnt[kRefSlabs];  // list cursors, before the queues are in use
-    };
-    uint16_t ids[kRefSlabCap];
-    uint16_t beg[kRefSlabs + 2];
+    // 16-bit counts of the cells, then their ends, then (filled backwards) their first
+    // entries; one more holds the end of the last
+    uint32_t cell[(1 << (2 * kGridLog2)) / 2 + 4];
+    uint32_t cq[2][64];  // queued crossings: edge of A << 16 | edge of B
+    uint16_t ids[kRefCellCap];
     uint32_t par_a[32], par_b[32];  // bit i % 32 of word i / 32: edge i is crossed an odd number of times
     int range[2][4];                // min x, max x, min y, max y of A and of B
+    unsigned long long q18[2], r56[2];  // each warp's crossing terms (ExactSum)
     double part[2];
     long long ends[2];
     long long e;
-    int sh;
-    int in0[2];  // first vertex of A inside B, of B inside A
+    int sum[2];  // each warp's edges in the common box, references
 };
 
 // the named barrier of pair slot g (0 or 1) of the block (barrier 0 is __syncthreads;
@@ -260,63 +291,6 @@ __device__ __forceinline__ void stage_ring(int2* dst, const int2* __restrict__ s
         const unsigned d = (unsigned)__cvta_generic_to_shared(dst + i);
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src + i) : "memory");
     }
-}
-
-// B's slab lists over the common box (rows [ry0, ry1], columns [rx0, rx1]), by one warp
-__device__ __forceinline__ void build_pair_slabs(const int2* v, int n, int rx0, int rx1, int ry0, int ry1,
-                                                 RefPair& P, int lane)
-{
-    int sh = 0;
-    while (((ry1 - ry0) >> sh) >= kRefSlabs) ++sh;
-    for (;; ++sh) {
-#pragma unroll
-        for (int u = 0; u < kSlabsPerLane; ++u) P.cnt[kSlabsPerLane * lane + u] = 0;
-        __syncwarp();
-        for (int e = lane; e < n; e += 32) {
-            const int2 a = v[e], b = v[e + 1 == n ? 0 : e + 1];
-            const int lo = max(min(a.y, b.y), ry0), hi = min(max(a.y, b.y), ry1);
-            if (lo > hi || max(a.x, b.x) < rx0 || min(a.x, b.x) > rx1) continue;
-            const int s0 = (lo - ry0) >> sh, s1 = (hi - ry0) >> sh;
-            for (int q = s0; q <= s1; ++q) atomicAdd(&P.cnt[q], 1);
-        }
-        __syncwarp();
-        int c[kSlabsPerLane], mine = 0;
-#pragma unroll
-        for (int u = 0; u < kSlabsPerLane; ++u) {
-            c[u] = P.cnt[kSlabsPerLane * lane + u];
-            mine += c[u];
-        }
-        int incl = mine;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += t;
-        }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        if (total > kRefSlabCap) {  // (one slab holds at most n <= kRefineBigVerts)
-            __syncwarp();
-            continue;
-        }
-        int run = incl - mine;
-#pragma unroll
-        for (int u = 0; u < kSlabsPerLane; ++u) {
-            P.beg[kSlabsPerLane * lane + u] = (uint16_t)run;
-            P.cnt[kSlabsPerLane * lane + u] = run;
-            run += c[u];
-        }
-        if (lane == 31) P.beg[kRefSlabs] = (uint16_t)total;
-        if (lane == 0) P.sh = sh;
-        __syncwarp();
-        break;
-    }
-    for (int e = lane; e < n; e += 32) {
-        const int2 a = v[e], b = v[e + 1 == n ? 0 : e + 1];
-        const int lo = max(min(a.y, b.y), ry0), hi = min(max(a.y, b.y), ry1);
-        if (lo > hi || max(a.x, b.x) < rx0 || min(a.x, b.x) > rx1) continue;
-        const int s0 = (lo - ry0) >> sh, s1 = (hi - ry0) >> sh;
-        for (int q = s0; q <= s1; ++q) P.ids[atomicAdd(&P.cnt[q], 1)] = (uint16_t)e;
-    }
-    __syncwarp();
 }
 
 // a + e inside B (shifted false: a is A's vertex), or c - e inside A (shifted true), by a warp
@@ -355,44 +329,123 @@ __device__ __forceinline__ long long ring_ends(const int2* v, int n, const uint3
     return sum;
 }
 
-// J of one pair by two warps (wip = 0, 1; every branch is uniform over both): both
-// rings staged in the pair's shared slice when they fit, else read from global
-// memory.  Warp 1 lists B's edges by y-slab over the rings' common box while warp 0
-// decides the two first vertices; the warps take alternate 32-edge groups of A's edges
-// and find their crossings in those lists, queueing them (the fp64 terms are evaluated
-// 32 at a time) and keeping each edge's crossing parity.  The state of every other
-// vertex follows from the parities along its ring (each crossing moves an edge across
-// the other boundary; the predicates are exact, so the parities are), which leaves the
-// end terms as one pass of integer sums: no vertex is tested against the other ring
-// and A needs no lists.  Bound by issue and by the predicates' dependent integer
-// chains.  77,824 pairs of 8 to 1,024 vertices (4,096 lists of 19): 1.10 ms, 1.76 when every
-// vertex was tested against the other ring's lists.
+// the common box of a pair and its grid of cells
+struct PairGrid {
+    int rx0, rx1, ry0, ry1, lg, shx, shy;
+    // cells of edge (a, b): columns c0 .. c1 of rows r0 .. r1; false: outside the box
+    __device__ __forceinline__ bool cells(int2 a, int2 b, int& c0, int& c1, int& r0, int& r1) const
+    {
+        const int x0 = max(min(a.x, b.x), rx0), x1 = min(max(a.x, b.x), rx1);
+        const int y0 = max(min(a.y, b.y), ry0), y1 = min(max(a.y, b.y), ry1);
+        c0 = (x0 - rx0) >> shx;
+        c1 = (x1 - rx0) >> shx;
+        r0 = (y0 - ry0) >> shy;
+        r1 = (y1 - ry0) >> shy;
+        return x0 <= x1 && y0 <= y1;
+    }
+};
+
+// B's cell lists over the common box, by the pair's 64 threads (t)
+__device__ __forceinline__ void build_pair_cells(const int2* v, int n, PairGrid& G, RefPair& P, int t, int g)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = t & 31, wip = t >> 5;
+    const int words = 1 << (2 * G.lg - 1);  // two cells each
+    const int per = max(words >> 6, 1);     // words per thread of the prefix sum (8, 2 or 1)
+    while (((G.rx1 - G.rx0) >> G.shx) >> G.lg) ++G.shx;
+    while (((G.ry1 - G.ry0) >> G.shy) >> G.lg) ++G.shy;
+    for (;; ++G.shx, ++G.shy) {
+        for (int i = t; i < words; i += 64) P.cell[i] = 0;
+        pair_sync(g);
+        for (int e = t; e < n; e += 64) {
+            int c0, c1, r, r1;
+            if (!G.cells(v[e], v[e + 1 == n ? 0 : e + 1], c0, c1, r, r1)) continue;
+            for (; r <= r1; ++r)
+                for (int c = (r << G.lg) + c0; c <= (r << G.lg) + c1; ++c)
+                    atomicAdd(&P.cell[c >> 1], 1u << (16 * (c & 1)));
+        }
+        pair_sync(g);
+        // counts to ends: each thread's words, then the warp's and the pair's prefix
+        const int w0 = t * per;
+        int mine = 0;
+        if (w0 < words)
+            for (int u = 0; u < per; ++u) {
+                const uint32_t w = P.cell[w0 + u];
+                mine += (int)(w & 0xFFFFu) + (int)(w >> 16);
+            }
+        int x = mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(full, x, d);
+            if (lane >= d) x += y;
+        }
+        if (lane == 31) P.sum[wip] = x;
+        pair_sync(g);
+        const int total = P.sum[0] + P.sum[1];
+        if (total > kRefCellCap) {  // (one cell holds at most n <= kRefineBigVerts)
+            pair_sync(g);
+            continue;
+        }
+        int run = x - mine + (wip ? P.sum[0] : 0);
+        if (w0 < words)
+            for (int u = 0; u < per; ++u) {
+                const uint32_t w = P.cell[w0 + u];
+                const int lo = run + (int)(w & 0xFFFFu), hi = lo + (int)(w >> 16);
+                P.cell[w0 + u] = (uint32_t)lo | ((uint32_t)hi << 16);
+                run = hi;
+            }
+        if (t == 0) P.cell[words] = (uint32_t)total;
+        pair_sync(g);
+        break;
+    }
+    for (int e = t; e < n; e += 64) {
+        int c0, c1, r, r1;
+        if (!G.cells(v[e], v[e + 1 == n ? 0 : e + 1], c0, c1, r, r1)) continue;
+        for (; r <= r1; ++r)
+            for (int c = (r << G.lg) + c0; c <= (r << G.lg) + c1; ++c) {
+                const uint32_t old = atomicSub(&P.cell[c >> 1], 1u << (16 * (c & 1)));
+                P.ids[((old >> (16 * (c & 1))) & 0xFFFFu) - 1] = (uint16_t)e;
+            }
+    }
+    pair_sync(g);
+}
+
+// J of one pair by two warps (wip = 0, 1; every branch is uniform over both), rings of at
+// most kRefineBigVerts vertices: B staged in the pair's shared slice, A too when both fit.
+// B's edges are listed by the cells of the rings' common box.  The warps take alternate
+// 32-edge groups of A's edges; a group's (edge, listed edge) visits are spread over the
+// lanes by a warp scan, so that no lane waits for the longest list, and the crossings
+// found are queued (their fp64 terms are evaluated 32 at a time) and flip both edges'
+// parities.  Each ring's first vertex is tested against the other ring; the state of
+// every other vertex follows from the parities along its ring (each crossing moves an
+// edge across the other boundary; the predicates are exact, so the parities are), which
+// leaves the end terms as one pass of integer sums.  The crossings' terms are summed as
+// integers too (ExactSum), so the lists' order (atomics of two warps) does not show.
+// Bound by issue and by the latency of dependent shared-memory and integer chains.
+// 77,824 pairs of 8 to 1,024 vertices (4,096 lists of 19): 0.71 ms; 1.10 with y-slabs listed
+// by one warp and a lane per edge, of which the listing took a third.
 __device__ double pair_jaccard(PairView A, PairView B, RefPair& P, int wip, int lane, int g)
 {
     if (A.sgn == 0 || B.sgn == 0) return 0.0;
     const unsigned full = 0xffffffffu;
+    const int t = 32 * wip + lane;
     double inter;
     if (max(A.n, B.n) > kRefineBigVerts) {  // (large rings where no queue takes them)
-        const double part = warp_intersection_area(A.v, A.n, A.sgn, B.v, B.n, B.sgn, P.cq[wip], lane, wip);
+        const double part = warp_intersection_area(A.v, A.n, A.sgn, B.v, B.n, B.sgn,
+                                                   reinterpret_cast<uint2*>(P.sv) + 64 * wip, lane, wip);
         if (lane == 0) P.part[wip] = part;
         pair_sync(g);
         inter = P.part[0] + P.part[1];
     } else {
-        const int2* a = A.v;
-        const int2* b = B.v;
-        // both rings staged when they fit the slice, else the one that fits (B first: its
-        // edges are the inner loop), else neither
-        const bool sa = A.n + B.n <= kWarpVerts || (B.n > kWarpVerts && A.n <= kWarpVerts);
-        const bool sb = A.n + B.n <= kWarpVerts || B.n <= kWarpVerts;
-        if (sa || sb) {
-            const int boff = sa ? A.n : 0;
-            if (sa) stage_ring(P.sv, A.v, A.n, 32 * wip + lane);
-            if (sb) stage_ring(P.sv + boff, B.v, B.n, 32 * wip + lane);
-            asm volatile("cp.async.wait_all;\n" ::: "memory");
-            pair_sync(g);
-            if (sa) a = P.sv;
-            if (sb) b = P.sv + boff;
-        }
+        const bool sa = A.n + B.n <= kWarpVerts;
+        stage_ring(P.sv, B.v, B.n, t);
+        if (sa) stage_ring(P.sv + B.n, A.v, A.n, t);
+        P.par_a[lane] = 0;  // (both warps write the same zeros)
+        P.par_b[lane] = 0;
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        pair_sync(g);
+        const int2* b = P.sv;
+        const int2* a = sa ? P.sv + B.n : A.v;
         {  // warp 0: A's range; warp 1: B's
             const int2* v = wip == 0 ? a : b;
             const int n = wip == 0 ? A.n : B.n;
@@ -414,103 +467,125 @@ __device__ double pair_jaccard(PairView A, PairView B, RefPair& P, int wip, int 
                 P.range[wip][2] = y0;
                 P.range[wip][3] = y1;
             }
-            P.par_a[lane] = 0;  // (both warps write the same zeros)
-            P.par_b[lane] = 0;
         }
         pair_sync(g);
-        const int rx0 = max(P.range[0][0], P.range[1][0]), rx1 = min(P.range[0][1], P.range[1][1]);
-        const int ry0 = max(P.range[0][2], P.range[1][2]), ry1 = min(P.range[0][3], P.range[1][3]);
-        if (rx0 > rx1 || ry0 > ry1) return 0.0;
-        if (wip == 1) {
-            build_pair_slabs(b, B.n, rx0, rx1, ry0, ry1, P, lane);
-        } else {
-            const int ia = warp_point_in_ring(a[0], b, B.n, false, lane);
-            const int ib = warp_point_in_ring(b[0], a, A.n, true, lane);
-            if (lane == 0) {
-                P.in0[0] = ia;
-                P.in0[1] = ib;
-            }
+        PairGrid G{max(P.range[0][0], P.range[1][0]), min(P.range[0][1], P.range[1][1]),
+                   max(P.range[0][2], P.range[1][2]), min(P.range[0][3], P.range[1][3]), 0, 0, 0};
+        if (G.rx0 > G.rx1 || G.ry0 > G.ry1) return 0.0;
+        // B's edges in the box (the grid's size), and the first vertices' states
+        int nb = 0;
+        for (int e0 = 32 * wip; e0 < B.n; e0 += 64) {
+            const int e = e0 + lane;
+            int c0, c1, r0, r1;
+            const bool in = e < B.n && G.cells(b[e], b[e + 1 == B.n ? 0 : e + 1], c0, c1, r0, r1);
+            nb += __popc(__ballot_sync(full, in));
         }
+        if (lane == 0) P.sum[wip] = nb;
+        // (warp 0: the first vertex of A inside B; warp 1: that of B inside A)
+        const int in0 = wip == 0 ? warp_point_in_ring(a[0], b, B.n, false, lane)
+                                 : warp_point_in_ring(b[0], a, A.n, true, lane);
         pair_sync(g);
-        const int sh = P.sh;
+        G.lg = pair_grid_log2(P.sum[0] + P.sum[1]);
+        build_pair_cells(b, B.n, G, P, t, g);
+        const uint16_t* beg = reinterpret_cast<const uint16_t*>(P.cell);
         const int2 org = b[0];
-        uint2* cq = P.cq[wip];
-        double acc = 0;
+        uint32_t* cq = P.cq[wip];
+        ExactSum sum;
         int nq = 0;  // warp-uniform queue length (< 32 between iterations)
         for (int i0 = 32 * wip; i0 < A.n; i0 += 64) {
-            const int i = i0 + lane;
-            int2 u = make_int2(0, 0), w = make_int2(0, 0);
-            int k = 0, kend = 0, q0 = 0;
-            if (i < A.n) {
-                u = a[i];
-                w = a[i + 1 == A.n ? 0 : i + 1];
-                const int lo = max(min(u.y, w.y), ry0), hi = min(max(u.y, w.y), ry1);
-                if ((u.x != w.x || u.y != w.y) && lo <= hi && max(u.x, w.x) >= rx0 && min(u.x, w.x) <= rx1) {
-                    q0 = (lo - ry0) >> sh;
-                    k = P.beg[q0];
-                    kend = P.beg[((hi - ry0) >> sh) + 1];
+            int c0 = 0, c1 = -1, r0 = 0, r1 = -1;  // the lane's edge's cells (none)
+            if (i0 + lane < A.n) {
+                const int2 u = a[i0 + lane], w = a[i0 + lane + 1 == A.n ? 0 : i0 + lane + 1];
+                if (!G.cells(u, w, c0, c1, r0, r1) || (u.x == w.x && u.y == w.y)) r1 = r0 - 1;
+            }
+            const int rows = __reduce_max_sync(full, r1 - r0 + 1);
+            const int first = (r0 << 16) | c0;
+            for (int dr = 0; dr < rows; ++dr) {
+                int k0 = 0, len = 0;  // the row's stretch of the lists
+                if (r0 + dr <= r1) {
+                    const int row = (r0 + dr) << G.lg;
+                    k0 = beg[row + c0];
+                    len = beg[row + c1 + 1] - k0;
+                }
+                int excl = len;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const int y = __shfl_up_sync(full, excl, d);
+                    if (lane >= d) excl += y;
+                }
+                const int visits = __shfl_sync(full, excl, 31);
+                excl -= len;
+                const int shift = k0 - excl;  // list position of visit x of this lane's edge: x + shift
+                for (int x0 = 0; x0 < visits; x0 += 32) {
+                    const int x = x0 + lane;
+                    int own = 0;  // the last lane whose first visit is <= x
+#pragma unroll
+                    for (int step = 16; step >= 1; step >>= 1)
+                        if (__shfl_sync(full, excl, own + step) <= x) own += step;
+                    const int k = x + __shfl_sync(full, shift, own);
+                    const int of = __shfl_sync(full, first, own);
+                    bool hit = false;
+                    int j = 0;
+                    const int i = i0 + own;
+                    if (x < visits) {
+                        j = P.ids[k];
+                        const int2 c = b[j], d = b[j + 1 == B.n ? 0 : j + 1];
+                        const int2 u = a[i], w = a[i + 1 == A.n ? 0 : i + 1];
+                        const int dx0 = min(c.x, d.x), dy0 = min(c.y, d.y);
+                        if (!(max(min(u.x, w.x), dx0) > min(max(u.x, w.x), max(c.x, d.x)) ||
+                              max(min(u.y, w.y), dy0) > min(max(u.y, w.y), max(c.y, d.y)) ||
+                              (c.x == d.x && c.y == d.y))) {
+                            // this pair is visited once: in the first cell listed for both
+                            const int ur = of >> 16, uc = of & 0xFFFF;
+                            const int cell = ((ur + dr) << G.lg) + max(uc, (max(dx0, G.rx0) - G.rx0) >> G.shx);
+                            if (ur + dr == max(ur, (max(dy0, G.ry0) - G.ry0) >> G.shy) && k >= beg[cell] && k < beg[cell + 1])
+                                hit = side_of_shifted_point(c, d, u) != side_of_shifted_point(c, d, w) &&
+                                      side_of_point_to_shifted(u, w, c) != side_of_point_to_shifted(u, w, d);
+                        }
+                    }
+                    const unsigned bal = __ballot_sync(full, hit);
+                    if (bal) {
+                        if (hit) {
+                            atomicXor(&P.par_a[i >> 5], 1u << (i & 31));
+                            atomicXor(&P.par_b[j >> 5], 1u << (j & 31));
+                            cq[nq + __popc(bal & pmh_lanemask_lt())] = ((uint32_t)i << 16) | (uint32_t)j;
+                        }
+                        nq += __popc(bal);
+                        __syncwarp();
+                        if (nq >= 32) {
+                            const uint32_t ij = cq[lane];
+                            sum.add(crossing_terms(a, A.n, A.sgn, b, B.n, B.sgn, org, make_uint2(ij >> 16, ij & 0xFFFFu)));
+                            nq -= 32;
+                            const uint32_t rest = lane < nq ? cq[32 + lane] : 0u;
+                            __syncwarp();
+                            if (lane < nq) cq[lane] = rest;
+                            __syncwarp();
+                        }
+                    }
                 }
             }
-            const int ux0 = min(u.x, w.x), ux1 = max(u.x, w.x), uy0 = min(u.y, w.y), uy1 = max(u.y, w.y);
-            const int steps = __reduce_max_sync(full, kend - k);
-            int q = q0, qend = k < kend ? P.beg[q0 + 1] : 0;  // slab of list position k, and its end
-            bool odd = false;
-            for (int t = 0; t < steps; ++t, ++k) {
-                bool hit = false;
-                int j = 0;
-                if (k < kend) {
-                    while (k >= qend) {
-                        ++q;
-                        qend = P.beg[q + 1];
-                    }
-                    j = P.ids[k];
-                    const int2 c = b[j], d = b[j + 1 == B.n ? 0 : j + 1];
-                    const int dy0 = min(c.y, d.y);
-                    // this pair is visited once: in the first listed slab of both
-                    if (!(max(ux0, min(c.x, d.x)) > min(ux1, max(c.x, d.x)) || max(uy0, dy0) > min(uy1, max(c.y, d.y)) ||
-                          (c.x == d.x && c.y == d.y)) &&
-                        q == max(q0, (max(dy0, ry0) - ry0) >> sh))
-                        hit = side_of_shifted_point(c, d, u) != side_of_shifted_point(c, d, w) &&
-                              side_of_point_to_shifted(u, w, c) != side_of_point_to_shifted(u, w, d);
-                }
-                const unsigned bal = __ballot_sync(full, hit);
-                if (bal) {
-                    if (hit) {
-                        odd = !odd;
-                        atomicXor(&P.par_b[j >> 5], 1u << (j & 31));
-                        cq[nq + __popc(bal & pmh_lanemask_lt())] = make_uint2((uint32_t)i, (uint32_t)j);
-                    }
-                    nq += __popc(bal);
-                    __syncwarp();
-                    if (nq >= 32) {
-                        acc += crossing_terms(a, A.n, A.sgn, b, B.n, B.sgn, org, cq[lane]);
-                        nq -= 32;
-                        const uint2 rest = lane < nq ? cq[32 + lane] : make_uint2(0u, 0u);
-                        __syncwarp();
-                        if (lane < nq) cq[lane] = rest;
-                        __syncwarp();
-                    }
-                }
-            }
-            const unsigned word = __ballot_sync(full, odd);
-            if (lane == 0) P.par_a[i0 >> 5] = word;
         }
-        if (lane < nq) acc += crossing_terms(a, A.n, A.sgn, b, B.n, B.sgn, org, cq[lane]);
-        __syncwarp();
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(full, acc, o);
-        if (lane == 0) P.part[wip] = acc;
+        if (lane < nq) {
+            const uint32_t ij = cq[lane];
+            sum.add(crossing_terms(a, A.n, A.sgn, b, B.n, B.sgn, org, make_uint2(ij >> 16, ij & 0xFFFFu)));
+        }
+        sum.reduce();
+        if (lane == 0) {
+            P.q18[wip] = sum.q18;
+            P.r56[wip] = sum.r56;
+        }
         pair_sync(g);
-        const long long ends = wip == 0 ? A.sgn * ring_ends(a, A.n, P.par_a, P.in0[0], org.x, lane)
-                                        : B.sgn * ring_ends(b, B.n, P.par_b, P.in0[1], org.x, lane);
+        const long long ends = wip == 0 ? A.sgn * ring_ends(a, A.n, P.par_a, in0, org.x, lane)
+                                        : B.sgn * ring_ends(b, B.n, P.par_b, in0, org.x, lane);
         if (lane == 0) P.ends[wip] = ends;
         pair_sync(g);
-        inter = (P.part[0] + P.part[1]) + 0.5 * (double)(P.ends[0] + P.ends[1]);
+        inter = ExactSum{P.q18[0] + P.q18[1], P.r56[0] + P.r56[1]}.total(P.ends[0] + P.ends[1]);
     }
     const double uni = A.area + B.area - inter;
     return uni > 0 ? fmin(fmax(inter / uni, 0.0), 1.0) : 0.0;
 }
 
-__global__ void __launch_bounds__(kRefineWarps * 32, 8)
+__global__ void __launch_bounds__(kRefineWarps * 32, 7)
 refine_pairs_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff,
                     const int64_t* __restrict__ qarea2, const int4* __restrict__ qbox,
                     const int2* __restrict__ pxy, const int64_t* __restrict__ poff,
@@ -668,18 +743,6 @@ __device__ bool build_big_lists(const int2* v, int n, int y0, int y1, int32_t* i
     sh_out = sh;
     return true;
 }
-
-// exact running sum of fp64 terms |x| < 2^44: multiples of 2^-18 and of 2^-56, modulo 2^64
-struct ExactSum {
-    unsigned long long q18 = 0, r56 = 0;
-    __device__ __forceinline__ void add(double x)
-    {
-        const long long q = __double2ll_rn(x * 262144.0);
-        const double r = fma((double)q, -1.0 / 262144.0, x);  // exact: |r| <= 2^-19
-        q18 += (unsigned long long)q;
-        r56 += (unsigned long long)__double2ll_rn(r * 72057594037927936.0);
-    }
-};
 
 __device__ __forceinline__ bool edges_cross(int2 a, int2 b, int2 c, int2 d)
 {
@@ -914,9 +977,8 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             en += __shfl_xor_sync(0xffffffffu, en, o);
-            sum.q18 += __shfl_xor_sync(0xffffffffu, sum.q18, o);
-            sum.r56 += __shfl_xor_sync(0xffffffffu, sum.r56, o);
         }
+        sum.reduce();
         if (lane == 0) {
             atomicAdd(&s.ends, en);
             atomicAdd(&s.q18, sum.q18);
@@ -924,8 +986,7 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
         }
         __syncthreads();
         if (tid == 0) {
-            const long long q18 = (long long)(s.q18 + (s.ends << 17));
-            const double inter = (double)q18 * (1.0 / 262144.0) + (double)(long long)s.r56 * (1.0 / 72057594037927936.0);
+            const double inter = ExactSum{s.q18, s.r56}.total((long long)s.ends);
             const double uni = va.area + vb.area - inter;
             out[e] = uni > 0 ? fmin(fmax(inter / uni, 0.0), 1.0) : 0.0;
         }
