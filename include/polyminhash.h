@@ -73,12 +73,11 @@ typedef struct pmh_rerank_s* pmh_rerank;
  *   flags     0 or PMH_FLAG_STREAM_INDEX | PMH_FLAG_COVERAGE_MASK */
 /* pmh_params.flags: sign through the stream index (same hashes, much less
  * work for small polygons).  The first call with a given (seed, K) builds the
- * index of the first 65,536 / 32,768 / 8,192 / 1,048,576 points of each stream,
- * bucketed by cell of a 128 x 128 / 64 x 64 / 32 x 32 / 512 x 512 grid (8 bytes
- * per point and per (cell, hash) record: about K * 11.5 MB of device memory,
+ * index of the first points of each stream, bucketed by cell of seven grids (8 x 8
+ * to 256 x 256 with half a point per cell, 512 x 512 with 1,048,576 points; 8 bytes
+ * per point and per (cell, hash): about K * 11 MB of device memory,
  * kept by the context; that call synchronises); later calls reuse it.
- * Each polygon's form (index or walk) and grid level are planned at upload from
- * its box and area. */
+ * Each polygon's form (index or walk) and grid follow from its box and area. */
 #define PMH_FLAG_STREAM_INDEX 1u
 /* pmh_params.flags: decide bounding-box candidates of the walk through a
  * precomputed per-polygon 16 x 16 coverage mask where it can (cells no edge

@@ -112,7 +112,8 @@ extern "C" int pmh_destroy(pmh_ctx ctx)
     if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
     for (cudaEvent_t e : ctx->sign_ev) cudaEventDestroy(e);
     for (int l = 0; l < kIndexLevels; ++l) {
-        if (ctx->sindex.cell[l]) cudaFree(ctx->sindex.cell[l]);
+        if (ctx->sindex.first[l]) cudaFree(ctx->sindex.first[l]);
+        if (ctx->sindex.beg[l]) cudaFree(ctx->sindex.beg[l]);
         if (ctx->sindex.ent[l]) cudaFree(ctx->sindex.ent[l]);
     }
     delete ctx;

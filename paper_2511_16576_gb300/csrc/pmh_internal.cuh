@@ -55,26 +55,23 @@ enum ScratchSlot {
     SCR_COUNT
 };
 
-// first kStreamIndexPoints points of every hash's stream, bucketed by cell of a
-// 2^kStreamGridBits-square grid (stream_index.cu); the other levels hold fewer
-// points on coarser grids or more points on a finer one (level l:
-// 2^index_level_gbits(l) cells per side, the first index_level_points(l)
-// points): 65,536 on 128^2, 32,768 on 64^2, 8,192 on 32^2 and 2^20 on 512^2
-// (about four points per (cell, hash) list on levels 0 and 3, eight on 1 and 2)
-constexpr int kStreamGridBits = 7;
-constexpr int kStreamIndexPoints = 65536;
-constexpr int kIndexLevels = 4;
-constexpr int kIndexMaxPoints = 1 << 20;  // the deepest level
-__host__ __device__ constexpr int index_level_gbits(int l) { return l == 0 ? 7 : l == 1 ? 6 : l == 2 ? 5 : 9; }
+// Stream index (stream_index.cu): per level l a 2^index_level_gbits(l)-square grid over
+// the domain (8^2 to 512^2 cells) and the first index_level_points(l) points of every
+// hash's stream bucketed by its cells: half a point per (cell, hash) on average, and
+// four on the finest level, whose polygons have no finer grid to go to.
+constexpr int kIndexLevels = 7;
+constexpr int kIndexMaxPoints = 1 << 20;  // the finest level
+__host__ __device__ constexpr int index_level_gbits(int l) { return 3 + l; }
 __host__ __device__ constexpr int index_level_points(int l)
 {
-    return l == 0 ? 65536 : l == 1 ? 32768 : l == 2 ? 8192 : kIndexMaxPoints;
+    return l == kIndexLevels - 1 ? kIndexMaxPoints : 1 << (2 * index_level_gbits(l) - 1);
 }
 // a level is built only if its entry offsets (K * points) fit in 31 bits
 __host__ __device__ constexpr bool index_level_fits(int l, int K)
 {
     return (long long)K * index_level_points(l) <= (1ll << 31);
 }
+constexpr int kWalkKernelLevel = 4;  // the level that sign_kernel's indexed form reads (128^2)
 // polygons of at most this many vertices are staged in shared memory by the
 // signing kernels; larger ones are read through their y-slab edge index
 constexpr int kStagedMaxVerts = 256;
@@ -89,19 +86,18 @@ constexpr int kChunkMinVerts = 4096;
 // under the bounding box, 32 per round of ~50 instructions, and sees about
 // lim * bbox / 2^32 candidates, with lim = 8 * 2^32 / area (a hit is then
 // missed with probability ~e^-8 and the walk resumes at lim).  Returns lim, or
-// 0 to walk.  The same function decides the class of a polygon at upload and
-// the limit in the signing kernels.
+// 0 to walk.  (sign_kernel only: polygons above the staged size, with coverage masks.)
 __host__ __device__ __forceinline__ uint32_t pmh_indexed_limit(int4 bb, long long area2)
 {
     // single precision: the estimate only picks a form and a limit (any limit
     // gives the exact result), and double precision is slow on this GPU
     if (bb.z <= bb.x || bb.w <= bb.y) return 0;
-    const int shift = 16 - kStreamGridBits;
+    const int shift = 16 - index_level_gbits(kWalkKernelLevel);
     const float area = 0.5f * (float)(area2 < 0 ? -area2 : area2);
     const float walk = 4294967296.0f / fmaxf(area, 1.0f);
     const float cells = (float)((((bb.z - 1) >> shift) - (bb.x >> shift) + 1) *
                                 (((bb.w - 1) >> shift) - (bb.y >> shift) + 1));
-    const float lim = fminf((float)kStreamIndexPoints, 8.0f * walk + 256.0f);
+    const float lim = fminf((float)index_level_points(kWalkKernelLevel), 8.0f * walk + 256.0f);
     const float cand = lim * ((float)(bb.z - bb.x) * (float)(bb.w - bb.y) * (1.0f / 4294967296.0f));
     const float walk_cost = ceilf(walk * (1.0f / 128.0f)) * 130.0f;
     const float index_cost = ceilf(cells * (1.0f / 32.0f)) * 50.0f + 40.0f;
@@ -109,100 +105,45 @@ __host__ __device__ __forceinline__ uint32_t pmh_indexed_limit(int4 bb, long lon
     return (uint32_t)lim;
 }
 
-// Cell records of the stream index, cell-major: record (cell c, hash k) is
-// cell[c * K + k]; .x = first entry of the list of (k, c), which ends where
-// record (c + 1, k) starts (row c = G*G is the end of every hash's lists);
-// .y = six 5-bit counts, bits [5t, 5t+5) = entries of the list with stream
-// index below M >> t.  The records of one cell for consecutive hashes are
-// adjacent, so a warp reading one cell for sixteen hashes reads 128 bytes.
-constexpr int kRankLevels = 6;
-// Plan of the indexed form for a polygon (sign_unified.cu),
-// in estimated warp instructions per hash.  The limit is lim = 11 * 2^32 / area (a
-// hit below it is missed with probability ~e^-11; the walk then resumes at lim),
-// capped at the shallow levels' 65,536 points where 8 * 2^32 / area fits there, and
-// at most ~24 box points below 8 * 2^32 / area are expected.  The gather first reads the
-// points below lim1 = 3.5 * 2^32 / area (an inside point exists there with
-// probability ~1 - e^-3.5); only the hashes without one read on up to lim.  On a
-// grid level holding at least lim points it costs ~4.9 per cell record under the
-// box and ~2.5 per first-pass point read (those below the smallest rank level >=
-// lim1 in those cells), plus ~20 for the mask, exact tests and setup; the walk
-// costs ~45 per round of 64 points plus ~40.  Returns lim (0 = walk), lim1 and
-// the cheapest level for each pass.  Any limit and levels give the exact result;
-// the plan only picks the cheaper work.
-struct PmhIndexPlan {
-    uint32_t lim;
-    int level;      // grid level holding every point below lim (the second pass)
-    uint32_t lim1;  // bound of the first gather pass: ~3.5 expected first hits
-    int level1;     // grid level of the first pass (holding every point below lim1)
-};
-__host__ __device__ __forceinline__ float pmh_level_cost(int4 bb, uint32_t lim1, uint32_t M, int shift)
+// Level of the indexed form for a polygon's clipped box (sign_unified.cu): the finest
+// grid that lays at most kPlanCells cells, and at most 32 a side, under the box.  Per
+// (cell, hash) the form reads one word, 128 hashes at a time, and only the points of
+// boundary cells below the hash's bound cost more, so finer cells are the cheaper ones
+// until the words read outweigh the points saved.  -1: an empty box.
+constexpr int kPlanCells = 128;
+__host__ __device__ __forceinline__ int pmh_index_level(int4 bb, int K)
 {
-    const float C = (float)((((bb.z - 1) >> shift) - (bb.x >> shift) + 1) *
-                            (((bb.w - 1) >> shift) - (bb.y >> shift) + 1));
-    uint32_t lvl = M;
-    for (int t = 1; t < 6 && (M >> t) >= lim1; ++t) lvl = M >> t;
-    const float pts = (float)lvl * C * (float)(1u << (2 * shift)) * (1.0f / 4294967296.0f);
-    return 4.9f * C + 2.5f * pts;
-}
-__host__ __device__ __forceinline__ PmhIndexPlan pmh_index_plan(int4 bb, long long area2)
-{
-    PmhIndexPlan plan{0u, 0, 0u, 0};
-    if (bb.z <= bb.x || bb.w <= bb.y) return plan;
-    const float area = 0.5f * (float)(area2 < 0 ? -area2 : area2);
-    const float walk = 4294967296.0f / fmaxf(area, 1.0f);
-    // a polygon is indexed when ~24 box points lie below 8 expected first hits; its limit
-    // is 11 of them, but not past the shallow levels' 65,536 points when 8 fit there
-    const float lim8 = 8.0f * walk + 256.0f;
-    float lim = fminf((float)kIndexMaxPoints, 11.0f * walk + 256.0f);
-    if (lim8 <= (float)kStreamIndexPoints) lim = fminf(lim, (float)kStreamIndexPoints);
-    const float box = (float)(bb.z - bb.x) * (float)(bb.w - bb.y) * (1.0f / 4294967296.0f);
-    if (fminf((float)kIndexMaxPoints, lim8) * box > 24.0f) return plan;
-    const uint32_t L = (uint32_t)lim, L1 = (uint32_t)fminf(lim, 3.5f * walk + 64.0f);
-    // the cheapest level holding every point below the bound: L for the second pass,
-    // L1 for the first (on a coarser shallow level the first pass reads a few cells
-    // where the deep level holding L would read many); the deep level (larger than
-    // L2) only for bounds the L2-resident levels cannot hold
-    float best = 3.0e38f, best1 = 3.0e38f;
-    int level = 0, level1 = 0;
-    for (int l = 0; l < kIndexLevels; ++l) {
-        const uint32_t M = (uint32_t)index_level_points(l);
-        const bool deep = M > (uint32_t)kStreamIndexPoints;
-        const float c = pmh_level_cost(bb, L1, M, 16 - index_level_gbits(l));
-        if (L <= M && !(deep && L <= (uint32_t)kStreamIndexPoints) && c < best) {
-            best = c;
-            level = l;
-        }
-        if (L1 <= M && !(deep && L1 <= (uint32_t)kStreamIndexPoints) && c < best1) {
-            best1 = c;
-            level1 = l;
-        }
+    if (bb.z <= bb.x || bb.w <= bb.y) return -1;
+    int level = 0;
+    for (int l = 1; l < kIndexLevels && index_level_fits(l, K); ++l) {
+        const int shift = 16 - index_level_gbits(l);
+        const int cx = ((bb.z - 1) >> shift) - (bb.x >> shift) + 1, cy = ((bb.w - 1) >> shift) - (bb.y >> shift) + 1;
+        if (cx > 32 || cy > 32 || cx * cy > kPlanCells) break;
+        level = l;
     }
-    const float walk_cost = ceilf(walk * (1.0f / 64.0f)) * 45.0f + 40.0f;
-    if (best1 + 20.0f >= walk_cost) return plan;
-    plan.lim = L;
-    plan.level = level;
-    plan.lim1 = L1;
-    plan.level1 = level1;
-    return plan;
+    return level;
 }
 
 struct StreamIndex {
     uint64_t seed = 0;
     int K = 0;
-    uint2* cell[kIndexLevels] = {};  // per level: [(G * G + 1) * K] records
-    uint2* ent[kIndexLevels] = {};   // per level: [K * M] (stream index, x | y << 16)
-    int ranked[kIndexLevels] = {};   // every list of the level fits the 5-bit counts
+    // rows of index_pitch(K) hashes per cell:
+    uint32_t* first[kIndexLevels] = {};  // [G * G][pitch]: 2 * the smallest index of the stream in the cell, + 1
+                                         // if the cell holds more of the level's points; all ones if none
+    uint32_t* beg[kIndexLevels] = {};    // [G * G + 1][pitch]: the first entry of (cell, hash)
+    uint2* ent[kIndexLevels] = {};       // [K * M] (stream index, x | y << 16) by (hash, cell, index)
 };
+// hashes per row of the index's tables: a multiple of four (16-byte reads)
+__host__ __device__ constexpr int index_pitch(int K) { return (K + 3) & ~3; }
 struct IndexLevelView {
-    const uint2* cell;
+    const uint32_t* first;
+    const uint32_t* beg;
     const uint2* ent;
-    int M, gbits, shift, ranked;
+    int M, gbits, shift;
 };
 struct StreamIndexView {
-    const uint2* cell;  // level 0 (nullptr: no index)
-    const uint2* ent;
-    int M, gbits, shift, ranked, K;
-    IndexLevelView lv[kIndexLevels];
+    int K, pitch;
+    IndexLevelView lv[kIndexLevels];  // lv[0].first nullptr: no index
 };
 
 struct pmh_ctx_s {
@@ -264,10 +205,9 @@ struct pmh_polys_s {
     int32_t* order = nullptr;       // polygons by expected signing cost, largest first (built
                                     // on the first signing call without the stream index)
     int32_t* order_cls = nullptr;   // class order: polygons above kChunkMinVerts vertices, then
-                                    // the other polygons signed in cost order (staged walk-form
-                                    // ones and those above kStagedMaxVerts), each by cost, then
-                                    // staged indexed-form polygons (Morton order)
-    int64_t n_indexed = 0;          // class 0: <= kStagedMaxVerts vertices, pmh_index_plan lim > 0
+                                    // the others above kStagedMaxVerts, each by cost, then the
+                                    // staged polygons (Morton order)
+    int64_t n_indexed = 0;          // class 0: <= kStagedMaxVerts vertices
     int64_t n_whole_cost = 0;       // class 1: the rest up to kChunkMinVerts vertices
     uint32_t* mask = nullptr;       // [n][16] coverage masks
 };

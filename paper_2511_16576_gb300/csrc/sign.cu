@@ -68,9 +68,10 @@ __device__ uint32_t sign_chunk_indexed(const Inside& inside, const StreamIndexVi
                                        int lane, Work& work)
 {
     const uint32_t w = (uint32_t)(bb.z - bb.x), h = (uint32_t)(bb.w - bb.y);
+    const IndexLevelView& L = S.lv[kWalkKernelLevel];
     lim = min(lim, T);
-    const int cx0 = bb.x >> S.shift, cx1 = (bb.z - 1) >> S.shift;
-    const int cy0 = bb.y >> S.shift, cy1 = (bb.w - 1) >> S.shift;
+    const int cx0 = bb.x >> L.shift, cx1 = (bb.z - 1) >> L.shift;
+    const int cy0 = bb.y >> L.shift, cy1 = (bb.w - 1) >> L.shift;
     const int ncx = cx1 - cx0 + 1, C = ncx * (cy1 - cy0 + 1);
     const int g = lane >> 3, gl = lane & 7;
     uint32_t mine = T;
@@ -80,16 +81,16 @@ __device__ uint32_t sign_chunk_indexed(const Inside& inside, const StreamIndexVi
         const int k = kb + g;
         int read = 0;
         if (k < kend) {
-            const uint2* cs = S.cell + k;  // record of cell c: cs[c * K]
+            const uint32_t* cs = L.beg + k;  // list start of cell c: cs[c * pitch]
             uint2* cb = cbuf + g * kCand;
             for (int c = gl; c < C; c += 8) {
-                const int cell = ((cy0 + c / ncx) << S.gbits) | (cx0 + c % ncx);
-                const uint32_t beg = cs[(int64_t)cell * S.K].x, end = cs[(int64_t)(cell + 1) * S.K].x;
+                const int cell = ((cy0 + c / ncx) << L.gbits) | (cx0 + c % ncx);
+                const uint32_t beg = cs[(int64_t)cell * S.pitch], end = cs[(int64_t)(cell + 1) * S.pitch];
                 for (uint32_t e = beg; e < end; e += 4) {
                     uint2 q[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
-                        q[u] = e + u < end ? S.ent[e + u] : make_uint2(0xFFFFFFFFu, 0u);
+                        q[u] = e + u < end ? L.ent[e + u] : make_uint2(0xFFFFFFFFu, 0u);
                     bool stop = false;
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
@@ -216,7 +217,7 @@ sign_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
         const int n = (int)(off[p + 1] - b);
         const int4 bb = bbox[p];
         // (with the stream index every polygon is signed by sign_unified.cu instead)
-        const uint32_t lim = area2 && S.cell && n > kSmemVerts ? pmh_indexed_limit(bb, area2[p]) : 0;
+        const uint32_t lim = area2 && S.lv[0].first && n > kSmemVerts ? pmh_indexed_limit(bb, area2[p]) : 0;
         uint32_t mine;
         if (n <= kSmemVerts) {
             // stage the vertices (closed: v[n] = v[0]; cp.async 8-byte copies), the
@@ -324,7 +325,7 @@ int pmh_launch_sign(pmh_ctx ctx, const int2* xy, const int64_t* off, const int4*
         ctx->sign_ev_used += 3;
         PMH_CUDA_TRY(cudaEventRecord(ev[0], s));
     }
-    if (S.cell && S.ranked && order_cls && area2 && !d_n && !masks) {
+    if (S.lv[0].first && order_cls && area2 && !d_n && !masks) {
         // every polygon in one launch: the class order puts the polygons above
         // kChunkMinVerts first (32-hash items), then the rest (whole polygons)
         const int U = kSignVariants[ctx->sign_variant >= 0 ? ctx->sign_variant : 0].U;
@@ -371,7 +372,7 @@ extern "C" int pmh_minhash_sign(pmh_ctx ctx, pmh_polys polys, const pmh_params* 
     const bool indexed = (params->flags & PMH_FLAG_STREAM_INDEX) != 0;
     const bool masked = (params->flags & PMH_FLAG_COVERAGE_MASK) != 0;
     if (indexed) PMH_TRY(pmh_stream_index_get(ctx, params, (cudaStream_t)stream, &sidx));
-    if ((!indexed || !sidx.ranked || masked) && !polys->order)
+    if ((!indexed || masked) && !polys->order)
         PMH_TRY(pmh_build_cost_order(polys, (cudaStream_t)stream));
     if (masked && !polys->mask) PMH_TRY(pmh_build_masks(polys, (cudaStream_t)stream));
     return pmh_launch_sign(ctx, polys->xy, polys->offsets, polys->bbox, polys->slab_info,
@@ -482,7 +483,7 @@ extern "C" int pmh_sign_autotune(pmh_ctx ctx, pmh_polys sample, const pmh_params
             const bool indexed = (params->flags & PMH_FLAG_STREAM_INDEX) != 0;
             const bool masked = (params->flags & PMH_FLAG_COVERAGE_MASK) != 0;
             if (indexed) rc = pmh_stream_index_get(ctx, params, 0, &sidx);
-            if (rc == PMH_OK && (!indexed || !sidx.ranked || masked) && !sample->order)
+            if (rc == PMH_OK && (!indexed || masked) && !sample->order)
                 rc = pmh_build_cost_order(sample, 0);
             if (rc == PMH_OK && masked && !sample->mask) rc = pmh_build_masks(sample, 0);
             if (rc == PMH_OK)

@@ -2,23 +2,24 @@
 // launch for polygons of every size, through the stream index.
 //
 // h_k(P) = min{ i : point i of stream k lies in P } is found, per polygon, in
-// the indexed form or in the walk form, as the polygon's plan says
-// (pmh_index_plan: the cheaper one by estimated warp instructions):
-//   * indexed form: every point of stream k with index below the limit L that
-//     falls in P's bounding box sits in one of the grid cells under the box
-//     (stream_index.cu), and a cell record tells how many of its points lie
-//     below each of six rank levels.  Sixteen hashes at a time, the (cell,
-//     hash) records under the box are read one per lane, and the points they
-//     hold are spread over the lanes by a warp scan (every lane loads one
-//     point, no lane walks a list).  A point in the box is classified by the
-//     polygon's 32 x 32 coverage mask: in an inside cell it is a hit and bounds
-//     the hash from above, in an outside cell it is dropped, in a boundary
-//     cell it is kept; kept points below their hash's smallest hit are tested
-//     32 at a time, one per lane (lane-local exact test).  A hash without an
-//     inside point below L (or whose kept points overflowed) walks on;
-//   * walk form: Algorithm 1 in warp rounds of 32 * U consecutive stream
-//     points; box candidates in index order (ballot + ffs), each decided by
-//     the mask or by the warp-cooperative exact test.
+// the indexed form or in the walk form:
+//   * indexed form: the cells of one grid of the stream index (stream_index.cu)
+//     under P's bounding box are classified as inside P, outside, or crossed by its
+//     boundary.  Of an inside cell only the first point of the stream in it can be
+//     the hash, and the index holds that index, so 128 hashes at a time (four a lane)
+//     the inside cells cost one 16-byte read and four minima per cell.  Of a
+//     boundary cell the first point is a candidate only if it is below the hash's
+//     bound so far -- few are, the inside cells having set a bound already.  The
+//     candidates of all lanes are queued and looked up 32 at a time (the point is
+//     recomputed from its index) in a 32 x 32 coverage mask, which decides most;
+//     the others are queued again and tested exactly 32 at a time, so that the long
+//     part runs with every lane.  An inside point lowers its hash's bound, an outside
+//     one is replaced by the next point of its cell below the bound.  A hash without
+//     a point below the level's limit walks on from there;
+//   * walk form (no index, or a very large polygon whose expected walk is short):
+//     Algorithm 1 in warp rounds of 32 * U consecutive stream points; box
+//     candidates in index order (ballot + ffs), each decided by the mask or by the
+//     warp-cooperative exact test.
 // Edge sources: a polygon of at most 256 vertices is staged in the warp's
 // shared-memory slice with its edges binned into 32 y-slabs; a larger one is
 // read from global memory through the y-slab edge lists built at upload
@@ -42,32 +43,27 @@
 
 namespace {
 
-// a kept point is packed as (hash within the group << 20 | stream index)
-constexpr int kIdxBits = 20;
-constexpr uint32_t kIdxMask = (1u << kIdxBits) - 1u;
-static_assert(kIndexMaxPoints <= (1 << kIdxBits), "point indices are packed in 20 bits");
-
 constexpr int kUniWarps = 4;       // warps per block
 constexpr int kUniMinBlocks = 8;   // resident blocks per SM the registers are sized for
-constexpr int kSub = 16;           // hashes gathered together
 constexpr int kMaskN = 32;         // coverage mask cells per side
-constexpr int kPool = 256;         // kept (boundary) points of one group of kSub hashes
-constexpr int kQueue = 64;         // exact-test queue (at most 31 + 32 entries)
+constexpr int kGroup = 128;        // hashes signed together, four a lane
+constexpr int kQueue = 192;        // candidates: at most 31, + 128 of a cell, + 32 that follow exact tests
+constexpr uint32_t kNoPoint = 0xFFFFFFFFu;
 constexpr int kIdxU = 4;           // points per lane per round of a resumed walk
 constexpr int kMaskMaxEdges = 4096;  // larger polygons skip the mask (every cell is a boundary cell)
 
-struct UniWarp {
+struct __align__(16) UniWarp {
+    uint32_t best[kGroup];   // per hash of the group: 2 * smallest inside index found (+ 1); 16-byte accesses
     int2 v[kSmemVerts + 1];  // staged vertices, v[n] = v[0]
     uint8_t ids[kSlabCap];   // staged edges by slab
     uint16_t beg[kSlabs + 1];
     int cnt[kSlabs];
     uint32_t bnd[kMaskN];    // bit i of row j: an edge touches cell (i, j)
     uint32_t inb[kMaskN];    // bit i of row j: untouched cell (i, j) lies inside
-    uint32_t best[kSub];     // per hash of the group: smallest inside index found
-    uint2 pool[kPool];       // (hash << 20 | index, x | y << 16)
-    uint2 queue[kQueue];
-    int npool;
-    uint32_t ovf;            // bit j: hash j lost kept points
+    uint32_t cell[kPlanCells];  // table rows of the inside cells (from the front) and of the boundary cells (from the back)
+    uint2 queue[kQueue];     // (depth in the cell's list << 16 | boundary cell << 7 | hash, 2 * stream index + more)
+    uint2 exact[64];         // the same, of candidates to test exactly
+    uint32_t exact_xy[64];   // x | y << 16
 };
 
 // ---------------------------------------------------------------------------
@@ -141,11 +137,20 @@ __device__ __forceinline__ bool warp_inside_src(const Src& s, int px, int py, in
     return __popc(__ballot_sync(0xffffffffu, par)) & 1;
 }
 
-__host__ __device__ __forceinline__ int mask32_log2(int w)
+// coverage mask frame of a clipped box: cells of 2^cwl x 2^chl lattice units aligned to
+// the lattice (so that the cells of any grid of the stream index with at most 32 cells a
+// side under the box are unions of mask cells), cell (0, 0) holding the box's corner
+struct MaskFrame {
+    int x0, y0, cwl, chl;
+};
+__device__ __forceinline__ MaskFrame mask_frame(int4 bb)
 {
-    int a = (w + kMaskN - 1) / kMaskN, l = 0;
-    while ((1 << l) < a) ++l;
-    return l;
+    MaskFrame f{0, 0, 0, 0};
+    while (((bb.z - 1) >> f.cwl) - (bb.x >> f.cwl) >= kMaskN) ++f.cwl;
+    while (((bb.w - 1) >> f.chl) - (bb.y >> f.chl) >= kMaskN) ++f.chl;
+    f.x0 = (bb.x >> f.cwl) << f.cwl;
+    f.y0 = (bb.y >> f.chl) << f.chl;
+    return f;
 }
 
 // one slab holding every staged edge: the exact test then reads all n edges
@@ -158,23 +163,25 @@ __device__ __forceinline__ int single_slab(UniWarp& m, int n, int lane)
     return 16;
 }
 
-// 32 x 32 coverage mask over the clipped box bb (cell (i, j): lattice points
-// bb.x + [i*cw, (i+1)*cw) by bb.y + [j*ch, (j+1)*ch)).  bnd marks every cell
+// 32 x 32 coverage mask of frame f over the clipped box bb (cell (i, j): lattice points
+// f.x0 + [i*cw, (i+1)*cw) by f.y0 + [j*ch, (j+1)*ch)).  bnd marks every cell
 // whose closed rectangle, grown by one unit on its low sides, meets an edge
 // (and possibly a few neighbours: the marking is conservative).  Every lattice
 // point of an unmarked cell (under the half-open reading, the point shifted up
 // and right by an infinitesimal) then shares the membership of the whole
 // rectangle.  Row j's unmarked cells are classified together from the edges
-// crossing the line y = bb.y + j*ch: a cell is inside iff an odd number of
-// crossings lies left of it.  A crossing lies in a marked cell of the row, at
+// crossing the line y = f.y0 + j*ch: a cell is inside iff an odd number of
+// crossings lies left of it (none does on a line below the box, which no edge
+// crosses).  A crossing lies in a marked cell of the row, at
 // least one unit left of or strictly right of every unmarked cell, so its
 // cell index -- computed in single precision, off by less than one unit --
 // never moves it across an unmarked cell, and the classification is exact.
 // Without a mask (use_mask false) every cell is a boundary cell.
 template <class Src, class W>
-__device__ __forceinline__ void build_mask(UniWarp& m, const Src& src, int n, int4 bb, int cwl,
-                                           int chl, bool use_mask, int lane, W& work)
+__device__ __forceinline__ void build_mask(UniWarp& m, const Src& src, int n, int4 bb, const MaskFrame& f,
+                                           bool use_mask, int lane, W& work)
 {
+    const int cwl = f.cwl, chl = f.chl;
     if (!use_mask) {
         m.bnd[lane] = 0xFFFFFFFFu;
         m.inb[lane] = 0u;
@@ -188,10 +195,10 @@ __device__ __forceinline__ void build_mask(UniWarp& m, const Src& src, int n, in
     for (int e = lane; e < n; e += 32) {
         const int2 a = src.vert(e), c = src.vert(e + 1);
         // rows whose grown band [j*ch - 1, (j+1)*ch] (relative) meets the edge's y-range
-        const int ylo = min(a.y, c.y) - bb.y, yhi = max(a.y, c.y) - bb.y;
+        const int ylo = min(a.y, c.y) - f.y0, yhi = max(a.y, c.y) - f.y0;
         const int j0 = max(0, ((ylo + ch - 1) >> chl) - 1);
         const int j1 = min(kMaskN - 1, (yhi + 1) >> chl);
-        const float ax = (float)(a.x - bb.x), ay = (float)(a.y - bb.y);
+        const float ax = (float)(a.x - f.x0), ay = (float)(a.y - f.y0);
         const float dx = (float)(c.x - a.x);
         const float inv_dy = c.y != a.y ? 1.0f / (float)(c.y - a.y) : 0.0f;
         for (int j = j0; j <= j1; ++j) {
@@ -212,11 +219,11 @@ __device__ __forceinline__ void build_mask(UniWarp& m, const Src& src, int n, in
         }
     }
     __syncwarp();
-    // lane j: parity of the crossings of the line y = bb.y + j*ch left of each cell
-    // (rows below the box's top only: the slab lists cover [bb.y, bb.w))
+    // lane j: parity of the crossings of the line y = f.y0 + j*ch left of each cell
+    // (lines inside the box only: the slab lists cover [bb.y, bb.w))
     uint32_t word = 0;
-    if ((lane << chl) < bb.w - bb.y) {
-        const int py = bb.y + (lane << chl);
+    const int py = f.y0 + (lane << chl);
+    if (py >= bb.y && py < bb.w) {
         int lo, hi;
         src.row(py, lo, hi);
         uint32_t par = 0;
@@ -224,7 +231,7 @@ __device__ __forceinline__ void build_mask(UniWarp& m, const Src& src, int n, in
             const int e = src.edge(t);
             const int2 a = src.vert(e), b = src.vert(e + 1);
             if ((a.y > py) != (b.y > py)) {
-                const float x = (float)(a.x - bb.x) +
+                const float x = (float)(a.x - f.x0) +
                                 (float)(b.x - a.x) * ((float)(py - a.y) / (float)(b.y - a.y));
                 const int ci = (int)floorf(x * inv_cw);
                 par ^= ci < 0 ? 0xFFFFFFFFu : (ci >= kMaskN - 1 ? 0u : (0xFFFFFFFFu << (ci + 1)));
@@ -256,20 +263,6 @@ struct MaskedWalker {
     }
 };
 
-// exact tests of queue[0 .. count), one per lane; an inside point lowers its hash's result
-template <class Src, class W>
-__device__ __forceinline__ void exact_batch(UniWarp& m, int count, const Src& src, int lane, W& work)
-{
-    if (lane < count) {
-        const uint2 c = m.queue[lane];
-        const int kl = (int)(c.x >> kIdxBits);
-        const uint32_t idx = c.x & kIdxMask;
-        if (idx < m.best[kl] && lane_inside(src, (int)(c.y & 0xFFFFu), (int)(c.y >> 16), work))
-            atomicMin(&m.best[kl], idx);
-    }
-    __syncwarp();
-}
-
 // per-lane counts of the gather (widened at the end), and the same compiled away
 struct GatherCounts {
     unsigned cells = 0, read = 0, cand = 0, masked = 0;
@@ -278,192 +271,230 @@ struct NoGather {
     Sink cells, read, cand, masked;
 };
 
-// Indexed form of hashes [k_begin, k_end) of polygon p (row `out` of the output).
+// The cells of level L under the box: inside cells to the front of m.cell, boundary
+// cells to its back (as cell * pitch).  A grid cell is a block of mask cells; it is inside
+// iff all of them are (a part outside the mask's frame is outside the box).
+__device__ __forceinline__ void classify_cells(UniWarp& m, const IndexLevelView& L, int pitch, int4 bb,
+                                               const MaskFrame& f, int& n_in, int& n_bnd, int lane)
+{
+    const unsigned full = 0xffffffffu;
+    const int cx0 = bb.x >> L.shift, cy0 = bb.y >> L.shift;
+    const int ncx = ((bb.z - 1) >> L.shift) - cx0 + 1, C = ncx * (((bb.w - 1) >> L.shift) - cy0 + 1);
+    const int cw = 1 << (L.shift - f.cwl), ch = 1 << (L.shift - f.chl);  // mask cells a side
+    n_in = n_bnd = 0;
+    for (int c0 = 0; c0 < C; c0 += 32) {
+        const int c = c0 + lane;
+        bool in = false, bnd = false;
+        uint32_t off = 0;
+        if (c < C) {
+            const int gy = c / ncx, gx = c - gy * ncx;
+            off = (uint32_t)(((cy0 + gy) << L.gbits) | (cx0 + gx)) * (uint32_t)pitch;
+            const int i0 = (((cx0 + gx) << L.shift) - f.x0) >> f.cwl, j0 = (((cy0 + gy) << L.shift) - f.y0) >> f.chl;
+            const int ia = max(i0, 0), ib = min(i0 + cw, kMaskN);
+            const uint32_t cols = (ib == 32 ? 0xFFFFFFFFu : (1u << ib) - 1u) & ~((1u << ia) - 1u);
+            uint32_t any = 0, all = cols;
+            for (int j = max(j0, 0); j < min(j0 + ch, kMaskN); ++j) {
+                const uint32_t w = m.inb[j];
+                any |= m.bnd[j] | w;
+                all &= w;
+            }
+            in = all == cols && i0 >= 0 && i0 + cw <= kMaskN && j0 >= 0 && j0 + ch <= kMaskN;
+            bnd = !in && (any & cols) != 0;
+        }
+        const unsigned bi = __ballot_sync(full, in), bb_ = __ballot_sync(full, bnd);
+        if (in) m.cell[n_in + __popc(bi & pmh_lanemask_lt())] = off;
+        if (bnd) m.cell[kPlanCells - 1 - (n_bnd + __popc(bb_ & pmh_lanemask_lt()))] = off;
+        n_in += __popc(bi);
+        n_bnd += __popc(bb_);
+    }
+    __syncwarp();
+}
+
+// Indexed form of hashes [k_begin, k_end) of polygon p (row `out` of the output).  Bound
+// by issue (the exact tests of spiky rings, the mask of every polygon) and by the latency
+// of the table reads, which stay in L2.  Against reading every point below a few expected
+// first hits from the cells under the box: 300,000 star polygons, K = 128, 5.3 ms (9.1);
+// 400,000 of the combined workload 6.4 ms (10.6).
+// A __syncwarp stands between every read of a queue and the next write to it: a vote
+// orders nothing in memory.
 template <class Src, class W, class G>
-__device__ __forceinline__ void indexed_range(UniWarp& m, const Src& src, const StreamIndexView& S,
-                                              PmhIndexPlan plan, int4 bb, uint64_t seed, uint32_t T,
+__device__ __forceinline__ void indexed_range(UniWarp& m, const Src& src, const StreamIndexView& S, int level,
+                                              int4 bb, const MaskFrame& f, float walk, uint64_t seed, uint32_t T,
                                               int k_begin, int k_end, uint32_t* __restrict__ out,
                                               int lane, W& work, G& gc)
 {
-    const unsigned full = 0xffffffffu;
+    const unsigned full = 0xffffffffu, lt = pmh_lanemask_lt();
     const uint32_t w = (uint32_t)(bb.z - bb.x), h = (uint32_t)(bb.w - bb.y);
-    const int cwl = mask32_log2((int)w), chl = mask32_log2((int)h);
-    uint32_t lim = min(plan.lim, T);
-    // grid levels of the plan's two passes (coarser ones for boxes that span many
-    // fine cells, the deep level for long walks); level 0 (second pass) or the
-    // second pass's level (first pass) where that level is not built
-    const int l2 = S.lv[plan.level].ranked && lim <= (uint32_t)S.lv[plan.level].M ? plan.level : 0;
-    lim = min(lim, (uint32_t)S.lv[l2].M);  // every point below lim is in the level's lists
-    const uint32_t lim1 = min(plan.lim1, lim);
-    const int l1 = S.lv[plan.level1].ranked && lim1 <= (uint32_t)S.lv[plan.level1].M ? plan.level1 : l2;
-    // first pass: the points below bound1 = M1 >> lev1, the smallest rank level >= lim1
-    int lev1 = 0;
-    while (lev1 + 1 < kRankLevels && ((uint32_t)S.lv[l1].M >> (lev1 + 1)) >= lim1) ++lev1;
-    const uint32_t bound1 = (uint32_t)S.lv[l1].M >> lev1;
-    // second pass: up to M2 >> lev (the smallest rank level >= lim), skipping the
-    // points below bound1 when that is a rank level of its level (else reading
-    // them again: they are outside the polygon or above their hash's bound)
-    int lev = 0;
-    while (lev + 1 < kRankLevels && ((uint32_t)S.lv[l2].M >> (lev + 1)) >= lim) ++lev;
-    int lev_skip = -1;
-    for (int t = lev; t < kRankLevels; ++t)
-        if (((uint32_t)S.lv[l2].M >> t) == bound1) lev_skip = t;
-    const bool second = ((uint32_t)S.lv[l2].M >> lev) > bound1;
-    const MaskedWalker<Src> walker{&m, src, bb.x, bb.y, cwl, chl};
-    const int hl = lane & (kSub - 1);
+    const IndexLevelView& L = S.lv[level];
+    const int pitch = S.pitch;
+    int n_in, n_bnd;
+    classify_cells(m, L, pitch, bb, f, n_in, n_bnd, lane);
+    // with few inside cells to bound the hashes, a first pass over the boundary cells keeps to
+    // the points below ~2 expected first hits: else every cell's first point would be tried
+    const uint32_t lim1 = 8 * n_in >= n_bnd ? kNoPoint : 2u * (uint32_t)fminf(2.0f * walk + 64.0f, 1.0e9f);
+    const MaskedWalker<Src> walker{&m, src, f.x0, f.y0, f.cwl, f.chl};
 
-    for (int kc = k_begin; kc < k_end; kc += kSub) {
-        const int kn = min(kSub, k_end - kc);
-        if (lane < kSub) m.best[lane] = 0xFFFFFFFFu;
-        if (lane == 0) m.ovf = 0;
-        // two passes over the cells: first the points below level lev1 (about
-        // 3.5x the expected first hit: most hashes find their answer there),
-        // then, for the hashes with no inside point yet, those up to level lev
-        uint32_t open = kn == 32 ? 0xFFFFFFFFu : ((1u << kn) - 1u);
-        for (int pass = 0; pass < 2 && lim > 0; ++pass) {
-            const int hi_lev = pass == 0 ? lev1 : lev;       // read entries below M >> hi_lev
-            const int lo_lev = pass == 0 ? -1 : lev_skip;    // ... skipping those below M >> lo_lev
-            if (pass == 1 && (!second || open == 0)) break;
-            // the pass's grid level: cells under the box, row-major; a round reads two
-            // cells for the kSub hashes of a group (lane: hash lane & 15, cell
-            // 2 * round + lane / 16)
-            const IndexLevelView& L = S.lv[pass == 0 ? l1 : l2];
-            const uint2* cells = L.cell;
-            const uint2* ents = L.ent;
-            const int gb = L.gbits, shf = L.shift;
-            const int cx0 = bb.x >> shf, cy0 = bb.y >> shf;
-            const int ncx = ((bb.z - 1) >> shf) - cx0 + 1;
-            const int C = ncx * (((bb.w - 1) >> shf) - cy0 + 1);
-            if (lane == 0) m.npool = 0;
-            __syncwarp();
-            const bool mine = hl < kn && ((open >> hl) & 1u);
-            const uint2* rec = cells + kc + hl;
-            int cx = lane >> 4, cy = 0;
-            if (cx >= ncx) {
-                cx -= ncx;
-                ++cy;
-            }
-            if (lane == 0) gc.cells += (unsigned)(C * __popc(open));
-            // the records of the next round are loaded while this round's points are read
-            uint2 rnext = make_uint2(0u, 0u);
-            if ((lane >> 4) < C && mine) rnext = rec[(int64_t)(((cy0 + cy) << gb) | (cx0 + cx)) * S.K];
-            for (int c0 = 0; c0 < C; c0 += 2) {
-                // one (hash, cell) record per lane: its points between the levels
-                const uint2 r = rnext;
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    cx += 1;
-                    if (cx >= ncx) {
-                        cx -= ncx;
-                        ++cy;
-                    }
-                }
-                rnext = make_uint2(0u, 0u);
-                if (c0 + 2 + (lane >> 4) < C && mine)
-                    rnext = rec[(int64_t)(((cy0 + cy) << gb) | (cx0 + cx)) * S.K];
-                const uint32_t below_lo = lo_lev < 0 ? 0u : (r.y >> (5 * lo_lev)) & 31u;
-                const uint32_t first = r.x + below_lo, cnt = ((r.y >> (5 * hi_lev)) & 31u) - below_lo;
-                uint32_t incl = cnt;
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const uint32_t t = __shfl_up_sync(full, incl, d);
-                    if (lane >= d) incl += t;
-                }
-                const uint32_t excl = incl - cnt;
-                const int E = (int)__shfl_sync(full, incl, 31);
-                gc.read += lane == 0 ? (unsigned)E : 0u;
-                // spread the points over the lanes: point e belongs to the last
-                // lane whose exclusive offset is <= e
-                for (int e0 = 0; e0 < E; e0 += 32) {
-                    const uint32_t e = (uint32_t)(e0 + lane);
-                    int own = 0;
-#pragma unroll
-                    for (int step = 16; step >= 1; step >>= 1)
-                        if (__shfl_sync(full, excl, own + step) <= e) own += step;
-                    const uint32_t o_first = __shfl_sync(full, first, own);
-                    const uint32_t o_excl = __shfl_sync(full, excl, own);
-                    const int o_hl = own & (kSub - 1);
-                    if ((int)e < E) {
-                        const uint2 q = ents[o_first + (e - o_excl)];
-                        const uint32_t rr = q.y;
-                        const uint32_t dx = (rr & 0xFFFFu) - (uint32_t)bb.x;
-                        const uint32_t dy = (rr >> 16) - (uint32_t)bb.y;
-                        if (q.x < lim && dx < w && dy < h) {
-                            ++gc.cand;
-                            const int i = (int)(dx >> cwl), j = (int)(dy >> chl);
-                            if ((m.bnd[j] >> i) & 1u) {
-                                const int slot = atomicAdd(&m.npool, 1);
-                                if (slot < kPool) m.pool[slot] = make_uint2(((uint32_t)o_hl << kIdxBits) | q.x, rr);
-                                else atomicOr(&m.ovf, 1u << o_hl);
-                            } else {
-                                ++gc.masked;
-                                if ((m.inb[j] >> i) & 1u) atomicMin(&m.best[o_hl], q.x);
-                            }
-                        }
-                    }
-                }
-            }
-            __syncwarp();
-            // kept points below their hash's smallest hit go to the queue, tested 32 at a time
-            const int np = min(m.npool, kPool);
-            int nq = 0;  // warp-uniform queue length
-            for (int t0 = 0; t0 < np; t0 += 32) {
-                const int t = t0 + lane;
-                uint2 c = make_uint2(0u, 0u);
-                bool keep = false;
-                if (t < np) {
-                    c = m.pool[t];
-                    keep = (c.x & kIdxMask) < m.best[c.x >> kIdxBits];
-                }
-                const unsigned bal = __ballot_sync(full, keep);
-                if (keep) m.queue[nq + __popc(bal & pmh_lanemask_lt())] = c;
-                nq += __popc(bal);
-                __syncwarp();
-                if (nq >= 32) {
-                    exact_batch(m, 32, src, lane, work);
-                    nq -= 32;
-                    const uint2 rest = lane < nq ? m.queue[32 + lane] : make_uint2(0u, 0u);
-                    __syncwarp();
-                    if (lane < nq) m.queue[lane] = rest;
-                    __syncwarp();
-                }
-            }
-            if (nq > 0) exact_batch(m, nq, src, lane, work);
-            // a hash with an inside point below the first level is final (every point
-            // below it was examined); one that lost kept points walks from the start
-            open &= __ballot_sync(full, lane < kn && m.best[lane] == 0xFFFFFFFFu) & ~m.ovf;
+    for (int kc = k_begin; kc < k_end; kc += kGroup) {
+        const int kn = min(kGroup, k_end - kc);
+        // lane: hashes 4 * vl .. 4 * vl + 3 of the group, cells sub, sub + nsub, .. (several
+        // cells at a time for few hashes)
+        const int nv = (kn + 3) >> 2, lgv = 32 - __clz(nv - 1);
+        const int nsub = 32 >> lgv, vl = lane & ((1 << lgv) - 1), sub = lane >> lgv;
+        const bool active = vl < nv;
+        const uint32_t* first = L.first + kc + 4 * (active ? vl : 0);
+        if (lane == 0) gc.cells += (unsigned)((n_in + n_bnd) * kn);
+        uint4 best = make_uint4(kNoPoint, kNoPoint, kNoPoint, kNoPoint);
+#pragma unroll 4
+        for (int i = sub; i < n_in; i += nsub) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4*>(first + m.cell[i]));
+            best.x = min(best.x, v.x);
+            best.y = min(best.y, v.y);
+            best.z = min(best.z, v.z);
+            best.w = min(best.w, v.w);
         }
-
-        // hashes without an inside point below lim resume the walk there; one
-        // that lost kept points walks from the start
-        const uint32_t overs = m.ovf;
-        unsigned todo =
-            __ballot_sync(full, lane < kn && (((overs >> lane) & 1u) || m.best[lane] == 0xFFFFFFFFu));
-        while (todo) {
-            const int j = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const uint32_t start = ((overs >> j) & 1u) ? 0u : lim;
-            uint32_t hk = T;
-            if (start < T) {
-                const uint64_t sk = pmh_mix64(seed + (uint64_t)(kc + j + 1) * PMH_GAMMA);
-                hk = sign_one_t<kIdxU>(walker, bb.x, bb.y, w, h, sk, T, lane, work, start);
-            }
-            if (lane == 0) m.best[j] = hk;
+        for (int o = 1 << lgv; o < 32; o <<= 1) {
+            best.x = min(best.x, __shfl_xor_sync(full, best.x, o));
+            best.y = min(best.y, __shfl_xor_sync(full, best.y, o));
+            best.z = min(best.z, __shfl_xor_sync(full, best.z, o));
+            best.w = min(best.w, __shfl_xor_sync(full, best.w, o));
+        }
+        if (sub == 0) {
+            m.best[4 * vl] = best.x;
+            m.best[4 * vl + 1] = best.y;
+            m.best[4 * vl + 2] = best.z;
+            m.best[4 * vl + 3] = best.w;
         }
         __syncwarp();
-        if (lane < kn) out[kc + lane] = m.best[lane];
+        uint32_t bound = lim1;
+        bool open = active;
+        int nq = 0, nx = 0;  // queued candidates, queued exact tests
+        const uint4 none = make_uint4(kNoPoint, kNoPoint, kNoPoint, kNoPoint);
+        // an inside point bounds its hash; an outside one is followed by the next of its cell, if
+        // that is still below the hash's bound
+        auto settle = [&](uint2 c, bool inside, bool fail) {
+            if (inside) atomicMin(&m.best[c.x & 127u], c.y);
+            bool again = false;
+            if (fail && (c.y & 1u)) {
+                const uint32_t row = m.cell[kPlanCells - 1 - (int)((c.x >> 7) & 127u)] + (uint32_t)kc + (c.x & 127u);
+                const uint32_t e = L.beg[row] + (c.x >> 16) + 1u, end = L.beg[row + (uint32_t)pitch];
+                c = make_uint2(c.x + 0x10000u, 2u * L.ent[e].x + (e + 1u < end));
+                again = c.y < min(m.best[c.x & 127u], bound);
+                ++gc.read;
+            }
+            const unsigned bal = __ballot_sync(full, again);
+            if (again) m.queue[nq + __popc(bal & lt)] = c;
+            nq += __popc(bal);
+            __syncwarp();
+        };
+        for (int i0 = 0;;) {
+            if (i0 < n_bnd) {
+                const int i = i0 + sub;
+                const uint4 v = open && i < n_bnd
+                                    ? __ldg(reinterpret_cast<const uint4*>(first + m.cell[kPlanCells - 1 - i]))
+                                    : none;
+                const uint32_t tag = (uint32_t)(i << 7 | 4 * vl);
+                const uint32_t vv[4] = {v.x, v.y, v.z, v.w};
+                const uint32_t bb4[4] = {best.x, best.y, best.z, best.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool cand = vv[u] < min(bb4[u], bound);
+                    const unsigned bal = __ballot_sync(full, cand);
+                    if (cand) m.queue[nq + __popc(bal & lt)] = make_uint2(tag + u, vv[u]);
+                    nq += __popc(bal);
+                }
+                i0 += nsub;
+                __syncwarp();
+            }
+            const bool scanned = i0 >= n_bnd;
+            for (;;) {
+                if (nx < 32 && (nq >= 32 || (scanned && nq > 0))) {
+                    // look 32 candidates up
+                    const int count = min(nq, 32);
+                    nq -= count;
+                    uint2 c = make_uint2(0u, kNoPoint);
+                    uint32_t r = 0;
+                    bool inside = false, fail = false, boundary = false;
+                    if (lane < count) c = m.queue[nq + lane];
+                    __syncwarp();
+                    if (c.y < m.best[c.x & 127u]) {
+                        const uint64_t sk = pmh_mix64(seed + (uint64_t)((uint32_t)kc + (c.x & 127u) + 1u) * PMH_GAMMA);
+                        r = pmh_mix64_lo(sk + (uint64_t)((c.y >> 1) + 1u) * PMH_GAMMA);
+                        const int px = (int)(r & 0xFFFFu), py = (int)(r >> 16);
+                        fail = true;
+                        if ((uint32_t)(px - bb.x) < w && (uint32_t)(py - bb.y) < h) {
+                            ++gc.cand;
+                            const int i = (px - f.x0) >> f.cwl, j = (py - f.y0) >> f.chl;
+                            boundary = (m.bnd[j] >> i) & 1u;
+                            inside = !boundary && ((m.inb[j] >> i) & 1u);
+                            fail = !boundary && !inside;
+                            gc.masked += boundary ? 0u : 1u;
+                        }
+                    }
+                    const unsigned bal = __ballot_sync(full, boundary);
+                    if (boundary) {
+                        m.exact[nx + __popc(bal & lt)] = c;
+                        m.exact_xy[nx + __popc(bal & lt)] = r;
+                    }
+                    nx += __popc(bal);
+                    settle(c, inside, fail);
+                } else if (nx >= 32 || (scanned && nx > 0)) {
+                    // test 32 exactly
+                    const int count = min(nx, 32);
+                    nx -= count;
+                    uint2 c = make_uint2(0u, kNoPoint);
+                    uint32_t r = 0;
+                    bool inside = false, fail = false;
+                    if (lane < count) {
+                        c = m.exact[nx + lane];
+                        r = m.exact_xy[nx + lane];
+                    }
+                    if (c.y < m.best[c.x & 127u]) {
+                        inside = lane_inside(src, (int)(r & 0xFFFFu), (int)(r >> 16), work);
+                        fail = !inside;
+                    }
+                    __syncwarp();
+                    settle(c, inside, fail);
+                } else {
+                    break;
+                }
+            }
+            best = make_uint4(m.best[4 * vl], m.best[4 * vl + 1], m.best[4 * vl + 2], m.best[4 * vl + 3]);
+            if (!scanned) continue;
+            // a hash with an inside point below the bound is final: every point below it was
+            // tried; the others take a second pass without one
+            if (bound == kNoPoint) break;
+            open = active && max(max(best.x, best.y), max(best.z, best.w)) >= bound;
+            if (!__any_sync(full, open)) break;
+            bound = kNoPoint;
+            i0 = 0;
+        }
+
+        // hashes without an inside point below the level's limit walk on from there
+        for (int j0 = 0; j0 < kn; j0 += 32) {
+            uint32_t v = j0 + lane < kn ? m.best[j0 + lane] : 0u;
+            unsigned todo = __ballot_sync(full, v == kNoPoint && (uint32_t)L.M < T);
+            v = v == kNoPoint ? T : min(v >> 1, T);
+            while (todo) {
+                const int j = __ffs(todo) - 1;
+                todo &= todo - 1;
+                const uint64_t sk = pmh_mix64(seed + (uint64_t)(kc + j0 + j + 1) * PMH_GAMMA);
+                const uint32_t hk = sign_one_t<kIdxU>(walker, bb.x, bb.y, w, h, sk, T, lane, work, (uint32_t)L.M);
+                if (lane == j) v = hk;
+            }
+            if (j0 + lane < kn) out[kc + j0 + lane] = v;
+        }
         __syncwarp();
     }
 }
 
 // Walk form of hashes [k_begin, k_end): lane j keeps hash k0 + j of each 32.
 template <int U, class Src, class W>
-__device__ __forceinline__ void walk_range(const UniWarp& m, const Src& src, int4 bb, uint64_t seed,
+__device__ __forceinline__ void walk_range(const UniWarp& m, const Src& src, int4 bb, const MaskFrame& f, uint64_t seed,
                                            uint32_t T, int k_begin, int k_end,
                                            uint32_t* __restrict__ out, int lane, W& work)
 {
     const uint32_t w = (uint32_t)(bb.z - bb.x), h = (uint32_t)(bb.w - bb.y);
-    const MaskedWalker<Src> walker{&m, src, bb.x, bb.y, mask32_log2((int)w), mask32_log2((int)h)};
+    const MaskedWalker<Src> walker{&m, src, f.x0, f.y0, f.cwl, f.chl};
     for (int k0 = k_begin; k0 < k_end; k0 += 32) {
         const int kend = min(k_end, k0 + 32);
         uint32_t mine = T;
@@ -479,12 +510,12 @@ __device__ __forceinline__ void walk_range(const UniWarp& m, const Src& src, int
 // Walk form of a staged polygon, kept out of line so that its registers do not
 // weigh on the indexed form's gather (Work by pointer: a local copy inside).
 template <int U, class W>
-__device__ __noinline__ void walk_staged(const UniWarp& m, StagedSrc src, int4 bb, uint64_t seed,
+__device__ __noinline__ void walk_staged(const UniWarp& m, StagedSrc src, int4 bb, MaskFrame f, uint64_t seed,
                                          uint32_t T, int k_begin, int k_end, uint32_t* out,
                                          int lane, W* work)
 {
     W local;
-    walk_range<U>(m, src, bb, seed, T, k_begin, k_end, out, lane, local);
+    walk_range<U>(m, src, bb, f, seed, T, k_begin, k_end, out, lane, local);
     work->walk += local.walk;
     work->cand += local.cand;
     work->edges += local.edges;
@@ -495,19 +526,20 @@ __device__ __noinline__ void walk_staged(const UniWarp& m, StagedSrc src, int4 b
 // A polygon above the staged size (read from global memory): the mask, then the
 // planned form, out of line for the same reason.
 template <int U, class W, class G>
-__device__ __noinline__ void sign_global(UniWarp& m, GlobalSrc src, int n, int4 bb, PmhIndexPlan plan,
+__device__ __noinline__ void sign_global(UniWarp& m, GlobalSrc src, int n, int4 bb, int level, float walk,
                                          const StreamIndexView& S, uint64_t seed, uint32_t T,
                                          int k_begin, int k_end, uint32_t* out, int lane, W* work,
                                          G* gc)
 {
     W local;
     G g;
-    build_mask(m, src, n, bb, mask32_log2(bb.z - bb.x), mask32_log2(bb.w - bb.y), n <= kMaskMaxEdges,
-               lane, local);
-    if (plan.lim > 0)
-        indexed_range(m, src, S, plan, bb, seed, T, k_begin, k_end, out, lane, local, g);
+    const MaskFrame f = mask_frame(bb);
+    build_mask(m, src, n, bb, f, n <= kMaskMaxEdges, lane, local);
+    // (without a mask every cell is a boundary cell: a walk of few rounds is cheaper)
+    if (level >= 0 && (n <= kMaskMaxEdges || walk > 1024.0f))
+        indexed_range(m, src, S, level, bb, f, walk, seed, T, k_begin, k_end, out, lane, local, g);
     else
-        walk_range<U>(m, src, bb, seed, T, k_begin, k_end, out, lane, local);
+        walk_range<U>(m, src, bb, f, seed, T, k_begin, k_end, out, lane, local);
     work->walk += local.walk;
     work->cand += local.cand;
     work->edges += local.edges;
@@ -577,25 +609,27 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
             for (int k = k_begin + lane; k < k_end; k += 32) row[k] = T;
             continue;
         }
-        // the form (indexed or walk) and grid level the polygon's cost model picks
-        const PmhIndexPlan plan = (S.cell && area2) ? pmh_index_plan(bb, area2[p]) : PmhIndexPlan{0u, 0, 0u, 0};
+        // the indexed form's grid level (-1: no index) and the expected walk
+        const int level = S.lv[0].first && area2 ? pmh_index_level(bb, K) : -1;
+        const long long a2 = area2 ? area2[p] : 0;
+        const float walk = 4294967296.0f / fmaxf(0.5f * (float)(a2 < 0 ? -a2 : a2), 1.0f);
         if (staged) {
             // stage the polygon (closed: v[n] = v[0]; cp.async 8-byte copies) and bin its edges
             stage_vertices(m.v, xy + b, n, lane);
             int sh = staged_slab_shift(bb.w - bb.y);
             if (!build_staged_slabs(m.v, n, bb.y, sh, m.ids, m.beg, m.cnt, lane)) sh = single_slab(m, n, lane);
             const StagedSrc src{m.v, m.ids, m.beg, bb.y, sh};
-            build_mask(m, src, n, bb, mask32_log2(bb.z - bb.x), mask32_log2(bb.w - bb.y), true, lane,
-                       work);
-            if (kIndexedOnly || plan.lim > 0)
-                indexed_range(m, src, S, plan, bb, seed, T, k_begin, k_end, row, lane, work, gc);
+            const MaskFrame f = mask_frame(bb);
+            build_mask(m, src, n, bb, f, true, lane, work);
+            if (kIndexedOnly || level >= 0)
+                indexed_range(m, src, S, level, bb, f, walk, seed, T, k_begin, k_end, row, lane, work, gc);
             else
-                walk_staged<U, W>(m, src, bb, seed, T, k_begin, k_end, row, lane, &work);
+                walk_staged<U, W>(m, src, bb, f, seed, T, k_begin, k_end, row, lane, &work);
         } else if (!kIndexedOnly) {
             const SlabInfo si = slabs ? slabs[p] : SlabInfo{0, 0, 0, 1, 0};
             const GlobalSrc src{xy + b, n, si.S > 0 ? slab_ptr + si.slab_base : nullptr,
                                 si.S > 0 ? slab_edges + si.edge_base : nullptr, si.slab_h, si.ymin};
-            sign_global<U, W, G>(m, src, n, bb, plan, S, seed, T, k_begin, k_end, row, lane, &work, &gc);
+            sign_global<U, W, G>(m, src, n, bb, level, walk, S, seed, T, k_begin, k_end, row, lane, &work, &gc);
         }
         __syncwarp();
     }

@@ -230,11 +230,10 @@ __device__ __forceinline__ uint32_t morton16(uint32_t x, uint32_t y)
 
 // class key: polygons of more than kChunkMinVerts vertices (class 2) first, by
 // decreasing expected cost -- the signing launch splits them into 32-hash items
-// and starts the longest first -- then the staged polygons of the walk form and
-// the polygons above kStagedMaxVerts (class 1), by decreasing expected cost,
-// then staged polygons of the indexed form (class 0) in Morton order of their
-// box centres -- warps running at the same time then read nearby cells of the
-// stream index, which keeps them in L2; counts classes 0 and 1 into n_cls[0],
+// and starts the longest first -- then the others above kStagedMaxVerts (class 1),
+// by decreasing expected cost, then the staged polygons (class 0) in Morton order
+// of their box centres -- warps running at the same time then read nearby cells of
+// the stream index, which keeps them in L2; counts classes 0 and 1 into n_cls[0],
 // n_cls[1]
 __global__ void class_key_kernel(const int4* __restrict__ bbox, const int64_t* __restrict__ area2,
                                  const int64_t* __restrict__ off, int64_t n,
@@ -249,8 +248,7 @@ __global__ void class_key_kernel(const int4* __restrict__ bbox, const int64_t* _
         const float cost = 8589934592.0f / fmaxf(aa, 1.0f);
         const int4 bb = bbox[p];
         const int64_t nv = off[p + 1] - off[p];
-        const int cls = nv > kChunkMinVerts ? 2
-                        : (nv > kStagedMaxVerts || pmh_index_plan(bb, a).lim == 0) ? 1 : 0;
+        const int cls = nv > kChunkMinVerts ? 2 : nv > kStagedMaxVerts ? 1 : 0;
         uint32_t key;
         if (cls == 0) {
             const uint32_t cx = (uint32_t)min((bb.x + bb.z) >> 1, 65535);

@@ -4,18 +4,17 @@
 // Every polygon draws from the same K point streams (Sec. 3.2: fixed seeds per
 // hash function), so the points themselves can be indexed once: for each hash
 // k the points i < M are sorted (stably) by their cell in a G x G grid over the
-// domain.  A polygon then reads only the cells under its bounding box, and in
-// each cell only the points below an index limit L; the smallest such index
-// whose point lies in the polygon is h_k exactly, because every point of the
-// stream with index < L that lies in the bounding box is in one of those
-// cells.  If no point below L hits, the ordinary walk continues from L.
+// domain.  In a cell that lies inside a polygon only the cell's first point can
+// be the hash, and in a cell that the boundary crosses only its points below the
+// smallest one known to be inside; the smallest index found that way is h_k
+// exactly if it is below M, because every point of the stream with index < M is
+// in one of the cells.  If there is none, the ordinary walk continues from M.
 //
-// Layout: the entries are sorted by (hash k, cell c, stream index); entry e =
-// (stream index, x | y << 16), one 8-byte load.  The list of (k, c) is
-// [cell[c*K + k].x, cell[(c+1)*K + k].x) (cell-major records).  cell[.].y holds
-// six 5-bit counts: the entries of the list below M, M/2, ..., M/32, so that a
-// reader with limit L knows how many entries to read (those below the smallest
-// level >= L) without reading past them.
+// Layout: rows of P = K rounded up to four per cell; first[c * P + k] = 2 * smallest
+// index of the list of (k, c), + 1 if the list goes on (all ones if it is empty): a warp
+// reads one cell's words for 128 consecutive hashes as 512 bytes.  The entries are
+// sorted by (hash k, cell c, stream index); entry e = (stream index, x | y << 16), one
+// 8-byte load.  The list of (k, c) is [beg[c*P + k], beg[(c+1)*P + k]).
 #include <algorithm>
 
 #include "pmh_internal.cuh"
@@ -59,48 +58,49 @@ __global__ void finish_index_kernel(const uint32_t* __restrict__ keys, const int
     }
 }
 
-// cell records (cell-major) from the k-major list starts: start and the rank
-// counts of each level; row G*G holds each hash's end.  *longest = longest list
+// list starts and first indexes (cell-major) from the k-major list starts; row G*G of beg
+// holds each hash's end
 __global__ void cell_record_kernel(const int64_t* __restrict__ starts, int K, int gbits,
-                                   const uint2* __restrict__ ent, int M, uint2* __restrict__ cell,
-                                   int* __restrict__ longest)
+                                   const uint2* __restrict__ ent, uint32_t* __restrict__ beg,
+                                   uint32_t* __restrict__ first)
 {
     const int64_t GG = (int64_t)1 << (2 * gbits);
-    const int64_t n_cells = GG * K;
-    int mine = 0;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_cells;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = c >> (2 * gbits), cl = c & (GG - 1);
-        const uint32_t b = (uint32_t)starts[c], e = (uint32_t)starts[c + 1];
-        mine = max(mine, (int)(e - b));
-        uint32_t counts = 0;
-        for (int t = 0; t < kRankLevels; ++t) {
-            const uint32_t level = (uint32_t)M >> t;
-            uint32_t cnt = 0;
-            for (uint32_t i = b; i < e && ent[i].x < level; ++i) ++cnt;
-            counts |= min(cnt, 31u) << (5 * t);
+    const int P = index_pitch(K);
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < GG * P;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t cl = t / P, k = t - cl * P;
+        uint32_t b = 0, e = 0, f = 0xFFFFFFFFu;
+        if (k < K) {  // (the row's padding holds empty lists)
+            const int64_t c = (k << (2 * gbits)) + cl;
+            b = (uint32_t)starts[c];
+            e = (uint32_t)starts[c + 1];
+            if (b < e) f = 2u * ent[b].x + (e - b > 1u);
         }
-        cell[cl * K + k] = make_uint2(b, counts);
-        if (cl == GG - 1) cell[GG * K + k] = make_uint2(e, 0u);
+        beg[t] = b;
+        first[t] = f;
+        if (cl == GG - 1) beg[GG * P + k] = e;
     }
-    if (mine) atomicMax(longest, mine);
 }
 
 }  // namespace
 
 // One level: the first M points of every hash's stream on a 2^gbits-square grid.
-// Allocates *cell and *ent; on failure frees what it allocated.
+// Allocates *first, *beg and *ent; on failure frees what it allocated.
 static int build_level(pmh_ctx ctx, const pmh_params* P, cudaStream_t s, int M, int gbits,
-                       uint2** cell_out, uint2** ent_out, int* ranked)
+                       uint32_t** first_out, uint32_t** beg_out, uint2** ent_out)
 {
     const int shift = 16 - gbits;
     const int64_t n = (int64_t)P->K * M;
     const int64_t n_cells = (int64_t)P->K << (2 * gbits);
-    uint2 *cell = nullptr, *ent = nullptr;
-    if (cudaMalloc(&cell, sizeof(uint2) * (n_cells + P->K)) != cudaSuccess ||
+    const int64_t rows = 1ll << (2 * gbits), pitch = index_pitch((int)P->K);
+    uint32_t *first = nullptr, *beg = nullptr;
+    uint2* ent = nullptr;
+    if (cudaMalloc(&first, sizeof(uint32_t) * rows * pitch) != cudaSuccess ||
+        cudaMalloc(&beg, sizeof(uint32_t) * (rows + 1) * pitch) != cudaSuccess ||
         cudaMalloc(&ent, sizeof(uint2) * n) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(cell);
+        cudaFree(first);
+        cudaFree(beg);
         cudaFree(ent);
         return pmh_set_error(PMH_ERR_NOMEM, "stream index allocation failed");
     }
@@ -109,15 +109,15 @@ static int build_level(pmh_ctx ctx, const pmh_params* P, cudaStream_t s, int M, 
     int64_t* counts = nullptr;
     if (cudaMalloc(&keys, sizeof(uint32_t) * n) != cudaSuccess ||
         cudaMalloc(&vals, sizeof(int32_t) * n) != cudaSuccess ||
-        cudaMalloc(&counts, sizeof(int64_t) * (n_cells + 2)) != cudaSuccess) {
+        cudaMalloc(&counts, sizeof(int64_t) * (n_cells + 1)) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(keys);
         cudaFree(vals);
-        cudaFree(cell);
+        cudaFree(first);
+        cudaFree(beg);
         cudaFree(ent);
         return pmh_set_error(PMH_ERR_NOMEM, "stream index scratch allocation failed");
     }
-    int* longest = reinterpret_cast<int*>(counts + n_cells + 1);
     int rc = PMH_OK;
     const int blocks = ctx->sm_count * 16;
     stream_points_kernel<<<blocks, 256, 0, s>>>(P->seed, (int)P->K, M, shift, gbits, keys, vals);
@@ -127,7 +127,7 @@ static int build_level(pmh_ctx ctx, const pmh_params* P, cudaStream_t s, int M, 
     int key_bits = 2 * gbits;
     while ((1ll << key_bits) < (int64_t)P->K << (2 * gbits)) ++key_bits;
     if (rc == PMH_OK) rc = pmh_radix_sort_u32(ctx, keys, vals, n, key_bits, s);
-    if (rc == PMH_OK && cudaMemsetAsync(counts, 0, sizeof(int64_t) * (n_cells + 2), s) != cudaSuccess)
+    if (rc == PMH_OK && cudaMemsetAsync(counts, 0, sizeof(int64_t) * (n_cells + 1), s) != cudaSuccess)
         rc = pmh_set_error(PMH_ERR_CUDA, "memset failed");
     if (rc == PMH_OK) {
         cell_count_kernel<<<blocks, 256, 0, s>>>(keys, n, counts);
@@ -137,29 +137,26 @@ static int build_level(pmh_ctx ctx, const pmh_params* P, cudaStream_t s, int M, 
     if (rc == PMH_OK) {
         finish_index_kernel<<<blocks, 256, 0, s>>>(keys, vals, n, P->seed, gbits, ent);
         g_pmh_launches.fetch_add(1);
-        cell_record_kernel<<<blocks, 256, 0, s>>>(counts, (int)P->K, gbits, ent, M, cell, longest);
+        cell_record_kernel<<<blocks, 256, 0, s>>>(counts, (int)P->K, gbits, ent, beg, first);
         g_pmh_launches.fetch_add(1);
         e = cudaGetLastError();
         if (e != cudaSuccess) rc = pmh_set_error(PMH_ERR_CUDA, "finish: %s", cudaGetErrorString(e));
     }
-    if (rc == PMH_OK && cudaMemcpyAsync(ctx->h_pinned, longest, sizeof(int), cudaMemcpyDeviceToHost, s) !=
-                            cudaSuccess)
-        rc = pmh_set_error(PMH_ERR_CUDA, "stream index: copy failed");
     cudaError_t e2 = cudaStreamSynchronize(s);
-    const int longest_list = rc == PMH_OK ? (int)*reinterpret_cast<int*>(ctx->h_pinned) : 0;
     cudaFree(keys);
     cudaFree(vals);
     cudaFree(counts);
     if (rc == PMH_OK && e2 != cudaSuccess)
         rc = pmh_set_error(PMH_ERR_CUDA, "stream index build: %s", cudaGetErrorString(e2));
     if (rc != PMH_OK) {
-        cudaFree(cell);
+        cudaFree(first);
+        cudaFree(beg);
         cudaFree(ent);
         return rc;
     }
-    *cell_out = cell;
+    *first_out = first;
+    *beg_out = beg;
     *ent_out = ent;
-    *ranked = longest_list <= 31;  // else the counts saturate: only the list ends are used
     return PMH_OK;
 }
 
@@ -167,22 +164,18 @@ static StreamIndexView view_of(const StreamIndex& si)
 {
     StreamIndexView v{};
     for (int l = 0; l < kIndexLevels; ++l)
-        v.lv[l] = IndexLevelView{si.cell[l], si.ent[l], index_level_points(l), index_level_gbits(l),
-                                 16 - index_level_gbits(l), si.ranked[l]};
-    v.cell = si.cell[0];
-    v.ent = si.ent[0];
-    v.M = index_level_points(0);
-    v.gbits = index_level_gbits(0);
-    v.shift = 16 - index_level_gbits(0);
-    v.ranked = si.ranked[0];
+        v.lv[l] = IndexLevelView{si.first[l], si.beg[l], si.ent[l], index_level_points(l), index_level_gbits(l),
+                                 16 - index_level_gbits(l)};
     v.K = si.K;
+    v.pitch = index_pitch(si.K);
     return v;
 }
 
 static void free_index(StreamIndex& si)
 {
     for (int l = 0; l < kIndexLevels; ++l) {
-        cudaFree(si.cell[l]);
+        cudaFree(si.first[l]);
+        cudaFree(si.beg[l]);
         cudaFree(si.ent[l]);
     }
     si = StreamIndex();
@@ -191,20 +184,20 @@ static void free_index(StreamIndex& si)
 int pmh_stream_index_get(pmh_ctx ctx, const pmh_params* P, cudaStream_t s, StreamIndexView* out)
 {
     StreamIndex& si = ctx->sindex;
-    if (si.cell[0] && si.seed == P->seed && si.K == (int)P->K) {
+    if (si.first[0] && si.seed == P->seed && si.K == (int)P->K) {
         *out = view_of(si);
         return PMH_OK;
     }
-    if (si.cell[0]) {
+    if (si.first[0]) {
         cudaDeviceSynchronize();
         free_index(si);
     }
     StreamIndex fresh;
     int rc = PMH_OK;
     for (int l = 0; l < kIndexLevels && rc == PMH_OK; ++l)
-        if (l == 0 || index_level_fits(l, (int)P->K))  // level 0 always fits (K <= 4096)
-            rc = build_level(ctx, P, s, index_level_points(l), index_level_gbits(l), &fresh.cell[l],
-                             &fresh.ent[l], &fresh.ranked[l]);
+        if (index_level_fits(l, (int)P->K))  // (all but the finest always do: K <= 4096)
+            rc = build_level(ctx, P, s, index_level_points(l), index_level_gbits(l), &fresh.first[l],
+                             &fresh.beg[l], &fresh.ent[l]);
     if (rc != PMH_OK) {
         free_index(fresh);
         return rc;

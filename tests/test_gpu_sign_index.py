@@ -1,0 +1,51 @@
+"""Signing through the stream index (A1): the counter-free kernels that production calls run against
+the counting build (which the other tests run) and the oracle, over the forms of the index."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2511_16576_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda", 0)
+SEED = 0x5EED
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2511_16576_gb300 import binding
+    binding.load()
+    return binding
+
+
+# every cell crossed by the boundary (finest grid, two passes) / most cells inside / spiky rings
+# with long slab lists / rings above 256 and above 4,096 vertices
+SHAPES = {
+    "smallest": dict(n=20_000, n_range=(4, 40), n_dist="loguniform", f_range=(1e-5, 5e-5)),
+    "combined": dict(n=20_000, n_range=(8, 1024), n_dist="loguniform", f_range=(1e-5, 1e-2), fractal=True,
+                     comonotone=True),
+    "stars": dict(n=8000, n_range=(16, 256), n_dist="loguniform", f_range=(1e-4, 1e-2)),
+    "large": dict(n=300, n_range=(200, 20_000), n_dist="loguniform", f_range=(1e-3, 1e-1), fractal=True,
+                  comonotone=True),
+}
+
+
+@pytest.mark.parametrize("shape", list(SHAPES))
+@pytest.mark.parametrize("K", [128, 3, 37, 300])
+def test_production_hashes(B, orc, shape, K):
+    kw = dict(SHAPES[shape])
+    n = max(64, kw.pop("n") * 32 // max(K, 32))
+    db = synth.star_polygons(n, 61 + K, **kw)
+    ctx = B.Context(0)
+    P = B.make_params(K, 1, 1 << 24, SEED, flags=B.FLAG_STREAM_INDEX)
+    polys = B.poly_upload(ctx, torch.from_numpy(db.xy).to(DEV), torch.from_numpy(db.offsets).to(DEV))
+    counted = B.minhash_sign(ctx, polys, P)
+    B.sign_count_work(ctx, False)
+    for _ in range(3):
+        assert torch.equal(B.minhash_sign(ctx, polys, P), counted)
+    rows = np.unique(np.concatenate([np.argsort(np.diff(db.offsets))[-2:],
+                                     np.random.default_rng(K).choice(db.n, 24, replace=False)]))
+    sub = db.subset(rows)
+    ref = orc.sign(sub.xy, sub.offsets, SEED, K, 1 << 24, nthreads=16)
+    assert np.array_equal(counted[torch.from_numpy(rows).to(DEV)].cpu().numpy().view(np.uint32), ref)
+    ctx.close()
