@@ -88,6 +88,7 @@ extern "C" int pmh_create(pmh_ctx* out, int device)
     c->sm_count = prop.multiProcessorCount;
     if (cudaMalloc(&c->d_status, 64 * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&c->d_tickets, 64 * sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMalloc(&c->walks, sizeof(WalkItem) * kWalkItems) != cudaSuccess ||
         cudaMallocHost(&c->h_pinned, 64 * sizeof(int64_t)) != cudaSuccess) {
         cudaGetLastError();
         pmh_destroy(c);
@@ -109,6 +110,7 @@ extern "C" int pmh_destroy(pmh_ctx ctx)
         if (ctx->scratch[i]) cudaFree(ctx->scratch[i]);
     if (ctx->d_status) cudaFree(ctx->d_status);
     if (ctx->d_tickets) cudaFree(ctx->d_tickets);
+    if (ctx->walks) cudaFree(ctx->walks);
     if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
     for (cudaEvent_t e : ctx->sign_ev) cudaEventDestroy(e);
     for (int l = 0; l < kIndexLevels; ++l) {

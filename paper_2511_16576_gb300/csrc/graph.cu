@@ -41,6 +41,7 @@ struct pmh_qgraph_s {
     int32_t* slab_cursor = nullptr;
     int32_t* slab_edges = nullptr;
     SlabPtrs* d_slabs = nullptr;
+    WalkItem* walks = nullptr;        // leftover walks of the batch's signing
     int32_t* ref_queue = nullptr;     // pairs of large rings (nullable)
     int64_t cap_ptr = 0, cap_edges = 0;
     int64_t* counts = nullptr;
@@ -68,7 +69,7 @@ struct pmh_qgraph_s {
     double* ref_j = nullptr;
     int* flags = nullptr;
     int64_t* d_n = nullptr;
-    unsigned long long* ticket = nullptr;  // [4]: signing grid, refinement grids
+    unsigned long long* ticket = nullptr;  // [8]: refinement grids at 1, signing at 4
     int64_t* scan_sums = nullptr;
     const uint32_t* sidx_first = nullptr;  // the stream index the graph captured (nullptr: none)
     int64_t kernels = 0;               // kernel launches per replay
@@ -96,7 +97,7 @@ extern "C" int pmh_qgraph_destroy(pmh_qgraph g)
                     g->flags,     g->d_n,        g->ticket,     g->scan_sums, g->sl_ids,
                     g->sl_n,      g->sl_counts,  g->sl_sums,    g->sl_row_ptr, g->sl_cand,
                     g->qfeat,     g->feat,       g->score,     g->join_stage,
-                    g->d_slabs,   g->ref_queue};
+                    g->d_slabs,   g->ref_queue,  g->walks};
     for (void* b : bufs)
         if (b) cudaFree(b);
     delete g;
@@ -187,7 +188,8 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
                           cudaMalloc(&g->ref_j, sizeof(double) * Q * k) == cudaSuccess)) &&
               cudaMalloc(&g->flags, sizeof(int) * 4) == cudaSuccess &&
               cudaMalloc(&g->d_n, sizeof(int64_t)) == cudaSuccess &&
-              cudaMalloc(&g->ticket, 4 * sizeof(unsigned long long)) == cudaSuccess &&
+              cudaMalloc(&g->ticket, 8 * sizeof(unsigned long long)) == cudaSuccess &&
+              cudaMalloc(&g->walks, sizeof(WalkItem) * kWalkItems) == cudaSuccess &&
               cudaMalloc(&g->d_slabs, sizeof(SlabPtrs)) == cudaSuccess &&
               // (a batch of a few small queries against small polygons has no large ring; a set
               // reloaded with larger ones is still refined, by the two-warp form)
@@ -222,7 +224,7 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
     if (rc == PMH_OK)
         rc = pmh_launch_sign_unified(ctx, U, g->xy, g->off, g->bbox, g->area2, g->slab_info, g->slab_ptr,
                                      g->slab_edges, nullptr, Q, Q, 0, g->d_n, g->flags, &g->P, sidx,
-                                     g->ticket, g->hashes, nullptr, cs);
+                                     WalkQueue{g->walks, g->ticket + 4}, g->hashes, nullptr, cs);
     if (rc == PMH_OK)
         rc = pmh_launch_query(index, g->hashes, Q, g->d_n, g->counts, nullptr, nullptr, 0, g->join_stage,
                               g->cap, g->flags, false, cs);

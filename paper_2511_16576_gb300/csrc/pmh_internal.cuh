@@ -146,11 +146,27 @@ struct StreamIndexView {
     IndexLevelView lv[kIndexLevels];  // lv[0].first nullptr: no index
 };
 
+// Walks that the indexed form leaves over: a hash without a point below its level's
+// limit, queued by the signing launches and walked by sign_walks_kernel.
+struct WalkItem {
+    int32_t p, k;    // polygon, hash
+    uint32_t start;  // first stream index to examine
+    uint32_t next;   // segments handed out
+};
+constexpr int kWalkItems = 32768;  // (beyond them a hash is marked in the output and found there)
+// device counters of a signing call: [0] work-queue ticket, [1] queued walks, [2] walk ticket
+constexpr int kSignTickets = 3;
+struct WalkQueue {
+    WalkItem* items;
+    unsigned long long* tickets;  // [kSignTickets]
+};
+
 struct pmh_ctx_s {
     int device = 0;
     int sm_count = 0;
     int* d_status = nullptr;              // device status word (0 = ok)
     unsigned long long* d_tickets = nullptr;  // work-queue tickets [64]
+    WalkItem* walks = nullptr;                // [kWalkItems]
     void* scratch[SCR_COUNT] = {};
     size_t scratch_bytes[SCR_COUNT] = {};
     int64_t* h_pinned = nullptr;          // small pinned host buffer [64]
@@ -311,13 +327,14 @@ int pmh_launch_sign(pmh_ctx ctx, const int2* xy, const int64_t* off, const int4*
 // per lane per round of the walk form (2, 4 or 8); work (optional) the six
 // work counters.  The last n_indexed_tail slots of a class list (staged polygons
 // of the indexed form, the class order's last class) get a launch of their own
-// through a build of the kernel without the other paths.
+// through a build of the kernel without the other paths.  wq: the call's counters and
+// the queue of leftover walks, which a last launch takes (with a stream index).
 int pmh_launch_sign_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* off,
                             const int4* bbox, const int64_t* area2, const SlabInfo* slabs,
                             const int32_t* slab_ptr, const int32_t* slab_edges, const int32_t* list,
                             int64_t n_slots, int64_t n_chunked, int64_t n_indexed_tail,
                             const int64_t* d_n, const int* d_flags, const pmh_params* P,
-                            const StreamIndexView& S, unsigned long long* ticket, uint32_t* out,
+                            const StreamIndexView& S, const WalkQueue& wq, uint32_t* out,
                             unsigned long long* work, cudaStream_t s);
 // bucket join (lsh.cu): the count pass (write false: counts) or the fill pass (write
 // true: the CSR rows).  `stage` (nullable, pmh_join_stage_bytes(Q, pool_ints) bytes,

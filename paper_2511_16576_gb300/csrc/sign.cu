@@ -42,6 +42,7 @@ namespace {
 constexpr int kWarps = 8;        // warps per block
 constexpr int kU = 4;            // points per lane per round
 constexpr int kWorkSlot = 8;     // context ticket slots 8..13: work counters of the walk kernel
+constexpr int kSignTicketSlot = 44;  // slots 44..46: counters of a call through the stream index
 constexpr int kIdxWorkSlot = 16; // slots 16..21: work counters of the unified kernel
 
 __device__ __forceinline__ uint32_t sign_one(const int2* __restrict__ v, int n, int x0, int y0,
@@ -332,7 +333,8 @@ int pmh_launch_sign(pmh_ctx ctx, const int2* xy, const int64_t* off, const int4*
         const int64_t n_big = n_polys - n_indexed - n_whole_cost;
         PMH_TRY(pmh_launch_sign_unified(ctx, U, xy, off, bbox, area2, slabs, slab_ptr, slab_edges,
                                         order_cls, n_polys, n_big, n_indexed, nullptr, nullptr, P, S,
-                                        ticket + 2, out, work ? ctx->d_tickets + kIdxWorkSlot : nullptr, s));
+                                        WalkQueue{ctx->walks, ctx->d_tickets + kSignTicketSlot}, out,
+                                        work ? ctx->d_tickets + kIdxWorkSlot : nullptr, s));
         if (timed) {
             PMH_CUDA_TRY(cudaEventRecord(ev[1], s));
             PMH_CUDA_TRY(cudaEventRecord(ev[2], s));

@@ -15,7 +15,7 @@
 //     the others are queued again and tested exactly 32 at a time, so that the long
 //     part runs with every lane.  An inside point lowers its hash's bound, an outside
 //     one is replaced by the next point of its cell below the bound.  A hash without
-//     a point below the level's limit walks on from there;
+//     a point below the level's limit is queued, and a last launch walks on from there;
 //   * walk form (no index, or a very large polygon whose expected walk is short):
 //     Algorithm 1 in warp rounds of 32 * U consecutive stream points; box
 //     candidates in index order (ballot + ffs), each decided by the mask or by the
@@ -49,7 +49,7 @@ constexpr int kMaskN = 32;         // coverage mask cells per side
 constexpr int kGroup = 128;        // hashes signed together, four a lane
 constexpr int kQueue = 192;        // candidates: at most 31, + 128 of a cell, + 32 that follow exact tests
 constexpr uint32_t kNoPoint = 0xFFFFFFFFu;
-constexpr int kIdxU = 4;           // points per lane per round of a resumed walk
+constexpr int kIdxU = 4;           // points per lane per round of a leftover walk
 constexpr int kMaskMaxEdges = 4096;  // larger polygons skip the mask (every cell is a boundary cell)
 
 struct __align__(16) UniWarp {
@@ -320,8 +320,8 @@ __device__ __forceinline__ void classify_cells(UniWarp& m, const IndexLevelView&
 template <class Src, class W, class G>
 __device__ __forceinline__ void indexed_range(UniWarp& m, const Src& src, const StreamIndexView& S, int level,
                                               int4 bb, const MaskFrame& f, float walk, uint64_t seed, uint32_t T,
-                                              int k_begin, int k_end, uint32_t* __restrict__ out,
-                                              int lane, W& work, G& gc)
+                                              int64_t p, int k_begin, int k_end, const WalkQueue& wq,
+                                              uint32_t* __restrict__ out, int lane, W& work, G& gc)
 {
     const unsigned full = 0xffffffffu, lt = pmh_lanemask_lt();
     const uint32_t w = (uint32_t)(bb.z - bb.x), h = (uint32_t)(bb.w - bb.y);
@@ -332,7 +332,6 @@ __device__ __forceinline__ void indexed_range(UniWarp& m, const Src& src, const 
     // with few inside cells to bound the hashes, a first pass over the boundary cells keeps to
     // the points below ~2 expected first hits: else every cell's first point would be tried
     const uint32_t lim1 = 8 * n_in >= n_bnd ? kNoPoint : 2u * (uint32_t)fminf(2.0f * walk + 64.0f, 1.0e9f);
-    const MaskedWalker<Src> walker{&m, src, f.x0, f.y0, f.cwl, f.chl};
 
     for (int kc = k_begin; kc < k_end; kc += kGroup) {
         const int kn = min(kGroup, k_end - kc);
@@ -469,17 +468,21 @@ __device__ __forceinline__ void indexed_range(UniWarp& m, const Src& src, const 
             i0 = 0;
         }
 
-        // hashes without an inside point below the level's limit walk on from there
+        // hashes without an inside point below the level's limit are queued for the walks, or,
+        // past the queue, marked for them in the output (no hash is above 2^31)
         for (int j0 = 0; j0 < kn; j0 += 32) {
             uint32_t v = j0 + lane < kn ? m.best[j0 + lane] : 0u;
-            unsigned todo = __ballot_sync(full, v == kNoPoint && (uint32_t)L.M < T);
+            const unsigned todo = __ballot_sync(full, v == kNoPoint && (uint32_t)L.M < T);
             v = v == kNoPoint ? T : min(v >> 1, T);
-            while (todo) {
-                const int j = __ffs(todo) - 1;
-                todo &= todo - 1;
-                const uint64_t sk = pmh_mix64(seed + (uint64_t)(kc + j0 + j + 1) * PMH_GAMMA);
-                const uint32_t hk = sign_one_t<kIdxU>(walker, bb.x, bb.y, w, h, sk, T, lane, work, (uint32_t)L.M);
-                if (lane == j) v = hk;
+            if (todo) {
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(wq.tickets + 1, (unsigned long long)__popc(todo));
+                base = __shfl_sync(full, base, 0);
+                if ((todo >> lane) & 1u) {
+                    const unsigned long long pos = base + __popc(todo & lt);
+                    if (pos < kWalkItems) wq.items[pos] = WalkItem{(int32_t)p, kc + j0 + lane, (uint32_t)L.M, 0u};
+                    else v = kNoPoint;
+                }
             }
             if (j0 + lane < kn) out[kc + j0 + lane] = v;
         }
@@ -528,8 +531,8 @@ __device__ __noinline__ void walk_staged(const UniWarp& m, StagedSrc src, int4 b
 template <int U, class W, class G>
 __device__ __noinline__ void sign_global(UniWarp& m, GlobalSrc src, int n, int4 bb, int level, float walk,
                                          const StreamIndexView& S, uint64_t seed, uint32_t T,
-                                         int k_begin, int k_end, uint32_t* out, int lane, W* work,
-                                         G* gc)
+                                         int64_t p, int k_begin, int k_end, const WalkQueue& wq,
+                                         uint32_t* out, int lane, W* work, G* gc)
 {
     W local;
     G g;
@@ -537,7 +540,7 @@ __device__ __noinline__ void sign_global(UniWarp& m, GlobalSrc src, int n, int4 
     build_mask(m, src, n, bb, f, n <= kMaskMaxEdges, lane, local);
     // (without a mask every cell is a boundary cell: a walk of few rounds is cheaper)
     if (level >= 0 && (n <= kMaskMaxEdges || walk > 1024.0f))
-        indexed_range(m, src, S, level, bb, f, walk, seed, T, k_begin, k_end, out, lane, local, g);
+        indexed_range(m, src, S, level, bb, f, walk, seed, T, p, k_begin, k_end, wq, out, lane, local, g);
     else
         walk_range<U>(m, src, bb, f, seed, T, k_begin, k_end, out, lane, local);
     work->walk += local.walk;
@@ -563,8 +566,8 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
                     const int32_t* __restrict__ slab_edges, const int32_t* __restrict__ list,
                     int64_t n_slots, int64_t n_chunked, const int64_t* __restrict__ d_n,
                     const int* __restrict__ d_flags, uint64_t seed, int K, uint32_t T,
-                    StreamIndexView S, unsigned long long* __restrict__ ticket,
-                    uint32_t* __restrict__ out, unsigned long long* __restrict__ work_out)
+                    StreamIndexView S, WalkQueue wq, uint32_t* __restrict__ out,
+                    unsigned long long* __restrict__ work_out)
 {
     __shared__ UniWarp smem[kUniWarps];
     __shared__ unsigned long long wsum[6];
@@ -585,7 +588,7 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
     const int64_t n_items = failed ? 0 : n_chunked * chunks + (n_slots - n_chunked);
     for (;;) {
         unsigned long long item = 0;
-        if (lane == 0) item = atomicAdd(ticket, 1ull);
+        if (lane == 0) item = atomicAdd(wq.tickets, 1ull);
         item = __shfl_sync(full, item, 0);
         if ((int64_t)item >= n_items) break;
         int64_t slot;
@@ -622,14 +625,15 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
             const MaskFrame f = mask_frame(bb);
             build_mask(m, src, n, bb, f, true, lane, work);
             if (kIndexedOnly || level >= 0)
-                indexed_range(m, src, S, level, bb, f, walk, seed, T, k_begin, k_end, row, lane, work, gc);
+                indexed_range(m, src, S, level, bb, f, walk, seed, T, p, k_begin, k_end, wq, row, lane, work, gc);
             else
                 walk_staged<U, W>(m, src, bb, f, seed, T, k_begin, k_end, row, lane, &work);
         } else if (!kIndexedOnly) {
             const SlabInfo si = slabs ? slabs[p] : SlabInfo{0, 0, 0, 1, 0};
             const GlobalSrc src{xy + b, n, si.S > 0 ? slab_ptr + si.slab_base : nullptr,
                                 si.S > 0 ? slab_edges + si.edge_base : nullptr, si.slab_h, si.ymin};
-            sign_global<U, W, G>(m, src, n, bb, level, walk, S, seed, T, k_begin, k_end, row, lane, &work, &gc);
+            sign_global<U, W, G>(m, src, n, bb, level, walk, S, seed, T, p, k_begin, k_end, wq, row, lane, &work,
+                                 &gc);
         }
         __syncwarp();
     }
@@ -659,6 +663,139 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
     }
 }
 
+// The leftover walks.  A walk is cut into segments of kWalkSegment stream points that
+// warps take in turn: a warp owns the item its ticket gives it and walks it segment by
+// segment; out of items, it helps with the unfinished ones, so that the last few long
+// walks (2^32 / area points each: 10^5 for the smallest polygons, up to T for one without
+// a lattice point) spread over the device -- walked by the warp that signed the polygon
+// they were the tail of the launch: 8,000 coastlines, K = 256, took 4.8 ms and take 0.97,
+// 0.10 of it here.  The smallest inside index of all segments is the hash; a segment past the best
+// one so far ends the item.  Box points are rare (a few per walk), so they are tested
+// over the polygon's slab or all its edges from global memory.
+constexpr uint32_t kWalkSegment = 4096;
+
+// segment [a, a + kWalkSegment) of one walk
+template <class W>
+__device__ __forceinline__ void walk_segment(const int2* xy, const int64_t* off, const int4* bbox, const SlabInfo* slabs,
+                                             const int32_t* slab_ptr, const int32_t* slab_edges, uint64_t seed,
+                                             uint32_t T, int64_t p, int k, uint32_t a, uint32_t* res, int lane,
+                                             W& work)
+{
+    const int64_t b = off[p];
+    const int n = (int)(off[p + 1] - b);
+    const int4 bb = bbox[p];
+    const SlabInfo si = slabs && n > kSmemVerts ? slabs[p] : SlabInfo{0, 0, 0, 1, 0};
+    const GlobalSrc src{xy + b, n, si.S > 0 ? slab_ptr + si.slab_base : nullptr,
+                        si.S > 0 ? slab_edges + si.edge_base : nullptr, si.slab_h, si.ymin};
+    auto inside = [&](int px, int py, int ln, W& w) { return warp_inside_src(src, px, py, ln, w); };
+    const uint64_t sk = pmh_mix64(seed + (uint64_t)(k + 1) * PMH_GAMMA);
+    const uint32_t end = T - a > kWalkSegment ? a + kWalkSegment : T;
+    const uint32_t r = sign_one_t<kIdxU>(inside, bb.x, bb.y, (uint32_t)(bb.z - bb.x), (uint32_t)(bb.w - bb.y), sk,
+                                         end, lane, work, a);
+    if (r < end && lane == 0) atomicMin(res, r);
+}
+
+template <bool kCount>
+__global__ void __launch_bounds__(256)
+sign_walks_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, const int4* __restrict__ bbox,
+                  const SlabInfo* __restrict__ slabs, const int32_t* __restrict__ slab_ptr,
+                  const int32_t* __restrict__ slab_edges, const int32_t* __restrict__ list, int64_t n_slots,
+                  const int64_t* __restrict__ d_n, const int* __restrict__ d_flags, uint64_t seed, int K, uint32_t T,
+                  WalkQueue wq, uint32_t* out, unsigned long long* __restrict__ work_out)
+{
+    if (d_flags && *d_flags) return;
+    const int lane = threadIdx.x & 31;
+    const unsigned full = 0xffffffffu;
+    using W = typename std::conditional<kCount, Work, NoWork>::type;
+    W work;
+    const unsigned long long queued = wq.tickets[1];
+    const int n = (int)min(queued, (unsigned long long)kWalkItems);
+    const int nwarps = (int)(gridDim.x * (blockDim.x >> 5)), warp = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    // the next segment's first index, past the walk's end when the item is finished
+    auto ahead = [&](const WalkItem& it, uint32_t next, uint32_t best) {
+        const uint64_t a = (uint64_t)it.start + (uint64_t)next * kWalkSegment;
+        return a < (uint64_t)min(T, best);
+    };
+    auto walk_item = [&](int i) {
+        WalkItem* it = wq.items + i;
+        const WalkItem w = *it;
+        uint32_t* res = out + (int64_t)w.p * K + w.k;
+        for (;;) {
+            uint32_t s = 0, best = 0;
+            if (lane == 0) {
+                s = atomicAdd(&it->next, 1u);
+                best = *reinterpret_cast<volatile uint32_t*>(res);
+            }
+            s = __shfl_sync(full, s, 0);
+            best = __shfl_sync(full, best, 0);
+            if (!ahead(w, s, best)) break;
+            walk_segment(xy, off, bbox, slabs, slab_ptr, slab_edges, seed, T, w.p, w.k, w.start + s * kWalkSegment,
+                         res, lane, work);
+        }
+    };
+    for (;;) {
+        unsigned long long i = 0;
+        if (lane == 0) i = atomicAdd(wq.tickets + 2, 1ull);
+        i = __shfl_sync(full, i, 0);
+        if (i >= (unsigned long long)n) break;
+        walk_item((int)i);
+    }
+    // help with unfinished items, 32 looked at a time from a place of the warp's own; done
+    // after a round of the queue without one
+    const int chunks = (n + 31) / 32;
+    int c = chunks > 0 ? warp % chunks : 0;
+    for (int idle = 0; idle < chunks; c = c + 1 == chunks ? 0 : c + 1) {
+        const int i = 32 * c + lane;
+        bool todo = false;
+        if (i < n) {
+            const WalkItem w = wq.items[i];
+            todo = ahead(w, *reinterpret_cast<volatile uint32_t*>(&wq.items[i].next),
+                         *reinterpret_cast<volatile uint32_t*>(out + (int64_t)w.p * K + w.k));
+        }
+        unsigned left = __ballot_sync(full, todo);
+        if (!left) {
+            ++idle;
+            continue;
+        }
+        // (the warps of one chunk spread over its items)
+        for (int skip = (warp / chunks) % __popc(left); skip > 0; --skip) left &= left - 1;
+        walk_item(32 * c + __ffs(left) - 1);
+        idle = 0;
+        c = c == 0 ? chunks - 1 : c - 1;  // look at this chunk again
+    }
+    // past the queue: the marked hashes, a warp each
+    if (queued > (unsigned long long)kWalkItems) {
+        if (d_n) n_slots = min(n_slots, *d_n);
+        for (int64_t slot = warp; slot < n_slots; slot += nwarps) {
+            const int64_t p = list ? (int64_t)list[slot] : slot;
+            const int level = pmh_index_level(bbox[p], K);
+            for (int k0 = 0; k0 < K; k0 += 32) {
+                uint32_t* row = out + p * (int64_t)K + k0;
+                unsigned left = __ballot_sync(full, k0 + lane < K && row[k0 + lane < K ? lane : 0] == kNoPoint);
+                while (left) {
+                    const int j = __ffs(left) - 1;
+                    left &= left - 1;
+                    __syncwarp();
+                    if (lane == 0) row[j] = T;
+                    __syncwarp();
+                    for (uint64_t a = (uint64_t)index_level_points(level); a < T; a += kWalkSegment) {
+                        walk_segment(xy, off, bbox, slabs, slab_ptr, slab_edges, seed, T, p, k0 + j, (uint32_t)a, row + j,
+                                     lane, work);
+                        uint32_t best = 0;
+                        if (lane == 0) best = *reinterpret_cast<volatile uint32_t*>(row + j);
+                        if (__shfl_sync(full, best, 0) < T) break;
+                    }
+                }
+            }
+        }
+    }
+    if (kCount && work_out && lane == 0) {  // (warp-uniform counts)
+        atomicAdd(&work_out[0], work.walk);
+        atomicAdd(&work_out[3], work.cand);
+        atomicAdd(&work_out[4], work.edges);
+    }
+}
+
 }  // namespace
 
 // one persistent launch over `n` slots of `list` (or slot order) with its own ticket
@@ -667,7 +804,7 @@ static int launch_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* off
                           const int64_t* area2, const SlabInfo* slabs, const int32_t* slab_ptr,
                           const int32_t* slab_edges, const int32_t* list, int64_t n_slots,
                           int64_t n_chunked, const int64_t* d_n, const int* d_flags, const pmh_params* P,
-                          const StreamIndexView& S, unsigned long long* ticket, uint32_t* out,
+                          const StreamIndexView& S, const WalkQueue& wq, uint32_t* out,
                           unsigned long long* work, cudaStream_t s)
 {
     auto fn = kIndexedOnly
@@ -684,10 +821,9 @@ static int launch_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* off
     const int64_t n_items = n_chunked * chunks + (n_slots - n_chunked);
     int64_t blocks = (int64_t)ctx->sm_count * std::max(per_sm, 1);
     blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, (n_items + kUniWarps - 1) / kUniWarps));
-    PMH_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned long long), s));
     fn<<<(int)blocks, kUniWarps * 32, 0, s>>>(xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list,
                                               n_slots, n_chunked, d_n, d_flags, P->seed, (int)P->K,
-                                              P->T, S, ticket, out, work);
+                                              P->T, S, wq, out, work);
     PMH_LAUNCHED(kIndexedOnly ? "sign_unified_kernel<indexed>" : "sign_unified_kernel");
     return PMH_OK;
 }
@@ -697,18 +833,28 @@ int pmh_launch_sign_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* o
                             const int32_t* slab_ptr, const int32_t* slab_edges, const int32_t* list,
                             int64_t n_slots, int64_t n_chunked, int64_t n_indexed_tail,
                             const int64_t* d_n, const int* d_flags, const pmh_params* P,
-                            const StreamIndexView& S, unsigned long long* ticket, uint32_t* out,
+                            const StreamIndexView& S, const WalkQueue& wq, uint32_t* out,
                             unsigned long long* work, cudaStream_t s)
 {
     if (n_slots <= 0) return PMH_OK;
+    PMH_CUDA_TRY(cudaMemsetAsync(wq.tickets, 0, sizeof(unsigned long long) * kSignTickets, s));
     // the indexed class at the list's end goes to its own launch (needs the class list)
     const int64_t tail = list && !d_n ? std::min(std::max<int64_t>(n_indexed_tail, 0), n_slots - n_chunked) : 0;
     if (n_slots - tail > 0)
         PMH_TRY(launch_unified<false>(ctx, U, xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list,
-                                      n_slots - tail, n_chunked, d_n, d_flags, P, S, ticket, out, work, s));
-    if (tail > 0)
+                                      n_slots - tail, n_chunked, d_n, d_flags, P, S, wq, out, work, s));
+    if (tail > 0) {
+        if (n_slots - tail > 0) PMH_CUDA_TRY(cudaMemsetAsync(wq.tickets, 0, sizeof(unsigned long long), s));
         PMH_TRY(launch_unified<true>(ctx, U, xy, off, bbox, area2, slabs, slab_ptr, slab_edges,
-                                     list + (n_slots - tail), tail, 0, nullptr, d_flags, P, S, ticket, out,
+                                     list + (n_slots - tail), tail, 0, nullptr, d_flags, P, S, wq, out,
                                      work, s));
+    }
+    if (S.lv[0].first) {
+        // (two blocks of eight warps per SM: the walks are bound by the generator's integer chain)
+        auto fn = work ? sign_walks_kernel<true> : sign_walks_kernel<false>;
+        fn<<<ctx->sm_count * 4, 256, 0, s>>>(xy, off, bbox, slabs, slab_ptr, slab_edges, list, n_slots, d_n, d_flags,
+                                             P->seed, (int)P->K, P->T, wq, out, work);
+        PMH_LAUNCHED("sign_walks_kernel");
+    }
     return PMH_OK;
 }
