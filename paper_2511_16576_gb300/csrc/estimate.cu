@@ -217,6 +217,67 @@ __device__ void bitonic_sort_u64(uint64_t* s, int n /* power of two */)
     }
 }
 
+// Short rows (at most kShortRow pairs), a warp each: every key's rank among the row's keys
+// (from shared memory) is its place in the list, so nothing is sorted and nothing waits
+// on a barrier.  4,096 rows of 64: 16 us with the block kernel's empty launch behind it, 30 us
+// with a block and a bitonic sort each.
+constexpr int kShortRow = 128;
+constexpr int kShortWarps = 8;
+
+__device__ __forceinline__ uint64_t topm_key(const int32_t* cand, const uint16_t* count, const float* score, int K,
+                                             int64_t x)
+{
+    const uint32_t hi = score ? ~f2ord(score[x]) : (uint32_t)(K - min((int)count[x], K));
+    return ((uint64_t)hi << 32) | (uint32_t)cand[x];
+}
+
+__global__ void __launch_bounds__(kShortWarps * 32)
+topm_short_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ cand,
+                  const uint16_t* __restrict__ count, const float* __restrict__ score, int64_t Q, int K, int m,
+                  int32_t* __restrict__ out_ids, int32_t* __restrict__ out_n, const int* __restrict__ d_flags)
+{
+    __shared__ uint64_t keys[kShortWarps][kShortRow];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t q = (int64_t)blockIdx.x * kShortWarps + wid;
+    if (q >= Q) return;
+    const bool failed = d_flags && *d_flags;
+    const int64_t b = failed ? 0 : row_ptr[q], e = failed ? 0 : row_ptr[q + 1];
+    if (e - b > kShortRow) return;  // topm_kernel's
+    const int n = (int)(e - b), kept = min(n, m);
+    uint64_t mine[kShortRow / 32];
+    int rank[kShortRow / 32];
+#pragma unroll
+    for (int u = 0; u < kShortRow / 32; ++u) {
+        const int i = 32 * u + lane;
+        mine[u] = i < n ? topm_key(cand, count, score, K, b + i) : ~0ull;
+        rank[u] = 0;
+        keys[wid][i] = mine[u];
+    }
+    __syncwarp();
+    const int nu = (n + 31) >> 5;  // (short rows skip the empty registers)
+    for (int j = 0; j < n; ++j) {
+        const uint64_t k = keys[wid][j];
+#pragma unroll
+        for (int u = 0; u < kShortRow / 32; ++u)
+            if (u < nu) rank[u] += k < mine[u];
+    }
+    // equal keys (the same pair twice) share a rank: their ranks' sum is short, and each is
+    // moved behind the equal ones before it
+    int sum = 0;
+#pragma unroll
+    for (int u = 0; u < kShortRow / 32; ++u) sum += 32 * u + lane < n ? rank[u] : 0;
+    if (__reduce_add_sync(0xffffffffu, sum) != n * (n - 1) / 2)
+        for (int j = 0; j < n; ++j)
+#pragma unroll
+            for (int u = 0; u < kShortRow / 32; ++u)
+                rank[u] += j < 32 * u + lane && keys[wid][j] == mine[u];
+#pragma unroll
+    for (int u = 0; u < kShortRow / 32; ++u)
+        if (32 * u + lane < n && rank[u] < m) out_ids[q * m + rank[u]] = (int32_t)(uint32_t)(mine[u] & 0xFFFFFFFFu);
+    for (int i = kept + lane; i < m; i += 32) out_ids[q * m + i] = -1;
+    if (lane == 0) out_n[q] = kept;
+}
+
 // one block per query.  Count form: a histogram of the row's counts (0..K) gives
 // the largest threshold c* with at least m pairs of count >= c*; every key of
 // those pairs is gathered and sorted, and the first m kept -- the m best keys
@@ -229,7 +290,7 @@ constexpr int kSelMax = 2048;
 __global__ void __launch_bounds__(kTopThreads)
 topm_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ cand,
             const uint16_t* __restrict__ count, const float* __restrict__ score, int K, int m,
-            int cap /* power of two >= max(m + kTopChunk, kSelMax) */, int32_t* __restrict__ out_ids,
+            int cap /* power of two >= max(m + kTopChunk, kSelMax) */, int min_row, int32_t* __restrict__ out_ids,
             int32_t* __restrict__ out_n, const int* __restrict__ d_flags)
 {
     extern __shared__ uint64_t s[];  // cap keys, then (count form) K + 1 histogram bins
@@ -237,6 +298,7 @@ topm_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ can
     const int64_t q = blockIdx.x;
     const bool failed = d_flags && *d_flags;
     const int64_t b = failed ? 0 : row_ptr[q], e = failed ? 0 : row_ptr[q + 1];
+    if (e - b < min_row) return;  // topm_short_kernel's
     int kept = 0;
     bool merged = true;
     if (!score && e - b > m) {
@@ -300,9 +362,7 @@ topm_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ can
         for (int i = threadIdx.x; i < sz; i += blockDim.x) {
             uint64_t key = ~0ull;
             if (i >= kept && i < kept + take) {
-                int64_t idx = base + (i - kept);
-                uint32_t hi = score ? ~f2ord(score[idx]) : (uint32_t)(K - min((int)count[idx], K));
-                key = ((uint64_t)hi << 32) | (uint32_t)cand[idx];
+                key = topm_key(cand, count, score, K, base + (i - kept));
             } else if (i < kept) {
                 key = s[i];
             }
@@ -408,8 +468,16 @@ int pmh_launch_topm(const int64_t* row_ptr, const int32_t* cand, const uint16_t*
     const size_t smem = sizeof(uint64_t) * cap + sizeof(int) * (size_t)(kb + 1);
     PMH_CUDA_TRY(cudaFuncSetAttribute(topm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem));
+    // large batches: the short rows a warp each, then a block per longer row (a batch of a few
+    // hundred rows fills the device either way and saves the launch)
+    const bool split = Q >= 512;
+    if (split) {
+        topm_short_kernel<<<(unsigned)((Q + kShortWarps - 1) / kShortWarps), kShortWarps * 32, 0, s>>>(
+            row_ptr, cand, count, score, Q, kb, m, out_ids, out_n, d_flags);
+        PMH_LAUNCHED("topm_short_kernel");
+    }
     topm_kernel<<<(unsigned)Q, kTopThreads, smem, s>>>(row_ptr, cand, count, score, kb, m, cap,
-                                                       out_ids, out_n, d_flags);
+                                                       split ? kShortRow + 1 : 0, out_ids, out_n, d_flags);
     PMH_LAUNCHED("topm_kernel");
     return PMH_OK;
 }

@@ -643,7 +643,12 @@ __device__ void tc_teardown(TcSmem& s, uint32_t tmem, int* err)
     if (threadIdx.x == 0 && s.stop && err) atomicOr(err, kTcErr);
 }
 
-__global__ void __launch_bounds__(kTcThreads, 1)
+// Four CTAs per SM (their accumulators fill its tensor memory): a tile is a chain of
+// loads, two MMA chains and two epilogues of 128 threads, so one CTA leaves the SM
+// waiting; the next tile's features are loaded while this one is computed.  262,144
+// rows: 24 us, 70 us with one CTA per SM and the loads at the head of each tile.
+constexpr int kTcCtas = 4;
+__global__ void __launch_bounds__(kTcThreads, kTcCtas)
 mlp_tc_kernel(const __nv_bfloat16* __restrict__ feat, int64_t n_rows, const __nv_bfloat16* __restrict__ w1b,
               const __nv_bfloat16* __restrict__ w2b, const __nv_bfloat16* __restrict__ w3b,
               const float* __restrict__ master, float* __restrict__ score, int* __restrict__ err)
@@ -651,16 +656,28 @@ mlp_tc_kernel(const __nv_bfloat16* __restrict__ feat, int64_t n_rows, const __nv
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TcSmem& s = *reinterpret_cast<TcSmem*>(smem_raw);
     const int tid = threadIdx.x;
+    constexpr int kLoads = kTcRows * (kInPad / 8) / kTcThreads;  // 16-byte chunks per thread and tile
+    uint4 v[kLoads];
+    // a tile's features (rows past n_rows are zero)
+    auto load = [&](int64_t base) {
+#pragma unroll
+        for (int u = 0; u < kLoads; ++u) {
+            const int i = tid + u * kTcThreads, r = i / (kInPad / 8), kc = i % (kInPad / 8);
+            v[u] = base + r < n_rows ? __ldg(reinterpret_cast<const uint4*>(feat + (base + r) * kInPad + 8 * kc))
+                                     : make_uint4(0u, 0u, 0u, 0u);
+        }
+    };
+    const int64_t first = (int64_t)blockIdx.x * kTcRows, step = (int64_t)gridDim.x * kTcRows;
+    load(first);
     const uint32_t tmem = tc_setup(s, w1b, w2b, w3b, master);
     uint32_t phase = 0;
-    for (int64_t base = (int64_t)blockIdx.x * kTcRows; base < n_rows; base += (int64_t)gridDim.x * kTcRows) {
-        // the tile's features (16-byte chunks; rows past n_rows are zero)
-        for (int i = tid; i < kTcRows * (kInPad / 8); i += kTcThreads) {
-            const int r = i / (kInPad / 8), kc = i % (kInPad / 8);
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (base + r < n_rows) v = *reinterpret_cast<const uint4*>(feat + (base + r) * kInPad + 8 * kc);
-            *reinterpret_cast<uint4*>(s.x + canon(r, 8 * kc, kInPad)) = v;
+    for (int64_t base = first; base < n_rows; base += step) {
+#pragma unroll
+        for (int u = 0; u < kLoads; ++u) {
+            const int i = tid + u * kTcThreads, r = i / (kInPad / 8), kc = i % (kInPad / 8);
+            *reinterpret_cast<uint4*>(s.x + canon(r, 8 * kc, kInPad)) = v[u];
         }
+        load(base + step);
         float y;
         if (!tc_tile(s, tmem, phase, y)) break;
         if (base + tid < n_rows) score[base + tid] = y;
@@ -859,7 +876,8 @@ struct pmh_rerank_s {
     __nv_bfloat16* w1b = nullptr;  // [64][48] bf16 operand copies
     __nv_bfloat16* w2b = nullptr;  // [64][64]
     __nv_bfloat16* w3b = nullptr;  // [64]
-    int* err = nullptr;            // tensor-core wait status of the public forward call
+    int* h_err = nullptr;          // tensor-core wait status of the public forward call, in pinned host
+    int* err = nullptr;            // memory (read after the call's synchronisation without a copy), mapped
     int64_t steps = 0;
 };
 
@@ -868,9 +886,10 @@ extern "C" int pmh_rerank_destroy(pmh_rerank r)
     if (!r) return PMH_OK;
     cudaSetDevice(r->device);
     cudaDeviceSynchronize();
-    void* bufs[] = {r->master, r->m1, r->m2, r->grads, r->loss, r->w1b, r->w2b, r->w3b, r->err};
+    void* bufs[] = {r->master, r->m1, r->m2, r->grads, r->loss, r->w1b, r->w2b, r->w3b};
     for (void* b : bufs)
         if (b) cudaFree(b);
+    if (r->h_err) cudaFreeHost(r->h_err);
     delete r;
     return PMH_OK;
 }
@@ -891,7 +910,8 @@ extern "C" int pmh_rerank_create(pmh_ctx ctx, pmh_rerank* out)
               cudaMalloc(&r->w1b, sizeof(__nv_bfloat16) * kH * kInPad) == cudaSuccess &&
               cudaMalloc(&r->w2b, sizeof(__nv_bfloat16) * kH * kH) == cudaSuccess &&
               cudaMalloc(&r->w3b, sizeof(__nv_bfloat16) * kH) == cudaSuccess &&
-              cudaMalloc(&r->err, sizeof(int)) == cudaSuccess;
+              cudaHostAlloc(&r->h_err, sizeof(int), cudaHostAllocMapped) == cudaSuccess &&
+              cudaHostGetDevicePointer(&r->err, r->h_err, 0) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         pmh_rerank_destroy(r);
@@ -900,7 +920,7 @@ extern "C" int pmh_rerank_create(pmh_ctx ctx, pmh_rerank* out)
     cudaMemset(r->master, 0, sizeof(float) * N_PARAMS);
     cudaMemset(r->m1, 0, sizeof(float) * N_PARAMS);
     cudaMemset(r->m2, 0, sizeof(float) * N_PARAMS);
-    cudaMemset(r->err, 0, sizeof(int));
+    *r->h_err = 0;
     refresh_bf16_kernel<<<8, 256>>>(r->master, r->w1b, r->w2b, r->w3b);
     g_pmh_launches.fetch_add(1);
     PMH_CUDA_TRY(cudaDeviceSynchronize());
@@ -949,14 +969,17 @@ extern "C" int pmh_rerank_features(pmh_ctx ctx, pmh_polys queries, pmh_polys db,
                                      (cudaStream_t)stream);
 }
 
-// forward pass: the tensor-core kernel (a few CTAs per SM at most, so that their
-// tensor-memory allocations, 128 columns each, always fit the SM's 512)
+// forward pass: the tensor-core kernel, at most four CTAs per SM (the shared memory keeps a
+// fifth out), so that their tensor-memory allocations, 128 columns each, always fit the
+// SM's 512
 static int tc_forward(pmh_rerank r, const uint16_t* d_feat, int64_t n, float* d_score, int* err,
                       cudaStream_t s)
 {
-    const size_t smem = std::max<size_t>(sizeof(TcSmem) + 1024, 60 * 1024);
+    const size_t smem = std::max<size_t>(sizeof(TcSmem) + 1024, 48 * 1024);
+    static_assert(sizeof(TcSmem) + 1024 <= 56 * 1024, "four CTAs per SM");
     PMH_CUDA_TRY(cudaFuncSetAttribute(mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int blocks = (int)std::min<int64_t>((n + kTcRows - 1) / kTcRows, (int64_t)r->ctx->sm_count);
+    PMH_CUDA_TRY(cudaFuncSetAttribute(mlp_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    const int blocks = (int)std::min<int64_t>((n + kTcRows - 1) / kTcRows, (int64_t)r->ctx->sm_count * kTcCtas);
     mlp_tc_kernel<<<std::max(blocks, 1), kTcThreads, smem, s>>>(
         reinterpret_cast<const __nv_bfloat16*>(d_feat), n, r->w1b, r->w2b, r->w3b, r->master, d_score, err);
     PMH_LAUNCHED("mlp_tc_kernel");
@@ -1021,12 +1044,11 @@ extern "C" int pmh_rerank_forward(pmh_rerank r, const uint16_t* d_feat, int64_t 
     PMH_TRY(pmh_check_device(r->ctx));
     if (n_rows == 0) return PMH_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    PMH_CUDA_TRY(cudaMemsetAsync(r->err, 0, sizeof(int), s));
+    volatile int* err = r->h_err;  // (the last call that could write it has synchronised)
+    *err = 0;
     PMH_TRY(tc_forward(r, d_feat, n_rows, d_score, r->err, s));
-    int h_err = 0;
-    PMH_CUDA_TRY(cudaMemcpyAsync(&h_err, r->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     PMH_CUDA_TRY(cudaStreamSynchronize(s));
-    if (h_err) return pmh_set_error(PMH_ERR_CUDA, "a tensor-core wait of the forward pass ran out");
+    if (*err) return pmh_set_error(PMH_ERR_CUDA, "a tensor-core wait of the forward pass ran out");
     return PMH_OK;
 }
 
