@@ -71,11 +71,6 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi)
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-__device__ __forceinline__ uint32_t pack_raw(__nv_bfloat16 lo, __nv_bfloat16 hi)
-{
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
-
 __device__ __forceinline__ float bfr(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
 __device__ __forceinline__ uint32_t ld32(const __nv_bfloat16* p)
@@ -83,56 +78,99 @@ __device__ __forceinline__ uint32_t ld32(const __nv_bfloat16* p)
     return *reinterpret_cast<const uint32_t*>(p);
 }
 
-struct MlpSmem {
-    __nv_bfloat16 w1[kH][XS];   // [out][in]   B operand of layer 1
-    __nv_bfloat16 w2[kH][HS];   // [out][in]   B operand of layer 2
-    __nv_bfloat16 w2t[kH][HS];  // [in][out]   B operand of dh1 = d2 . W2
+// four 8 x 8 bf16 blocks, transposed on the way (lane l gives the address of row l % 8 of
+// block l / 8): thread (g, t) receives elements (2t, g) and (2t + 1, g) of each block
+__device__ __forceinline__ void ldsm_t4(const __nv_bfloat16* p, uint32_t* r)
+{
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a)
+                 : "memory");
+}
+
+// asynchronous copy of 16 or 4 bytes to shared memory; zero bytes when !ok (src must be
+// readable either way)
+__device__ __forceinline__ void cp16(void* dst, const void* src, bool ok = true)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(ok ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp4(void* dst, const void* src, bool ok)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(ok ? 4 : 0)
+                 : "memory");
+}
+
+struct __align__(16) MlpSmem {
+    __nv_bfloat16 w1[kH][XS];   // [out][in]
+    __nv_bfloat16 w2[kH][HS];   // [out][in]
     __nv_bfloat16 w3[8][HS];    // row 0 = w3, rows 1..7 zero
     float b1[kH], b2[kH], w3f[kH], b3;
-    __nv_bfloat16 x[kChunk][XS];
-    __nv_bfloat16 h1[kChunk][HS];
-    __nv_bfloat16 d2[kChunk][HS];
-    __nv_bfloat16 d1[kChunk][HS];
-    float g3[kChunk];
-    float gb1[kH], gb2[kH], gw3[kH], gb3, loss;
+    __align__(16) __nv_bfloat16 x[kChunk][XS];  // (16-byte copies and ldmatrix rows)
+    __align__(16) __nv_bfloat16 h1[kChunk][HS];
+    __align__(16) __nv_bfloat16 d2[kChunk][HS];
+    __align__(16) __nv_bfloat16 d1[kChunk][HS];
+    float g3[kChunk], label[kChunk];
+    float part[kWarpsMlp][3 * kH + 2];  // each warp's sums: b2, w3, b1, b3, loss
 };
 
-// load the bf16 weights into shared memory (padding zeroed)
+// the bf16 weights to shared memory (16-byte asynchronous copies; the caller waits)
 __device__ void load_weights(MlpSmem& s, const __nv_bfloat16* __restrict__ w1b,
                              const __nv_bfloat16* __restrict__ w2b,
                              const __nv_bfloat16* __restrict__ w3b, const float* __restrict__ master)
 {
-    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-    for (int i = threadIdx.x; i < kH * XS; i += blockDim.x) {
-        int o = i / XS, c = i % XS;
-        s.w1[o][c] = c < kInPad ? w1b[o * kInPad + c] : zero;
+    for (int i = threadIdx.x; i < kH * (kInPad / 8); i += blockDim.x) {
+        const int o = i / (kInPad / 8), c = 8 * (i % (kInPad / 8));
+        cp16(&s.w1[o][c], w1b + o * kInPad + c);
     }
-    for (int i = threadIdx.x; i < kH * HS; i += blockDim.x) {
-        int o = i / HS, c = i % HS;
-        s.w2[o][c] = c < kH ? w2b[o * kH + c] : zero;
-        s.w2t[o][c] = c < kH ? w2b[c * kH + o] : zero;
+    for (int i = threadIdx.x; i < kH * (kH / 8); i += blockDim.x) {
+        const int o = i / (kH / 8), c = 8 * (i % (kH / 8));
+        cp16(&s.w2[o][c], w2b + o * kH + c);
     }
-    for (int i = threadIdx.x; i < 8 * HS; i += blockDim.x) {
-        int r = i / HS, c = i % HS;
-        s.w3[r][c] = (r == 0 && c < kH) ? w3b[c] : zero;
+    for (int i = threadIdx.x; i < 8 * (kH / 2); i += blockDim.x) {
+        const int r = i / (kH / 2), c = 2 * (i % (kH / 2));
+        *reinterpret_cast<uint32_t*>(&s.w3[r][c]) = r == 0 ? ld32(w3b + c) : 0u;
     }
     for (int i = threadIdx.x; i < kH; i += blockDim.x) {
         s.b1[i] = master[OFF_B1 + i];
         s.b2[i] = master[OFF_B2 + i];
         s.w3f[i] = __bfloat162float(w3b[i]);
-        s.gb1[i] = 0.f;
-        s.gb2[i] = 0.f;
-        s.gw3[i] = 0.f;
     }
-    if (threadIdx.x == 0) {
-        s.b3 = master[OFF_B3];
-        s.gb3 = 0.f;
-        s.loss = 0.f;
+    if (threadIdx.x == 0) s.b3 = master[OFF_B3];
+}
+
+// sums of sixteen values over the eight row groups g of a warp (lanes of equal t): the
+// lanes halve the values they keep at each exchange, 14 shuffles instead of 48.  Returns the sums
+// of values 2 * (bits of g reversed) and the next
+__device__ __forceinline__ void sum_groups(const float* v, int lane, float& lo, float& hi)
+{
+    float a[8], b[4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {  // lanes of g bit 2 (lane bit 4) keep the upper eight
+        const float give = (lane & 16) ? v[i] : v[8 + i], keep = (lane & 16) ? v[8 + i] : v[i];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float give = (lane & 8) ? a[i] : a[4 + i], keep = (lane & 8) ? a[4 + i] : a[i];
+        b[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+    }
+    const float g0 = (lane & 4) ? b[0] : b[2], k0 = (lane & 4) ? b[2] : b[0];
+    const float g1 = (lane & 4) ? b[1] : b[3], k1 = (lane & 4) ? b[3] : b[1];
+    lo = k0 + __shfl_xor_sync(0xffffffffu, g0, 4);
+    hi = k1 + __shfl_xor_sync(0xffffffffu, g1, 4);
 }
 
 // Training pass: forward + backward, accumulating the gradients of the mean
-// squared error over n_total rows (the forward pass alone runs on tcgen05 below).
+// squared error over n_total rows (the forward pass alone runs on tcgen05 below).  A
+// minibatch of 4,096 rows is 32 chunks, one per CTA, so the launch takes as long as one
+// chunk's chain: the weights and the first features arrive together in 16-byte copies, the
+// transposed operands of the weight gradients come from ldmatrix, the bias and output-layer
+// gradients stay in registers until the end and are summed without atomics.  4,096
+// rows: 11 us, 25 before.
 __global__ void __launch_bounds__(kWarpsMlp * 32, 1)
 mlp_train_kernel(const __nv_bfloat16* __restrict__ feat, const float* __restrict__ label, int64_t n_rows,
                  int64_t n_total, const __nv_bfloat16* __restrict__ w1b,
@@ -143,25 +181,44 @@ mlp_train_kernel(const __nv_bfloat16* __restrict__ feat, const float* __restrict
     MlpSmem& s = *reinterpret_cast<MlpSmem*>(smem_raw);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
+    // a chunk's features and labels (rows past n_rows are zero); 4-byte copies where the
+    // features are not 16-byte aligned
+    const bool wide = (reinterpret_cast<uintptr_t>(feat) & 15) == 0;
+    auto stage = [&](int64_t base) {
+        if (wide) {
+            for (int i = threadIdx.x; i < kChunk * (kInPad / 8); i += blockDim.x) {
+                const int r = i / (kInPad / 8), c = 8 * (i % (kInPad / 8));
+                const bool ok = base + r < n_rows;
+                cp16(&s.x[r][c], feat + (ok ? base + r : 0) * kInPad + c, ok);
+            }
+        } else {
+            for (int i = threadIdx.x; i < kChunk * (kInPad / 2); i += blockDim.x) {
+                const int r = i / (kInPad / 2), c = 2 * (i % (kInPad / 2));
+                const bool ok = base + r < n_rows;
+                cp4(&s.x[r][c], feat + (ok ? base + r : 0) * kInPad + c, ok);
+            }
+        }
+        for (int r = threadIdx.x; r < kChunk; r += blockDim.x) s.label[r] = base + r < n_rows ? label[base + r] : 0.f;
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        __syncthreads();
+    };
     load_weights(s, w1b, w2b, w3b, master);
-    __syncthreads();
 
     // weight-gradient accumulators of this warp, kept across chunks:
     // gW2 slice: out units 16*(wid/2).., in units 32*(wid%2).. (4 n-tiles);
     // gW1 slice: out units 16*(wid/2).., in units 24*(wid%2).. (3 n-tiles)
     float acc_w2[4][4] = {};
     float acc_w1[3][4] = {};
+    // this thread's parts of the sums over its rows, columns 8 * nt + 2 * t + c: b2, w3, b1
+    float s_b2[16] = {}, s_w3[16] = {}, s_b1[16] = {};
+    float s_b3 = 0.f, s_loss = 0.f;
     const float inv_n = 1.f / (float)(n_total > 1 ? n_total : 1);
+    // ldmatrix row addresses of the transposed operands: blocks (row 0, col 0), (row 8, col 0),
+    // (row 0, col 8), (row 8, col 8) for B, the middle two exchanged for A
+    const int lr = lane & 7, l8 = (lane >> 3) & 1, l16 = lane >> 4;
 
     for (int64_t base = (int64_t)blockIdx.x * kChunk; base < n_rows; base += (int64_t)gridDim.x * kChunk) {
-        // stage the chunk's features (rows past n_rows are zero)
-        for (int i = threadIdx.x; i < kChunk * (kInPad / 2); i += blockDim.x) {
-            int r = i / (kInPad / 2), c2 = i % (kInPad / 2);
-            uint32_t v = 0;
-            if (base + r < n_rows) v = ld32(feat + (base + r) * kInPad + 2 * c2);
-            *reinterpret_cast<uint32_t*>(&s.x[r][2 * c2]) = v;
-        }
-        __syncthreads();
+        stage(base);
         const int r0 = wid * 16;  // this warp's rows within the chunk
 
         // ---- layer 1: [16 x 48] x [48 x 64]
@@ -234,21 +291,20 @@ mlp_train_kernel(const __nv_bfloat16* __restrict__ feat, const float* __restrict
         float pB = 1.f / (1.f + expf(-(acc3[2] + s.b3)));
         // ---- backward
         if (t == 0) {
-            float gA = 0.f, gB = 0.f, l = 0.f;
+            float gA = 0.f, gB = 0.f;
             if (rowA < n_rows) {
-                float err = pA - label[rowA];
-                l += err * err;
+                float err = pA - s.label[r0 + g];
+                s_loss += err * err;
                 gA = 2.f * err * inv_n * pA * (1.f - pA);
             }
             if (rowB < n_rows) {
-                float err = pB - label[rowB];
-                l += err * err;
+                float err = pB - s.label[r0 + g + 8];
+                s_loss += err * err;
                 gB = 2.f * err * inv_n * pB * (1.f - pB);
             }
             s.g3[r0 + g] = gA;
             s.g3[r0 + g + 8] = gB;
-            atomicAdd(&s.loss, l);
-            atomicAdd(&s.gb3, gA + gB);
+            s_b3 += gA + gB;
         }
         __syncwarp();
         const float g3A = s.g3[r0 + g], g3B = s.g3[r0 + g + 8];
@@ -257,7 +313,7 @@ mlp_train_kernel(const __nv_bfloat16* __restrict__ feat, const float* __restrict
         uint32_t a4f[4][4];
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
-            float d[4], gw[2], gb[2];
+            float d[4];
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int col = nt * 8 + 2 * t + c;
@@ -265,24 +321,8 @@ mlp_train_kernel(const __nv_bfloat16* __restrict__ feat, const float* __restrict
                 const bool mA = (mask2 >> (nt * 4 + c)) & 1u, mB = (mask2 >> (nt * 4 + 2 + c)) & 1u;
                 d[c] = mA ? w3 * g3rA : 0.f;
                 d[2 + c] = mB ? w3 * g3rB : 0.f;
-                gb[c] = d[c] + d[2 + c];
-                gw[c] = g3rA * h2v[nt][c] + g3rB * h2v[nt][2 + c];
-            }
-            // reduce over the 8 row groups g (lanes with equal t)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-#pragma unroll
-                for (int o = 4; o < 32; o <<= 1) {
-                    gb[c] += __shfl_xor_sync(0xffffffffu, gb[c], o);
-                    gw[c] += __shfl_xor_sync(0xffffffffu, gw[c], o);
-                }
-            }
-            if (g == 0) {
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    atomicAdd(&s.gb2[nt * 8 + 2 * t + c], gb[c]);
-                    atomicAdd(&s.gw3[nt * 8 + 2 * t + c], gw[c]);
-                }
+                s_b2[2 * nt + c] += d[c] + d[2 + c];
+                s_w3[2 * nt + c] += g3rA * h2v[nt][c] + g3rB * h2v[nt][2 + c];
             }
             uint32_t lo = pack2(d[0], d[1]), hi = pack2(d[2], d[3]);
             a4f[nt >> 1][(nt & 1) * 2 + 0] = lo;
@@ -295,28 +335,21 @@ mlp_train_kernel(const __nv_bfloat16* __restrict__ feat, const float* __restrict
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt) {
-                uint32_t b[2] = {ld32(&s.w2t[nt * 8 + g][16 * kk + 2 * t]),
-                                 ld32(&s.w2t[nt * 8 + g][16 * kk + 2 * t + 8])};
+            for (int nt = 0; nt < 8; nt += 2) {
+                uint32_t b[4];
+                ldsm_t4(&s.w2[16 * kk + 8 * l8 + lr][nt * 8 + 8 * l16], b);
                 mma_bf16(acc4[nt], a4f[kk], b);
+                mma_bf16(acc4[nt + 1], a4f[kk], b + 2);
             }
         }
         // d1 = relu'(z1) * dh1; gb1 += d1; d1 (bf16) to shared memory
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
-            float d[4], gb[2];
+            float d[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) d[i] = ((mask1 >> (nt * 4 + i)) & 1u) ? acc4[nt][i] : 0.f;
-            gb[0] = d[0] + d[2];
-            gb[1] = d[1] + d[3];
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int o = 4; o < 32; o <<= 1) gb[c] += __shfl_xor_sync(0xffffffffu, gb[c], o);
-            if (g == 0) {
-                atomicAdd(&s.gb1[nt * 8 + 2 * t], gb[0]);
-                atomicAdd(&s.gb1[nt * 8 + 2 * t + 1], gb[1]);
-            }
+            s_b1[2 * nt] += d[0] + d[2];
+            s_b1[2 * nt + 1] += d[1] + d[3];
             *reinterpret_cast<uint32_t*>(&s.d1[r0 + g][nt * 8 + 2 * t]) = pack2(d[0], d[1]);
             *reinterpret_cast<uint32_t*>(&s.d1[r0 + g + 8][nt * 8 + 2 * t]) = pack2(d[2], d[3]);
         }
@@ -326,30 +359,23 @@ mlp_train_kernel(const __nv_bfloat16* __restrict__ feat, const float* __restrict
 #pragma unroll
         for (int kk = 0; kk < kChunk / 16; ++kk) {
             const int k0 = 16 * kk;
-            // A[m = out][k = row] = d2[row][out]
-            uint32_t a[4] = {pack_raw(s.d2[k0 + 2 * t][m0 + g], s.d2[k0 + 2 * t + 1][m0 + g]),
-                             pack_raw(s.d2[k0 + 2 * t][m0 + g + 8], s.d2[k0 + 2 * t + 1][m0 + g + 8]),
-                             pack_raw(s.d2[k0 + 2 * t + 8][m0 + g], s.d2[k0 + 2 * t + 9][m0 + g]),
-                             pack_raw(s.d2[k0 + 2 * t + 8][m0 + g + 8], s.d2[k0 + 2 * t + 9][m0 + g + 8])};
+            // A[m = out][k = row] = d2[row][out], B[k = row][n = in] = h1[row][in]
+            uint32_t a[4], bb[4];
+            ldsm_t4(&s.d2[k0 + 8 * l16 + lr][m0 + 8 * l8], a);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int n0 = 32 * (wid & 1) + 8 * j;
-                // B[k = row][n = in] = h1[row][in]
-                uint32_t b[2] = {pack_raw(s.h1[k0 + 2 * t][n0 + g], s.h1[k0 + 2 * t + 1][n0 + g]),
-                                 pack_raw(s.h1[k0 + 2 * t + 8][n0 + g], s.h1[k0 + 2 * t + 9][n0 + g])};
-                mma_bf16(acc_w2[j], a, b);
+            for (int j = 0; j < 4; j += 2) {
+                ldsm_t4(&s.h1[k0 + 8 * l8 + lr][32 * (wid & 1) + 8 * j + 8 * l16], bb);
+                mma_bf16(acc_w2[j], a, bb);
+                mma_bf16(acc_w2[j + 1], a, bb + 2);
             }
-            uint32_t a1[4] = {pack_raw(s.d1[k0 + 2 * t][m0 + g], s.d1[k0 + 2 * t + 1][m0 + g]),
-                              pack_raw(s.d1[k0 + 2 * t][m0 + g + 8], s.d1[k0 + 2 * t + 1][m0 + g + 8]),
-                              pack_raw(s.d1[k0 + 2 * t + 8][m0 + g], s.d1[k0 + 2 * t + 9][m0 + g]),
-                              pack_raw(s.d1[k0 + 2 * t + 8][m0 + g + 8], s.d1[k0 + 2 * t + 9][m0 + g + 8])};
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const int n0 = 24 * (wid & 1) + 8 * j;
-                uint32_t b[2] = {pack_raw(s.x[k0 + 2 * t][n0 + g], s.x[k0 + 2 * t + 1][n0 + g]),
-                                 pack_raw(s.x[k0 + 2 * t + 8][n0 + g], s.x[k0 + 2 * t + 9][n0 + g])};
-                mma_bf16(acc_w1[j], a1, b);
-            }
+            ldsm_t4(&s.d1[k0 + 8 * l16 + lr][m0 + 8 * l8], a);
+            // (three tiles of 24 inputs: the last read's second tile is not used, and stays in the row)
+            const int n1 = 24 * (wid & 1);
+            ldsm_t4(&s.x[k0 + 8 * l8 + lr][n1 + 8 * l16], bb);
+            mma_bf16(acc_w1[0], a, bb);
+            mma_bf16(acc_w1[1], a, bb + 2);
+            ldsm_t4(&s.x[k0 + 8 * l8 + lr][n1 + 16], bb);
+            mma_bf16(acc_w1[2], a, bb);
         }
         __syncthreads();
     }
@@ -372,16 +398,46 @@ mlp_train_kernel(const __nv_bfloat16* __restrict__ feat, const float* __restrict
             if (c < kIn) atomicAdd(&grads[OFF_W1 + o * kIn + c], acc_w1[j][i]);
         }
     }
+    // the warp's column sums: thread (g, t) holds columns 8 * (v / 2) + 2 * t + v % 2 of values v
+    const int v0 = 2 * (((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1));
+    const int col = 4 * v0 + 2 * t;
+    float lo, hi;
+    sum_groups(s_b2, lane, lo, hi);
+    s.part[wid][col] = lo;
+    s.part[wid][col + 1] = hi;
+    sum_groups(s_w3, lane, lo, hi);
+    s.part[wid][kH + col] = lo;
+    s.part[wid][kH + col + 1] = hi;
+    sum_groups(s_b1, lane, lo, hi);
+    s.part[wid][2 * kH + col] = lo;
+    s.part[wid][2 * kH + col + 1] = hi;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s_b3 += __shfl_xor_sync(0xffffffffu, s_b3, o);
+        s_loss += __shfl_xor_sync(0xffffffffu, s_loss, o);
+    }
+    if (lane == 0) {
+        s.part[wid][3 * kH] = s_b3;
+        s.part[wid][3 * kH + 1] = s_loss;
+    }
     __syncthreads();
-    for (int i = threadIdx.x; i < kH; i += blockDim.x) {
-        atomicAdd(&grads[OFF_B1 + i], s.gb1[i]);
-        atomicAdd(&grads[OFF_B2 + i], s.gb2[i]);
-        atomicAdd(&grads[OFF_W3 + i], s.gw3[i]);
+    for (int i = threadIdx.x; i < 3 * kH + 2; i += blockDim.x) {
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWarpsMlp; ++w) v += s.part[w][i];
+        float* dst = i < kH ? &grads[OFF_B2 + i] : i < 2 * kH ? &grads[OFF_W3 + i - kH]
+                     : i < 3 * kH ? &grads[OFF_B1 + i - 2 * kH] : i == 3 * kH ? &grads[OFF_B3] : loss_out;
+        atomicAdd(dst, i == 3 * kH + 1 ? v * inv_n : v);
     }
-    if (threadIdx.x == 0) {
-        atomicAdd(&grads[OFF_B3], s.gb3);
-        atomicAdd(loss_out, s.loss * inv_n);
-    }
+}
+
+// the gradients and the loss to the caller's arrays, in one launch
+__global__ void __launch_bounds__(256)
+export_kernel(const float* __restrict__ grads, float* __restrict__ d_grads, float* __restrict__ d_loss)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N_PARAMS && d_grads) d_grads[i] = grads[i];
+    if (i == N_PARAMS && d_loss) *d_loss = grads[i];
 }
 
 // Adam on the fp32 master weights (the bf16 operand copies are refreshed after it)
@@ -865,14 +921,18 @@ rerank_select_kernel(const uint32_t* __restrict__ qh, const uint32_t* __restrict
 
 }  // namespace
 
+// shared memory of the forward pass: a fifth CTA must not fit
+constexpr size_t kTcSmemBytes = sizeof(TcSmem) + 1024 > 48 * 1024 ? sizeof(TcSmem) + 1024 : 48 * 1024;
+static_assert(kTcSmemBytes <= 56 * 1024, "four CTAs per SM");
+
 struct pmh_rerank_s {
     pmh_ctx ctx = nullptr;
     int device = 0;
     float* master = nullptr;  // packed fp32 weights
     float* m1 = nullptr;      // Adam moments
     float* m2 = nullptr;
-    float* grads = nullptr;
-    float* loss = nullptr;
+    float* grads = nullptr;   // [N_PARAMS + 1]: the gradients, then the loss
+    float* loss = nullptr;    // grads + N_PARAMS
     __nv_bfloat16* w1b = nullptr;  // [64][48] bf16 operand copies
     __nv_bfloat16* w2b = nullptr;  // [64][64]
     __nv_bfloat16* w3b = nullptr;  // [64]
@@ -886,7 +946,7 @@ extern "C" int pmh_rerank_destroy(pmh_rerank r)
     if (!r) return PMH_OK;
     cudaSetDevice(r->device);
     cudaDeviceSynchronize();
-    void* bufs[] = {r->master, r->m1, r->m2, r->grads, r->loss, r->w1b, r->w2b, r->w3b};
+    void* bufs[] = {r->master, r->m1, r->m2, r->grads, r->w1b, r->w2b, r->w3b};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (r->h_err) cudaFreeHost(r->h_err);
@@ -905,8 +965,7 @@ extern "C" int pmh_rerank_create(pmh_ctx ctx, pmh_rerank* out)
     bool ok = cudaMalloc(&r->master, sizeof(float) * N_PARAMS) == cudaSuccess &&
               cudaMalloc(&r->m1, sizeof(float) * N_PARAMS) == cudaSuccess &&
               cudaMalloc(&r->m2, sizeof(float) * N_PARAMS) == cudaSuccess &&
-              cudaMalloc(&r->grads, sizeof(float) * N_PARAMS) == cudaSuccess &&
-              cudaMalloc(&r->loss, sizeof(float)) == cudaSuccess &&
+              cudaMalloc(&r->grads, sizeof(float) * (N_PARAMS + 1)) == cudaSuccess &&
               cudaMalloc(&r->w1b, sizeof(__nv_bfloat16) * kH * kInPad) == cudaSuccess &&
               cudaMalloc(&r->w2b, sizeof(__nv_bfloat16) * kH * kH) == cudaSuccess &&
               cudaMalloc(&r->w3b, sizeof(__nv_bfloat16) * kH) == cudaSuccess &&
@@ -916,6 +975,17 @@ extern "C" int pmh_rerank_create(pmh_ctx ctx, pmh_rerank* out)
         cudaGetLastError();
         pmh_rerank_destroy(r);
         return pmh_set_error(PMH_ERR_NOMEM, "reranker allocation failed");
+    }
+    r->loss = r->grads + N_PARAMS;
+    cudaError_t e = cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(MlpSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(mlp_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) {
+        pmh_rerank_destroy(r);
+        return pmh_set_error(PMH_ERR_CUDA, "reranker kernels: %s", cudaGetErrorString(e));
     }
     cudaMemset(r->master, 0, sizeof(float) * N_PARAMS);
     cudaMemset(r->m1, 0, sizeof(float) * N_PARAMS);
@@ -975,27 +1045,26 @@ extern "C" int pmh_rerank_features(pmh_ctx ctx, pmh_polys queries, pmh_polys db,
 static int tc_forward(pmh_rerank r, const uint16_t* d_feat, int64_t n, float* d_score, int* err,
                       cudaStream_t s)
 {
-    const size_t smem = std::max<size_t>(sizeof(TcSmem) + 1024, 48 * 1024);
-    static_assert(sizeof(TcSmem) + 1024 <= 56 * 1024, "four CTAs per SM");
-    PMH_CUDA_TRY(cudaFuncSetAttribute(mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PMH_CUDA_TRY(cudaFuncSetAttribute(mlp_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     const int blocks = (int)std::min<int64_t>((n + kTcRows - 1) / kTcRows, (int64_t)r->ctx->sm_count * kTcCtas);
-    mlp_tc_kernel<<<std::max(blocks, 1), kTcThreads, smem, s>>>(
+    mlp_tc_kernel<<<std::max(blocks, 1), kTcThreads, kTcSmemBytes, s>>>(
         reinterpret_cast<const __nv_bfloat16*>(d_feat), n, r->w1b, r->w2b, r->w3b, r->master, d_score, err);
     PMH_LAUNCHED("mlp_tc_kernel");
     return PMH_OK;
 }
 
 static int train_launch(pmh_rerank r, const uint16_t* d_feat, const float* d_label, int64_t n,
-                        cudaStream_t s)
+                        float* d_grads, float* d_loss, cudaStream_t s)
 {
-    const size_t smem = sizeof(MlpSmem);
-    PMH_CUDA_TRY(cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = sizeof(MlpSmem);  // (allowed for the kernel by pmh_rerank_create)
     int blocks = (int)std::min<int64_t>((n + kChunk - 1) / kChunk, (int64_t)r->ctx->sm_count);
     mlp_train_kernel<<<std::max(blocks, 1), kWarpsMlp * 32, smem, s>>>(
         reinterpret_cast<const __nv_bfloat16*>(d_feat), d_label, n, n, r->w1b, r->w2b, r->w3b,
         r->master, r->grads, r->loss);
     PMH_LAUNCHED("mlp_train_kernel");
+    if (d_grads || d_loss) {
+        export_kernel<<<(N_PARAMS + 1 + 255) / 256, 256, 0, s>>>(r->grads, d_grads, d_loss);
+        PMH_LAUNCHED("export_kernel");
+    }
     return PMH_OK;
 }
 
@@ -1058,14 +1127,8 @@ extern "C" int pmh_rerank_gradients(pmh_rerank r, const uint16_t* d_feat, const 
     if (!r || n_rows < 1 || !d_feat || !d_label) return pmh_set_error(PMH_ERR_ARG, "bad arguments");
     PMH_TRY(pmh_check_device(r->ctx));
     cudaStream_t s = (cudaStream_t)stream;
-    PMH_CUDA_TRY(cudaMemsetAsync(r->grads, 0, sizeof(float) * N_PARAMS, s));
-    PMH_CUDA_TRY(cudaMemsetAsync(r->loss, 0, sizeof(float), s));
-    PMH_TRY(train_launch(r, d_feat, d_label, n_rows, s));
-    if (d_grads)
-        PMH_CUDA_TRY(cudaMemcpyAsync(d_grads, r->grads, sizeof(float) * N_PARAMS,
-                                     cudaMemcpyDeviceToDevice, s));
-    if (d_loss) PMH_CUDA_TRY(cudaMemcpyAsync(d_loss, r->loss, sizeof(float), cudaMemcpyDeviceToDevice, s));
-    return PMH_OK;
+    PMH_CUDA_TRY(cudaMemsetAsync(r->grads, 0, sizeof(float) * (N_PARAMS + 1), s));
+    return train_launch(r, d_feat, d_label, n_rows, d_grads, d_loss, s);
 }
 
 extern "C" int pmh_rerank_adam_step(pmh_rerank r, float lr, float beta1, float beta2, float eps,
