@@ -161,7 +161,7 @@ __device__ __forceinline__ uint32_t sign_chunk_walk(const Inside& inside, int4 b
     uint32_t mine = T;
     for (int k = k0; k < kend; ++k) {
         uint64_t sk = pmh_mix64(seed + (uint64_t)(k + 1) * PMH_GAMMA);
-        uint32_t hk = sign_one_t<U>(inside, bb.x, bb.y, w, h, sk, T, lane, work);
+        uint32_t hk = sign_one_t<U, true>(inside, bb.x, bb.y, w, h, sk, T, lane, work);
         if (lane == k - k0) mine = hk;
     }
     return mine;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(W * 32, MinBlocks)
 sign_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
             const int4* __restrict__ bbox, const SlabInfo* __restrict__ slabs,
             const int32_t* __restrict__ slab_ptr, const int32_t* __restrict__ slab_edges,
-            const int32_t* __restrict__ order, uint64_t seed, int K, uint32_t T, int chunks,
+            const int32_t* __restrict__ order, uint64_t seed, int K, uint32_t T, int per_item, int chunks,
             int64_t n_polys, const int64_t* __restrict__ d_n, const int* __restrict__ d_flags,
             unsigned long long* __restrict__ ticket, uint32_t* __restrict__ out,
             const int64_t* __restrict__ area2, StreamIndexView S,
@@ -212,8 +212,8 @@ sign_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
         if ((int64_t)item >= n_items) break;
         const int64_t slot = (int64_t)(item / (unsigned)chunks);
         const int64_t p = order ? (int64_t)order[slot] : slot;
-        const int k0 = (int)(item % (unsigned)chunks) * 32;
-        const int kend = min(K, k0 + 32);
+        const int k0 = (int)(item % (unsigned)chunks) * per_item;
+        const int kend = min(K, k0 + per_item);
         const int64_t b = off[p];
         const int n = (int)(off[p + 1] - b);
         const int4 bb = bbox[p];
@@ -226,7 +226,8 @@ sign_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
             if (masks && lane < 16) smask[wid][lane] = masks[p * 16 + lane];
             stage_vertices(sv[wid], xy + b, n, lane);
             const int sh = staged_slab_shift(max(bb.w - bb.y, 1));
-            const bool staged = bb.w > bb.y && bb.z > bb.x &&
+            // (a ring of two edges a lane is tested whole: binning its edges costs more)
+            const bool staged = (masks || n > 64) && bb.w > bb.y && bb.z > bb.x &&
                                 build_staged_slabs(sv[wid], n, bb.y, sh, sid[wid], sbeg[wid], scnt[wid], lane);
             const int cwl = mask_cell_log2(bb.z - bb.x), chl = mask_cell_log2(bb.w - bb.y);
             if (staged) {
@@ -237,7 +238,7 @@ sign_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
                 else
                     mine = sign_chunk_walk<U>(st, bb, seed, k0, kend, T, lane, work);
             } else {
-                // too many slab references (or an empty box): every edge, no mask
+                // few edges, too many slab references, or an empty box: every edge, no mask
                 mine = sign_chunk_walk<U>(AllEdges{sv[wid], n}, bb, seed, k0, kend, T, lane, work);
             }
         } else if (slabs && slabs[p].S > 0) {
@@ -271,7 +272,7 @@ sign_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
 }
 
 using SignFn = void (*)(const int2*, const int64_t*, const int4*, const SlabInfo*, const int32_t*,
-                        const int32_t*, const int32_t*, uint64_t, int, uint32_t, int, int64_t,
+                        const int32_t*, const int32_t*, uint64_t, int, uint32_t, int, int, int64_t,
                         const int64_t*, const int*, unsigned long long*, uint32_t*, const int64_t*,
                         StreamIndexView, unsigned long long*, const uint32_t*);
 struct SignVariant {
@@ -309,9 +310,10 @@ int pmh_launch_sign(pmh_ctx ctx, const int2* xy, const int64_t* off, const int4*
     const StreamIndexView S = sidx ? *sidx : StreamIndexView{};
     if (n_polys <= 0) return PMH_OK;
     unsigned long long* work = d_n ? nullptr : ctx->d_tickets + kWorkSlot;
+    // (tickets and both kernels' counts lie together: one clear)
+    const bool cleared = work && ticket >= ctx->d_tickets && ticket < ctx->d_tickets + kWorkSlot;
     if (work) {
-        PMH_CUDA_TRY(cudaMemsetAsync(work, 0, sizeof(unsigned long long) * 6, s));
-        PMH_CUDA_TRY(cudaMemsetAsync(ctx->d_tickets + kIdxWorkSlot, 0, sizeof(unsigned long long) * 6, s));
+        PMH_CUDA_TRY(cudaMemsetAsync(ctx->d_tickets, 0, sizeof(unsigned long long) * (kIdxWorkSlot + 6), s));
         if (!ctx->sign_count) work = nullptr;  // counts stay zero: the counter-free kernels run
     }
     const bool timed = ctx->sign_timing && !d_n && ctx->sign_ev_used + 3 <= 3 * 1024;
@@ -347,15 +349,20 @@ int pmh_launch_sign(pmh_ctx ctx, const int2* xy, const int64_t* off, const int4*
         return PMH_OK;
     }
     const SignVariant& v = kSignVariants[ctx->sign_variant >= 0 ? ctx->sign_variant : 0];
-    const int chunks = (int)((P->K + 31) / 32);
-    const int64_t n_items = n_polys * chunks;
     int per_sm = 0;
     PMH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, v.fn, v.W * 32, 0));
     int64_t blocks = (int64_t)ctx->sm_count * std::max(per_sm, 1);
+    // hashes per item: 32, fewer for a set with less than two such items per resident warp (an
+    // item's hashes are signed one after the other; its staging is a few hashes' worth, so
+    // not below four).  1,000 polygons, K = 32: a call 53.6 us with 32-hash items and every ring binned, 28.5 now
+    int per_item = 32;
+    while (per_item > 4 && n_polys * (int64_t)((P->K + per_item - 1) / per_item) < 2 * blocks * v.W) per_item /= 2;
+    const int chunks = (int)((P->K + per_item - 1) / per_item);
+    const int64_t n_items = n_polys * chunks;
     blocks = std::min<int64_t>(blocks, (n_items + v.W - 1) / v.W);
-    PMH_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned long long), s));
+    if (!cleared) PMH_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned long long), s));
     v.fn<<<(int)blocks, v.W * 32, 0, s>>>(xy, off, bbox, slabs, slab_ptr, slab_edges, order,
-                                          P->seed, (int)P->K, P->T, chunks, n_polys, d_n, d_flags,
+                                          P->seed, (int)P->K, P->T, per_item, chunks, n_polys, d_n, d_flags,
                                           ticket, out, area2, S, work, masks);
     PMH_LAUNCHED("sign_kernel");
     if (timed) PMH_CUDA_TRY(cudaEventRecord(ev[2], s));

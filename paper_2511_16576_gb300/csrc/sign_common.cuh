@@ -221,7 +221,7 @@ __device__ __forceinline__ bool build_staged_slabs(const int2* v, int n, int y0,
     return true;
 }
 
-template <int U, class Inside, class W>
+template <int U, bool kLazy, class Inside, class W>
 __device__ __forceinline__ uint32_t sign_walk(const Inside& inside, int x0, int y0, uint32_t w,
                                               uint32_t h, uint64_t sk, uint32_t T, int lane,
                                               W& work, uint32_t start);
@@ -247,25 +247,41 @@ struct Masked {
 };
 
 // One hash of one polygon; every lane returns the same value.  U points per
-// lane per round: one round covers 32 * U consecutive stream indices.
-template <int U, class Inside, class W>
+// lane per round: one round covers 32 * U consecutive stream indices.  kLazy: the first
+// 128 points 32 at a time (a polygon of 1% of the domain or more has its hash among
+// them more often than not, and the generator is most of a round's work).
+template <int U, bool kLazy = false, class Inside, class W>
 __device__ __forceinline__ uint32_t sign_one_t(const Inside& inside, int x0, int y0, uint32_t w,
                                                uint32_t h, uint64_t sk, uint32_t T, int lane,
                                                W& work, uint32_t start = 0)
 {
     if (w == 0 || h == 0) return T;
-    const uint32_t r = sign_walk<U>(inside, x0, y0, w, h, sk, T, lane, work, start);
+    const uint32_t r = sign_walk<U, kLazy>(inside, x0, y0, w, h, sk, T, lane, work, start);
     work.walk += (r < T ? r + 1 : T) - start;
     return r;
 }
 
-template <int U, class Inside, class W>
+template <int U, bool kLazy, class Inside, class W>
 __device__ __forceinline__ uint32_t sign_walk(const Inside& inside, int x0, int y0, uint32_t w,
                                               uint32_t h, uint64_t sk, uint32_t T, int lane,
                                               W& work, uint32_t start)
 {
     uint64_t z = sk + (uint64_t)(start + lane + 1) * PMH_GAMMA;
     const uint64_t step = 32ull * PMH_GAMMA;
+    if (kLazy) {
+#pragma unroll 1
+        for (int j = 0; j < 4 && start < T; ++j, start += 32u, z += step) {
+            const uint32_t pt = pmh_mix64_lo(z);
+            unsigned b = __ballot_sync(0xffffffffu, ((pt & 0xFFFFu) - (uint32_t)x0 < w) & ((pt >> 16) - (uint32_t)y0 < h));
+            while (b) {
+                const int l = __ffs(b) - 1;
+                b &= b - 1;
+                if (start + (uint32_t)l >= T) return T;
+                const uint32_t r = __shfl_sync(0xffffffffu, pt, l);
+                if (inside((int)(r & 0xFFFFu), (int)(r >> 16), lane, work)) return start + (uint32_t)l;
+            }
+        }
+    }
     for (uint32_t i0 = start; i0 < T; i0 += 32u * U) {
         uint32_t pts[U];
         unsigned m = 0;
