@@ -127,88 +127,124 @@ extern "C" int pmh_destroy(pmh_ctx ctx)
 // (clipped to the lattice domain, half-open), twice the signed area.
 // status[0] |= 1 bad offsets, 2 < 3 vertices, 4 coordinate out of range;
 // status[1] = max vertex count.
+//
+// kCopy: the vertices are copied from src to dst on the way (a device-to-device upload).
+// sz.info: the sizes of every polygon's slab index too, from a second look at vertices that
+// the caches still hold.
+// Bound by memory at large sets (each vertex is read once, written once under kCopy): a
+// lane keeps four vertices in flight, and an edge's start vertex is the lane before's (a
+// rotation), so that no vertex is loaded twice.  400,000 polygons of 8 to 1,024 vertices (0.7 GB):
+// 352 us; before, 297 us of preparation and 202 us of sizes followed a copy of the vertices
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, 6) prep_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
-                            int64_t n_polys, const int64_t* __restrict__ d_n, int64_t n_vertices,
-                            int4* __restrict__ bbox, int64_t* __restrict__ area2,
-                            int* __restrict__ status)
+template <bool kCopy>
+__global__ void __launch_bounds__(256, 6)
+prep_kernel(const int2* __restrict__ src, int2* __restrict__ dst, const int64_t* __restrict__ off,
+            int64_t n_polys, const int64_t* __restrict__ d_n, int64_t n_vertices,
+            int4* __restrict__ bbox, int64_t* __restrict__ area2, SlabSizes sz, int* __restrict__ status)
 {
     const int lane = threadIdx.x & 31;
-    if (d_n) n_polys = min(n_polys, *d_n);
-    int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    // (slots at or past the device-side count get empty sizes)
+    const int64_t n_live = d_n ? min(n_polys, *d_n) : n_polys;
     const int LIM = 1 << 20;
     int nmax = 0;  // largest vertex count of the warp's polygons (one atomic at the end)
     for (int64_t p = warp; p < n_polys; p += nwarps) {
-        int64_t b = off[p], e = off[p + 1];
-        int flags = 0;
-        if (b < 0 || e > n_vertices || e < b) flags |= 1;
-        int64_t n = e - b;
-        if (n < 3) flags |= 2;
-        if (flags) {
-            if (lane == 0) {
-                atomicOr(&status[0], flags);
-                bbox[p] = make_int4(0, 0, 0, 0);
-                area2[p] = 0;
-            }
-            continue;
-        }
-        int x0 = INT_MAX, y0 = INT_MAX, x1 = INT_MIN, y1 = INT_MIN;
-        long long a2 = 0;
-        // four vertices per lane in flight; edge i's end vertex is lane + 1's vertex
-        // (a shuffle), lane 31 reads it
-        for (int64_t i0 = 0; i0 < n; i0 += 128) {
-            int2 v[4], w[4];
+        SlabInfo si{0, 0, 0, 1, 0};
+        long long entries = 0;
+        if (p < n_live) {
+            const int64_t b = off[p], e = off[p + 1];
+            int flags = 0;
+            if (b < 0 || e > n_vertices || e < b) flags |= 1;
+            const int64_t n = e - b;
+            if (n < 3) flags |= 2;
+            if (flags) {
+                if (lane == 0) {
+                    atomicOr(&status[0], flags);
+                    bbox[p] = make_int4(0, 0, 0, 0);
+                    area2[p] = 0;
+                }
+            } else {
+                int x0 = INT_MAX, y0 = INT_MAX, x1 = INT_MIN, y1 = INT_MIN;
+                long long a2 = 0;
+                int2 carry = src[e - 1];
+                for (int64_t i0 = 0; i0 < n; i0 += 128) {
+                    int2 v[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t i = i0 + 32 * u + lane;
-                v[u] = i < n ? xy[b + i] : xy[b];
-                w[u] = lane == 31 && i < n ? xy[b + (i + 1 == n ? 0 : i + 1)] : v[u];
-            }
+                    for (int u = 0; u < 4; ++u) {
+                        const int64_t i = i0 + 32 * u + lane;
+                        v[u] = i < n ? src[b + i] : make_int2(0, 0);
+                    }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t i = i0 + 32 * u + lane;
-                const int wx = __shfl_down_sync(0xffffffffu, v[u].x, 1);
-                const int wy = __shfl_down_sync(0xffffffffu, v[u].y, 1);
-                if (lane < 31) w[u] = make_int2(wx, wy);
-                if (i < n) {
-                    if (i + 1 == n) w[u] = xy[b];
-                    if (v[u].x < -LIM || v[u].x > LIM || v[u].y < -LIM || v[u].y > LIM) flags |= 4;
-                    x0 = min(x0, v[u].x);
-                    x1 = max(x1, v[u].x);
-                    y0 = min(y0, v[u].y);
-                    y1 = max(y1, v[u].y);
-                    a2 += (long long)v[u].x * w[u].y - (long long)w[u].x * v[u].y;
+                    for (int u = 0; u < 4; ++u) {
+                        const int64_t i = i0 + 32 * u + lane;
+                        const int rx = __shfl_sync(0xffffffffu, v[u].x, (lane + 31) & 31);
+                        const int ry = __shfl_sync(0xffffffffu, v[u].y, (lane + 31) & 31);
+                        const int wx = lane == 0 ? carry.x : rx, wy = lane == 0 ? carry.y : ry;
+                        carry = make_int2(rx, ry);
+                        if (i < n) {
+                            if (kCopy) dst[b + i] = v[u];
+                            x0 = min(x0, v[u].x);
+                            x1 = max(x1, v[u].x);
+                            y0 = min(y0, v[u].y);
+                            y1 = max(y1, v[u].y);
+                            a2 += (long long)wx * v[u].y - (long long)v[u].x * wy;
+                        }
+                    }
+                }
+                x0 = __reduce_min_sync(0xffffffffu, x0);
+                y0 = __reduce_min_sync(0xffffffffu, y0);
+                x1 = __reduce_max_sync(0xffffffffu, x1);
+                y1 = __reduce_max_sync(0xffffffffu, y1);
+                for (int o = 16; o > 0; o >>= 1) a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+                const bool bad = x0 < -LIM || x1 > LIM || y0 < -LIM || y1 > LIM;
+                if (lane == 0) {
+                    if (bad) atomicOr(&status[0], 4);
+                    // clip to the lattice domain [0, 65536)
+                    int cx0 = max(x0, 0), cy0 = max(y0, 0), cx1 = min(x1, 65536), cy1 = min(y1, 65536);
+                    if (cx1 < cx0) cx1 = cx0;
+                    if (cy1 < cy0) cy1 = cy0;
+                    bbox[p] = make_int4(cx0, cy0, cx1, cy1);
+                    area2[p] = a2;
+                    nmax = max(nmax, (int)(n < INT_MAX ? n : INT_MAX));
+                }
+                if (sz.info && n > kSlabMinVerts && n <= INT_MAX && !bad) {
+                    const int nv = (int)n, S = slab_count_for(nv, y1 - y0);
+                    const int h = max((y1 - y0 + S - 1) / S, 1);
+                    const uint64_t hm = slab_div_magic(h);
+                    int cy = src[e - 1].y;
+                    for (int e0 = 0; e0 < nv; e0 += 128) {
+                        int ay[4], by[4];
+                        ring_edge_ys(src, b, nv, e0, lane, cy, ay, by);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            if (e0 + 32 * u + lane >= nv || ay[u] == by[u]) continue;
+                            const int lo = min(ay[u], by[u]) - y0, hi = max(ay[u], by[u]) - 1 - y0;
+                            entries += slab_div(hi, hm) - slab_div(lo, hm) + 1;
+                        }
+                    }
+                    for (int o = 16; o > 0; o >>= 1) entries += __shfl_xor_sync(0xffffffffu, entries, o);
+                    si = SlabInfo{0, 0, S, h, y0};
                 }
             }
         }
-        x0 = __reduce_min_sync(0xffffffffu, x0);
-        y0 = __reduce_min_sync(0xffffffffu, y0);
-        x1 = __reduce_max_sync(0xffffffffu, x1);
-        y1 = __reduce_max_sync(0xffffffffu, y1);
-        flags = __reduce_or_sync(0xffffffffu, flags);
-        for (int o = 16; o > 0; o >>= 1) a2 += __shfl_xor_sync(0xffffffffu, a2, o);
-        if (lane == 0) {
-            if (flags) atomicOr(&status[0], flags);
-            // clip to the lattice domain [0, 65536)
-            int cx0 = max(x0, 0), cy0 = max(y0, 0), cx1 = min(x1, 65536), cy1 = min(y1, 65536);
-            if (cx1 < cx0) cx1 = cx0;
-            if (cy1 < cy0) cy1 = cy0;
-            bbox[p] = make_int4(cx0, cy0, cx1, cy1);
-            area2[p] = a2;
-            nmax = max(nmax, (int)(n < INT_MAX ? n : INT_MAX));
+        if (sz.info && lane == 0) {
+            sz.info[p] = si;
+            sz.ptr[p] = si.S > 0 ? si.S + 1 : 0;
+            sz.edge[p] = entries;
         }
     }
     if (lane == 0 && nmax > 0) atomicMax(&status[1], nmax);
 }
 
-int pmh_launch_prep(int sm_count, const int2* xy, const int64_t* off, int64_t n_polys,
-                    const int64_t* d_n, int64_t n_vertices, int4* bbox, int64_t* area2,
+int pmh_launch_prep(int sm_count, const int2* src, int2* dst, const int64_t* off, int64_t n_polys,
+                    const int64_t* d_n, int64_t n_vertices, int4* bbox, int64_t* area2, SlabSizes sz,
                     int* status, cudaStream_t s)
 {
     if (n_polys <= 0) return PMH_OK;
-    int blocks = (int)std::min<int64_t>((n_polys + 7) / 8, (int64_t)sm_count * 16);
-    prep_kernel<<<blocks, 256, 0, s>>>(xy, off, n_polys, d_n, n_vertices, bbox, area2, status);
+    const int blocks = (int)std::min<int64_t>((n_polys + 7) / 8, (int64_t)sm_count * 32);
+    auto fn = dst ? prep_kernel<true> : prep_kernel<false>;
+    fn<<<blocks, 256, 0, s>>>(src, dst, off, n_polys, d_n, n_vertices, bbox, area2, sz, status);
     PMH_LAUNCHED("prep_kernel");
     return PMH_OK;
 }
@@ -236,16 +272,34 @@ static int upload_fill(pmh_polys P, const int32_t* xy, const int64_t* offsets, b
     pmh_ctx ctx = P->ctx;
     const int64_t n_polys = P->n, n_vertices = P->nv;
     cudaMemcpyKind kind = host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+    // vertices that are on the device are copied by the kernel that reads them (an int2 load
+    // wants 8-byte alignment; others are copied first)
+    const bool fused = !host && n_polys > 0 && reinterpret_cast<uintptr_t>(xy) % sizeof(int2) == 0;
     cudaError_t e = cudaSuccess;
-    if (n_vertices > 0) e = cudaMemcpyAsync(P->xy, xy, sizeof(int2) * n_vertices, kind, s);
+    if (n_vertices > 0 && !fused) e = cudaMemcpyAsync(P->xy, xy, sizeof(int2) * n_vertices, kind, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(P->offsets, offsets, sizeof(int64_t) * (n_polys + 1), kind, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_status, 0, 2 * sizeof(int), s);
     if (e != cudaSuccess) return pmh_set_error(PMH_ERR_CUDA, "upload copy failed: %s", cudaGetErrorString(e));
     // offsets[0] and offsets[n] are checked by the kernel through b/e bounds
-    if (n_polys > 0)
-        PMH_TRY(pmh_launch_prep(ctx->sm_count, P->xy, P->offsets, n_polys, nullptr, n_vertices, P->bbox,
-                                P->area2, ctx->d_status, s));
+    int64_t* sizes = nullptr;
+    if (n_polys > 0) {
+        if (!P->slab_info && cudaMalloc(&P->slab_info, sizeof(SlabInfo) * n_polys) != cudaSuccess) {
+            cudaGetLastError();
+            return pmh_set_error(PMH_ERR_NOMEM, "slab info allocation failed");
+        }
+        PMH_TRY(pmh_scratch(ctx, SCR_MISC, sizeof(int64_t) * (size_t)(2 * (n_polys + 1)), (void**)&sizes));
+        int64_t* edge = sizes + n_polys + 1;
+        PMH_TRY(pmh_launch_prep(ctx->sm_count, fused ? reinterpret_cast<const int2*>(xy) : P->xy,
+                                fused ? P->xy : nullptr, P->offsets, n_polys, nullptr, n_vertices, P->bbox,
+                                P->area2, SlabSizes{P->slab_info, sizes, edge}, ctx->d_status, s));
+        PMH_TRY(pmh_exclusive_scan_i64(ctx, sizes, sizes, n_polys, s));
+        PMH_TRY(pmh_exclusive_scan_i64(ctx, edge, edge, n_polys, s));
+        e = cudaMemcpyAsync(ctx->h_pinned + 1, sizes + n_polys, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(ctx->h_pinned + 2, edge + n_polys, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess) return pmh_set_error(PMH_ERR_CUDA, "upload failed: %s", cudaGetErrorString(e));
+    }
     int st[2] = {0, 0};
     e = cudaMemcpyAsync(ctx->h_pinned, ctx->d_status, 2 * sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -255,6 +309,7 @@ static int upload_fill(pmh_polys P, const int32_t* xy, const int64_t* offsets, b
     if (st[0] & 2) return pmh_set_error(PMH_ERR_RANGE, "a polygon has fewer than 3 vertices");
     if (st[0] & 4) return pmh_set_error(PMH_ERR_RANGE, "a coordinate exceeds |2^20|");
     P->max_n = st[1];
+    const int64_t n_ptr = n_polys > 0 ? ctx->h_pinned[1] : 0, n_edges = n_polys > 0 ? ctx->h_pinned[2] : 0;
     if (n_polys > 0) {
         int blocks = (int)std::min<int64_t>((n_polys + 255) / 256, (int64_t)ctx->sm_count * 32);
         poly_feat_kernel<<<blocks, 256, 0, s>>>(P->area2, P->offsets, n_polys, nullptr, P->feat);
@@ -262,7 +317,7 @@ static int upload_fill(pmh_polys P, const int32_t* xy, const int64_t* offsets, b
         if ((e = cudaGetLastError()) != cudaSuccess)
             return pmh_set_error(PMH_ERR_CUDA, "feature kernel: %s", cudaGetErrorString(e));
     }
-    PMH_TRY(pmh_build_slabs(P, s));
+    PMH_TRY(pmh_build_slabs(P, sizes, sizes + n_polys + 1, n_ptr, n_edges, s));
     return pmh_build_class_order(P, s);
 }
 
@@ -311,17 +366,23 @@ static int upload_common(pmh_ctx ctx, const int32_t* xy, const int64_t* offsets,
     return PMH_OK;
 }
 
-// the per-polygon products that a reload rebuilds (their sizes follow the data)
-static void free_derived(pmh_polys p)
+// release the per-polygon products that are built later than the upload (a reload drops them),
+// and with `all` those of the upload itself
+static void free_derived(pmh_polys p, bool all)
 {
-    void* bufs[] = {p->slab_info, p->slab_ptr, p->slab_edges, p->order, p->order_cls, p->mask};
+    void* late[] = {p->order, p->mask};
+    for (void* b : late)
+        if (b) cudaFree(b);
+    p->order = nullptr;
+    p->mask = nullptr;
+    p->n_indexed = p->n_whole_cost = 0;
+    if (!all) return;
+    void* bufs[] = {p->slab_info, p->slab_ptr, p->slab_edges, p->order_cls};
     for (void* b : bufs)
         if (b) cudaFree(b);
     p->slab_info = nullptr;
-    p->slab_ptr = p->slab_edges = nullptr;
-    p->order = p->order_cls = nullptr;
-    p->mask = nullptr;
-    p->n_indexed = p->n_whole_cost = 0;
+    p->slab_ptr = p->slab_edges = p->order_cls = nullptr;
+    p->cap_slab_ptr = p->cap_slab_edges = 0;
 }
 
 extern "C" int pmh_poly_reload(pmh_polys polys, const int32_t* xy, const int64_t* offsets,
@@ -334,11 +395,19 @@ extern "C" int pmh_poly_reload(pmh_polys polys, const int32_t* xy, const int64_t
                              "vertices; got %lld, %lld)", (long long)polys->n, (long long)polys->nv,
                              (long long)n_polys, (long long)n_vertices);
     cudaStream_t s = (cudaStream_t)stream;
-    PMH_CUDA_TRY(cudaStreamSynchronize(s));  // no kernel of this stream may still read the old data
-    // (a reload that fails leaves no slab index behind)
+    // no kernel of any stream may still read the old data.  The slab lists and the class order
+    // keep their buffers while the new lists fit (releasing and taking half a gigabyte was a
+    // third of a reload of 400,000 polygons)
+    PMH_CUDA_TRY(cudaDeviceSynchronize());
     if (polys->d_slabs) PMH_CUDA_TRY(cudaMemsetAsync(polys->d_slabs, 0, sizeof(SlabPtrs), s));
-    free_derived(polys);
-    return upload_fill(polys, xy, offsets, host_memory != 0, s);
+    free_derived(polys, false);
+    const int rc = upload_fill(polys, xy, offsets, host_memory != 0, s);
+    if (rc != PMH_OK) {  // a reload that fails leaves no slab index behind
+        if (polys->d_slabs) cudaMemsetAsync(polys->d_slabs, 0, sizeof(SlabPtrs), s);
+        cudaDeviceSynchronize();
+        free_derived(polys, true);
+    }
+    return rc;
 }
 
 extern "C" int pmh_poly_upload(pmh_ctx ctx, const int32_t* d_xy, const int64_t* d_offsets,

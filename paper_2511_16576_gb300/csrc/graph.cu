@@ -38,7 +38,6 @@ struct pmh_qgraph_s {
     int64_t* slab_sizes = nullptr;
     int64_t* slab_sums = nullptr;
     int32_t* slab_ptr = nullptr;
-    int32_t* slab_cursor = nullptr;
     int32_t* slab_edges = nullptr;
     SlabPtrs* d_slabs = nullptr;
     WalkItem* walks = nullptr;        // leftover walks of the batch's signing
@@ -91,7 +90,7 @@ extern "C" int pmh_qgraph_destroy(pmh_qgraph g)
     if (g->exec) cudaGraphExecDestroy(g->exec);
     if (g->graph) cudaGraphDestroy(g->graph);
     void* bufs[] = {g->xy,        g->off,        g->bbox,       g->area2,     g->hashes,
-                    g->slab_info, g->slab_sizes, g->slab_sums,  g->slab_ptr,  g->slab_cursor,
+                    g->slab_info, g->slab_sizes, g->slab_sums,  g->slab_ptr,
                     g->slab_edges, g->counts,    g->row_ptr,    g->cand,      g->count16,
                     g->top_ids,   g->top_n,      g->jv,         g->ref_ids,   g->ref_j,
                     g->flags,     g->d_n,        g->ticket,     g->scan_sums, g->sl_ids,
@@ -165,7 +164,6 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
               cudaMalloc(&g->slab_sizes, sizeof(int64_t) * 2 * (Q + 1)) == cudaSuccess &&
               cudaMalloc(&g->slab_sums, sizeof(int64_t) * 2 * pmh_scan_sums_size(Q)) == cudaSuccess &&
               cudaMalloc(&g->slab_ptr, sizeof(int32_t) * g->cap_ptr) == cudaSuccess &&
-              cudaMalloc(&g->slab_cursor, sizeof(int32_t) * g->cap_ptr) == cudaSuccess &&
               cudaMalloc(&g->slab_edges, sizeof(int32_t) * g->cap_edges) == cudaSuccess &&
               cudaMalloc(&g->counts, sizeof(int64_t) * Q) == cudaSuccess &&
               cudaMalloc(&g->join_stage, pmh_join_stage_bytes(index, Q, g->cap)) == cudaSuccess &&
@@ -215,12 +213,12 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
     if (rc == PMH_OK && cudaMemsetAsync(g->flags, 0, sizeof(int) * 4, cs) != cudaSuccess)
         rc = pmh_set_error(PMH_ERR_CUDA, "capture memset failed");
     if (rc == PMH_OK)
-        rc = pmh_launch_prep(ctx->sm_count, g->xy, g->off, Q, g->d_n, max_vertices, g->bbox, g->area2,
+        rc = pmh_launch_prep(ctx->sm_count, g->xy, nullptr, g->off, Q, g->d_n, max_vertices, g->bbox,
+                             g->area2, SlabSizes{g->slab_info, g->slab_sizes, g->slab_sizes + Q + 1},
                              g->flags, cs);
     if (rc == PMH_OK)
         rc = pmh_launch_slabs_fixed(ctx, g->xy, g->off, Q, g->d_n, g->slab_info, g->slab_sizes,
-                                    g->slab_sums, g->slab_ptr, g->cap_ptr, g->slab_cursor, g->slab_edges,
-                                    g->cap_edges, cs);
+                                    g->slab_sums, g->slab_ptr, g->cap_ptr, g->slab_edges, g->cap_edges, cs);
     if (rc == PMH_OK)
         rc = pmh_launch_sign_unified(ctx, U, g->xy, g->off, g->bbox, g->area2, g->slab_info, g->slab_ptr,
                                      g->slab_edges, nullptr, Q, Q, 0, g->d_n, g->flags, &g->P, sidx,

@@ -202,6 +202,43 @@ struct SlabPtrs {
 // 2^21 / 64 for polygons above 256 vertices, or 1), so the floor is exact
 __host__ __device__ __forceinline__ uint64_t slab_div_magic(int h) { return (1ull << 40) / (uint64_t)h + 1ull; }
 __host__ __device__ __forceinline__ int slab_div(int x, uint64_t m) { return (int)(((uint64_t)x * m) >> 40); }
+// slabs of a polygon of n vertices and the given height
+__host__ __device__ __forceinline__ int slab_count_for(int n, int height)
+{
+    int s = n / 4;
+    s = s > 1 ? s : 1;
+    const int hmax = height > 1 ? height : 1;
+    s = s < hmax ? s : hmax;
+    return s < (1 << 16) ? s : 1 << 16;
+}
+// where A0 writes the sizes of each polygon's slab table (S + 1) and edge lists (zero for
+// polygons without an index)
+struct SlabSizes {
+    SlabInfo* info = nullptr;
+    int64_t* ptr = nullptr;
+    int64_t* edge = nullptr;
+};
+#ifdef __CUDACC__
+// y of the two end points of the edges that end at vertices e0 + 32u + lane (u < 4) of the ring
+// of n vertices at xy + b, four loads in flight per lane: an edge starts at the lane before's
+// vertex (a rotation; lane 0 takes the round before's last one, first the ring's last vertex).
+// Edge id of the edge that ends at vertex i: i - 1, or n - 1 for i = 0
+__device__ __forceinline__ void ring_edge_ys(const int2* __restrict__ xy, int64_t b, int n, int e0, int lane,
+                                             int& carry, int (&ay)[4], int (&by)[4])
+{
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int i = e0 + 32 * u + lane;
+        by[u] = i < n ? xy[b + i].y : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int r = __shfl_sync(0xffffffffu, by[u], (lane + 31) & 31);
+        ay[u] = lane == 0 ? carry : r;
+        carry = r;
+    }
+}
+#endif
 
 // Handles record their device so that they can be released after their context.
 struct pmh_polys_s {
@@ -215,8 +252,9 @@ struct pmh_polys_s {
     int32_t max_n = 0;         // largest vertex count
     float2* feat = nullptr;         // [n] log2(area) / 32, log2(n) / 16 (reranker inputs)
     SlabInfo* slab_info = nullptr;  // [n]
-    int32_t* slab_ptr = nullptr;
+    int32_t* slab_ptr = nullptr;    // (kept by a reload while its lists fit)
     int32_t* slab_edges = nullptr;
+    int64_t cap_slab_ptr = 0, cap_slab_edges = 0;
     SlabPtrs* d_slabs = nullptr;    // the three above, device-resident (rewritten by a reload)
     int32_t* order = nullptr;       // polygons by expected signing cost, largest first (built
                                     // on the first signing call without the stream index)
@@ -228,11 +266,13 @@ struct pmh_polys_s {
     uint32_t* mask = nullptr;       // [n][16] coverage masks
 };
 
-int pmh_build_slabs(pmh_polys P, cudaStream_t s);
+// the slab lists of P from the exclusive scans of its SlabSizes, whose totals the host knows
+int pmh_build_slabs(pmh_polys P, const int64_t* ptr_base, const int64_t* edge_base, int64_t n_ptr,
+                    int64_t n_edges, cudaStream_t s);
 int pmh_launch_slabs_fixed(pmh_ctx ctx, const int2* xy, const int64_t* off, int64_t max_polys,
                            const int64_t* d_n, SlabInfo* info, int64_t* sizes, int64_t* sums,
-                           int32_t* slab_ptr, int64_t cap_ptr, int32_t* cursor, int32_t* slab_edges,
-                           int64_t cap_edges, cudaStream_t s);
+                           int32_t* slab_ptr, int64_t cap_ptr, int32_t* slab_edges, int64_t cap_edges,
+                           cudaStream_t s);
 int pmh_build_masks(pmh_polys P, cudaStream_t s);
 
 // coverage masks (masks.cu): 16 x 16 cells of 2^cwl x 2^chl lattice units over the
@@ -309,8 +349,8 @@ int64_t pmh_scan_sums_size(int64_t n);
 // 2 fewer than 3 vertices, 4 coordinate range), bit 3 = candidate overflow (set
 // by the join).  Kernels after a failed stage do nothing.
 // ---------------------------------------------------------------------------
-int pmh_launch_prep(int sm_count, const int2* xy, const int64_t* off, int64_t n_polys,
-                    const int64_t* d_n, int64_t n_vertices, int4* bbox, int64_t* area2,
+int pmh_launch_prep(int sm_count, const int2* src, int2* dst, const int64_t* off, int64_t n_polys,
+                    const int64_t* d_n, int64_t n_vertices, int4* bbox, int64_t* area2, SlabSizes sz,
                     int* status, cudaStream_t s);
 int pmh_launch_sign(pmh_ctx ctx, const int2* xy, const int64_t* off, const int4* bbox,
                     const SlabInfo* slabs, const int32_t* slab_ptr, const int32_t* slab_edges,

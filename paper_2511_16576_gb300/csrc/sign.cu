@@ -354,7 +354,8 @@ int pmh_launch_sign(pmh_ctx ctx, const int2* xy, const int64_t* off, const int4*
     int64_t blocks = (int64_t)ctx->sm_count * std::max(per_sm, 1);
     // hashes per item: 32, fewer for a set with less than two such items per resident warp (an
     // item's hashes are signed one after the other; its staging is a few hashes' worth, so
-    // not below four).  1,000 polygons, K = 32: a call 53.6 us with 32-hash items and every ring binned, 28.5 now
+    // not below four).  1,000 polygons, K = 32: a call 53.6 us with 32-hash items and every
+    // ring binned, 28.5 now
     int per_item = 32;
     while (per_item > 4 && n_polys * (int64_t)((P->K + per_item - 1) / per_item) < 2 * blocks * v.W) per_item /= 2;
     const int chunks = (int)((P->K + per_item - 1) / per_item);
