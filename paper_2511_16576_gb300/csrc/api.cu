@@ -293,8 +293,7 @@ static int upload_fill(pmh_polys P, const int32_t* xy, const int64_t* offsets, b
         PMH_TRY(pmh_launch_prep(ctx->sm_count, fused ? reinterpret_cast<const int2*>(xy) : P->xy,
                                 fused ? P->xy : nullptr, P->offsets, n_polys, nullptr, n_vertices, P->bbox,
                                 P->area2, SlabSizes{P->slab_info, sizes, edge}, ctx->d_status, s));
-        PMH_TRY(pmh_exclusive_scan_i64(ctx, sizes, sizes, n_polys, s));
-        PMH_TRY(pmh_exclusive_scan_i64(ctx, edge, edge, n_polys, s));
+        PMH_TRY(pmh_exclusive_scan_i64(ctx, sizes, sizes, n_polys, s, nullptr, 2));  // sizes, edge
         e = cudaMemcpyAsync(ctx->h_pinned + 1, sizes + n_polys, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(ctx->h_pinned + 2, edge + n_polys, sizeof(int64_t), cudaMemcpyDeviceToHost, s);

@@ -162,7 +162,7 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
               cudaMalloc(&g->hashes, sizeof(uint32_t) * Q * K) == cudaSuccess &&
               cudaMalloc(&g->slab_info, sizeof(SlabInfo) * Q) == cudaSuccess &&
               cudaMalloc(&g->slab_sizes, sizeof(int64_t) * 2 * (Q + 1)) == cudaSuccess &&
-              cudaMalloc(&g->slab_sums, sizeof(int64_t) * 2 * pmh_scan_sums_size(Q)) == cudaSuccess &&
+              cudaMalloc(&g->slab_sums, sizeof(int64_t) * pmh_scan_sums_size(Q)) == cudaSuccess &&
               cudaMalloc(&g->slab_ptr, sizeof(int32_t) * g->cap_ptr) == cudaSuccess &&
               cudaMalloc(&g->slab_edges, sizeof(int32_t) * g->cap_edges) == cudaSuccess &&
               cudaMalloc(&g->counts, sizeof(int64_t) * Q) == cudaSuccess &&

@@ -336,9 +336,10 @@ __device__ __forceinline__ uint32_t pmh_mix64_lo(uint64_t z)
 // exclusive prefix sum of n int64 values in place-able form: out[i] = sum in[0..i-1],
 // out[n] = total (out has n + 1 entries).  in may alias out.
 // sums_buffer (optional, pmh_scan_sums_size(n) entries) replaces the context scratch,
-// so that a captured graph owns every buffer it touches.
+// so that a captured graph owns every buffer it touches.  arrays > 1: as many scans, the
+// arrays n + 1 entries apart.
 int pmh_exclusive_scan_i64(pmh_ctx ctx, const int64_t* in, int64_t* out, int64_t n,
-                           cudaStream_t s, int64_t* sums_buffer = nullptr);
+                           cudaStream_t s, int64_t* sums_buffer = nullptr, int arrays = 1);
 int64_t pmh_scan_sums_size(int64_t n);
 
 // ---------------------------------------------------------------------------

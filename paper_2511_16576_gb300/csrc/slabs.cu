@@ -302,7 +302,7 @@ int pmh_build_class_order(pmh_polys P, cudaStream_t s)
 // wrote (zero past *d_n), and the lists of every polygon whose lists fit the
 // buffers (slab_ptr: cap_ptr entries; slab_edges: cap_edges entries); a polygon
 // whose lists do not fit gets S = 0 and is tested over all its edges.
-// sizes: 2 * (max_polys + 1) entries; sums: 2 * pmh_scan_sums_size(max_polys).
+// sizes: 2 * (max_polys + 1) entries; sums: pmh_scan_sums_size(max_polys).
 int pmh_launch_slabs_fixed(pmh_ctx ctx, const int2* xy, const int64_t* off, int64_t max_polys,
                            const int64_t* d_n, SlabInfo* info, int64_t* sizes, int64_t* sums,
                            int32_t* slab_ptr, int64_t cap_ptr, int32_t* slab_edges, int64_t cap_edges,
@@ -311,9 +311,7 @@ int pmh_launch_slabs_fixed(pmh_ctx ctx, const int2* xy, const int64_t* off, int6
     if (max_polys <= 0) return PMH_OK;
     int64_t* ptr_sizes = sizes;
     int64_t* edge_sizes = sizes + (max_polys + 1);
-    PMH_TRY(pmh_exclusive_scan_i64(ctx, ptr_sizes, ptr_sizes, max_polys, s, sums));
-    PMH_TRY(pmh_exclusive_scan_i64(ctx, edge_sizes, edge_sizes, max_polys, s,
-                                   sums + pmh_scan_sums_size(max_polys)));
+    PMH_TRY(pmh_exclusive_scan_i64(ctx, sizes, sizes, max_polys, s, sums, 2));
     const int blocks = (int)std::min<int64_t>((max_polys + 7) / 8, (int64_t)ctx->sm_count * 16);
     slab_fill_kernel<<<blocks, kFillThreads, 0, s>>>(xy, off, max_polys, d_n, info, ptr_sizes, edge_sizes,
                                                      slab_ptr, cap_ptr, slab_edges, cap_edges);
