@@ -22,10 +22,137 @@ namespace {
 
 constexpr int kMaxK = 4096;
 constexpr int kAgreeWarps = 4;
-constexpr int kAgreeChunk = 64;  // consecutive pairs per warp turn
+constexpr int kAgreeChunk = 64;  // consecutive pairs per warp turn, fewer in a small batch
 constexpr int kAgreeGroup = 4;   // pairs compared at a time (their loads in flight together)
 
-// Warps take chunks of kAgreeChunk consecutive pairs (the row of the first by
+// pairs per warp turn: kAgreeChunk, or so many that every warp of the grid gets a turn (a
+// multiple of the pairs compared at a time).  32 pairs with features: 51 us by one
+// warp, 8.9 us by sixteen
+__device__ __forceinline__ int64_t agree_chunk(int64_t total, int64_t nwarps, int group)
+{
+    const int64_t per = (total + nwarps - 1) / nwarps;
+    return min((int64_t)kAgreeChunk, (per + group - 1) / group * group);
+}
+
+// the row holding pair x: the last q with row_ptr[q] <= x
+__device__ __forceinline__ int64_t agree_row_of(const int64_t* __restrict__ row_ptr, int64_t Q, int64_t x)
+{
+    int64_t lo = 0, hi = Q;
+    while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (row_ptr[mid] <= x) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// Rows of at most 128 hashes (K % 4 == 0): a lane holds four hashes of the query, read once per
+// row of candidates, and eight pairs' rows are in flight at a time.  The band bits come from
+// the lanes' four equality bits with one shuffle or ballot (bands whose hashes do not straddle
+// lanes unevenly: rows 1, 2, or a multiple of 4).  Bound by the issue rate and L2: with the
+// query reloaded and the equality words built in shared memory for every pair it was 170
+// issue slots a pair.  4,096 queries, 4.0M pairs of 300,000 rows, 64 x 2 bands: 606 -> 352 us
+// (5.9 TB/s of rows, two thirds of them out of L2)
+constexpr int kAgreeRowK = 128;
+constexpr int kAgreeRowGroup = 8;
+
+template <bool kFeat>  // (kFeat: K = 128)
+__global__ void __launch_bounds__(kAgreeWarps * 32, kFeat ? 6 : 8)
+agree_short_kernel(const uint32_t* __restrict__ qh, const uint32_t* __restrict__ ph,
+                   const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ cand, int64_t Q,
+                   int64_t cap, int K, int bands, int rows, uint32_t T, uint16_t* __restrict__ count,
+                   uint32_t* __restrict__ bandmask, __nv_bfloat16* __restrict__ feat, FeatSrc qf,
+                   FeatSrc pf, const int* __restrict__ d_flags)
+{
+    constexpr int G = kAgreeRowGroup;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (d_flags && *d_flags) return;  // failed validation or candidate overflow
+    const int64_t total = min(row_ptr[Q], cap);
+    const int64_t nwarps = (int64_t)gridDim.x * kAgreeWarps;
+    // (a pair's feature inputs are fetched pair by pair: two pairs a warp while that fills no grid)
+    const int64_t chunk = agree_chunk(total, nwarps, kFeat ? 2 : G);
+    const bool in = lane < K / 4;
+    // band `lane` in the equality bits: bits [bsh, bsh + rows) of lane bsrc, or (rows % 4 == 0) the
+    // rows / 4 lanes from lane bsh on
+    const bool whole = rows >= 4, band = lane < bands;
+    const int bsrc = whole ? 0 : (lane * rows) >> 2, bsh = whole ? (rows / 4) * lane : (lane * rows) & 3;
+    const uint32_t bneed = whole ? (rows >= 128 ? ~0u : (1u << (rows / 4)) - 1u) : (1u << rows) - 1u;
+    uint4 u = make_uint4(0u, 0u, 0u, 0u);
+    unsigned live = 0;  // this lane's hashes of the query that were found (not T)
+    int64_t uq = -1;    // the query u holds
+    for (int64_t ch = (int64_t)blockIdx.x * kAgreeWarps + wid; ch * chunk < total; ch += nwarps) {
+        const int64_t x0 = ch * chunk, x1 = min(x0 + chunk, total);
+        const int64_t q0 = agree_row_of(row_ptr, Q, x0);
+        for (int64_t xb = x0; xb < x1; xb += 32) {
+            const int nvalid = (int)min((int64_t)32, x1 - xb);
+            int64_t ql = q0;
+            int32_t pl = 0;
+            if (lane < nvalid) {
+                while (row_ptr[ql + 1] <= xb + lane) ++ql;
+                pl = cand[xb + lane];
+            }
+            const int64_t qprev = __shfl_up_sync(0xffffffffu, ql, 1);
+            const unsigned turns = __ballot_sync(0xffffffffu, lane < nvalid && ql != (lane ? qprev : uq));
+            int my_count = 0;
+            unsigned my_bands = 0;
+            for (int t0 = 0; t0 < nvalid; t0 += G) {
+                uint4 v[G];
+#pragma unroll
+                for (int t = 0; t < G; ++t) {
+                    const int64_t pp = __shfl_sync(0xffffffffu, pl, t0 + t);
+                    v[t] = make_uint4(0u, 0u, 0u, 0u);
+                    if (in && t0 + t < nvalid) v[t] = __ldg(reinterpret_cast<const uint4*>(ph + pp * K) + lane);
+                }
+#pragma unroll
+                for (int t = 0; t < G; ++t) {
+                    if (t0 + t >= nvalid) continue;  // warp-uniform
+                    if ((turns >> (t0 + t)) & 1u) {
+                        uq = __shfl_sync(0xffffffffu, ql, t0 + t);
+                        if (in) u = __ldg(reinterpret_cast<const uint4*>(qh + uq * K) + lane);
+                        live = in ? (unsigned)(u.x != T) | ((unsigned)(u.y != T) << 1) |
+                                        ((unsigned)(u.z != T) << 2) | ((unsigned)(u.w != T) << 3)
+                                  : 0u;
+                    }
+                    const unsigned bits = ((unsigned)(u.x == v[t].x) | ((unsigned)(u.y == v[t].y) << 1) |
+                                           ((unsigned)(u.z == v[t].z) << 2) | ((unsigned)(u.w == v[t].w) << 3)) &
+                                          live;
+                    int ct = __popc(bits), lt = 0, gt = 0;
+                    if (kFeat) {  // the three counts in one sum (10 bits each)
+                        lt = (u.x < v[t].x) + (u.y < v[t].y) + (u.z < v[t].z) + (u.w < v[t].w);
+                        gt = (u.x > v[t].x) + (u.y > v[t].y) + (u.z > v[t].z) + (u.w > v[t].w);
+                        const int sum = __reduce_add_sync(0xffffffffu, ct | (lt << 10) | (gt << 20));
+                        ct = sum & 1023;
+                        lt = (sum >> 10) & 1023;
+                        gt = sum >> 20;
+                    } else {
+                        ct = __reduce_add_sync(0xffffffffu, ct);
+                    }
+                    if (lane == t0 + t) my_count = ct;
+                    if (bandmask) {
+                        const uint32_t from = whole ? __ballot_sync(0xffffffffu, bits == 0xFu)
+                                                    : __shfl_sync(0xffffffffu, bits, bsrc);
+                        const unsigned mb = __ballot_sync(0xffffffffu, band && ((from >> (bsh & 31)) & bneed) == bneed);
+                        if (lane == t0 + t) my_bands = mb;
+                    }
+                    if (kFeat) {
+                        const int64_t q = __shfl_sync(0xffffffffu, ql, t0 + t);
+                        const int64_t pp = __shfl_sync(0xffffffffu, pl, t0 + t);
+                        const float fhi = pmh_feature_col(lane, K, ct, lt, gt, pmh_feat_pair(qf, pf, q, pp));
+                        __nv_bfloat16* f = feat + (xb + t0 + t) * 48;
+                        f[lane] = __float2bfloat16_rn(bits == 0xFu ? 1.f : 0.f);
+                        if (lane < 16) f[32 + lane] = __float2bfloat16_rn(fhi);
+                    }
+                }
+            }
+            if (lane < nvalid) {
+                if (count) count[xb + lane] = (uint16_t)my_count;
+                if (bandmask) bandmask[xb + lane] = my_bands;
+            }
+        }
+    }
+}
+
+// Rows of any K.  Warps take chunks of consecutive pairs (the row of the first by
 // binary search over row_ptr); 32 pairs at a time each lane reads one pair's
 // candidate id and steps its row on from there, and the warp then compares the
 // pairs four at a time (ids and rows by shuffle).  Per pair:
@@ -49,16 +176,10 @@ agree_rows_kernel(const uint32_t* __restrict__ qh, const uint32_t* __restrict__ 
     // equality words in shared memory: for the band bits, and for the features' groups
     // unless K = 128 (then lane l holds group l's four hashes)
     const bool need_eq = bandmask || (kFeat && K != 128);
-    for (int64_t ch = (int64_t)blockIdx.x * kAgreeWarps + wid; ch * kAgreeChunk < total; ch += nwarps) {
-        const int64_t x0 = ch * kAgreeChunk, x1 = min(x0 + kAgreeChunk, total);
-        // the row holding pair x0: the last q with row_ptr[q] <= x0
-        int64_t lo = 0, hi = Q;
-        while (hi - lo > 1) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (row_ptr[mid] <= x0) lo = mid;
-            else hi = mid;
-        }
-        const int64_t q0 = lo;
+    const int64_t chunk = agree_chunk(total, nwarps, kAgreeGroup);
+    for (int64_t ch = (int64_t)blockIdx.x * kAgreeWarps + wid; ch * chunk < total; ch += nwarps) {
+        const int64_t x0 = ch * chunk, x1 = min(x0 + chunk, total);
+        const int64_t q0 = agree_row_of(row_ptr, Q, x0);
         for (int64_t xb = x0; xb < x1; xb += 32) {
             const int nvalid = (int)min((int64_t)32, x1 - xb);
             const int64_t xl = xb + lane;
@@ -449,11 +570,17 @@ int pmh_launch_agree_features(pmh_ctx ctx, const uint32_t* qh, const uint32_t* p
 {
     if (Q <= 0) return PMH_OK;
     const int blocks = ctx->sm_count * 16;  // persistent: pair chunks are handed out in turn
-    auto fn = feat ? agree_rows_kernel<true> : agree_rows_kernel<false>;
+    // rows of at most 128 hashes that 16-byte loads can read, if the bands are whole lanes or lie
+    // inside one; features only at K = 128 (a lane's hashes are then a feature's group)
+    const bool bands_fit = !bandmask || P->rows <= 2 || P->rows % 4 == 0;
+    const bool aligned = ((reinterpret_cast<uintptr_t>(qh) | reinterpret_cast<uintptr_t>(ph)) & 15) == 0;
+    const bool short_rows = P->K % 4 == 0 && P->K <= kAgreeRowK && (!feat || P->K == 128) && bands_fit && aligned;
+    auto fn = short_rows ? (feat ? agree_short_kernel<true> : agree_short_kernel<false>)
+                         : (feat ? agree_rows_kernel<true> : agree_rows_kernel<false>);
     fn<<<blocks, kAgreeWarps * 32, 0, s>>>(qh, ph, row_ptr, cand, Q, cap, (int)P->K, (int)P->bands, (int)P->rows,
                                            P->T, count, bandmask, reinterpret_cast<__nv_bfloat16*>(feat), qf,
                                            pf, d_flags);
-    PMH_LAUNCHED("agree_rows_kernel");
+    PMH_LAUNCHED(short_rows ? "agree_short_kernel" : "agree_rows_kernel");
     return PMH_OK;
 }
 
