@@ -279,12 +279,16 @@ __device__ __forceinline__ uint32_t slot_hash(int32_t p)
 }
 
 // candidate p's tuple of band j equals the query's, both tuples read at once (16-byte
-// loads for 4 or 8 rows when vec: K % 4 == 0)
+// loads for 4 or 8 rows, 8-byte ones for 2, when vec: K % 4 == 0)
 __device__ __forceinline__ bool tuple_match2(const uint32_t* __restrict__ qh, const uint32_t* __restrict__ dbrow,
                                              int j, int rows, bool vec)
 {
     const uint32_t* a = qh + j * rows;
     const uint32_t* b = dbrow + j * rows;
+    if (vec && rows == 2) {
+        const uint2 u = __ldg(reinterpret_cast<const uint2*>(a)), v = __ldg(reinterpret_cast<const uint2*>(b));
+        return u.x == v.x && u.y == v.y;
+    }
     if (vec && rows == 4) {
         const uint4 u = __ldg(reinterpret_cast<const uint4*>(a)), v = __ldg(reinterpret_cast<const uint4*>(b));
         return u.x == v.x && u.y == v.y && u.z == v.z && u.w == v.w;
@@ -778,8 +782,8 @@ warp_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int ban
 // sorting a row of a few hundred costs; the block grows with the bitmap (256 threads
 // while four blocks fit an SM) so that its time per row stays the same.  Bound by the
 // latency of hashes -> directory -> entries -> tuples, and by the tuples' sectors.
-// 4,096 queries of 64 x 2 bands against 300,000 polygons (880 candidates a query): 0.51 ms
-// a pass, 1.12 with the open-addressing set.
+// 4,096 queries of 64 x 2 bands against 300,000 polygons (880 candidates a query): 0.33 ms
+// a pass, 0.54 when every entry's tuple was read, 1.12 with the open-addressing set.
 //
 // Which sets: with tuples of one or two hashes (rows of hundreds to thousands) up to
 // 2^20 ids, where one bitmap still fits an SM (4,096 queries of 64 x 2 bands, 520,000
@@ -802,7 +806,8 @@ bitmap_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int b
                    const int64_t* __restrict__ d_n, int* __restrict__ d_flags)
 {
     extern __shared__ uint4 bits[];
-    __shared__ JoinBands jb;
+    // (32 bits: at most 2^20 ids under 128 bands)
+    __shared__ int blo[kMaxBandsPerLane * 32], boff[kMaxBandsPerLane * 32 + 1];
     __shared__ uint32_t bcomp[kMaxBandsPerLane * 32];
     __shared__ int wsum[32];
     __shared__ long long stage_off;
@@ -830,57 +835,64 @@ bitmap_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int b
         // the bands' directory slots, the bitmap cleared meanwhile
         for (int j = threadIdx.x; j < bands; j += blockDim.x) {
             const uint64_t key = band_key(qh, j, rows, T, lsh_seed);
-            int64_t lo = 0, n = 0;
+            int lo = 0, n = 0;
             uint32_t c = 0;
             if (key != PMH_INVALID_KEY) {
                 c = composite(key, j, band_bits);
-                lo = dir[c >> dsh];
-                n = dir[(c >> dsh) + 1] - lo;
+                lo = (int)dir[c >> dsh];
+                n = (int)dir[(c >> dsh) + 1] - lo;
             }
             bcomp[j] = c;
-            jb.lo[j] = lo;
-            jb.off[j + 1] = n;
+            blo[j] = lo;
+            boff[j + 1] = n;
         }
         for (int i = threadIdx.x; i < words4; i += blockDim.x) bits[i] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
         if (wid == 0) {  // prefix of the bands' entry counts
-            int64_t carry = 0;
+            int carry = 0;
             for (int j0 = 0; j0 < bands; j0 += 32) {
                 const int j = j0 + lane;
-                int64_t x = j < bands ? jb.off[j + 1] : 0;
+                int x = j < bands ? boff[j + 1] : 0;
                 for (int o = 1; o < 32; o <<= 1) {
-                    const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+                    const int y = __shfl_up_sync(0xffffffffu, x, o);
                     if (lane >= o) x += y;
                 }
-                if (j < bands) jb.off[j + 1] = carry + x;
+                if (j < bands) boff[j + 1] = carry + x;
                 carry += __shfl_sync(0xffffffffu, x, 31);
             }
-            if (lane == 0) jb.off[0] = 0;
+            if (lane == 0) boff[0] = 0;
         }
         __syncthreads();
-        const int64_t total = jb.off[bands];
-        for (int64_t g0 = (int64_t)wid * (32 * kBitmapU); g0 < total; g0 += (int64_t)nw * (32 * kBitmapU)) {
+        const int total = boff[bands];
+        const volatile uint32_t* found = word;
+        for (int g0 = wid * (32 * kBitmapU); g0 < total; g0 += nw * (32 * kBitmapU)) {
             int jj[kBitmapU];
             int32_t pp[kBitmapU];
             bool in[kBitmapU];
+            int lo = 0, hi = bands;  // the band holding the lane's first entry: the last j with boff[j] <= g
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (boff[mid] <= g0 + lane) lo = mid;
+                else hi = mid;
+            }
 #pragma unroll
             for (int u = 0; u < kBitmapU; ++u) {
-                const int64_t g = g0 + 32 * u + lane;
+                const int g = g0 + 32 * u + lane;
                 in[u] = g < total;
-                int lo = 0, hi = bands;  // the band holding entry g: the last j with off[j] <= g
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (jb.off[mid] <= g) lo = mid;
-                    else hi = mid;
-                }
-                jj[u] = lo;
                 pp[u] = 0;
                 if (in[u]) {
-                    const int64_t x = jb.lo[lo] + (g - jb.off[lo]);
+                    while (boff[lo + 1] <= g) ++lo;  // (boff[bands] = total > g)
+                    const int x = blo[lo] + (g - boff[lo]);
                     pp[u] = ids[x];
                     in[u] = comp[x] == bcomp[lo];
                 }
+                jj[u] = lo;
             }
+            // (an id that another band has found needs no second look: its tuple's sector is the
+            // walk's largest cost, and most entries of short tuples are such)
+#pragma unroll
+            for (int u = 0; u < kBitmapU; ++u)
+                in[u] = in[u] && !((found[pp[u] >> 5] >> (pp[u] & 31)) & 1u);
 #pragma unroll
             for (int u = 0; u < kBitmapU; ++u)
                 if (in[u] && tuple_match2(qh, dbh + (int64_t)pp[u] * K, jj[u], rows, vec))
