@@ -779,11 +779,11 @@ warp_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int ban
 // by the composite read beside the id, instead of a bisection of dependent reads),
 // concatenated and split evenly over the warps, four entries per lane in flight.
 // Clearing and reading the bitmap costs n / 128 shared vectors per row, about what
-// sorting a row of a few hundred costs; the block grows with the bitmap (256 threads
-// while four blocks fit an SM) so that its time per row stays the same.  Bound by the
+// sorting a row of a few hundred costs; the block grows with the bitmap, so that an SM's
+// warps stay the same.  Bound by the
 // latency of hashes -> directory -> entries -> tuples, and by the tuples' sectors.
-// 4,096 queries of 64 x 2 bands against 300,000 polygons (880 candidates a query): 0.33 ms
-// a pass, 0.54 when every entry's tuple was read, 1.12 with the open-addressing set.
+// 4,096 queries of 64 x 2 bands against 300,000 polygons (880 candidates a query): 0.22 ms
+// a pass, 0.54 when every entry's tuple was read by 256 threads, 1.12 with the open-addressing set.
 //
 // Which sets: with tuples of one or two hashes (rows of hundreds to thousands) up to
 // 2^20 ids, where one bitmap still fits an SM (4,096 queries of 64 x 2 bands, 520,000
@@ -1230,7 +1230,9 @@ static JoinStage stage_view(void* buf, int64_t Q, int64_t pool_ints)
     return st;
 }
 
-// the bitmap join's pass: 256 threads while four bitmaps fit an SM, more as they grow
+// the bitmap join's pass: as many threads as fill an SM beside the bitmaps that fit it, since its
+// time is the latency of dependent reads (4,096 queries of 64 x 2 bands, 300,000 polygons, five
+// 37 KB bitmaps an SM: 331 us with 256 threads, 218 with 512; 32 x 4 bands, 400,000: 122 and 99)
 static int launch_bitmap(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* d_n, int64_t* counts,
                          const int64_t* row_ptr, int32_t* cand, int64_t cap, const JoinStage& st,
                          bool deferred, int* d_flags, bool write, cudaStream_t s)
@@ -1240,8 +1242,8 @@ static int launch_bitmap(pmh_index X, const uint32_t* qh, int64_t Q, const int64
     const size_t smem = sizeof(uint4) * (size_t)std::max(words4, 1);
     // (a batch that leaves SMs with one or two queries gives those the threads instead: one query
     // of 64 x 2 bands, 200,000 polygons: 33 us with 256 threads, 17 with 1,024)
-    const int64_t sms = X->ctx->sm_count;
-    const int threads = smem > 104 * 1024 || Q <= sms ? 1024 : smem > 50 * 1024 || Q <= 2 * sms ? 512 : 256;
+    const int64_t sms = X->ctx->sm_count, fit = (225 * 1024) / ((int64_t)smem + 2048);
+    const int threads = fit < 4 || Q <= sms ? 1024 : fit < 8 || Q <= 2 * sms ? 512 : 256;
     auto fn = write ? bitmap_join_kernel<true> : bitmap_join_kernel<false>;
     PMH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 1;
