@@ -20,10 +20,14 @@
 // fp64 in coordinates relative to B's first vertex, summed exactly.  GB300's fp64 rate is low,
 // so the fp64 work is kept to the crossings (a few per edge) and one Newton
 // reciprocal each.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <climits>
 
 #include "pmh_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -640,7 +644,7 @@ refine_pairs_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qo
 }
 
 // ---------------------------------------------------------------------------
-// Pairs with a ring above kRefineBigVerts vertices: a block each.  The two-warp form
+// Pairs with a ring above kRefineBigVerts vertices: a cluster each.  The two-warp form
 // keeps both rings' slab lists in 2,048 shared references; above ~1,700 vertices they
 // overflow and every edge pair was tested (n * m predicates by 64 threads).  Here a
 // ring's lists are the y-slab index of its set (slabs.cu: about n / 4 slabs, read from
@@ -657,10 +661,14 @@ refine_pairs_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qo
 // added as two integers (multiples of 2^-18, and the remainder's of 2^-56, modulo 2^64):
 // sums of integers do not depend on their order, so neither the list order (atomics)
 // nor the split over the threads shows in the result.
-// Bound by the latency of list entry -> two vertices, from L1/L2; 512 threads a pair.
-// 512 pairs of coastlines of 4 to 16,384 vertices: 0.94 ms, 153 ms before.
+// Bound by the latency of list entry -> two vertices, from L1/L2, and by each vertex's own
+// list.  Two blocks a pair: with one the launch ended with its largest pairs, with four or eight
+// the shared set-up weighed more.  512 pairs of coastlines of 4 to 16,384 vertices: 0.53 ms;
+// 0.82 with one block, 0.62 with four, 0.83 with eight; 153 ms in the two-warp form.
 // ---------------------------------------------------------------------------
-constexpr int kBigThreads = 512;
+constexpr int kBigThreads = 512;  // per block of a pair's cluster
+constexpr int kBigBlocks = 1024 / kBigThreads;  // resident an SM
+constexpr int kBigCluster = 2;
 constexpr int kBigWarps = kBigThreads / 32;
 constexpr int kBigCap = 2048;     // shared references of a ring without a slab index
 constexpr int kBigSlabs = 256;
@@ -773,7 +781,7 @@ __device__ __forceinline__ void push_crossings(bool hit, int i, int j, uint2* cq
     }
 }
 
-__global__ void __launch_bounds__(kBigThreads, 2)
+__global__ void __cluster_dims__(kBigCluster, 1, 1) __launch_bounds__(kBigThreads, kBigBlocks)
 refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff,
                   const int64_t* __restrict__ qarea2, const SlabPtrs* __restrict__ qslabs,
                   const int2* __restrict__ pxy, const int64_t* __restrict__ poff,
@@ -785,22 +793,30 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
     __shared__ BigSmem s;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const long long queued = (long long)ticket[1];
+    // the cluster's blocks share a pair: its vertices and edges are dealt to their threads in turn,
+    // its ranges and sums are added up in their shared memories
+    const cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), ctid = rank * kBigThreads + tid;
+    constexpr int kStride = kBigThreads * kBigCluster;
     for (;;) {
-        __syncthreads();
-        if (tid == 0) s.e = (long long)atomicAdd(ticket + 2, 1ull);
+        cl.sync();
+        if (tid == 0 && rank == 0) {
+            const long long next = (long long)atomicAdd(ticket + 2, 1ull);
+            for (int r = 0; r < kBigCluster; ++r) *cl.map_shared_rank(&s.e, r) = next;
+        }
         if (tid < 2) {
             s.range[tid][0] = s.range[tid][2] = INT_MAX;
             s.range[tid][1] = s.range[tid][3] = INT_MIN;
         }
         if (tid == 0) s.ends = s.q18 = s.r56 = 0;
-        __syncthreads();
+        cl.sync();
         if (s.e >= queued) break;
         const int64_t e = e0 + big[s.e];
         const int64_t q = qid_list ? (int64_t)qid_list[e] : e / m;
         const int64_t p = ids[e];
         const PairView va = view(qxy, qoff, qarea2, q), vb = view(pxy, poff, parea2, p);
-        if (va.sgn == 0 || vb.sgn == 0) {  // (uniform over the block)
-            if (tid == 0) out[e] = 0.0;
+        if (va.sgn == 0 || vb.sgn == 0) {  // (uniform over the cluster)
+            if (ctid == 0) out[e] = 0.0;
             continue;
         }
         // both rings' ranges
@@ -810,7 +826,7 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
             const int n = r ? vb.n : va.n;
             int x0 = INT_MAX, x1 = INT_MIN, y0 = INT_MAX, y1 = INT_MIN;
 #pragma unroll 4
-            for (int i = tid; i < n; i += kBigThreads) {
+            for (int i = ctid; i < n; i += kStride) {
                 const int2 u = v[i];
                 x0 = min(x0, u.x);
                 x1 = max(x1, u.x);
@@ -821,14 +837,15 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
             x1 = __reduce_max_sync(0xffffffffu, x1);
             y0 = __reduce_min_sync(0xffffffffu, y0);
             y1 = __reduce_max_sync(0xffffffffu, y1);
-            if (lane == 0) {
-                atomicMin(&s.range[r][0], x0);
-                atomicMax(&s.range[r][1], x1);
-                atomicMin(&s.range[r][2], y0);
-                atomicMax(&s.range[r][3], y1);
+            if (lane < kBigCluster) {
+                int* range = cl.map_shared_rank(s.range[r], lane);
+                atomicMin(range + 0, x0);
+                atomicMax(range + 1, x1);
+                atomicMin(range + 2, y0);
+                atomicMax(range + 3, y1);
             }
         }
-        __syncthreads();
+        cl.sync();
         ListRing A{va.v, va.n, nullptr, nullptr, 0, 0, 0, s.range[0][0], s.range[0][1]};
         ListRing B{vb.v, vb.n, nullptr, nullptr, 0, 0, 0, s.range[1][0], s.range[1][1]};
         // lists: the set's slab index, else shared lists (warp r builds ring r's), else
@@ -867,7 +884,7 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
         long long ends = 0;  // twice the end terms
         ExactSum sum;
         // end terms of A's edges: vertex a_i + e inside B closes edge i - 1
-        for (int i = tid; i < A.n; i += kBigThreads) {
+        for (int i = ctid; i < A.n; i += kStride) {
             const int2 a = A.v[i];
             if (a.y < yb0 || a.y > yb1 || a.x < B.x0 || a.x > B.x1) continue;
             int lo, hi;
@@ -888,7 +905,7 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
             }
         }
         // end terms of B's edges: vertex c_j - e inside A closes edge j - 1
-        for (int j = tid; j < B.n; j += kBigThreads) {
+        for (int j = ctid; j < B.n; j += kStride) {
             const int2 c = B.v[j];
             if (c.y < ya0 || c.y > ya1 || c.x < A.x0 || c.x > A.x1) continue;
             int lo, hi;
@@ -910,7 +927,7 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
         }
         // crossings of A's edges with B's non-horizontal edges
         int nq = 0;  // warp-uniform queue length
-        for (int i0 = 32 * wid; i0 < A.n; i0 += kBigThreads) {
+        for (int i0 = ctid & ~31; i0 < A.n; i0 += kStride) {
             const int i = i0 + lane;
             int2 a = make_int2(0, 0), b = make_int2(0, 0);
             int k0 = 0, cntk = 0, q0 = 0;
@@ -951,7 +968,7 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
             }
         }
         // crossings of B's horizontal edges with A's edges
-        for (int j0 = 32 * wid; j0 < B.n; j0 += kBigThreads) {
+        for (int j0 = ctid & ~31; j0 < B.n; j0 += kStride) {
             const int j = j0 + lane;
             int2 c = make_int2(0, 0), d = make_int2(0, 0);
             int lo = 0, hi = 0;
@@ -980,12 +997,13 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
         }
         sum.reduce();
         if (lane == 0) {
-            atomicAdd(&s.ends, en);
-            atomicAdd(&s.q18, sum.q18);
-            atomicAdd(&s.r56, sum.r56);
+            BigSmem* first = cl.map_shared_rank(&s, 0);
+            atomicAdd(&first->ends, en);
+            atomicAdd(&first->q18, sum.q18);
+            atomicAdd(&first->r56, sum.r56);
         }
-        __syncthreads();
-        if (tid == 0) {
+        cl.sync();
+        if (ctid == 0) {
             const double inter = ExactSum{s.q18, s.r56}.total((long long)s.ends);
             const double uni = va.area + vb.area - inter;
             out[e] = uni > 0 ? fmin(fmax(inter / uni, 0.0), 1.0) : 0.0;
@@ -1078,7 +1096,7 @@ static int launch_refine(pmh_ctx ctx, const RefineQueries& qs, pmh_polys db, con
             e0, e1, out, tickets, big, d_n);
         PMH_LAUNCHED("refine_pairs_kernel");
         if (!big) continue;
-        const int bblocks = (int)std::min<int64_t>(e1 - e0, (int64_t)ctx->sm_count * 2);
+        const int bblocks = kBigCluster * (int)std::min<int64_t>(e1 - e0, std::max(ctx->sm_count * kBigBlocks / kBigCluster, 1));
         refine_big_kernel<<<bblocks, kBigThreads, 0, s>>>(qs.xy, qs.off, qs.area2, qs.slabs, db->xy, db->offsets,
                                                           db->area2, db->d_slabs, ids, m, qid_list, e0, out,
                                                           tickets, big);
