@@ -49,6 +49,12 @@ constexpr int kMaskN = 32;         // coverage mask cells per side
 constexpr int kGroup = 128;        // hashes signed together, four a lane
 constexpr int kQueue = 192;        // candidates: at most 31, + 128 of a cell, + 32 that follow exact tests
 constexpr uint32_t kNoPoint = 0xFFFFFFFFu;
+// A few hashes of a polygon of large area are walked: K walks of 2^32 / area points cost less than
+// classifying the cells under the box.  The staged class keeps its own build, without the walk,
+// unless K = 1.  K = 1, 149,000 centred polygons of 9 vertices: 503 us (692 indexed); K = 3,
+// 100,000 of 317 vertices: 1,669 (1,845); from K = 16 on the index is the faster form.
+constexpr int kBriefMaxK = 12;
+constexpr float kBriefWalk = 3000.0f;
 constexpr int kIdxU = 4;           // points per lane per round of a leftover walk
 constexpr int kMaskMaxEdges = 4096;  // larger polygons skip the mask (every cell is a boundary cell)
 
@@ -618,9 +624,10 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
             continue;
         }
         // the indexed form's grid level (-1: no index) and the expected walk
-        const int level = S.lv[0].first && area2 ? pmh_index_level(bb, K) : -1;
         const long long a2 = area2 ? area2[p] : 0;
         const float walk = 4294967296.0f / fmaxf(0.5f * (float)(a2 < 0 ? -a2 : a2), 1.0f);
+        const bool brief = !kIndexedOnly && K <= kBriefMaxK && (float)K * walk < kBriefWalk;
+        const int level = S.lv[0].first && area2 && !brief ? pmh_index_level(bb, K) : -1;
         if (staged) {
             // stage the polygon (closed: v[n] = v[0]; cp.async 8-byte copies) and bin its edges
             stage_vertices(m.v, xy + b, n, lane);
@@ -844,7 +851,8 @@ int pmh_launch_sign_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* o
     if (n_slots <= 0) return PMH_OK;
     PMH_CUDA_TRY(cudaMemsetAsync(wq.tickets, 0, sizeof(unsigned long long) * kSignTickets, s));
     // the indexed class at the list's end goes to its own launch (needs the class list)
-    const int64_t tail = list && !d_n ? std::min(std::max<int64_t>(n_indexed_tail, 0), n_slots - n_chunked) : 0;
+    // (of a single hash most of it walks: the other build)
+    const int64_t tail = list && !d_n && P->K > 1 ? std::min(std::max<int64_t>(n_indexed_tail, 0), n_slots - n_chunked) : 0;
     if (n_slots - tail > 0)
         PMH_TRY(launch_unified<false>(ctx, U, xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list,
                                       n_slots - tail, n_chunked, d_n, d_flags, P, S, wq, out, work, s));

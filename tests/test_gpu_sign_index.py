@@ -49,3 +49,17 @@ def test_production_hashes(B, orc, shape, K):
     ref = orc.sign(sub.xy, sub.offsets, SEED, K, 1 << 24, nthreads=16)
     assert np.array_equal(counted[torch.from_numpy(rows).to(DEV)].cpu().numpy().view(np.uint32), ref)
     ctx.close()
+
+
+@pytest.mark.parametrize("K", [1, 2, 12, 13])
+def test_few_hashes(B, orc, K):
+    """Large polygons of few hashes: walked or indexed by their area, staged or not."""
+    ctx = B.Context(0)
+    B.sign_count_work(ctx, False)
+    P = B.make_params(K, 1, 1 << 22, SEED, flags=B.FLAG_STREAM_INDEX)
+    for n_range in ((3, 40), (250, 600)):
+        db = synth.star_polygons(1500, 9 + K, n_range=n_range, n_dist="loguniform", f_range=(1e-4, 0.1))
+        polys = B.poly_upload(ctx, torch.from_numpy(db.xy).to(DEV), torch.from_numpy(db.offsets).to(DEV))
+        got = B.minhash_sign(ctx, polys, P).cpu().numpy().view(np.uint32)
+        assert np.array_equal(got, orc.sign(db.xy, db.offsets, SEED, K, 1 << 22, nthreads=16))
+    ctx.close()
