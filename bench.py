@@ -41,13 +41,14 @@ sys.path.insert(0, ROOT)
 #  walked stream point: 64-bit counter add (2), two xor-shift rounds (4 + 4), two
 #    low-64-bit 64x64 multiplies (4 + 4), final xor-shift of the low word (2), field
 #    extraction and half-open bbox test (6) = 26;
-#  grid cell read by the indexed form: two offsets and the cell address = 8;
-#  stream-index entry read: index and point loads, limit compare, bbox test = 10;
-#  bbox candidate classified = 6;
+#  (cell, hash) first point read by the indexed form: a minimum or a comparison, and the
+#    vote = 2;
+#  next point of a cell's list read: two offsets, the limit compare and the new tag = 10;
+#  bbox candidate: its point from the generator and bbox test (26) and its classification = 32;
 #  polygon edge tested: straddle test (3), two 32x32->64 products (4), difference (2),
 #    sign test and parity (3) = 12;
 #  candidate decided by the coverage mask: cell address and code lookup = 6.
-SIGN_OP_WEIGHTS = {"walk_points": 26, "cells": 8, "index_entries": 10, "candidates": 6,
+SIGN_OP_WEIGHTS = {"walk_points": 26, "cells": 2, "index_entries": 10, "candidates": 32,
                    "edge_tests": 12, "mask_decisions": 6}
 # the signing kernel's sources: a profile summary applies only to the source it was taken on
 SIGN_SOURCES = ["paper_2511_16576_gb300/csrc/sign_unified.cu",
@@ -703,7 +704,7 @@ def main():
                           "frac": ops / (kms * 1e-3) / peak if kms > 0 else None}
     dom = max(kernels, key=lambda k: kernels[k]["ms"])
     units = kernels[dom]["work_units_per_launch"]
-    gather_bytes = 8 * (units["cells"] + units["index_entries"])
+    gather_bytes = 4 * units["cells"] + 16 * units["index_entries"]
     prof = profiled_counters(N, w.name) if dom == "sign_unified_kernel" else None
     roofline = {"bound": "alu", "kernel": dom, "achieved": kernels[dom]["achieved"],
                 "peak": peak / 1e12, "unit": "Tintop/s", "frac": kernels[dom]["frac"],
@@ -716,8 +717,9 @@ def main():
                 "peak_source": "measured: pmh_probe_int_peak (integer mad/add/xor/shl mix, all SMs)",
                 "peak_nominal": nominal_int_peak(dev, clk),
                 "kernels": kernels, "timed_launches": kernel_ms["calls"],
-                # the index gather: cell records and entries read (8 B each), against the L2
-                # sector bytes ncu counted for the launch
+                # the index gather: the cells' first points (4 B per hash) and the points read
+                # after them (two list offsets and an entry, 16 B), against the L2 sector bytes
+                # ncu counted for the launch
                 "l2_gather": {"algorithmic_bytes": gather_bytes,
                               "lts_bytes": prof["lts_bytes"] if prof else None,
                               "lts_over_algorithmic": prof["lts_bytes"] / gather_bytes

@@ -4,14 +4,15 @@
 // agreeing positions estimates J.  The candidate pairs of all rows are cut into
 // chunks of consecutive pairs that warps take in turn (rows range from a few
 // candidates to thousands, so a block per row would leave the grid waiting on
-// the longest); a warp reads both rows' K hashes as 16-byte vectors (512 bytes
-// per row at K = 128, the query's from L1/L2); equality bits are gathered with
-// shuffles, the count is a warp reduction, and the band-match bits and the
-// reranker's features (A7) come from the same bits.
+// the longest).  Rows of at most 128 hashes: a lane holds four of the query's hashes
+// and reads the candidates' as 16-byte vectors (512 bytes per row at K = 128), the count
+// is a warp reduction, and the band-match bits and the reranker's features (A7) come from
+// the same equality bits; longer rows read both sides and gather the bits in shared memory.
 //
-// A6 sorts each candidate row by a 64-bit key in shared memory (bitonic),
-// keeping the first m: key = (K - count) << 32 | id for the plain form,
-// or (~orderable(score)) << 32 | id for a learned score.
+// A6 orders each candidate row by a 64-bit key (ranks by a warp for short rows of a large
+// batch, else a block's bitonic sort in shared memory), keeping the first m:
+// key = (K - count) << 32 | id for the plain form, or (~orderable(score)) << 32 | id for a
+// learned score.
 #include <cuda_bf16.h>
 
 #include <algorithm>

@@ -464,7 +464,7 @@ int pmh_launch_agree_features(pmh_ctx ctx, const uint32_t* qh, const uint32_t* p
 // (J desc, id asc) (refine.cu); jv: Q * m doubles of scratch; tickets: the grids' three
 // counters; d_n (optional) caps Q on the device.  big (pmh_refine_queue_bytes(Q * m);
 // nullable) is the queue of the pairs with a ring above kRefineBigVerts vertices, which
-// then go to a block each; without it every pair takes the two-warp form.
+// then go to a cluster each; without it every pair takes the two-warp form.
 struct RefineQueries {
     const int2* xy;
     const int64_t* off;
