@@ -18,6 +18,7 @@
 // memory (sets above the bitmap's), or a warp's merge of the ascending lists.
 #include <algorithm>
 
+#include "directory.cuh"
 #include "pmh_internal.cuh"
 
 namespace {
@@ -71,37 +72,18 @@ __global__ void fill_entries_kernel(const uint32_t* __restrict__ hashes, int64_t
     }
 }
 
-// The directory covers the composites of valid entries, [0, cmax) with
-// cmax = bands << (32 - band_bits) (invalid entries, all ones, sort last and are
-// never looked up): dir[s] = first sorted entry whose composite >> sh is >= s,
-// for s in [0, ceil(cmax / 2^sh)].  Thread e writes the slots after its predecessor's,
-// up to its own (thread m: up to the last), so every slot is written once; the
-// keys are uniform, so gaps are a slot or two (a band without one valid entry
-// leaves one thread a gap of 2^(32 - band_bits - sh) slots).
+// The directory (directory.cuh): thread e writes entry e's slots.  The keys are uniform, so
+// gaps are a slot or two (a band without one valid entry leaves one thread a gap of
+// 2^(32 - band_bits - sh) slots).
 __global__ void dir_kernel(const uint32_t* __restrict__ comp, int64_t m, int sh, int64_t cmax,
                            int64_t* __restrict__ dir)
 {
-    const int64_t top = (cmax + (1ll << sh) - 1) >> sh;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e <= m;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t cs = e < m ? min((int64_t)comp[e], cmax) >> sh : top;
-        const int64_t ps = e == 0 ? 0 : (min((int64_t)comp[e - 1], cmax) >> sh) + 1;
-        for (int64_t s = ps; s <= cs; ++s) dir[s] = e;
+        int64_t from, to;
+        pmh_dir_slots(comp, m, e, sh, cmax, &from, &to);
+        for (int64_t s = from; s <= to; ++s) dir[s] = e;
     }
-}
-
-// first sorted entry whose composite is >= c
-__device__ __forceinline__ int64_t comp_lower_bound(const uint32_t* __restrict__ comp,
-                                                    const int64_t* __restrict__ dir, int sh, uint32_t c)
-{
-    const uint32_t s = c >> sh;
-    int64_t lo = dir[s], hi = dir[s + 1];
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (comp[mid] < c) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
 }
 
 constexpr int kMaxBandsPerLane = 4;  // bands <= 128
@@ -184,7 +166,7 @@ __global__ void query_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, in
         uint64_t key = band_key(qh, j, rows, T, lsh_seed);
         if (key == PMH_INVALID_KEY) continue;
         cur[t].comp = composite(key, j, band_bits);
-        cur[t].cur = comp_lower_bound(comp, dir, dsh, cur[t].comp);
+        cur[t].cur = pmh_comp_lower_bound(comp, dir, dsh, cur[t].comp);
         advance(cur[t], comp, ids, dbh, qh, m, K, bands, rows);
     }
     int64_t out = kWrite ? row_ptr[q] : 0;
@@ -253,7 +235,7 @@ __device__ int64_t merge_row(const uint32_t* __restrict__ qh, int K, int bands, 
         uint64_t key = band_key(qh, j, rows, T, lsh_seed);
         if (key == PMH_INVALID_KEY) continue;
         cur[t].comp = composite(key, j, band_bits);
-        cur[t].cur = comp_lower_bound(comp, dir, dsh, cur[t].comp);
+        cur[t].cur = pmh_comp_lower_bound(comp, dir, dsh, cur[t].comp);
         advance(cur[t], comp, ids, dbh, qh, m, K, bands, rows);
     }
     int64_t cnt = 0;
@@ -332,7 +314,7 @@ template <bool kBig>
 __device__ int join_walk(const uint32_t* __restrict__ qh, int K, int bands, int rows, uint32_t T,
                          uint64_t lsh_seed, int band_bits, const uint32_t* __restrict__ comp,
                          const int32_t* __restrict__ ids, const uint32_t* __restrict__ dbh,
-                         const int64_t* __restrict__ dir, int dsh, int64_t m, int32_t id_lo, int32_t id_hi,
+                         const int64_t* __restrict__ dir, int dsh, int32_t id_lo, int32_t id_hi,
                          int32_t* table, int* n_unique, JoinBands& jb)
 {
     using S = JoinShape<kBig>;
@@ -348,9 +330,8 @@ __device__ int join_walk(const uint32_t* __restrict__ qh, int K, int bands, int 
         int64_t lo = 0, n = 0;
         if (key != PMH_INVALID_KEY) {
             const uint32_t c = composite(key, j, band_bits);
-            lo = comp_lower_bound(comp, dir, dsh, c);
-            const int64_t hi = c == 0xFFFFFFFFu ? m : comp_lower_bound(comp, dir, dsh, c + 1);
-            n = hi - lo;
+            lo = pmh_comp_lower_bound(comp, dir, dsh, c);
+            n = pmh_comp_lower_bound(comp, dir, dsh, c + 1) - lo;
         }
         jb.lo[j] = lo;
         jb.off[j + 1] = n;
@@ -525,7 +506,7 @@ join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int bands, i
             for (int r = 0; r < passes; ++r) {
                 const int32_t lo = (int32_t)(n_db * r / passes), hi = (int32_t)(n_db * (r + 1) / passes);
                 const int nu = join_walk<kBig>(qh, K, bands, rows, T, lsh_seed, band_bits, comp, ids, dbh, dir,
-                                               dsh, m, lo, hi, table, &n_unique, jb);
+                                               dsh, lo, hi, table, &n_unique, jb);
                 if (nu > kJoinMaxUnique) {
                     over = true;
                     break;
@@ -671,8 +652,8 @@ warp_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int ban
             const uint64_t key = band_key(qh, j, rows, T, lsh_seed);
             if (key != PMH_INVALID_KEY) {
                 const uint32_t c = composite(key, j, band_bits);
-                lo = comp_lower_bound(comp, dir, dsh, c);
-                n = comp_lower_bound(comp, dir, dsh, c + 1) - lo;  // (c is never all ones)
+                lo = pmh_comp_lower_bound(comp, dir, dsh, c);
+                n = pmh_comp_lower_bound(comp, dir, dsh, c + 1) - lo;
             }
         }
         int x = (int)min(n, (int64_t)(kWarpList + 1));
@@ -971,7 +952,7 @@ __global__ void __launch_bounds__(kRangeWarps * 32)
 range_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int rows, uint32_t T,
                   uint64_t lsh_seed, int band_bits, const uint32_t* __restrict__ comp,
                   const int32_t* __restrict__ ids, const uint32_t* __restrict__ dbh,
-                  const int64_t* __restrict__ dir, int dsh, int64_t m, int segs, int32_t* __restrict__ seg,
+                  const int64_t* __restrict__ dir, int dsh, int segs, int32_t* __restrict__ seg,
                   int64_t* __restrict__ counts, const int64_t* __restrict__ row_ptr,
                   int32_t* __restrict__ cand, int64_t cap, const int64_t* __restrict__ d_n,
                   int* __restrict__ d_flags)
@@ -998,8 +979,8 @@ range_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int ro
         int64_t lo = 0, n = 0;
         if (key != PMH_INVALID_KEY) {
             const uint32_t c = composite(key, 0, band_bits);
-            lo = comp_lower_bound(comp, dir, dsh, c);
-            n = (c == 0xFFFFFFFFu ? m : comp_lower_bound(comp, dir, dsh, c + 1)) - lo;
+            lo = pmh_comp_lower_bound(comp, dir, dsh, c);
+            n = pmh_comp_lower_bound(comp, dir, dsh, c + 1) - lo;
         }
         int64_t out = 0;
         if (kWrite) {
@@ -1054,15 +1035,9 @@ extern "C" int pmh_band_keys(pmh_ctx ctx, const uint32_t* d_hashes, int64_t n,
     return PMH_OK;
 }
 
-// end of the composites of valid entries (the directory's range), and the directory's
-// length (slots + 1)
-static int64_t dir_cmax(pmh_index X)
-{
-    return (int64_t)X->params.bands << (32 - X->band_bits);
-}
 static size_t dir_len(pmh_index X)
 {
-    return (size_t)((dir_cmax(X) + (1ll << X->dir_shift) - 1) >> X->dir_shift) + 1;
+    return (size_t)pmh_dir_len(pmh_dir_cmax(X->params.bands, X->band_bits), X->dir_shift);
 }
 
 // hashes copied in, band keys, (band, key) entries radix-sorted with ids, full keys gathered
@@ -1086,17 +1061,10 @@ static int index_fill(pmh_ctx ctx, pmh_index X, const uint32_t* d_hashes, cudaSt
     PMH_LAUNCHED("fill_entries_kernel");
     PMH_TRY(pmh_radix_sort_u32(ctx, X->sorted_comp, X->sorted_id, entries, 32, s));
     const int dblocks = (int)std::min<int64_t>((entries + 256) / 256, (int64_t)ctx->sm_count * 32);
-    dir_kernel<<<dblocks, 256, 0, s>>>(X->sorted_comp, entries, X->dir_shift, dir_cmax(X), X->dir);
+    dir_kernel<<<dblocks, 256, 0, s>>>(X->sorted_comp, entries, X->dir_shift,
+                                     pmh_dir_cmax(params->bands, bb), X->dir);
     PMH_LAUNCHED("dir_kernel");
     return PMH_OK;
-}
-
-// directory shift: about eight sorted entries per slot over [0, cmax), at most 2^24 slots
-static int dir_shift_for(int64_t entries, int64_t cmax)
-{
-    int sh = 31;
-    while (sh > 0 && (cmax >> (sh - 1)) <= (int64_t)1 << 24 && (cmax >> (sh - 1)) * 8 <= entries) --sh;
-    return sh;
 }
 
 extern "C" int pmh_lsh_build(pmh_ctx ctx, const uint32_t* d_hashes, int64_t n,
@@ -1114,11 +1082,9 @@ extern "C" int pmh_lsh_build(pmh_ctx ctx, const uint32_t* d_hashes, int64_t n,
     X->device = ctx->device;
     X->n = n;
     X->params = *params;
-    int bb = 1;
-    while ((1u << bb) - 1 < params->bands) ++bb;  // band index < 2^bb - 1: comp never all ones
-    X->band_bits = bb;
+    X->band_bits = pmh_band_bits(params->bands);
     const int64_t entries = n * params->bands;
-    X->dir_shift = dir_shift_for(entries, dir_cmax(X));
+    X->dir_shift = pmh_dir_shift(entries, pmh_dir_cmax(params->bands, X->band_bits));
     const size_t nn = (size_t)std::max<int64_t>(n, 1), ne = (size_t)std::max<int64_t>(entries, 1);
     if (cudaMalloc(&X->hashes, sizeof(uint32_t) * nn * params->K) != cudaSuccess ||
         cudaMalloc(&X->sorted_comp, sizeof(uint32_t) * ne) != cudaSuccess ||
@@ -1212,7 +1178,7 @@ static int launch_range(pmh_index X, const uint32_t* qh, int64_t Q, const int64_
     auto fn = write ? range_join_kernel<true> : range_join_kernel<false>;
     fn<<<blocks, kRangeWarps * 32, 0, s>>>(qh, Q, (int)P.K, (int)P.rows, P.T, P.lsh_seed, X->band_bits,
                                            X->sorted_comp, X->sorted_id, X->hashes, X->dir, X->dir_shift,
-                                           X->n, segs, seg, counts, row_ptr, cand, cap, d_n, d_flags);
+                                           segs, seg, counts, row_ptr, cand, cap, d_n, d_flags);
     PMH_LAUNCHED(write ? "range_join_kernel<fill>" : "range_join_kernel<count>");
     return PMH_OK;
 }

@@ -296,10 +296,7 @@ struct pmh_index_s {
     uint32_t* hashes = nullptr;     // [n][K]
     uint32_t* sorted_comp = nullptr;  // [n * bands] composite (band, key) sort keys
     int32_t* sorted_id = nullptr;     // [n * bands]
-    // directory of the sorted composites: dir[s] = first entry whose composite >> dir_shift
-    // is >= s, for s in [0, ceil((bands << (32 - band_bits)) / 2^dir_shift)] (a lower bound
-    // of a valid composite reads one short range)
-    int64_t* dir = nullptr;
+    int64_t* dir = nullptr;  // directory of the sorted composites (directory.cuh)
     int dir_shift = 32;
 };
 
