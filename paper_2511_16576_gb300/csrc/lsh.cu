@@ -1211,7 +1211,10 @@ static int launch_bitmap(pmh_index X, const uint32_t* qh, int64_t Q, const int64
     const int64_t sms = X->ctx->sm_count, fit = (225 * 1024) / ((int64_t)smem + 2048);
     const int threads = fit < 4 || Q <= sms ? 1024 : fit < 8 || Q <= 2 * sms ? 512 : 256;
     auto fn = write ? bitmap_join_kernel<true> : bitmap_join_kernel<false>;
-    PMH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // (the largest bitmap's, not this one's: the attribute is the process's, and a host thread with a
+    // small index must not take it from another between its set and its launch)
+    PMH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(kBitmapMaxIdsShort / 8)));
     int per_sm = 1;
     PMH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem));
     const unsigned blocks = (unsigned)std::min<int64_t>(Q, (int64_t)X->ctx->sm_count * std::max(per_sm, 1));
