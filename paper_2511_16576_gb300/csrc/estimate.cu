@@ -408,6 +408,10 @@ topm_short_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict
 // form, take the merge form: the running top-m kept in s[0..m), each new chunk
 // of the row appended and sorted with it.
 constexpr int kSelMax = 2048;
+constexpr int kTopMaxM = 1024;   // of the callers
+constexpr int kTopCap = 4096;    // keys of the longest list: a power of two
+static_assert(kTopCap >= kTopMaxM + kTopChunk && kTopCap >= kSelMax, "the longest list fits");
+constexpr int kTopSmemMax = (int)(sizeof(uint64_t) * kTopCap + sizeof(int) * (kMaxK + 1));
 
 __global__ void __launch_bounds__(kTopThreads)
 topm_kernel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ cand,
@@ -631,8 +635,9 @@ int pmh_launch_topm(const int64_t* row_ptr, const int32_t* cand, const uint16_t*
     while (cap < m + kTopChunk || cap < kSelMax) cap <<= 1;
     const int kb = (K > 0 && K <= kMaxK) ? K : kMaxK;  // counts are <= K
     const size_t smem = sizeof(uint64_t) * cap + sizeof(int) * (size_t)(kb + 1);
-    PMH_CUDA_TRY(cudaFuncSetAttribute(topm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+    // (the largest list's and histogram's: the attribute is shared by all host threads, and a call
+    // that set its own could lower it between another's set and its launch)
+    PMH_CUDA_TRY(cudaFuncSetAttribute(topm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopSmemMax));
     // large batches: the short rows a warp each, then a block per longer row (a batch of a few
     // hundred rows fills the device either way and saves the launch)
     const bool split = Q >= 512;

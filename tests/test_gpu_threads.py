@@ -45,3 +45,42 @@ def test_bitmap_joins_of_a_large_and_small_sets():
     for t in threads:
         t.join()
     assert not bad, (len(bad), bad[0])
+
+
+def test_topm_beside_the_capture_of_graphs():
+    """Top-m of counts up to 4,096 (49 KB of shared memory) beside a thread that captures query graphs at
+    K = 8 (33 KB)."""
+    from paper_2511_16576_gb300 import binding as B
+    lib = B.load()
+    bad = []
+    n = 300
+    rows = torch.arange(0, 601, n, dtype=torch.int64, device=DEV)
+    cand = torch.arange(600, dtype=torch.int32, device=DEV)
+    count = torch.arange(600, dtype=torch.int16, device=DEV)
+    ids, nn = torch.empty((2, 64), dtype=torch.int32, device=DEV), torch.empty(2, dtype=torch.int32, device=DEV)
+    P = B.make_params(8, 2)
+    ctx1 = B.Context(0)
+    index = B.lsh_build(ctx1, torch.zeros((64, 8), dtype=torch.int32, device=DEV), P)
+    ctx0, stream = B.Context(0), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    done = threading.Event()
+
+    def capture():
+        while not done.is_set():
+            B.QueryGraph(ctx1, index, 4, 64, 256, 8).close()
+
+    def topm():
+        for _ in range(40_000):
+            rc = lib.pmh_topm(ctx0.handle, rows.data_ptr(), cand.data_ptr(), count.data_ptr(), None, 2, 64,
+                              ids.data_ptr(), nn.data_ptr(), stream.cuda_stream)
+            if rc != 0:
+                bad.append((rc, lib.pmh_last_error()))
+        done.set()
+    threads = [threading.Thread(target=f) for f in (capture, topm)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not bad, (len(bad), bad[0])
+    assert torch.equal(ids[0].cpu(), torch.arange(299, 235, -1, dtype=torch.int32))
