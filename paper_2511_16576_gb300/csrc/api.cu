@@ -11,6 +11,7 @@
 #include <climits>
 
 #include "pmh_internal.cuh"
+#include "upload.cuh"
 
 std::atomic<int64_t> g_pmh_launches{0};
 
@@ -264,6 +265,8 @@ __global__ void poly_feat_kernel(const int64_t* __restrict__ area2, const int64_
     }
 }
 
+static_assert(kPointerOnDevice == cudaMemoryTypeDevice, "upload.cuh's memory type");
+
 // copy the arrays in, validate them and compute every per-polygon product (bbox,
 // 2 x area, reranker inputs, slab lists, class order) into P's buffers
 static int upload_fill(pmh_polys P, const int32_t* xy, const int64_t* offsets, bool host,
@@ -272,9 +275,15 @@ static int upload_fill(pmh_polys P, const int32_t* xy, const int64_t* offsets, b
     pmh_ctx ctx = P->ctx;
     const int64_t n_polys = P->n, n_vertices = P->nv;
     cudaMemcpyKind kind = host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
-    // vertices that are on the device are copied by the kernel that reads them (an int2 load
-    // wants 8-byte alignment; others are copied first)
-    const bool fused = !host && n_polys > 0 && reinterpret_cast<uintptr_t>(xy) % sizeof(int2) == 0;
+    // vertices that lie on this device are copied by the kernel that reads them (upload.cuh)
+    bool fused = false;
+    if (!host && n_polys > 0) {
+        cudaPointerAttributes at{};
+        if (cudaPointerGetAttributes(&at, xy) == cudaSuccess)
+            fused = pmh_reads_in_place((int)at.type, at.device, ctx->device, reinterpret_cast<uintptr_t>(xy));
+        else
+            cudaGetLastError();
+    }
     cudaError_t e = cudaSuccess;
     if (n_vertices > 0 && !fused) e = cudaMemcpyAsync(P->xy, xy, sizeof(int2) * n_vertices, kind, s);
     if (e == cudaSuccess)
