@@ -70,7 +70,7 @@ struct pmh_qgraph_s {
     int64_t* d_n = nullptr;
     unsigned long long* ticket = nullptr;  // [8]: refinement grids at 1, signing at 4
     int64_t* scan_sums = nullptr;
-    const uint32_t* sidx_first = nullptr;  // the stream index the graph captured (nullptr: none)
+    uint64_t sidx_build = 0;           // the build of the stream index the graph captured (0: none)
     int64_t kernels = 0;               // kernel launches per replay
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -153,7 +153,7 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
             delete g;
             return rc;
         }
-        g->sidx_first = sidx.lv[0].first;
+        g->sidx_build = ctx->sindex.build;
     }
     bool ok = cudaMalloc(&g->xy, sizeof(int2) * max_vertices) == cudaSuccess &&
               cudaMalloc(&g->off, sizeof(int64_t) * (Q + 1)) == cudaSuccess &&
@@ -296,7 +296,7 @@ extern "C" int pmh_qgraph_run(pmh_qgraph g, const int32_t* xy, const int64_t* of
 {
     if (!g) return pmh_set_error(PMH_ERR_ARG, "null graph");
     PMH_TRY(pmh_check_device(g->ctx));
-    if (g->sidx_first && g->ctx->sindex.first[0] != g->sidx_first)
+    if (g->sidx_build && g->ctx->sindex.build != g->sidx_build)
         return pmh_set_error(PMH_ERR_STATE, "the context's stream index was rebuilt for other "
                                             "parameters since the graph was captured: recreate the graph");
     if (n_queries < 0 || n_queries > g->maxQ || n_vertices < 0 || n_vertices > g->maxV ||

@@ -125,6 +125,7 @@ __host__ __device__ __forceinline__ int pmh_index_level(int4 bb, int K)
 }
 
 struct StreamIndex {
+    uint64_t build = 0;  // the context's count of builds (0: none); buffers' addresses come back
     uint64_t seed = 0;
     int K = 0;
     // rows of index_pitch(K) hashes per cell:
@@ -172,6 +173,7 @@ struct pmh_ctx_s {
     int64_t* h_pinned = nullptr;          // small pinned host buffer [64]
     int sign_variant = -1;                // autotuned signing kernel (-1 = default)
     StreamIndex sindex;                   // cached stream index (PMH_FLAG_STREAM_INDEX)
+    uint64_t sindex_builds = 0;
     int sign_timing = 0;                  // record per-kernel events in pmh_minhash_sign
     int sign_count = 1;                   // signing launches record their work counts
     std::vector<cudaEvent_t> sign_ev;     // three per recorded call

@@ -204,6 +204,7 @@ int pmh_stream_index_get(pmh_ctx ctx, const pmh_params* P, cudaStream_t s, Strea
     }
     fresh.seed = P->seed;
     fresh.K = (int)P->K;
+    fresh.build = ++ctx->sindex_builds;
     si = fresh;
     *out = view_of(si);
     return PMH_OK;

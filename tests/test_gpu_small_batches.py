@@ -34,3 +34,29 @@ def test_hashes(orc, K, maxq):
     finally:
         g.close()
         ctx.close()
+
+
+def test_graph_refuses_a_rebuilt_stream_index():
+    """The index rebuilt for another seed and the same K (buffers of the same sizes, whose addresses may
+    come back): the graph captured on the first one is refused, also after a rebuild for its own seed."""
+    from paper_2511_16576_gb300 import binding as B
+    db = synth.star_polygons(300, 3, f_range=(1e-3, 1e-2))
+    up = lambda ps: (torch.from_numpy(ps.xy).to(DEV), torch.from_numpy(ps.offsets).to(DEV))
+    ctx = B.Context(0)
+    P = [B.make_params(32, 8, 1 << 22, seed, 5, B.FLAG_STREAM_INDEX) for seed in (11, 12)]
+    index = B.lsh_build(ctx, B.minhash_sign(ctx, B.poly_upload(ctx, *up(db)), P[0]), P[0])
+    xy, off = up(db.subset(np.arange(4)))
+    g = B.QueryGraph(ctx, index, 4, xy.shape[0], 4096, 4)
+    g.run(xy, off)
+    first = g.hashes[:4].clone()
+    for p in (P[1], P[0]):
+        B.stream_index_build(ctx, p)
+        with pytest.raises(B.PmhError) as e:
+            g.run(xy, off)
+        assert e.value.code == -6  # PMH_ERR_STATE
+    g.close()
+    g = B.QueryGraph(ctx, index, 4, xy.shape[0], 4096, 4)
+    g.run(xy, off)
+    assert torch.equal(g.hashes[:4], first)
+    g.close()
+    ctx.close()
