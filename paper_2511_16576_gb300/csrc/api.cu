@@ -414,6 +414,7 @@ extern "C" int pmh_poly_reload(pmh_polys polys, const int32_t* xy, const int64_t
         if (polys->d_slabs) cudaMemsetAsync(polys->d_slabs, 0, sizeof(SlabPtrs), s);
         cudaDeviceSynchronize();
         free_derived(polys, true);
+        polys->max_n = INT32_MAX;  // (unknown)
     }
     return rc;
 }

@@ -72,6 +72,10 @@ struct pmh_qgraph_s {
     int64_t* scan_sums = nullptr;
     uint64_t sidx_build = 0;           // the build of the stream index the graph captured (0: none)
     int64_t kernels = 0;               // kernel launches per replay
+    // the launches of large rings, left out of a replay without one (an empty launch is 2 us of a
+    // query's 126)
+    std::vector<cudaGraphNode_t> big_nodes;
+    bool big_on = true;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -100,6 +104,24 @@ extern "C" int pmh_qgraph_destroy(pmh_qgraph g)
     for (void* b : bufs)
         if (b) cudaFree(b);
     delete g;
+    return PMH_OK;
+}
+
+// the nodes of `graph` that launch `func`
+static int find_kernel_nodes(cudaGraph_t graph, const void* func, std::vector<cudaGraphNode_t>* out)
+{
+    size_t n = 0;
+    PMH_CUDA_TRY(cudaGraphGetNodes(graph, nullptr, &n));
+    std::vector<cudaGraphNode_t> nodes(n);
+    PMH_CUDA_TRY(cudaGraphGetNodes(graph, nodes.data(), &n));
+    for (cudaGraphNode_t node : nodes) {
+        cudaGraphNodeType type;
+        PMH_CUDA_TRY(cudaGraphNodeGetType(node, &type));
+        if (type != cudaGraphNodeTypeKernel) continue;
+        cudaKernelNodeParams params{};
+        PMH_CUDA_TRY(cudaGraphKernelNodeGetParams(node, &params));
+        if (params.func == func) out->push_back(node);
+    }
     return PMH_OK;
 }
 
@@ -189,10 +211,8 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
               cudaMalloc(&g->ticket, 8 * sizeof(unsigned long long)) == cudaSuccess &&
               cudaMalloc(&g->walks, sizeof(WalkItem) * kWalkItems) == cudaSuccess &&
               cudaMalloc(&g->d_slabs, sizeof(SlabPtrs)) == cudaSuccess &&
-              // (a batch of a few small queries against small polygons has no large ring; a set
-              // reloaded with larger ones is still refined, by the two-warp form)
-              (k == 0 || std::max<int64_t>(max_vertices, db->max_n) <= kRefineBigVerts ||
-               cudaMalloc(&g->ref_queue, pmh_refine_queue_bytes(Q * m)) == cudaSuccess) &&
+              // (also without a large ring: the set may be reloaded with some)
+              (k == 0 || cudaMalloc(&g->ref_queue, pmh_refine_queue_bytes(Q * m)) == cudaSuccess) &&
               cudaMalloc(&g->scan_sums, sizeof(int64_t) * pmh_scan_sums_size(Q)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -280,6 +300,7 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
         e = cudaGraphInstantiate(&g->exec, graph, 0);
         if (e != cudaSuccess) rc = pmh_set_error(PMH_ERR_CUDA, "instantiate: %s", cudaGetErrorString(e));
     }
+    if (rc == PMH_OK && k > 0) rc = find_kernel_nodes(graph, pmh_refine_big_func(), &g->big_nodes);
     cudaStreamDestroy(cs);
     if (rc != PMH_OK) {
         cudaGetLastError();
@@ -311,8 +332,15 @@ extern "C" int pmh_qgraph_run(pmh_qgraph g, const int32_t* xy, const int64_t* of
         PMH_CUDA_TRY(cudaMemcpyAsync(g->off, offsets, sizeof(int64_t) * (n_queries + 1), kind, s));
     set_batch_kernel<<<1, 1, 0, s>>>(g->d_n, n_queries);
     PMH_LAUNCHED("set_batch_kernel");
+    // (a ring of the batch has at most its vertices; the set may have been reloaded since)
+    const bool big = !g->big_nodes.empty() && std::max<int64_t>(n_vertices, g->db->max_n) > kRefineBigVerts;
+    if (big != g->big_on) {
+        for (cudaGraphNode_t node : g->big_nodes) PMH_CUDA_TRY(cudaGraphNodeSetEnabled(g->exec, node, big));
+        g->big_on = big;
+    }
     PMH_CUDA_TRY(cudaGraphLaunch(g->exec, s));
-    g_pmh_launches.fetch_add(g->kernels);  // the kernels the graph holds
+    // the kernels the graph launches
+    g_pmh_launches.fetch_add(g->kernels - (big ? 0 : (int64_t)g->big_nodes.size()));
     return PMH_OK;
 }
 

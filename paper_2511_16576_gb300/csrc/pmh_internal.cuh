@@ -473,6 +473,7 @@ struct RefineQueries {
 };
 constexpr int kRefineBigVerts = 1024;
 size_t pmh_refine_queue_bytes(int64_t n_pairs);
+const void* pmh_refine_big_func();  // the kernel that takes the queue (a no-op when it is empty)
 int pmh_launch_refine_topk(pmh_ctx ctx, const RefineQueries& qs, pmh_polys db, const int32_t* ids,
                            const int32_t* nlist, int64_t Q, const int64_t* d_n, int32_t m, int32_t k,
                            double* jv, unsigned long long* tickets, int32_t* big, int32_t* top_ids,

@@ -1074,6 +1074,8 @@ size_t pmh_refine_queue_bytes(int64_t n_pairs)
     return sizeof(int32_t) * (size_t)std::min(std::max<int64_t>(n_pairs, 1), kRefineSlice);
 }
 
+const void* pmh_refine_big_func() { return reinterpret_cast<const void*>(refine_big_kernel); }
+
 // persistent grids (SM count x resident blocks) over the pairs, kRefineSlice at a time; with
 // a queue, the pairs of large rings are left to refine_big_kernel
 static int launch_refine(pmh_ctx ctx, const RefineQueries& qs, pmh_polys db, const int32_t* ids,

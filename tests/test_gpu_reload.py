@@ -92,3 +92,57 @@ def test_class_order_of_many(B, orc):
         got = B.minhash_sign(ctx, polys, P).cpu().numpy().view(np.uint32)
         assert np.array_equal(got, orc.sign(db.xy, db.offsets, SEED, K, T, nthreads=16))
     ctx.close()
+
+
+def _star(n, cx, cy, r, seed):
+    rng = np.random.default_rng(seed)
+    a = (np.arange(n) + rng.uniform(0.1, 0.9, n)) * (2 * np.pi / n)
+    rad = r * rng.uniform(0.8, 1.2, n)
+    return np.rint(np.stack([cx + rad * np.cos(a), cy + rad * np.sin(a)], 1)).astype(np.int32)
+
+
+def test_graph_on_a_set_reloaded_with_large_rings(B):
+    """A graph captured while every ring is small refines a reloaded set's large rings by the launches that
+    a graph captured on them takes, to the plain call's values; and leaves them out again."""
+    small = [600] * 8
+    large = [3000] + [257] * 6 + [258]
+    assert sum(small) == sum(large)
+    rings = lambda sizes: np.concatenate([_star(n, 20000 + 1500 * i, 30000 - 900 * i, 9000, i)
+                                          for i, n in enumerate(sizes)])
+    off = lambda sizes: np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    ctx = B.Context(0)
+    P = B.make_params(32, 16, 1 << 16, SEED)
+    up = lambda xy, o: (torch.from_numpy(xy).to(DEV), torch.from_numpy(o).to(DEV))
+    sets = [up(rings(s), off(s)) for s in (small, large)]
+    polys = B.poly_upload(ctx, *sets[0])
+    index = B.lsh_build(ctx, B.minhash_sign(ctx, polys, P), P)
+    q = up(rings(small)[:600], off(small[:1]))
+    qp = B.poly_upload(ctx, *q)
+
+    def graph():
+        return B.QueryGraph(ctx, index, 1, 900, 4096, 8, db=polys, k=8)
+
+    def replay(g):
+        before = B.launch_count()
+        g.run(*q)
+        launches = B.launch_count() - before
+        assert g.status()[0] == 0
+        n = int(g.top_n[0])
+        assert n > 0
+        ids = g.ref_ids[0, :n]
+        j = B.pair_jaccard(ctx, qp, polys, torch.zeros(n, dtype=torch.int32, device=DEV), ids.contiguous())
+        assert torch.equal(g.ref_j[0, :n], j)
+        return launches
+
+    g = graph()
+    launches = []
+    for s in (0, 1, 0, 1):
+        if launches:
+            B.poly_reload(polys, *sets[s])
+        fresh = graph()
+        launches.append((replay(g), replay(fresh)))
+        fresh.close()
+    assert all(a == b for a, b in launches), launches
+    assert launches[0][0] == launches[2][0] == launches[1][0] - 1 == launches[3][0] - 1
+    g.close()
+    ctx.close()
