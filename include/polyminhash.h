@@ -234,9 +234,12 @@ int pmh_index_destroy(pmh_index index);
  * total, d_cand is left unwritten, d_row_ptr is still written, and the call
  * returns PMH_ERR_CAPACITY: call again with a larger buffer.  With two bands or
  * more and a capacity, the counting pass keeps its sorted rows in context scratch (8
- * bytes per query and up to 4,096 ids per query, at most 64M ids) and the filling pass
- * copies them; rows past that pool (all of them without a capacity or without room
- * for it) are joined again.  Errors also: PMH_ERR_NOMEM (scratch). */
+ * bytes per query, and a pool of up to 4,096 ids per query, at most 64M ids and at most
+ * the capacity; a quarter more is taken, and kept for the context's life) and the
+ * filling pass copies them; rows past that pool (all of them without a capacity or
+ * without room for it) are joined again.  Sets above 409,600 polygons (2^20 with tuples
+ * of one or two hashes) under fewer than 16 bands keep no rows.  Errors also:
+ * PMH_ERR_NOMEM (scratch). */
 int pmh_lsh_query(pmh_ctx ctx, pmh_index index, const uint32_t* d_qhashes, int64_t Q,
                   int64_t* d_row_ptr, int32_t* d_cand, int64_t cand_capacity, int64_t* h_total,
                   void* stream);

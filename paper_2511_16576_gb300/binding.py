@@ -398,7 +398,11 @@ def lsh_rebuild(ctx: Context, index: Index, hashes: torch.Tensor, stream=None):
 
 def lsh_query(ctx: Context, index: Index, qhashes: torch.Tensor, capacity: int | None = None,
               stream=None):
-    """A4: CSR (row_ptr int64 [Q+1], cand int32 [total]); sizes the buffer itself."""
+    """A4: CSR (row_ptr int64 [Q+1], cand int32 [total]); sizes the buffer itself.
+
+    Without a capacity the call first takes room for 1,024 ids per query (8 to 128 MB, given back
+    when the result is short), and the context keeps a staging pool of as many ids, and a
+    quarter more, for its life."""
     Q = qhashes.shape[0]
     dev = qhashes.device
     row_ptr = torch.empty(Q + 1, dtype=torch.int64, device=dev)

@@ -177,6 +177,7 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
         }
         g->sidx_build = ctx->sindex.build;
     }
+    const size_t stage_bytes = pmh_join_stage_bytes(index, Q, g->cap);
     bool ok = cudaMalloc(&g->xy, sizeof(int2) * max_vertices) == cudaSuccess &&
               cudaMalloc(&g->off, sizeof(int64_t) * (Q + 1)) == cudaSuccess &&
               cudaMalloc(&g->bbox, sizeof(int4) * Q) == cudaSuccess &&
@@ -188,7 +189,7 @@ extern "C" int pmh_qgraph_create(pmh_ctx ctx, pmh_index index, const pmh_qgraph_
               cudaMalloc(&g->slab_ptr, sizeof(int32_t) * g->cap_ptr) == cudaSuccess &&
               cudaMalloc(&g->slab_edges, sizeof(int32_t) * g->cap_edges) == cudaSuccess &&
               cudaMalloc(&g->counts, sizeof(int64_t) * Q) == cudaSuccess &&
-              cudaMalloc(&g->join_stage, pmh_join_stage_bytes(index, Q, g->cap)) == cudaSuccess &&
+              (stage_bytes == 0 || cudaMalloc(&g->join_stage, stage_bytes) == cudaSuccess) &&
               cudaMalloc(&g->row_ptr, sizeof(int64_t) * (Q + 1)) == cudaSuccess &&
               cudaMalloc(&g->cand, sizeof(int32_t) * cand_capacity) == cudaSuccess &&
               cudaMalloc(&g->count16, sizeof(uint16_t) * cand_capacity) == cudaSuccess &&

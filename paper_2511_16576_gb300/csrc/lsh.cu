@@ -1160,9 +1160,26 @@ static int range_segs(pmh_index X, int64_t Q)
     return (int)std::min<int64_t>(std::max<int64_t>(want, 1), 512);
 }
 
+// The join of an index (the warp join may come before the bitmap or the set):
+//  * one hashmap: the bucket's range, no merge;
+//  * bitmap: sets that fit it (kBitmapMaxIds, kBitmapMaxIdsShort);
+//  * merge: a larger set under few bands: rows are mostly empty or short, and the warp merge's one
+//    launch a pass beats the sets' two (8 x 16 bands of 520,000: 73 against 110 us);
+//  * set: the others
+enum class JoinForm { kRange, kBitmap, kMerge, kSet };
+static JoinForm join_form(pmh_index X)
+{
+    const pmh_params& P = X->params;
+    if (P.bands == 1) return JoinForm::kRange;
+    if (X->n <= (P.rows <= 2 ? kBitmapMaxIdsShort : kBitmapMaxIds)) return JoinForm::kBitmap;
+    return P.bands < 16 ? JoinForm::kMerge : JoinForm::kSet;
+}
+
 size_t pmh_join_stage_bytes(pmh_index X, int64_t Q, int64_t pool_ints)
 {
-    if (X->params.bands == 1) return sizeof(int32_t) * (size_t)(Q * range_segs(X, Q));
+    const JoinForm form = join_form(X);
+    if (form == JoinForm::kMerge) return 0;  // stages nothing
+    if (form == JoinForm::kRange) return sizeof(int32_t) * (size_t)(Q * range_segs(X, Q));
     return 16 + sizeof(int64_t) * (size_t)Q + sizeof(int32_t) * (size_t)pool_ints;
 }
 
@@ -1231,15 +1248,13 @@ int pmh_launch_query(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* 
 {
     if (Q <= 0) return PMH_OK;
     const pmh_params& P = X->params;
-    if (P.bands == 1) {  // one hashmap: the bucket's range, no merge
+    const JoinForm form = join_form(X);
+    if (form == JoinForm::kRange) {
         int32_t* seg = static_cast<int32_t*>(stage);
         if (!write) PMH_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(int64_t) * (size_t)Q, s));
         return launch_range(X, qh, Q, d_n, seg, counts, row_ptr, cand, cap, d_flags, write, s);
     }
-    const bool bitmap = X->n <= (P.rows <= 2 ? kBitmapMaxIdsShort : kBitmapMaxIds);
-    if (!bitmap && P.bands < 16) {
-        // a large set under few bands: rows are mostly empty or short, and the warp merge's one
-        // launch a pass beats the sets' two (8 x 16 bands of 520,000: 73 against 110 us)
+    if (form == JoinForm::kMerge) {
         const int wpb = 8;
         auto fn = write ? query_kernel<true> : query_kernel<false>;
         fn<<<(unsigned)((Q + wpb - 1) / wpb), wpb * 32, 0, s>>>(
@@ -1274,7 +1289,7 @@ int pmh_launch_query(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* 
     }
     // (without a pool and without the warp join's marks every row is the block join's)
     const JoinStage sb = write && !staged && !warp ? JoinStage{} : st;
-    if (bitmap) {
+    if (form == JoinForm::kBitmap) {
         // (a pool of the whole capacity holds every row of a total that may be written)
         if (write && staged && pool_ints >= cap) return PMH_OK;
         return launch_bitmap(X, qh, Q, d_n, counts, row_ptr, cand, cap, sb, warp, d_flags, write, s);
@@ -1299,14 +1314,15 @@ extern "C" int pmh_lsh_query(pmh_ctx ctx, pmh_index X, const uint32_t* d_qhashes
     int64_t* counts = nullptr;
     PMH_TRY(pmh_scratch(ctx, SCR_QUERY, sizeof(int64_t) * (size_t)Q, (void**)&counts));
     // the count pass stages its sorted rows in a pool of up to 4,096 ids per query
-    // (at most 64M ids); rows past the pool are joined again by the fill pass.  A call
-    // that cannot fill (no capacity) stages nothing
+    // (at most 64M ids, and no more than can be filled); rows past the pool are joined again
+    // by the fill pass.  A call that cannot fill (no capacity) stages nothing
     void* stage = nullptr;
     int64_t pool_ints = 0;
-    if (X->params.bands == 1) {
+    const JoinForm form = join_form(X);
+    if (form == JoinForm::kRange) {
         PMH_TRY(pmh_scratch(ctx, SCR_JOIN, pmh_join_stage_bytes(X, Q, 0), &stage));
-    } else if (cand_capacity > 0) {
-        pool_ints = std::min<int64_t>(Q * 4096, 64ll << 20);
+    } else if (form != JoinForm::kMerge && cand_capacity > 0) {
+        pool_ints = std::min<int64_t>(std::min<int64_t>(Q * 4096, 64ll << 20), cand_capacity);
         // (without room for a pool the fill pass joins every row again)
         if (pmh_scratch(ctx, SCR_JOIN, pmh_join_stage_bytes(X, Q, pool_ints), &stage) != PMH_OK) {
             stage = nullptr;
@@ -1340,11 +1356,13 @@ extern "C" int pmh_lsh_query_fill(pmh_ctx ctx, pmh_index X, const uint32_t* d_qh
     if (Q == 0) return PMH_OK;
     cudaStream_t s = (cudaStream_t)stream;
     void* stage = nullptr;
-    if (X->params.bands == 1) {  // the segments' counts, taken again
+    const JoinForm form = join_form(X);
+    if (form == JoinForm::kRange) {  // the segments' counts, taken again
         PMH_TRY(pmh_scratch(ctx, SCR_JOIN, pmh_join_stage_bytes(X, Q, 0), &stage));
         PMH_TRY(launch_range(X, d_qhashes, Q, nullptr, static_cast<int32_t*>(stage), nullptr, nullptr, nullptr,
                              0, nullptr, false, s));
-    } else if (pmh_scratch(ctx, SCR_JOIN, pmh_join_stage_bytes(X, Q, 0), &stage) != PMH_OK) {
+    } else if (form != JoinForm::kMerge &&
+               pmh_scratch(ctx, SCR_JOIN, pmh_join_stage_bytes(X, Q, 0), &stage) != PMH_OK) {
         stage = nullptr;  // no marks for the warp join: the block joins take every row
     }
     return pmh_launch_query(X, d_qhashes, Q, nullptr, nullptr, d_row_ptr, d_cand, cand_capacity,

@@ -381,7 +381,8 @@ int pmh_launch_sign_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* o
 // the same buffer for both passes, 16-byte aligned) lets the count pass keep the rows
 // it sorted, up to pool_ints ids in all, so that the fill pass copies them; the fill
 // pass of a call whose count pass had no stage gets none either.  With one band the
-// stage holds the count pass's segment counts instead and both passes need it
+// stage holds the count pass's segment counts instead and both passes need it; a join
+// that stages nothing asks for 0 bytes and takes nullptr
 size_t pmh_join_stage_bytes(pmh_index X, int64_t Q, int64_t pool_ints);
 int pmh_launch_query(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* d_n,
                      int64_t* counts, const int64_t* row_ptr, int32_t* cand, int64_t cap,

@@ -184,3 +184,40 @@ def test_warp_join_and_what_it_leaves(B, ctx, orc, n, values):
                                          cand.data_ptr(), cand.numel(), None))
     assert np.array_equal(cand.cpu().numpy(), full[1])
     index.close()
+
+
+def taken(f):
+    """Device bytes that a call took and kept."""
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    f()
+    torch.cuda.synchronize()
+    return free - torch.cuda.mem_get_info()[0]
+
+
+def test_staging_memory(B, orc):
+    """The staging pool holds no more than the capacity, and a join that stages nothing takes none, in a
+    plain call and in a captured graph."""
+    rng = np.random.default_rng(5)
+    Q, slack = 16_384, 8 << 20
+    for n, K, bands, pool in ((5000, 64, 8, 1 << 20), (409_601, 64, 8, 0)):
+        ph, qh = hashes(rng, n, K, 500), hashes(rng, Q, K, 500)
+        qh[:50] = ph[:50]
+        c = B.Context(0)
+        index = B.lsh_build(c, on_device(ph), B.make_params(K, bands))
+        q = on_device(qh)
+        row_ptr = torch.empty(Q + 1, dtype=torch.int64, device=DEV)
+        cand = torch.empty(1 << 20, dtype=torch.int32, device=DEV)
+        B.lsh_query(c, index, q[:8], capacity=8)  # (kernels loaded)
+        out = []
+        assert taken(lambda: out.append(B.lsh_query(c, index, q, capacity=1 << 20))) <= 5 * pool + slack
+        rp_ref, cand_ref = orc.candidates(np.ascontiguousarray(qh[:100]), ph, bands, K // bands, T)
+        assert np.array_equal(out[0][0].cpu().numpy()[:101], rp_ref)
+        assert np.array_equal(out[0][1].cpu().numpy()[:rp_ref[-1]], cand_ref)
+        if pool == 0:  # two result arrays of 6 bytes a candidate, no third of 4
+            cap = 64 << 20
+            g = []
+            assert taken(lambda: g.append(B.QueryGraph(c, index, 64, 4096, cap, 8))) <= 6 * cap + 8 * slack
+            g[0].close()
+        index.close()
+        c.close()
