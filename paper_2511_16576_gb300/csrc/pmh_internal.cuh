@@ -155,8 +155,9 @@ struct WalkItem {
     uint32_t next;   // segments handed out
 };
 constexpr int kWalkItems = 32768;  // (beyond them a hash is marked in the output and found there)
-// device counters of a signing call: [0] work-queue ticket, [1] queued walks, [2] walk ticket
-constexpr int kSignTickets = 3;
+// device counters of a signing call: [0] work-queue ticket, [1] queued walks, [2] walk ticket,
+// [3] ticket of the marked hashes
+constexpr int kSignTickets = 4;
 struct WalkQueue {
     WalkItem* items;
     unsigned long long* tickets;  // [kSignTickets]

@@ -42,7 +42,7 @@ namespace {
 constexpr int kWarps = 8;        // warps per block
 constexpr int kU = 4;            // points per lane per round
 constexpr int kWorkSlot = 8;     // context ticket slots 8..13: work counters of the walk kernel
-constexpr int kSignTicketSlot = 44;  // slots 44..46: counters of a call through the stream index
+constexpr int kSignTicketSlot = 44;  // slots 44..47: counters of a call through the stream index
 constexpr int kIdxWorkSlot = 16; // slots 16..21: work counters of the unified kernel
 
 __device__ __forceinline__ uint32_t sign_one(const int2* __restrict__ v, int n, int x0, int y0,

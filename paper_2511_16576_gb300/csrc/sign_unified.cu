@@ -183,8 +183,8 @@ __device__ __forceinline__ int single_slab(UniWarp& m, int n, int lane)
 // cell index -- computed in single precision, off by less than one unit --
 // never moves it across an unmarked cell, and the classification is exact.
 // Without a mask (use_mask false) every cell is a boundary cell.
-template <class Src, class W>
-__device__ __forceinline__ void build_mask(UniWarp& m, const Src& src, int n, int4 bb, const MaskFrame& f,
+template <class M, class Src, class W>
+__device__ __forceinline__ void build_mask(M& m /* its bnd and inb */, const Src& src, int n, int4 bb, const MaskFrame& f,
                                            bool use_mask, int lane, W& work)
 {
     const int cwl = f.cwl, chl = f.chl;
@@ -682,44 +682,154 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
 // a lattice point) spread over the device -- walked by the warp that signed the polygon
 // they were the tail of the launch: 8,000 coastlines, K = 256, took 4.8 ms and take 0.97,
 // 0.10 of it here.  The smallest inside index of all segments is the hash; a segment past the best
-// one so far ends the item.  Box points are rare (a few per walk), so they are tested
-// over the polygon's slab or all its edges from global memory.
+// one so far ends the item.  Box points are tested over the polygon's slab or all its
+// edges from global memory: most polygons meet a few per walk.  A thin one whose box is a
+// thousand times its area meets as many: from kWalkMaskRatio on they go through the coverage
+// mask first, and what is left is gathered and tested a lane each where that is cheaper than
+// a warp each.  Bound by the generator's integer chain, and by those tests for thin polygons.
 constexpr uint32_t kWalkSegment = 4096;
+constexpr int kWalkWarps = 8;
+constexpr int kWalkBuf = 32 * (kIdxU + 1);  // box points: fewer than 32 kept, and a round's
+constexpr float kWalkMaskRatio = 32.0f;     // (a mask costs about as much as a segment's points)
+struct WalkWarp {
+    uint2 buf[kWalkBuf];  // (stream index << 1 | inside by the mask, x | y << 16), in order
+    uint32_t bnd[kMaskN], inb[kMaskN];
+};
 
-// segment [a, a + kWalkSegment) of one walk
+// a polygon as the walks read it
+struct WalkPoly {
+    GlobalSrc src;
+    int4 bb;
+    int edges;    // of one test, about
+    int batch;    // box points gathered before they are tested
+    bool masked;  // box points go through the mask
+    MaskFrame f;
+};
 template <class W>
-__device__ __forceinline__ void walk_segment(const int2* xy, const int64_t* off, const int4* bbox, const SlabInfo* slabs,
-                                             const int32_t* slab_ptr, const int32_t* slab_edges, uint64_t seed,
-                                             uint32_t T, int64_t p, int k, uint32_t a, uint32_t* res, int lane,
-                                             W& work)
+__device__ __forceinline__ WalkPoly walk_poly(WalkWarp& m, const int2* xy, const int64_t* off, const int4* bbox,
+                                              const int64_t* area2, const SlabInfo* slabs, const int32_t* slab_ptr,
+                                              const int32_t* slab_edges, int64_t p, int lane, W& work)
 {
     const int64_t b = off[p];
     const int n = (int)(off[p + 1] - b);
-    const int4 bb = bbox[p];
     const SlabInfo si = slabs && n > kSmemVerts ? slabs[p] : SlabInfo{0, 0, 0, 1, 0};
-    const GlobalSrc src{xy + b, n, si.S > 0 ? slab_ptr + si.slab_base : nullptr,
-                        si.S > 0 ? slab_edges + si.edge_base : nullptr, si.slab_h, si.ymin};
-    auto inside = [&](int px, int py, int ln, W& w) { return warp_inside_src(src, px, py, ln, w); };
-    const uint64_t sk = pmh_mix64(seed + (uint64_t)(k + 1) * PMH_GAMMA);
-    const uint32_t end = T - a > kWalkSegment ? a + kWalkSegment : T;
-    const uint32_t r = sign_one_t<kIdxU>(inside, bb.x, bb.y, (uint32_t)(bb.z - bb.x), (uint32_t)(bb.w - bb.y), sk,
-                                         end, lane, work, a);
-    if (r < end && lane == 0) atomicMin(res, r);
+    WalkPoly w{{xy + b, n, si.S > 0 ? slab_ptr + si.slab_base : nullptr,
+                si.S > 0 ? slab_edges + si.edge_base : nullptr, si.slab_h, si.ymin},
+               bbox[p], si.S > 0 ? min(n, 32) : n, 1, false, {}};
+    // a walk meets box / area box points on average (of which the mask leaves an eighth or so): an
+    // eighth of those to test at a time walks on past the hash by that much at most
+    const long long a2 = area2[p];
+    const float area = fmaxf(0.5f * (float)(a2 < 0 ? -a2 : a2), 1.0f);
+    const float ratio = (float)(w.bb.z - w.bb.x) * (float)(w.bb.w - w.bb.y) / area;
+    w.masked = ratio >= kWalkMaskRatio && n <= kMaskMaxEdges;
+    w.batch = (int)fminf(fmaxf(ratio * (w.masked ? 1.0f / 64.0f : 0.125f), 1.0f), 32.0f);
+    if (w.masked) {
+        w.f = mask_frame(w.bb);
+        build_mask(m, w.src, n, w.bb, w.f, true, lane, work);
+    }
+    return w;
+}
+
+// the smallest inside index of stream points [a, end), or end
+template <class W>
+__device__ __forceinline__ uint32_t walk_points(const WalkPoly& P, uint64_t sk, uint32_t a, uint32_t end, WalkWarp& m,
+                                                int lane, W& work)
+{
+    const unsigned full = 0xffffffffu, lt = pmh_lanemask_lt();
+    const uint32_t w = (uint32_t)(P.bb.z - P.bb.x), h = (uint32_t)(P.bb.w - P.bb.y);
+    const uint64_t step = 32ull * PMH_GAMMA;
+    uint64_t z = sk + (uint64_t)(a + lane + 1) * PMH_GAMMA;
+    uint32_t found = end;
+    int np = 0;  // gathered box points
+    for (uint64_t i0 = a;; i0 += 32u * kIdxU) {
+        const bool last = i0 >= end;
+        bool sure = false;  // a gathered point is inside by the mask
+        if (!last) {
+            uint32_t pt[kIdxU];
+            unsigned box = 0;
+#pragma unroll
+            for (int j = 0; j < kIdxU; ++j) {
+                pt[j] = pmh_mix64_lo(z + (uint64_t)j * step);
+                const uint32_t dx = (pt[j] & 0xFFFFu) - (uint32_t)P.bb.x, dy = (pt[j] >> 16) - (uint32_t)P.bb.y;
+                box |= (unsigned)((dx < w) & (dy < h)) << j;
+            }
+            z += (uint64_t)kIdxU * step;
+            if (!__any_sync(full, box)) continue;
+#pragma unroll
+            for (int j = 0; j < kIdxU; ++j) {
+                const uint32_t i = (uint32_t)i0 + 32u * j + (uint32_t)lane;
+                bool hit = ((box >> j) & 1u) && i < end, in = false;
+                if (P.masked && hit) {
+                    const int cx = ((int)(pt[j] & 0xFFFFu) - P.f.x0) >> P.f.cwl;
+                    const int cy = ((int)(pt[j] >> 16) - P.f.y0) >> P.f.chl;
+                    in = (m.inb[cy] >> cx) & 1u;
+                    hit = in || ((m.bnd[cy] >> cx) & 1u);
+                    work.masked += 1;
+                }
+                const unsigned bal = __ballot_sync(full, hit);
+                if (hit) m.buf[np + __popc(bal & lt)] = make_uint2(2u * i + in, pt[j]);
+                np += __popc(bal);
+                sure |= in;
+            }
+            __syncwarp();
+        }
+        const bool all = last || __any_sync(full, sure);
+        int head = 0;
+        while (np - head >= P.batch || (all && np > head)) {
+            const int count = min(np - head, 32);
+            const uint2 c = lane < count ? m.buf[head + lane] : make_uint2(0u, 0u);
+            head += count;
+            unsigned in = 0;
+            // (instructions of a lane's and of the warp's tests)
+            if (18 * P.edges < count * (20 * ((P.edges + 31) >> 5) + 25)) {
+                const bool inside = lane < count && ((c.x & 1u) || lane_inside(P.src, (int)(c.y & 0xFFFFu),
+                                                                               (int)(c.y >> 16), work));
+                in = __ballot_sync(full, inside);
+            } else {
+                for (int t = 0; t < count && !in; ++t) {
+                    const uint32_t r = __shfl_sync(full, c.y, t);
+                    if ((__shfl_sync(full, c.x, t) & 1u) ||
+                        warp_inside_src(P.src, (int)(r & 0xFFFFu), (int)(r >> 16), lane, work)) in = 1u << t;
+                }
+            }
+            if (in) {
+                found = __shfl_sync(full, c.x, __ffs(in) - 1) >> 1;
+                break;
+            }
+        }
+        if (last || found < end) break;
+        if (head > 0) {  // fewer than a batch are left: to the front
+            const uint2 c = lane < np - head ? m.buf[head + lane] : make_uint2(0u, 0u);
+            np -= head;
+            __syncwarp();
+            if (lane < np) m.buf[lane] = c;
+            __syncwarp();
+        }
+    }
+    __syncwarp();
+    work.walk += (found < end ? found + 1 : end) - a;
+    return found;
 }
 
 template <bool kCount>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kWalkWarps * 32, 3)
 sign_walks_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, const int4* __restrict__ bbox,
-                  const SlabInfo* __restrict__ slabs, const int32_t* __restrict__ slab_ptr,
+                  const int64_t* __restrict__ area2, const SlabInfo* __restrict__ slabs, const int32_t* __restrict__ slab_ptr,
                   const int32_t* __restrict__ slab_edges, const int32_t* __restrict__ list, int64_t n_slots,
                   const int64_t* __restrict__ d_n, const int* __restrict__ d_flags, uint64_t seed, int K, uint32_t T,
                   WalkQueue wq, uint32_t* out, unsigned long long* __restrict__ work_out)
 {
+    __shared__ WalkWarp smem[kWalkWarps];
     if (d_flags && *d_flags) return;
     const int lane = threadIdx.x & 31;
+    WalkWarp& m = smem[threadIdx.x >> 5];
     const unsigned full = 0xffffffffu;
     using W = typename std::conditional<kCount, Work, NoWork>::type;
     W work;
+    auto poly = [&](int64_t p) {
+        return walk_poly(m, xy, off, bbox, area2, slabs, slab_ptr, slab_edges, p, lane, work);
+    };
+    auto stream = [&](int k) { return pmh_mix64(seed + (uint64_t)(k + 1) * PMH_GAMMA); };
     const unsigned long long queued = wq.tickets[1];
     const int n = (int)min(queued, (unsigned long long)kWalkItems);
     const int nwarps = (int)(gridDim.x * (blockDim.x >> 5)), warp = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
@@ -732,6 +842,8 @@ sign_walks_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, 
         WalkItem* it = wq.items + i;
         const WalkItem w = *it;
         uint32_t* res = out + (int64_t)w.p * K + w.k;
+        const WalkPoly P = poly(w.p);
+        const uint64_t sk = stream(w.k);
         for (;;) {
             uint32_t s = 0, best = 0;
             if (lane == 0) {
@@ -741,8 +853,9 @@ sign_walks_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, 
             s = __shfl_sync(full, s, 0);
             best = __shfl_sync(full, best, 0);
             if (!ahead(w, s, best)) break;
-            walk_segment(xy, off, bbox, slabs, slab_ptr, slab_edges, seed, T, w.p, w.k, w.start + s * kWalkSegment,
-                         res, lane, work);
+            const uint32_t a = w.start + s * kWalkSegment, end = T - a > kWalkSegment ? a + kWalkSegment : T;
+            const uint32_t r = walk_points(P, sk, a, end, m, lane, work);
+            if (r < end && lane == 0) atomicMin(res, r);
         }
     };
     for (;;) {
@@ -775,36 +888,48 @@ sign_walks_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, 
         idle = 0;
         c = c == 0 ? chunks - 1 : c - 1;  // look at this chunk again
     }
-    // past the queue: the marked hashes, a warp each
+    // past the queue: the marked hashes, a warp each, found in groups of `per` consecutive ones that
+    // are handed out in turn: 32, or so few that every warp gets some.  5,000 thin polygons of 8
+    // vertices, K = 128 (640,000 walks of 17,000 points, of which 1,400 in the box): 28 ms, 161 with
+    // a polygon a warp and a warp a box point; of 64 vertices 35 and 192
     if (queued > (unsigned long long)kWalkItems) {
         if (d_n) n_slots = min(n_slots, *d_n);
-        for (int64_t slot = warp; slot < n_slots; slot += nwarps) {
-            const int64_t p = list ? (int64_t)list[slot] : slot;
-            const int level = pmh_index_level(bbox[p], K);
-            for (int k0 = 0; k0 < K; k0 += 32) {
-                uint32_t* row = out + p * (int64_t)K + k0;
-                unsigned left = __ballot_sync(full, k0 + lane < K && row[k0 + lane < K ? lane : 0] == kNoPoint);
-                while (left) {
-                    const int j = __ffs(left) - 1;
-                    left &= left - 1;
-                    __syncwarp();
-                    if (lane == 0) row[j] = T;
-                    __syncwarp();
-                    for (uint64_t a = (uint64_t)index_level_points(level); a < T; a += kWalkSegment) {
-                        walk_segment(xy, off, bbox, slabs, slab_ptr, slab_edges, seed, T, p, k0 + j, (uint32_t)a, row + j,
-                                     lane, work);
-                        uint32_t best = 0;
-                        if (lane == 0) best = *reinterpret_cast<volatile uint32_t*>(row + j);
-                        if (__shfl_sync(full, best, 0) < T) break;
-                    }
-                }
+        int per = 32;
+        while (per > 1 && n_slots * ((K + per - 1) / per) < 4ll * nwarps) per >>= 1;
+        const int groups = (K + per - 1) / per;
+        for (;;) {
+            unsigned long long t = 0;
+            if (lane == 0) t = atomicAdd(wq.tickets + 3, 1ull);
+            t = __shfl_sync(full, t, 0);
+            if ((int64_t)t >= n_slots * groups) break;
+            const int64_t slot = (int64_t)t / groups, p = list ? (int64_t)list[slot] : slot;
+            const int k0 = (int)((int64_t)t - slot * groups) * per;
+            uint32_t* row = out + p * (int64_t)K + k0;
+            const bool mine = lane < per && k0 + lane < K;
+            unsigned left = __ballot_sync(full, mine && row[mine ? lane : 0] == kNoPoint);
+            if (!left) continue;
+            const WalkPoly P = poly(p);
+            const uint32_t from = (uint32_t)index_level_points(pmh_index_level(P.bb, K));
+            while (left) {
+                const int j = __ffs(left) - 1;
+                left &= left - 1;
+                const uint32_t r = walk_points(P, stream(k0 + j), from, T, m, lane, work);
+                if (lane == 0) row[j] = r;
             }
         }
     }
-    if (kCount && work_out && lane == 0) {  // (warp-uniform counts)
-        atomicAdd(&work_out[0], work.walk);
-        atomicAdd(&work_out[3], work.cand);
-        atomicAdd(&work_out[4], work.edges);
+    if (kCount && work_out) {
+        unsigned long long le = work.lane_edges, ma = work.masked;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            le += __shfl_xor_sync(full, le, o);
+            ma += __shfl_xor_sync(full, ma, o);
+        }
+        if (lane == 0) {  // (the other counts are warp-uniform)
+            atomicAdd(&work_out[0], work.walk);
+            atomicAdd(&work_out[4], work.edges + le);
+            atomicAdd(&work_out[5], ma);
+        }
     }
 }
 
@@ -863,9 +988,9 @@ int pmh_launch_sign_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* o
                                      work, s));
     }
     if (S.lv[0].first) {
-        // (two blocks of eight warps per SM: the walks are bound by the generator's integer chain)
+        // (three blocks of eight warps per SM: the walks are bound by the generator's integer chain)
         auto fn = work ? sign_walks_kernel<true> : sign_walks_kernel<false>;
-        fn<<<ctx->sm_count * 4, 256, 0, s>>>(xy, off, bbox, slabs, slab_ptr, slab_edges, list, n_slots, d_n, d_flags,
+        fn<<<ctx->sm_count * 3, kWalkWarps * 32, 0, s>>>(xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list, n_slots, d_n, d_flags,
                                              P->seed, (int)P->K, P->T, wq, out, work);
         PMH_LAUNCHED("sign_walks_kernel");
     }

@@ -63,3 +63,42 @@ def test_few_hashes(B, orc, K):
         got = B.minhash_sign(ctx, polys, P).cpu().numpy().view(np.uint32)
         assert np.array_equal(got, orc.sign(db.xy, db.offsets, SEED, K, 1 << 22, nthreads=16))
     ctx.close()
+
+
+def _strips(n, length, seed):
+    """Thin slanted strips of 4 to 300 vertices and widths from nothing (no lattice point) to 60."""
+    rng = np.random.default_rng(seed)
+    rings = []
+    for i in range(n):
+        h = int(rng.choice([2, 4, 32, 40, 150]))
+        a, w = rng.uniform(0.2, 1.3), rng.choice([0.3, 2.0, 8.0, 60.0])
+        d, t = np.array([np.cos(a), np.sin(a)]), np.linspace(0, length, h)[:, None]
+        o = rng.uniform(1000, 64000 - length, 2)
+        side = np.array([-d[1], d[0]]) * w * (0.5 + np.sin(np.pi * t / length))
+        rings.append(np.rint(np.concatenate([o + d * t + side / 2, (o + d * t - side / 2)[::-1]])))
+    off = np.concatenate([[0], np.cumsum([len(r) for r in rings])]).astype(np.int64)
+    return np.concatenate(rings).astype(np.int32), off
+
+
+@pytest.mark.parametrize("n,K,T", [(300, 256, 6000), (5000, 33, 3000), (9000, 130, 1500), (40, 128, 9000)])
+@pytest.mark.parametrize("count", [True, False])
+def test_more_leftover_walks_than_the_queue_holds(orc, n, K, T, count):
+    """Thin polygons under large boxes: 70,000 to a million hashes without a point of the level's (the
+    last set: fewer than the queue holds), through the plain call and a captured graph."""
+    from paper_2511_16576_gb300 import binding as B
+    ctx = B.Context(0)
+    B.sign_count_work(ctx, count)
+    P = B.make_params(K, 1, T, 0x5EED, flags=B.FLAG_STREAM_INDEX)
+    xy, off = _strips(n, 20_000, n)
+    up = [torch.from_numpy(a).to(DEV) for a in (xy, off)]
+    polys = B.poly_upload(ctx, *up)
+    ref = orc.sign(xy, off, 0x5EED, K, T, nthreads=16)
+    assert (ref == T).any() and (ref < T).any()
+    h = B.minhash_sign(ctx, polys, P)
+    assert np.array_equal(h.cpu().numpy().view(np.uint32), ref)
+    index = B.lsh_build(ctx, h, P)
+    g = B.QueryGraph(ctx, index, max_queries=n + 7, max_vertices=xy.shape[0], cand_capacity=1 << 20, m=4)
+    g.run(*up)
+    assert np.array_equal(g.hashes[:n].cpu().numpy().view(np.uint32).reshape(n, K), ref)
+    g.close()
+    ctx.close()
