@@ -16,7 +16,8 @@
 //     part runs with every lane.  An inside point lowers its hash's bound, an outside
 //     one is replaced by the next point of its cell below the bound.  A hash without
 //     a point below the level's limit is queued, and a last launch walks on from there;
-//   * walk form (no index, or a very large polygon whose expected walk is short):
+//   * walk form (no index, a very large polygon whose expected walk is short, or, in a launch of its
+//     own, a few hashes of a polygon of large area):
 //     Algorithm 1 in warp rounds of 32 * U consecutive stream points; box
 //     candidates in index order (ballot + ffs), each decided by the mask or by the
 //     warp-cooperative exact test.
@@ -49,11 +50,13 @@ constexpr int kMaskN = 32;         // coverage mask cells per side
 constexpr int kGroup = 128;        // hashes signed together, four a lane
 constexpr int kQueue = 192;        // candidates: at most 31, + 128 of a cell, + 32 that follow exact tests
 constexpr uint32_t kNoPoint = 0xFFFFFFFFu;
-// A few hashes of a polygon of large area are walked: K walks of 2^32 / area points cost less than
-// classifying the cells under the box.  The staged class keeps its own build, without the walk,
-// unless K = 1.  K = 1, 149,000 centred polygons of 9 vertices: 503 us (692 indexed); K = 3,
-// 100,000 of 317 vertices: 1,669 (1,845); from K = 16 on the index is the faster form.
-constexpr int kBriefMaxK = 12;
+// A few hashes of a polygon of large area are walked in a launch of their own (sign_brief_kernel):
+// K walks of 2^32 / area points cost less than the mask and the cells under the box.  Rings above
+// the staged size, whose masks cost more, gain up to K = 32 (100,000 of 317 vertices, K = 32: 2,659
+// us through the index, 2,470), staged ones up to K = 8 (100,000 stars of 16 to 256 vertices and
+// 1e-4 to 1e-2 of the domain: K = 3 946 -> 754, 8 994 -> 970, 10 1,024 -> 1,050); points per
+// polygon from 1,500 to 4,500 measure within 5% of each other
+constexpr int kBriefMaxK = 8, kBriefMaxKLarge = 32;  // (of staged rings, and of larger ones)
 constexpr float kBriefWalk = 3000.0f;
 constexpr int kIdxU = 4;           // points per lane per round of a leftover walk
 constexpr int kMaskMaxEdges = 4096;  // larger polygons skip the mask (every cell is a boundary cell)
@@ -141,6 +144,16 @@ __device__ __forceinline__ bool warp_inside_src(const Src& s, int px, int py, in
         par ^= edge_parity(s.vert(e), s.vert(e + 1), px, py);
     }
     return __popc(__ballot_sync(0xffffffffu, par)) & 1;
+}
+
+// stream points examined per hash, on average
+__device__ __forceinline__ float expected_walk(long long area2)
+{
+    return 4294967296.0f / fmaxf(0.5f * (float)(area2 < 0 ? -area2 : area2), 1.0f);
+}
+__device__ __forceinline__ bool signed_briefly(int K, int64_t n, float walk)
+{
+    return K <= (n <= kSmemVerts ? kBriefMaxK : kBriefMaxKLarge) && (float)K * walk < kBriefWalk;
 }
 
 // coverage mask frame of a clipped box: cells of 2^cwl x 2^chl lattice units aligned to
@@ -624,10 +637,9 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
             continue;
         }
         // the indexed form's grid level (-1: no index) and the expected walk
-        const long long a2 = area2 ? area2[p] : 0;
-        const float walk = 4294967296.0f / fmaxf(0.5f * (float)(a2 < 0 ? -a2 : a2), 1.0f);
-        const bool brief = !kIndexedOnly && K <= kBriefMaxK && (float)K * walk < kBriefWalk;
-        const int level = S.lv[0].first && area2 && !brief ? pmh_index_level(bb, K) : -1;
+        const float walk = area2 ? expected_walk(area2[p]) : 0.0f;
+        const int level = S.lv[0].first && area2 ? pmh_index_level(bb, K) : -1;
+        if (level >= 0 && signed_briefly(K, n, walk)) continue;  // sign_brief_kernel's
         if (staged) {
             // stage the polygon (closed: v[n] = v[0]; cp.async 8-byte copies) and bin its edges
             stage_vertices(m.v, xy + b, n, lane);
@@ -672,6 +684,78 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
         }
         __syncthreads();
         if (threadIdx.x < 6) atomicAdd(&work_out[threadIdx.x], wsum[threadIdx.x]);
+    }
+}
+
+// Few hashes of polygons of large area (signed_briefly), a warp a polygon: Algorithm 1 without
+// mask, cells or slab lists for a ring that is staged -- a hash is among its first few dozen
+// points, and a box point's test over all the edges is a few instructions a lane.  Bound by
+// issue.  149,000 centred polygons of 9 vertices, K = 3: 378 us (763 through the index, 697 with the
+// index's earlier form); 100,000 of 317: 676 (1,680, 1,525).
+constexpr int kBriefWarps = 8;
+constexpr int kBriefChunk = 8;  // slots looked at together
+template <bool kCount>
+__global__ void __launch_bounds__(kBriefWarps * 32, 4)
+sign_brief_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, const int4* __restrict__ bbox,
+                  const int64_t* __restrict__ area2, const SlabInfo* __restrict__ slabs,
+                  const int32_t* __restrict__ slab_ptr, const int32_t* __restrict__ slab_edges,
+                  const int32_t* __restrict__ list, int64_t n_slots, const int64_t* __restrict__ d_n,
+                  const int* __restrict__ d_flags, uint64_t seed, int K, uint32_t T, uint32_t* __restrict__ out,
+                  unsigned long long* __restrict__ work_out)
+{
+    __shared__ int2 sv[kBriefWarps][kSmemVerts + 1];
+    if (d_flags && *d_flags) return;
+    if (d_n) n_slots = min(n_slots, *d_n);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    using W = typename std::conditional<kCount, Work, NoWork>::type;
+    W work;
+    int64_t chunk = (int64_t)blockIdx.x * kBriefWarps + wid;
+    unsigned left = 0;  // slots of the chunk to sign, a lane each
+    int64_t lp = 0;     // the lane's polygon
+    for (;;) {
+        if (!left) {
+            const int64_t slot = chunk * kBriefChunk + lane;
+            if (chunk * kBriefChunk >= n_slots) break;
+            chunk += (int64_t)gridDim.x * kBriefWarps;
+            bool mine = false;
+            if (lane < kBriefChunk && slot < n_slots) {
+                lp = list ? (int64_t)list[slot] : slot;
+                const int4 bb = bbox[lp];
+                mine = bb.z > bb.x && bb.w > bb.y &&
+                       signed_briefly(K, off[lp + 1] - off[lp], expected_walk(area2[lp]));
+            }
+            left = __ballot_sync(0xffffffffu, mine);
+            continue;
+        }
+        const int64_t p = __shfl_sync(0xffffffffu, lp, __ffs(left) - 1);
+        left &= left - 1;
+        const int4 bb = bbox[p];
+        const int64_t b = off[p];
+        const int n = (int)(off[p + 1] - b);
+        const uint32_t w = (uint32_t)(bb.z - bb.x), h = (uint32_t)(bb.w - bb.y);
+        uint32_t mine = T;
+        auto sign = [&](const auto& inside) {
+            for (int k = 0; k < K; ++k) {
+                const uint64_t sk = pmh_mix64(seed + (uint64_t)(k + 1) * PMH_GAMMA);
+                const uint32_t hk = sign_one_t<kIdxU, true>(inside, bb.x, bb.y, w, h, sk, T, lane, work);
+                if (lane == k) mine = hk;
+            }
+        };
+        if (n <= kSmemVerts) {
+            stage_vertices(sv[wid], xy + b, n, lane);
+            sign(AllEdges{sv[wid], n});
+        } else {
+            const SlabInfo si = slabs ? slabs[p] : SlabInfo{0, 0, 0, 1, 0};
+            const GlobalSrc src{xy + b, n, si.S > 0 ? slab_ptr + si.slab_base : nullptr,
+                                si.S > 0 ? slab_edges + si.edge_base : nullptr, si.slab_h, si.ymin};
+            sign([&](int px, int py, int ln, W& wk) { return warp_inside_src(src, px, py, ln, wk); });
+        }
+        if (lane < K) out[p * (int64_t)K + lane] = mine;
+        __syncwarp();
+    }
+    if (kCount && work_out && lane == 0) {  // (warp-uniform counts)
+        atomicAdd(&work_out[0], work.walk);
+        atomicAdd(&work_out[4], work.edges);
     }
 }
 
@@ -976,8 +1060,19 @@ int pmh_launch_sign_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* o
     if (n_slots <= 0) return PMH_OK;
     PMH_CUDA_TRY(cudaMemsetAsync(wq.tickets, 0, sizeof(unsigned long long) * kSignTickets, s));
     // the indexed class at the list's end goes to its own launch (needs the class list)
-    // (of a single hash most of it walks: the other build)
-    const int64_t tail = list && !d_n && P->K > 1 ? std::min(std::max<int64_t>(n_indexed_tail, 0), n_slots - n_chunked) : 0;
+    const int64_t tail = list && !d_n ? std::min(std::max<int64_t>(n_indexed_tail, 0), n_slots - n_chunked) : 0;
+    // (the class list's tail is staged: not looked at when only larger rings can be signed briefly)
+    const int64_t brief = !S.lv[0].first || !area2 ? 0
+                          : P->K <= (uint32_t)kBriefMaxK ? n_slots
+                          : P->K <= (uint32_t)kBriefMaxKLarge ? n_slots - tail : 0;
+    if (brief > 0) {
+        auto fn = work ? sign_brief_kernel<true> : sign_brief_kernel<false>;
+        constexpr int kPer = kBriefWarps * kBriefChunk;
+        const int64_t blocks = std::min<int64_t>((brief + kPer - 1) / kPer, (int64_t)ctx->sm_count * 4);
+        fn<<<(unsigned)blocks, kBriefWarps * 32, 0, s>>>(xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list,
+                                                         brief, d_n, d_flags, P->seed, (int)P->K, P->T, out, work);
+        PMH_LAUNCHED("sign_brief_kernel");
+    }
     if (n_slots - tail > 0)
         PMH_TRY(launch_unified<false>(ctx, U, xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list,
                                       n_slots - tail, n_chunked, d_n, d_flags, P, S, wq, out, work, s));

@@ -102,3 +102,35 @@ def test_more_leftover_walks_than_the_queue_holds(orc, n, K, T, count):
     assert np.array_equal(g.hashes[:n].cpu().numpy().view(np.uint32).reshape(n, K), ref)
     g.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("K", [1, 2, 3, 8, 9, 31, 32, 33])
+@pytest.mark.parametrize("count", [True, False])
+def test_few_hashes(orc, K, count):
+    """Polygons of every size and area around the forms of few hashes (walked briefly or through the index,
+    staged or larger rings), and their queries through a captured graph."""
+    from paper_2511_16576_gb300 import binding as B
+    ctx = B.Context(0)
+    B.sign_count_work(ctx, count)
+    T = 1 << 20
+    P = B.make_params(K, 1, T, SEED, flags=B.FLAG_STREAM_INDEX)
+    parts = [synth.star_polygons(n, 40 + i, n_range=r, n_dist="loguniform", f_range=f)
+             for i, (n, r, f) in enumerate([(300, (3, 60), (1e-2, 2e-1)), (300, (200, 300), (1e-4, 1e-1)),
+                                            (200, (4, 256), (1e-5, 1e-3)), (30, (3000, 9000), (1e-3, 1e-1))])]
+    far = np.array([[70_000, 70_000], [70_009, 70_000], [70_000, 70_009]], np.int32)  # no lattice point
+    xy = np.concatenate([p.xy for p in parts] + [far])
+    sizes = np.concatenate([np.diff(p.offsets) for p in parts] + [[3]])
+    order = np.random.default_rng(K).permutation(len(sizes))
+    first = np.concatenate([[0], np.cumsum(sizes)])
+    xy = np.ascontiguousarray(np.concatenate([xy[first[i]:first[i] + sizes[i]] for i in order]))
+    off = np.concatenate([[0], np.cumsum(sizes[order])]).astype(np.int64)
+    ref = orc.sign(xy, off, SEED, K, T, nthreads=16)
+    up = [torch.from_numpy(a).to(DEV) for a in (xy, off)]
+    h = B.minhash_sign(ctx, B.poly_upload(ctx, *up), P)
+    assert np.array_equal(h.cpu().numpy().view(np.uint32), ref)
+    n = len(sizes)
+    g = B.QueryGraph(ctx, B.lsh_build(ctx, h, P), n + 3, xy.shape[0], 1 << 21, 4)
+    g.run(*up)
+    assert np.array_equal(g.hashes[:n].cpu().numpy().view(np.uint32).reshape(n, K), ref)
+    g.close()
+    ctx.close()
