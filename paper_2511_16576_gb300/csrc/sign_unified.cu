@@ -151,10 +151,14 @@ __device__ __forceinline__ float expected_walk(long long area2)
 {
     return 4294967296.0f / fmaxf(0.5f * (float)(area2 < 0 ? -area2 : area2), 1.0f);
 }
-__device__ __forceinline__ bool signed_briefly(int K, int64_t n, float walk)
-{
-    return K <= (n <= kSmemVerts ? kBriefMaxK : kBriefMaxKLarge) && (float)K * walk < kBriefWalk;
-}
+// the walks signed briefly are shorter than this: of staged rings, and of larger ones
+struct BriefLimits {
+    float staged, large;
+    explicit BriefLimits(int K)
+        : staged(K <= kBriefMaxK ? kBriefWalk / (float)K : 0.0f), large(K <= kBriefMaxKLarge ? kBriefWalk / (float)K : 0.0f)
+    {
+    }
+};
 
 // coverage mask frame of a clipped box: cells of 2^cwl x 2^chl lattice units aligned to
 // the lattice (so that the cells of any grid of the stream index with at most 32 cells a
@@ -585,7 +589,7 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
                     const int32_t* __restrict__ slab_edges, const int32_t* __restrict__ list,
                     int64_t n_slots, int64_t n_chunked, const int64_t* __restrict__ d_n,
                     const int* __restrict__ d_flags, uint64_t seed, int K, uint32_t T,
-                    StreamIndexView S, WalkQueue wq, uint32_t* __restrict__ out,
+                    StreamIndexView S, WalkQueue wq, BriefLimits brief, uint32_t* __restrict__ out,
                     unsigned long long* __restrict__ work_out)
 {
     __shared__ UniWarp smem[kUniWarps];
@@ -639,7 +643,7 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
         // the indexed form's grid level (-1: no index) and the expected walk
         const float walk = area2 ? expected_walk(area2[p]) : 0.0f;
         const int level = S.lv[0].first && area2 ? pmh_index_level(bb, K) : -1;
-        if (level >= 0 && signed_briefly(K, n, walk)) continue;  // sign_brief_kernel's
+        if (level >= 0 && walk < (kIndexedOnly || staged ? brief.staged : brief.large)) continue;  // sign_brief_kernel's
         if (staged) {
             // stage the polygon (closed: v[n] = v[0]; cp.async 8-byte copies) and bin its edges
             stage_vertices(m.v, xy + b, n, lane);
@@ -687,7 +691,7 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
     }
 }
 
-// Few hashes of polygons of large area (signed_briefly), a warp a polygon: Algorithm 1 without
+// Few hashes of polygons of large area (BriefLimits), a warp a polygon: Algorithm 1 without
 // mask, cells or slab lists for a ring that is staged -- a hash is among its first few dozen
 // points, and a box point's test over all the edges is a few instructions a lane.  Bound by
 // issue.  149,000 centred polygons of 9 vertices, K = 3: 378 us (763 through the index, 697 with the
@@ -700,8 +704,8 @@ sign_brief_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, 
                   const int64_t* __restrict__ area2, const SlabInfo* __restrict__ slabs,
                   const int32_t* __restrict__ slab_ptr, const int32_t* __restrict__ slab_edges,
                   const int32_t* __restrict__ list, int64_t n_slots, const int64_t* __restrict__ d_n,
-                  const int* __restrict__ d_flags, uint64_t seed, int K, uint32_t T, uint32_t* __restrict__ out,
-                  unsigned long long* __restrict__ work_out)
+                  const int* __restrict__ d_flags, uint64_t seed, int K, uint32_t T, BriefLimits brief,
+                  uint32_t* __restrict__ out, unsigned long long* __restrict__ work_out)
 {
     __shared__ int2 sv[kBriefWarps][kSmemVerts + 1];
     if (d_flags && *d_flags) return;
@@ -722,7 +726,8 @@ sign_brief_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, 
                 lp = list ? (int64_t)list[slot] : slot;
                 const int4 bb = bbox[lp];
                 mine = bb.z > bb.x && bb.w > bb.y &&
-                       signed_briefly(K, off[lp + 1] - off[lp], expected_walk(area2[lp]));
+                       expected_walk(area2[lp]) <
+                           (off[lp + 1] - off[lp] <= kSmemVerts ? brief.staged : brief.large);
             }
             left = __ballot_sync(0xffffffffu, mine);
             continue;
@@ -1044,7 +1049,7 @@ static int launch_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* off
     blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, (n_items + kUniWarps - 1) / kUniWarps));
     fn<<<(int)blocks, kUniWarps * 32, 0, s>>>(xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list,
                                               n_slots, n_chunked, d_n, d_flags, P->seed, (int)P->K,
-                                              P->T, S, wq, out, work);
+                                              P->T, S, wq, BriefLimits((int)P->K), out, work);
     PMH_LAUNCHED(kIndexedOnly ? "sign_unified_kernel<indexed>" : "sign_unified_kernel");
     return PMH_OK;
 }
@@ -1070,7 +1075,8 @@ int pmh_launch_sign_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* o
         constexpr int kPer = kBriefWarps * kBriefChunk;
         const int64_t blocks = std::min<int64_t>((brief + kPer - 1) / kPer, (int64_t)ctx->sm_count * 4);
         fn<<<(unsigned)blocks, kBriefWarps * 32, 0, s>>>(xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list,
-                                                         brief, d_n, d_flags, P->seed, (int)P->K, P->T, out, work);
+                                                         brief, d_n, d_flags, P->seed, (int)P->K, P->T, BriefLimits((int)P->K), out,
+                                                         work);
         PMH_LAUNCHED("sign_brief_kernel");
     }
     if (n_slots - tail > 0)
