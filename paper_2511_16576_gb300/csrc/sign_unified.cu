@@ -51,22 +51,18 @@ constexpr int kGroup = 128;        // hashes signed together, four a lane
 constexpr int kQueue = 192;        // candidates: at most 31, + 128 of a cell, + 32 that follow exact tests
 constexpr uint32_t kNoPoint = 0xFFFFFFFFu;
 // A few hashes of a polygon of large area are walked in a launch of their own (sign_brief_kernel):
-// K walks of 2^32 / area points cost less than the mask and the cells under the box.  Rings above
-// the staged size, whose masks cost more, gain up to K = 32 (100,000 of 317 vertices, K = 32: 2,659
-// us through the index, 2,470), staged ones up to K = 8 (100,000 stars of 16 to 256 vertices and
-// 1e-4 to 1e-2 of the domain: K = 3 946 -> 754, 8 994 -> 970, 10 1,024 -> 1,050); points per
-// polygon from 1,500 to 4,500 measure within 5% of each other
-constexpr int kBriefMaxK = 8, kBriefMaxKLarge = 32;  // (of staged rings, and of larger ones)
+// K walks of 2^32 / area points cost less than the mask and the cells under the box.  100,000 stars
+// of 16 to 256 vertices and 1e-4 to 1e-2 of the domain: K = 3 946 us through the index, 754; 8 994,
+// 970; 10 1,024, 1,050; 5,000 fractal rings of 300 to 4,000 vertices: K = 3 168, 139; 8 176, 170;
+// 16 180, 218.  Points per polygon from 1,500 to 4,500 measure within 5% of each other
+constexpr int kBriefMaxK = 8;
 constexpr float kBriefWalk = 3000.0f;
 constexpr int kIdxU = 4;           // points per lane per round of a leftover walk
 constexpr int kMaskMaxEdges = 4096;  // larger polygons skip the mask (every cell is a boundary cell)
 
-struct __align__(16) UniWarp {
+// a warp's shared slice, and a staged ring's part of it
+struct __align__(16) UniSlice {
     uint32_t best[kGroup];   // per hash of the group: 2 * smallest inside index found (+ 1); 16-byte accesses
-    int2 v[kSmemVerts + 1];  // staged vertices, v[n] = v[0]
-    uint8_t ids[kSlabCap];   // staged edges by slab
-    uint16_t beg[kSlabs + 1];
-    int cnt[kSlabs];
     uint32_t bnd[kMaskN];    // bit i of row j: an edge touches cell (i, j)
     uint32_t inb[kMaskN];    // bit i of row j: untouched cell (i, j) lies inside
     uint32_t cell[kPlanCells];  // table rows of the inside cells (from the front) and of the boundary cells (from the back)
@@ -74,6 +70,15 @@ struct __align__(16) UniWarp {
     uint2 exact[64];         // the same, of candidates to test exactly
     uint32_t exact_xy[64];   // x | y << 16
 };
+struct UniWarp : UniSlice {
+    int2 v[kSmemVerts + 1];  // staged vertices, v[n] = v[0]
+    uint8_t ids[kSlabCap];   // staged edges by slab
+    uint16_t beg[kSlabs + 1];
+    int cnt[kSlabs];
+};
+// which polygons a build of the kernel takes: staged ones of the indexed form, larger ones, or all.
+// The class order puts them apart; a captured batch is mixed.
+enum class UniForm { kStaged, kLarge, kMixed };
 
 // ---------------------------------------------------------------------------
 // Edge sources.  vert(e) for e in [0, n] (vert(n) = vert(0)); row(py) gives the
@@ -100,12 +105,13 @@ struct GlobalSrc {
     int n;
     const int32_t* sp;   // slab table (nullptr: one list of every edge)
     const int32_t* se;   // edge lists
-    int slab_h, ymin;
+    int ymin;
+    uint64_t magic;      // of the slab height
     __device__ __forceinline__ int2 vert(int e) const { return v[e == n ? 0 : e]; }
     __device__ __forceinline__ void row(int py, int& lo, int& hi) const
     {
         if (sp) {
-            const int s = (py - ymin) / slab_h;
+            const int s = slab_div(py - ymin, magic);
             lo = sp[s];
             hi = sp[s + 1];
         } else {
@@ -151,14 +157,8 @@ __device__ __forceinline__ float expected_walk(long long area2)
 {
     return 4294967296.0f / fmaxf(0.5f * (float)(area2 < 0 ? -area2 : area2), 1.0f);
 }
-// the walks signed briefly are shorter than this: of staged rings, and of larger ones
-struct BriefLimits {
-    float staged, large;
-    explicit BriefLimits(int K)
-        : staged(K <= kBriefMaxK ? kBriefWalk / (float)K : 0.0f), large(K <= kBriefMaxKLarge ? kBriefWalk / (float)K : 0.0f)
-    {
-    }
-};
+// walks shorter than this are signed briefly
+static float brief_limit(int K) { return K <= kBriefMaxK ? kBriefWalk / (float)K : 0.0f; }
 
 // coverage mask frame of a clipped box: cells of 2^cwl x 2^chl lattice units aligned to
 // the lattice (so that the cells of any grid of the stream index with at most 32 cells a
@@ -271,7 +271,7 @@ __device__ __forceinline__ void build_mask(M& m /* its bnd and inb */, const Src
 // untouched cells by their code, boundary cells by the exact test.
 template <class Src>
 struct MaskedWalker {
-    const UniWarp* m;
+    const UniSlice* m;
     Src src;
     int x0, y0, cwl, chl;
     template <class W>
@@ -297,7 +297,7 @@ struct NoGather {
 // The cells of level L under the box: inside cells to the front of m.cell, boundary
 // cells to its back (as cell * pitch).  A grid cell is a block of mask cells; it is inside
 // iff all of them are (a part outside the mask's frame is outside the box).
-__device__ __forceinline__ void classify_cells(UniWarp& m, const IndexLevelView& L, int pitch, int4 bb,
+__device__ __forceinline__ void classify_cells(UniSlice& m, const IndexLevelView& L, int pitch, int4 bb,
                                                const MaskFrame& f, int& n_in, int& n_bnd, int lane)
 {
     const unsigned full = 0xffffffffu;
@@ -341,7 +341,7 @@ __device__ __forceinline__ void classify_cells(UniWarp& m, const IndexLevelView&
 // A __syncwarp stands between every read of a queue and the next write to it: a vote
 // orders nothing in memory.
 template <class Src, class W, class G>
-__device__ __forceinline__ void indexed_range(UniWarp& m, const Src& src, const StreamIndexView& S, int level,
+__device__ __forceinline__ void indexed_range(UniSlice& m, const Src& src, const StreamIndexView& S, int level,
                                               int4 bb, const MaskFrame& f, float walk, uint64_t seed, uint32_t T,
                                               int64_t p, int k_begin, int k_end, const WalkQueue& wq,
                                               uint32_t* __restrict__ out, int lane, W& work, G& gc)
@@ -515,7 +515,7 @@ __device__ __forceinline__ void indexed_range(UniWarp& m, const Src& src, const 
 
 // Walk form of hashes [k_begin, k_end): lane j keeps hash k0 + j of each 32.
 template <int U, class Src, class W>
-__device__ __forceinline__ void walk_range(const UniWarp& m, const Src& src, int4 bb, const MaskFrame& f, uint64_t seed,
+__device__ __forceinline__ void walk_range(const UniSlice& m, const Src& src, int4 bb, const MaskFrame& f, uint64_t seed,
                                            uint32_t T, int k_begin, int k_end,
                                            uint32_t* __restrict__ out, int lane, W& work)
 {
@@ -536,7 +536,7 @@ __device__ __forceinline__ void walk_range(const UniWarp& m, const Src& src, int
 // Walk form of a staged polygon, kept out of line so that its registers do not
 // weigh on the indexed form's gather (Work by pointer: a local copy inside).
 template <int U, class W>
-__device__ __noinline__ void walk_staged(const UniWarp& m, StagedSrc src, int4 bb, MaskFrame f, uint64_t seed,
+__device__ __noinline__ void walk_staged(const UniSlice& m, StagedSrc src, int4 bb, MaskFrame f, uint64_t seed,
                                          uint32_t T, int k_begin, int k_end, uint32_t* out,
                                          int lane, W* work)
 {
@@ -549,23 +549,31 @@ __device__ __noinline__ void walk_staged(const UniWarp& m, StagedSrc src, int4 b
     work->lane_edges += local.lane_edges;
 }
 
-// A polygon above the staged size (read from global memory): the mask, then the
-// planned form, out of line for the same reason.
+// A polygon above the staged size (read from global memory): the mask, then the planned form.
 template <int U, class W, class G>
-__device__ __noinline__ void sign_global(UniWarp& m, GlobalSrc src, int n, int4 bb, int level, float walk,
+__device__ __forceinline__ void sign_large(UniSlice& m, const GlobalSrc& src, int n, int4 bb, int level, float walk,
+                                           const StreamIndexView& S, uint64_t seed, uint32_t T, int64_t p, int k_begin,
+                                           int k_end, const WalkQueue& wq, uint32_t* out, int lane, W& work, G& gc)
+{
+    const MaskFrame f = mask_frame(bb);
+    build_mask(m, src, n, bb, f, n <= kMaskMaxEdges, lane, work);
+    // (without a mask every cell is a boundary cell: a walk of few rounds is cheaper)
+    if (level >= 0 && (n <= kMaskMaxEdges || walk > 1024.0f))
+        indexed_range(m, src, S, level, bb, f, walk, seed, T, p, k_begin, k_end, wq, out, lane, work, gc);
+    else
+        walk_range<U>(m, src, bb, f, seed, T, k_begin, k_end, out, lane, work);
+}
+
+// The same out of line, for the mixed build.
+template <int U, class W, class G>
+__device__ __noinline__ void sign_global(UniSlice& m, GlobalSrc src, int n, int4 bb, int level, float walk,
                                          const StreamIndexView& S, uint64_t seed, uint32_t T,
                                          int64_t p, int k_begin, int k_end, const WalkQueue& wq,
                                          uint32_t* out, int lane, W* work, G* gc)
 {
     W local;
     G g;
-    const MaskFrame f = mask_frame(bb);
-    build_mask(m, src, n, bb, f, n <= kMaskMaxEdges, lane, local);
-    // (without a mask every cell is a boundary cell: a walk of few rounds is cheaper)
-    if (level >= 0 && (n <= kMaskMaxEdges || walk > 1024.0f))
-        indexed_range(m, src, S, level, bb, f, walk, seed, T, p, k_begin, k_end, wq, out, lane, local, g);
-    else
-        walk_range<U>(m, src, bb, f, seed, T, k_begin, k_end, out, lane, local);
+    sign_large<U>(m, src, n, bb, level, walk, S, seed, T, p, k_begin, k_end, wq, out, lane, local, g);
     work->walk += local.walk;
     work->cand += local.cand;
     work->edges += local.edges;
@@ -577,11 +585,13 @@ __device__ __noinline__ void sign_global(UniWarp& m, GlobalSrc src, int n, int4 
     gc->masked += g.masked;
 }
 
-// kIndexedOnly: a launch over staged polygons of the indexed form only (the class
-// order's last class), compiled without the walk-form and large-polygon paths, so that
-// the gather keeps its values in registers (a fraction of the unified build's spills
-// and no call frames)
-template <int U, bool kCount, bool kIndexedOnly>
+// Builds for the classes of the class order: staged polygons of the indexed form without the
+// walk and the large-polygon paths, so that the gather keeps its values in registers (a
+// fraction of the mixed build's spills and no call frames); larger ones without the staged ring's
+// part of the shared memory (115 of 203 KB an SM), which leaves their vertices, read many times
+// from global memory, twice the L1 cache.  20,000 rings of 300 to 1,000 vertices and 2e-5 of the
+// domain: K = 32 1,115 us in the mixed build, 828; K = 128 2,447, 1,601
+template <int U, bool kCount, UniForm kForm>
 __global__ void __launch_bounds__(kUniWarps * 32, kUniMinBlocks)
 sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
                     const int4* __restrict__ bbox, const int64_t* __restrict__ area2,
@@ -589,15 +599,16 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
                     const int32_t* __restrict__ slab_edges, const int32_t* __restrict__ list,
                     int64_t n_slots, int64_t n_chunked, const int64_t* __restrict__ d_n,
                     const int* __restrict__ d_flags, uint64_t seed, int K, uint32_t T,
-                    StreamIndexView S, WalkQueue wq, BriefLimits brief, uint32_t* __restrict__ out,
+                    StreamIndexView S, WalkQueue wq, float brief_walk, uint32_t* __restrict__ out,
                     unsigned long long* __restrict__ work_out)
 {
-    __shared__ UniWarp smem[kUniWarps];
+    using Slice = typename std::conditional<kForm == UniForm::kLarge, UniSlice, UniWarp>::type;
+    __shared__ Slice smem[kUniWarps];
     __shared__ unsigned long long wsum[6];
     if (threadIdx.x < 6) wsum[threadIdx.x] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    UniWarp& m = smem[threadIdx.x >> 5];
+    Slice& m = smem[threadIdx.x >> 5];
     const unsigned full = 0xffffffffu;
     // work counters only in launches that report them
     using W = typename std::conditional<kCount, Work, NoWork>::type;
@@ -629,7 +640,7 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
         const int64_t p = list ? (int64_t)list[slot] : slot;
         const int64_t b = off[p];
         const int n = (int)(off[p + 1] - b);
-        const bool staged = n <= kSmemVerts;
+        const bool staged = kForm == UniForm::kMixed ? n <= kSmemVerts : kForm == UniForm::kStaged;
         const bool whole = chunk < 0 || (staged && !split);
         if (whole && chunk > 0) continue;  // signed whole by its chunk 0
         const int k_begin = whole ? 0 : 32 * chunk;
@@ -643,27 +654,36 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
         // the indexed form's grid level (-1: no index) and the expected walk
         const float walk = area2 ? expected_walk(area2[p]) : 0.0f;
         const int level = S.lv[0].first && area2 ? pmh_index_level(bb, K) : -1;
-        if (level >= 0 && walk < (kIndexedOnly || staged ? brief.staged : brief.large)) continue;  // sign_brief_kernel's
-        if (staged) {
-            // stage the polygon (closed: v[n] = v[0]; cp.async 8-byte copies) and bin its edges
-            stage_vertices(m.v, xy + b, n, lane);
-            int sh = staged_slab_shift(bb.w - bb.y);
-            if (!build_staged_slabs(m.v, n, bb.y, sh, m.ids, m.beg, m.cnt, lane)) sh = single_slab(m, n, lane);
-            const StagedSrc src{m.v, m.ids, m.beg, bb.y, sh};
-            const MaskFrame f = mask_frame(bb);
-            build_mask(m, src, n, bb, f, true, lane, work);
-            if (kIndexedOnly || level >= 0)
-                indexed_range(m, src, S, level, bb, f, walk, seed, T, p, k_begin, k_end, wq, row, lane, work, gc);
-            else
-                walk_staged<U, W>(m, src, bb, f, seed, T, k_begin, k_end, row, lane, &work);
-        } else if (!kIndexedOnly) {
-            const SlabInfo si = slabs ? slabs[p] : SlabInfo{0, 0, 0, 1, 0};
-            const GlobalSrc src{xy + b, n, si.S > 0 ? slab_ptr + si.slab_base : nullptr,
-                                si.S > 0 ? slab_edges + si.edge_base : nullptr, si.slab_h, si.ymin};
-            sign_global<U, W, G>(m, src, n, bb, level, walk, S, seed, T, p, k_begin, k_end, wq, row, lane, &work,
-                                 &gc);
+        if (level >= 0 && walk < brief_walk) continue;  // sign_brief_kernel's
+        if constexpr (kForm != UniForm::kLarge) {
+            if (staged) {
+                // stage the polygon (closed: v[n] = v[0]; cp.async 8-byte copies) and bin its edges
+                stage_vertices(m.v, xy + b, n, lane);
+                int sh = staged_slab_shift(bb.w - bb.y);
+                if (!build_staged_slabs(m.v, n, bb.y, sh, m.ids, m.beg, m.cnt, lane)) sh = single_slab(m, n, lane);
+                const StagedSrc src{m.v, m.ids, m.beg, bb.y, sh};
+                const MaskFrame f = mask_frame(bb);
+                build_mask(m, src, n, bb, f, true, lane, work);
+                if (kForm == UniForm::kStaged || level >= 0)
+                    indexed_range(m, src, S, level, bb, f, walk, seed, T, p, k_begin, k_end, wq, row, lane, work, gc);
+                else
+                    walk_staged<U, W>(m, src, bb, f, seed, T, k_begin, k_end, row, lane, &work);
+                __syncwarp();
+            }
         }
-        __syncwarp();
+        if constexpr (kForm != UniForm::kStaged) {
+            if (!staged) {
+                const SlabInfo si = slabs ? slabs[p] : SlabInfo{0, 0, 0, 1, 0};
+                const GlobalSrc src{xy + b, n, si.S > 0 ? slab_ptr + si.slab_base : nullptr,
+                                    si.S > 0 ? slab_edges + si.edge_base : nullptr, si.ymin, slab_div_magic(si.slab_h)};
+                if (kForm == UniForm::kLarge)
+                    sign_large<U>(m, src, n, bb, level, walk, S, seed, T, p, k_begin, k_end, wq, row, lane, work, gc);
+                else
+                    sign_global<U, W, G>(m, src, n, bb, level, walk, S, seed, T, p, k_begin, k_end, wq, row, lane, &work,
+                                         &gc);
+                __syncwarp();
+            }
+        }
     }
     if (kCount && work_out) {
         unsigned long long le = work.lane_edges, en = gc.read, ca = gc.cand, ma = gc.masked,
@@ -691,20 +711,20 @@ sign_unified_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off
     }
 }
 
-// Few hashes of polygons of large area (BriefLimits), a warp a polygon: Algorithm 1 without
+// Few hashes of polygons of large area (walks below kBriefWalk / K points), a warp a polygon: Algorithm 1 without
 // mask, cells or slab lists for a ring that is staged -- a hash is among its first few dozen
 // points, and a box point's test over all the edges is a few instructions a lane.  Bound by
 // issue.  149,000 centred polygons of 9 vertices, K = 3: 378 us (763 through the index, 697 with the
 // index's earlier form); 100,000 of 317: 676 (1,680, 1,525).
 constexpr int kBriefWarps = 8;
-constexpr int kBriefChunk = 8;  // slots looked at together
+constexpr int kBriefChunk = 8;  // slots looked at together, at most
 template <bool kCount>
 __global__ void __launch_bounds__(kBriefWarps * 32, 4)
 sign_brief_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, const int4* __restrict__ bbox,
                   const int64_t* __restrict__ area2, const SlabInfo* __restrict__ slabs,
                   const int32_t* __restrict__ slab_ptr, const int32_t* __restrict__ slab_edges,
                   const int32_t* __restrict__ list, int64_t n_slots, const int64_t* __restrict__ d_n,
-                  const int* __restrict__ d_flags, uint64_t seed, int K, uint32_t T, BriefLimits brief,
+                  const int* __restrict__ d_flags, uint64_t seed, int K, uint32_t T, float brief_walk,
                   uint32_t* __restrict__ out, unsigned long long* __restrict__ work_out)
 {
     __shared__ int2 sv[kBriefWarps][kSmemVerts + 1];
@@ -713,21 +733,21 @@ sign_brief_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, 
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     using W = typename std::conditional<kCount, Work, NoWork>::type;
     W work;
+    const int64_t nwarps = (int64_t)gridDim.x * kBriefWarps;
+    const int look = (int)max((int64_t)1, min((int64_t)kBriefChunk, n_slots / (2 * nwarps)));
     int64_t chunk = (int64_t)blockIdx.x * kBriefWarps + wid;
     unsigned left = 0;  // slots of the chunk to sign, a lane each
     int64_t lp = 0;     // the lane's polygon
     for (;;) {
         if (!left) {
-            const int64_t slot = chunk * kBriefChunk + lane;
-            if (chunk * kBriefChunk >= n_slots) break;
-            chunk += (int64_t)gridDim.x * kBriefWarps;
+            const int64_t slot = chunk * look + lane;
+            if (chunk * look >= n_slots) break;
+            chunk += nwarps;
             bool mine = false;
-            if (lane < kBriefChunk && slot < n_slots) {
+            if (lane < look && slot < n_slots) {
                 lp = list ? (int64_t)list[slot] : slot;
                 const int4 bb = bbox[lp];
-                mine = bb.z > bb.x && bb.w > bb.y &&
-                       expected_walk(area2[lp]) <
-                           (off[lp + 1] - off[lp] <= kSmemVerts ? brief.staged : brief.large);
+                mine = bb.z > bb.x && bb.w > bb.y && expected_walk(area2[lp]) < brief_walk;
             }
             left = __ballot_sync(0xffffffffu, mine);
             continue;
@@ -752,7 +772,7 @@ sign_brief_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, 
         } else {
             const SlabInfo si = slabs ? slabs[p] : SlabInfo{0, 0, 0, 1, 0};
             const GlobalSrc src{xy + b, n, si.S > 0 ? slab_ptr + si.slab_base : nullptr,
-                                si.S > 0 ? slab_edges + si.edge_base : nullptr, si.slab_h, si.ymin};
+                                si.S > 0 ? slab_edges + si.edge_base : nullptr, si.ymin, slab_div_magic(si.slab_h)};
             sign([&](int px, int py, int ln, W& wk) { return warp_inside_src(src, px, py, ln, wk); });
         }
         if (lane < K) out[p * (int64_t)K + lane] = mine;
@@ -803,7 +823,7 @@ __device__ __forceinline__ WalkPoly walk_poly(WalkWarp& m, const int2* xy, const
     const int n = (int)(off[p + 1] - b);
     const SlabInfo si = slabs && n > kSmemVerts ? slabs[p] : SlabInfo{0, 0, 0, 1, 0};
     WalkPoly w{{xy + b, n, si.S > 0 ? slab_ptr + si.slab_base : nullptr,
-                si.S > 0 ? slab_edges + si.edge_base : nullptr, si.slab_h, si.ymin},
+                si.S > 0 ? slab_edges + si.edge_base : nullptr, si.ymin, slab_div_magic(si.slab_h)},
                bbox[p], si.S > 0 ? min(n, 32) : n, 1, false, {}};
     // a walk meets box / area box points on average (of which the mask leaves an eighth or so): an
     // eighth of those to test at a time walks on past the hash by that much at most
@@ -1025,7 +1045,7 @@ sign_walks_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off, 
 }  // namespace
 
 // one persistent launch over `n` slots of `list` (or slot order) with its own ticket
-template <bool kIndexedOnly>
+template <UniForm kForm>
 static int launch_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* off, const int4* bbox,
                           const int64_t* area2, const SlabInfo* slabs, const int32_t* slab_ptr,
                           const int32_t* slab_edges, const int32_t* list, int64_t n_slots,
@@ -1033,14 +1053,14 @@ static int launch_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* off
                           const StreamIndexView& S, const WalkQueue& wq, uint32_t* out,
                           unsigned long long* work, cudaStream_t s)
 {
-    auto fn = kIndexedOnly
-                  ? (work ? sign_unified_kernel<2, true, true> : sign_unified_kernel<2, false, true>)
-                  : work ? (U <= 2   ? sign_unified_kernel<2, true, false>
-                            : U <= 4 ? sign_unified_kernel<4, true, false>
-                                     : sign_unified_kernel<8, true, false>)
-                         : (U <= 2   ? sign_unified_kernel<2, false, false>
-                            : U <= 4 ? sign_unified_kernel<4, false, false>
-                                     : sign_unified_kernel<8, false, false>);
+    using Fn = decltype(&sign_unified_kernel<2, true, kForm>);
+    // (points per lane per round of the walk form; the staged build has none)
+    const Fn fns[3][2] = {{sign_unified_kernel<2, false, kForm>, sign_unified_kernel<2, true, kForm>},
+                          {sign_unified_kernel<kForm == UniForm::kStaged ? 2 : 4, false, kForm>,
+                           sign_unified_kernel<kForm == UniForm::kStaged ? 2 : 4, true, kForm>},
+                          {sign_unified_kernel<kForm == UniForm::kStaged ? 2 : 8, false, kForm>,
+                           sign_unified_kernel<kForm == UniForm::kStaged ? 2 : 8, true, kForm>}};
+    const Fn fn = fns[U <= 2 ? 0 : U <= 4 ? 1 : 2][work != nullptr];
     int per_sm = 0;
     PMH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kUniWarps * 32, 0));
     const int chunks = (int)((P->K + 31) / 32);
@@ -1049,8 +1069,8 @@ static int launch_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* off
     blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, (n_items + kUniWarps - 1) / kUniWarps));
     fn<<<(int)blocks, kUniWarps * 32, 0, s>>>(xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list,
                                               n_slots, n_chunked, d_n, d_flags, P->seed, (int)P->K,
-                                              P->T, S, wq, BriefLimits((int)P->K), out, work);
-    PMH_LAUNCHED(kIndexedOnly ? "sign_unified_kernel<indexed>" : "sign_unified_kernel");
+                                              P->T, S, wq, brief_limit((int)P->K), out, work);
+    PMH_LAUNCHED(kForm == UniForm::kStaged ? "sign_unified_kernel<staged>" : "sign_unified_kernel");
     return PMH_OK;
 }
 
@@ -1065,28 +1085,27 @@ int pmh_launch_sign_unified(pmh_ctx ctx, int U, const int2* xy, const int64_t* o
     if (n_slots <= 0) return PMH_OK;
     PMH_CUDA_TRY(cudaMemsetAsync(wq.tickets, 0, sizeof(unsigned long long) * kSignTickets, s));
     // the indexed class at the list's end goes to its own launch (needs the class list)
-    const int64_t tail = list && !d_n ? std::min(std::max<int64_t>(n_indexed_tail, 0), n_slots - n_chunked) : 0;
-    // (the class list's tail is staged: not looked at when only larger rings can be signed briefly)
-    const int64_t brief = !S.lv[0].first || !area2 ? 0
-                          : P->K <= (uint32_t)kBriefMaxK ? n_slots
-                          : P->K <= (uint32_t)kBriefMaxKLarge ? n_slots - tail : 0;
-    if (brief > 0) {
+    const bool classes = list && !d_n;
+    const int64_t tail = classes ? std::min(std::max<int64_t>(n_indexed_tail, 0), n_slots - n_chunked) : 0;
+    if (S.lv[0].first && area2 && brief_limit((int)P->K) > 0.0f) {
         auto fn = work ? sign_brief_kernel<true> : sign_brief_kernel<false>;
-        constexpr int kPer = kBriefWarps * kBriefChunk;
-        const int64_t blocks = std::min<int64_t>((brief + kPer - 1) / kPer, (int64_t)ctx->sm_count * 4);
+        const int64_t blocks = std::min<int64_t>((n_slots + kBriefWarps - 1) / kBriefWarps, (int64_t)ctx->sm_count * 4);
         fn<<<(unsigned)blocks, kBriefWarps * 32, 0, s>>>(xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list,
-                                                         brief, d_n, d_flags, P->seed, (int)P->K, P->T, BriefLimits((int)P->K), out,
-                                                         work);
+                                                         n_slots, d_n, d_flags, P->seed, (int)P->K, P->T,
+                                                         brief_limit((int)P->K), out, work);
         PMH_LAUNCHED("sign_brief_kernel");
     }
-    if (n_slots - tail > 0)
-        PMH_TRY(launch_unified<false>(ctx, U, xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list,
-                                      n_slots - tail, n_chunked, d_n, d_flags, P, S, wq, out, work, s));
+    if (n_slots - tail > 0) {
+        // (the class list's head holds larger rings only)
+        auto launch = classes ? launch_unified<UniForm::kLarge> : launch_unified<UniForm::kMixed>;
+        PMH_TRY(launch(ctx, U, xy, off, bbox, area2, slabs, slab_ptr, slab_edges, list, n_slots - tail, n_chunked, d_n,
+                       d_flags, P, S, wq, out, work, s));
+    }
     if (tail > 0) {
         if (n_slots - tail > 0) PMH_CUDA_TRY(cudaMemsetAsync(wq.tickets, 0, sizeof(unsigned long long), s));
-        PMH_TRY(launch_unified<true>(ctx, U, xy, off, bbox, area2, slabs, slab_ptr, slab_edges,
-                                     list + (n_slots - tail), tail, 0, nullptr, d_flags, P, S, wq, out,
-                                     work, s));
+        PMH_TRY(launch_unified<UniForm::kStaged>(ctx, U, xy, off, bbox, area2, slabs, slab_ptr, slab_edges,
+                                                 list + (n_slots - tail), tail, 0, nullptr, d_flags, P, S, wq, out, work,
+                                                 s));
     }
     if (S.lv[0].first) {
         // (three blocks of eight warps per SM: the walks are bound by the generator's integer chain)
