@@ -71,7 +71,7 @@ __host__ __device__ constexpr bool index_level_fits(int l, int K)
 {
     return (long long)K * index_level_points(l) <= (1ll << 31);
 }
-constexpr int kWalkKernelLevel = 4;  // the level that sign_kernel's indexed form reads (128^2)
+constexpr int kWalkKernelLevel = 4;  // the coarsest level that sign_kernel's indexed form reads (128^2)
 // polygons of at most this many vertices are staged in shared memory by the
 // signing kernels; larger ones are read through their y-slab edge index
 constexpr int kStagedMaxVerts = 256;
@@ -80,29 +80,45 @@ constexpr int kStagedMaxVerts = 256;
 // staging, slab lists and coverage mask are then built once per polygon)
 constexpr int kChunkMinVerts = 4096;
 
-// Cost model of the indexed form for one polygon (clipped box bb, twice its
+// Cost model of sign_kernel's indexed form for one polygon (clipped box bb, twice its
 // area), in warp instructions per hash: the walk examines about 2^32 / area
 // points, 128 per round of ~130 instructions; the indexed form reads the cells
-// under the bounding box, 32 per round of ~50 instructions, and sees about
-// lim * bbox / 2^32 candidates, with lim = 8 * 2^32 / area (a hit is then
-// missed with probability ~e^-8 and the walk resumes at lim).  Returns lim, or
-// 0 to walk.  (sign_kernel only: polygons above the staged size, with coverage masks.)
-__host__ __device__ __forceinline__ uint32_t pmh_indexed_limit(int4 bb, long long area2)
+// under the bounding box, and sees about lim * bbox / 2^32 candidates, with lim = 8 * 2^32 /
+// area or all of the level's points; a hash without one below lim (e^(-lim / walk) of them) walks
+// on from there.  Returns lim (0: walk) and the cheapest level: a longer walk belongs to a
+// smaller polygon, so a finer grid lays no more cells under its box, but the finest level's
+// tables do not fit the L2 cache.  K = 128, one level of 8,192 points before: 20,000 rings of 300
+// to 1,000 vertices and 2e-5 of the domain 115 ms, 3.6; 5,000 of 300 to 4,000 and 1e-4 to 1e-3 1.55,
+// 1.21.  (Polygons above the staged size, with coverage masks.)
+struct WalkIndexPlan {
+    uint32_t lim;
+    int level;
+};
+__host__ __device__ __forceinline__ WalkIndexPlan pmh_walk_index_plan(int4 bb, long long area2, int K)
 {
     // single precision: the estimate only picks a form and a limit (any limit
     // gives the exact result), and double precision is slow on this GPU
-    if (bb.z <= bb.x || bb.w <= bb.y) return 0;
-    const int shift = 16 - index_level_gbits(kWalkKernelLevel);
+    WalkIndexPlan plan{0u, kWalkKernelLevel};
+    if (bb.z <= bb.x || bb.w <= bb.y) return plan;
     const float area = 0.5f * (float)(area2 < 0 ? -area2 : area2);
     const float walk = 4294967296.0f / fmaxf(area, 1.0f);
-    const float cells = (float)((((bb.z - 1) >> shift) - (bb.x >> shift) + 1) *
-                                (((bb.w - 1) >> shift) - (bb.y >> shift) + 1));
-    const float lim = fminf((float)index_level_points(kWalkKernelLevel), 8.0f * walk + 256.0f);
-    const float cand = lim * ((float)(bb.z - bb.x) * (float)(bb.w - bb.y) * (1.0f / 4294967296.0f));
     const float walk_cost = ceilf(walk * (1.0f / 128.0f)) * 130.0f;
-    const float index_cost = ceilf(cells * (1.0f / 32.0f)) * 50.0f + 40.0f;
-    if (index_cost >= walk_cost || cand > 24.0f) return 0;
-    return (uint32_t)lim;
+    const float box = (float)(bb.z - bb.x) * (float)(bb.w - bb.y) * (1.0f / 4294967296.0f);
+    float best = walk_cost;
+    for (int l = kWalkKernelLevel; l < kIndexLevels && index_level_fits(l, K); ++l) {
+        const int shift = 16 - index_level_gbits(l);
+        const float cells = (float)((((bb.z - 1) >> shift) - (bb.x >> shift) + 1) *
+                                    (((bb.w - 1) >> shift) - (bb.y >> shift) + 1));
+        const float lim = fminf((float)index_level_points(l), 8.0f * walk + 256.0f);
+        if (lim * box > 24.0f) continue;  // (too many candidates)
+        const float cost = 40.0f + cells * (l == kIndexLevels - 1 ? 8.0f : 2.0f) + expf(-lim / walk) * walk_cost;
+        if (cost < best) {
+            best = cost;
+            plan.lim = (uint32_t)lim;
+            plan.level = l;
+        }
+    }
+    return plan;
 }
 
 // Level of the indexed form for a polygon's clipped box (sign_unified.cu): the finest

@@ -64,13 +64,13 @@ constexpr int kCand = 64;
 // repeated warp argmin, exact test, walk resumed at lim if none is inside.
 template <int U, class Inside>
 __device__ uint32_t sign_chunk_indexed(const Inside& inside, const StreamIndexView& S, int4 bb,
-                                       uint64_t seed, int k0, int kend, uint32_t T, uint32_t lim,
+                                       uint64_t seed, int k0, int kend, uint32_t T, WalkIndexPlan plan,
                                        uint2* cbuf /* [4][kCand] */, int* ccount /* [4] */,
                                        int lane, Work& work)
 {
     const uint32_t w = (uint32_t)(bb.z - bb.x), h = (uint32_t)(bb.w - bb.y);
-    const IndexLevelView& L = S.lv[kWalkKernelLevel];
-    lim = min(lim, T);
+    const IndexLevelView& L = S.lv[plan.level];
+    const uint32_t lim = min(plan.lim, T);
     const int cx0 = bb.x >> L.shift, cx1 = (bb.z - 1) >> L.shift;
     const int cy0 = bb.y >> L.shift, cy1 = (bb.w - 1) >> L.shift;
     const int ncx = cx1 - cx0 + 1, C = ncx * (cy1 - cy0 + 1);
@@ -151,7 +151,7 @@ __device__ uint32_t sign_chunk_indexed(const Inside& inside, const StreamIndexVi
     return mine;
 }
 
-// the hashes k0 .. k0+31 of one polygon; lane j returns hash k0 + j.  lim > 0
+// the hashes k0 .. k0+31 of one polygon; lane j returns hash k0 + j.  plan.lim > 0
 // selects the indexed form (stream points below lim read from the index).
 template <int U, class Inside>
 __device__ __forceinline__ uint32_t sign_chunk_walk(const Inside& inside, int4 bb, uint64_t seed,
@@ -170,10 +170,10 @@ __device__ __forceinline__ uint32_t sign_chunk_walk(const Inside& inside, int4 b
 template <int U, class Inside>
 __device__ __forceinline__ uint32_t sign_chunk(const Inside& inside, int4 bb, uint64_t seed, int k0,
                                                int kend, uint32_t T, int lane,
-                                               const StreamIndexView& S, uint32_t lim,
+                                               const StreamIndexView& S, WalkIndexPlan plan,
                                                uint2* cbuf, int* ccount, Work& work)
 {
-    if (lim) return sign_chunk_indexed<U>(inside, S, bb, seed, k0, kend, T, lim, cbuf, ccount, lane, work);
+    if (plan.lim) return sign_chunk_indexed<U>(inside, S, bb, seed, k0, kend, T, plan, cbuf, ccount, lane, work);
     return sign_chunk_walk<U>(inside, bb, seed, k0, kend, T, lane, work);
 }
 
@@ -218,7 +218,8 @@ sign_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
         const int n = (int)(off[p + 1] - b);
         const int4 bb = bbox[p];
         // (with the stream index every polygon is signed by sign_unified.cu instead)
-        const uint32_t lim = area2 && S.lv[0].first && n > kSmemVerts ? pmh_indexed_limit(bb, area2[p]) : 0;
+        const WalkIndexPlan plan = area2 && S.lv[0].first && n > kSmemVerts ? pmh_walk_index_plan(bb, area2[p], K)
+                                                                            : WalkIndexPlan{0u, 0};
         uint32_t mine;
         if (n <= kSmemVerts) {
             // stage the vertices (closed: v[n] = v[0]; cp.async 8-byte copies), the
@@ -245,9 +246,9 @@ sign_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
             const SlabInfo si = slabs[p];
             mine = sign_chunk<U>(SlabEdges{xy + b, n, slab_ptr + si.slab_base,
                                            slab_edges + si.edge_base, si.slab_h, si.ymin},
-                                 bb, seed, k0, kend, T, lane, S, lim, cbuf[wid], ccount[wid], work);
+                                 bb, seed, k0, kend, T, lane, S, plan, cbuf[wid], ccount[wid], work);
         } else {
-            mine = sign_chunk<U>(AllEdges{xy + b, n}, bb, seed, k0, kend, T, lane, S, lim,
+            mine = sign_chunk<U>(AllEdges{xy + b, n}, bb, seed, k0, kend, T, lane, S, plan,
                                  cbuf[wid], ccount[wid], work);
         }
         if (k0 + lane < kend) out[p * (int64_t)K + k0 + lane] = mine;

@@ -134,3 +134,20 @@ def test_few_hashes(orc, K, count):
     assert np.array_equal(g.hashes[:n].cpu().numpy().view(np.uint32).reshape(n, K), ref)
     g.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("K,f,T", [(40, (2e-5, 2.1e-5), 1 << 20), (40, (1e-4, 1e-3), 1 << 20), (33, (1e-3, 2e-1), 1 << 20),
+                                   (40, (1e-6, 3e-6), 1 << 17), (2050, (2e-4, 1e-3), 1 << 16)])
+def test_index_with_coverage_masks(orc, K, f, T):
+    """Rings above the staged size through the index and the masks: limits of every level that the form
+    reads (and, at K = 2,050, without the finest)."""
+    from paper_2511_16576_gb300 import binding as B
+    ctx = B.Context(0)
+    db = synth.star_polygons(60 if K < 2000 else 8, 21, n_range=(257, 1500), n_dist="loguniform", f_range=f)
+    P = B.make_params(K, 1, T, SEED, flags=B.FLAG_STREAM_INDEX | B.FLAG_COVERAGE_MASK)
+    polys = B.poly_upload(ctx, torch.from_numpy(db.xy).to(DEV), torch.from_numpy(db.offsets).to(DEV))
+    h = B.minhash_sign(ctx, polys, P).cpu().numpy().view(np.uint32)
+    assert np.array_equal(h, orc.sign(db.xy, db.offsets, SEED, K, T, nthreads=16))
+    if K < 2000 and 1e-5 < f[0] < 1e-3:  # (the others walk: larger ones by cost, smaller ones past the index)
+        assert B.sign_work(ctx)["walk_points"] < 0.2 * h.astype(np.int64).sum()
+    ctx.close()
