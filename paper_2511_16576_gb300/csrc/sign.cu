@@ -227,8 +227,11 @@ sign_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
             if (masks && lane < 16) smask[wid][lane] = masks[p * 16 + lane];
             stage_vertices(sv[wid], xy + b, n, lane);
             const int sh = staged_slab_shift(max(bb.w - bb.y, 1));
-            // (a ring of two edges a lane is tested whole: binning its edges costs more)
-            const bool staged = (masks || n > 64) && bb.w > bb.y && bb.z > bb.x &&
+            // (a ring of two edges a lane with short walks is tested whole: binning its edges costs
+            // more.  100,000 polygons of 8 to 64 vertices and 1e-2 to 5e-2 of the domain, K = 7: 371
+            // us binned, 316; 20,000 of 1e-4 to 1e-2, K = 96: 5.10 ms binned, 5.58)
+            const bool staged = (masks || n > 64 || !lazy_box((uint32_t)(bb.z - bb.x), (uint32_t)(bb.w - bb.y))) &&
+                                bb.w > bb.y && bb.z > bb.x &&
                                 build_staged_slabs(sv[wid], n, bb.y, sh, sid[wid], sbeg[wid], scnt[wid], lane);
             const int cwl = mask_cell_log2(bb.z - bb.x), chl = mask_cell_log2(bb.w - bb.y);
             if (staged) {

@@ -221,6 +221,11 @@ __device__ __forceinline__ bool build_staged_slabs(const int2* v, int n, int y0,
     return true;
 }
 
+// A clipped box of 1/128 of the domain or more: the hash is among the first 128 points more often
+// than not, and the generator is most of a round's work; under smaller boxes the short rounds
+// cost a few percent.
+__device__ __forceinline__ bool lazy_box(uint32_t w, uint32_t h) { return (uint64_t)w * h >= 1ull << (32 - 7); }
+
 template <int U, bool kLazy, class Inside, class W>
 __device__ __forceinline__ uint32_t sign_walk(const Inside& inside, int x0, int y0, uint32_t w,
                                               uint32_t h, uint64_t sk, uint32_t T, int lane,
@@ -247,9 +252,8 @@ struct Masked {
 };
 
 // One hash of one polygon; every lane returns the same value.  U points per
-// lane per round: one round covers 32 * U consecutive stream indices.  kLazy: the first
-// 128 points 32 at a time (a polygon of 1% of the domain or more has its hash among
-// them more often than not, and the generator is most of a round's work).
+// lane per round: one round covers 32 * U consecutive stream indices.  kLazy: under a large
+// box (lazy_box) the first 128 points 32 at a time.
 template <int U, bool kLazy = false, class Inside, class W>
 __device__ __forceinline__ uint32_t sign_one_t(const Inside& inside, int x0, int y0, uint32_t w,
                                                uint32_t h, uint64_t sk, uint32_t T, int lane,
@@ -268,7 +272,7 @@ __device__ __forceinline__ uint32_t sign_walk(const Inside& inside, int x0, int 
 {
     uint64_t z = sk + (uint64_t)(start + lane + 1) * PMH_GAMMA;
     const uint64_t step = 32ull * PMH_GAMMA;
-    if (kLazy) {
+    if (kLazy && lazy_box(w, h)) {
 #pragma unroll 1
         for (int j = 0; j < 4 && start < T; ++j, start += 32u, z += step) {
             const uint32_t pt = pmh_mix64_lo(z);
