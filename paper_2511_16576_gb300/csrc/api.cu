@@ -292,16 +292,18 @@ static int upload_fill(pmh_polys P, const int32_t* xy, const int64_t* offsets, b
     if (e != cudaSuccess) return pmh_set_error(PMH_ERR_CUDA, "upload copy failed: %s", cudaGetErrorString(e));
     // offsets[0] and offsets[n] are checked by the kernel through b/e bounds
     int64_t* sizes = nullptr;
+    SlabInfo* info = P->slab_info;
     if (n_polys > 0) {
-        if (!P->slab_info && cudaMalloc(&P->slab_info, sizeof(SlabInfo) * n_polys) != cudaSuccess) {
-            cudaGetLastError();
-            return pmh_set_error(PMH_ERR_NOMEM, "slab info allocation failed");
-        }
-        PMH_TRY(pmh_scratch(ctx, SCR_MISC, sizeof(int64_t) * (size_t)(2 * (n_polys + 1)), (void**)&sizes));
+        // (a set without a ring that gets a slab index keeps no info: its sizes go to scratch.
+        // 100,000 polygons: 671 us with an array of its own, 384)
+        const size_t size_bytes = sizeof(int64_t) * (size_t)(2 * (n_polys + 1));
+        PMH_TRY(pmh_scratch(ctx, SCR_MISC, size_bytes + (info ? 0 : sizeof(SlabInfo) * (size_t)n_polys),
+                            (void**)&sizes));
         int64_t* edge = sizes + n_polys + 1;
+        if (!info) info = reinterpret_cast<SlabInfo*>(edge + n_polys + 1);
         PMH_TRY(pmh_launch_prep(ctx->sm_count, fused ? reinterpret_cast<const int2*>(xy) : P->xy,
                                 fused ? P->xy : nullptr, P->offsets, n_polys, nullptr, n_vertices, P->bbox,
-                                P->area2, SlabSizes{P->slab_info, sizes, edge}, ctx->d_status, s));
+                                P->area2, SlabSizes{info, sizes, edge}, ctx->d_status, s));
         PMH_TRY(pmh_exclusive_scan_i64(ctx, sizes, sizes, n_polys, s, nullptr, 2));  // sizes, edge
         e = cudaMemcpyAsync(ctx->h_pinned + 1, sizes + n_polys, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess)
@@ -325,7 +327,7 @@ static int upload_fill(pmh_polys P, const int32_t* xy, const int64_t* offsets, b
         if ((e = cudaGetLastError()) != cudaSuccess)
             return pmh_set_error(PMH_ERR_CUDA, "feature kernel: %s", cudaGetErrorString(e));
     }
-    PMH_TRY(pmh_build_slabs(P, sizes, sizes + n_polys + 1, n_ptr, n_edges, s));
+    PMH_TRY(pmh_build_slabs(P, info, sizes, sizes + n_polys + 1, n_ptr, n_edges, s));
     return pmh_build_class_order(P, s);
 }
 
@@ -357,7 +359,7 @@ static int upload_common(pmh_ctx ctx, const int32_t* xy, const int64_t* offsets,
     const size_t np = (size_t)(n_polys > 0 ? n_polys : 1);
     if (cudaMalloc(&P->xy, sizeof(int2) * (size_t)(n_vertices > 0 ? n_vertices : 1)) != cudaSuccess ||
         cudaMalloc(&P->offsets, sizeof(int64_t) * (size_t)(n_polys + 1)) != cudaSuccess ||
-        cudaMalloc(&P->bbox, sizeof(int4) * np) != cudaSuccess ||
+        cudaMalloc(&P->bbox, sizeof(int4) * np + sizeof(SlabPtrs)) != cudaSuccess ||
         cudaMalloc(&P->area2, sizeof(int64_t) * np) != cudaSuccess ||
         cudaMalloc(&P->feat, sizeof(float2) * np) != cudaSuccess) {
         cudaGetLastError();
@@ -365,6 +367,7 @@ static int upload_common(pmh_ctx ctx, const int32_t* xy, const int64_t* offsets,
         return pmh_set_error(PMH_ERR_NOMEM, "polygon allocation failed (%lld vertices)",
                              (long long)n_vertices);
     }
+    if (n_polys > 0) P->d_slabs = reinterpret_cast<SlabPtrs*>(P->bbox + n_polys);
     const int rc = upload_fill(P, xy, offsets, host, (cudaStream_t)stream);
     if (rc != PMH_OK) {
         pmh_polys_destroy(P);
@@ -459,7 +462,7 @@ extern "C" int pmh_polys_destroy(pmh_polys p)
     cudaSetDevice(p->device);
     if (p->xy || p->offsets || p->bbox || p->area2) cudaDeviceSynchronize();
     void* bufs[] = {p->xy, p->offsets, p->bbox, p->area2, p->feat, p->slab_info, p->slab_ptr,
-                    p->slab_edges, p->d_slabs, p->order, p->order_cls, p->mask};
+                    p->slab_edges, p->order, p->order_cls, p->mask};
     for (void* b : bufs)
         if (b) cudaFree(b);
     delete p;

@@ -54,8 +54,8 @@ __device__ __forceinline__ void for_slab_entries(const int2* __restrict__ xy, in
 }
 
 __global__ void __launch_bounds__(kFillThreads, 8) slab_fill_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
-                                 int64_t n_polys, const int64_t* __restrict__ d_n, SlabInfo* __restrict__ info,
-                                 const int64_t* __restrict__ ptr_base, const int64_t* __restrict__ edge_base,
+                                 int64_t n_polys, const int64_t* __restrict__ d_n, const SlabInfo* sized,
+                                 SlabInfo* info, const int64_t* __restrict__ ptr_base, const int64_t* __restrict__ edge_base,
                                  int32_t* slab_ptr, int64_t cap_ptr, int32_t* __restrict__ slab_edges,
                                  int64_t cap_edges)
 {
@@ -65,22 +65,26 @@ __global__ void __launch_bounds__(kFillThreads, 8) slab_fill_kernel(const int2* 
     if (d_n) n_polys = min(n_polys, *d_n);
     for (int64_t p = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); p < n_polys;
          p += nwarps) {
-        const SlabInfo si = info[p];
+        SlabInfo si = sized[p];
         const int S = si.S, y0 = si.ymin;
-        if (S <= 0) continue;
+        if (S <= 0) {
+            if (lane == 0 && sized != info) info[p] = si;
+            continue;
+        }
         const int64_t b = off[p];
         const int n = (int)(off[p + 1] - b);
         const uint64_t hm = slab_div_magic(si.slab_h);
         const int64_t pb = ptr_base[p], eb = edge_base[p];
         if (ptr_base[p + 1] > cap_ptr || edge_base[p + 1] > cap_edges) {
             // the lists do not fit the fixed buffers: this polygon is tested over all its edges
-            if (lane == 0) info[p].S = 0;
+            si.S = 0;
+            if (lane == 0) info[p] = si;
             continue;
         }
-        if (lane == 0) {
-            info[p].slab_base = pb;
-            info[p].edge_base = eb;
-        }
+        si.slab_base = pb;
+        si.edge_base = eb;
+        __syncwarp();  // (sized may be info: every lane has read its entry)
+        if (lane == 0) info[p] = si;
         int32_t* sp = slab_ptr + pb;
         int32_t* le = slab_edges + eb;
         const bool small = S <= kFillSmemSlabs;
@@ -219,25 +223,28 @@ static int grow_list(int32_t** buf, int64_t* cap, int64_t need)
     return PMH_OK;
 }
 
-int pmh_build_slabs(pmh_polys P, const int64_t* ptr_base, const int64_t* edge_base, int64_t n_ptr,
-                    int64_t n_edges, cudaStream_t s)
+int pmh_build_slabs(pmh_polys P, const SlabInfo* sized, const int64_t* ptr_base, const int64_t* edge_base,
+                    int64_t n_ptr, int64_t n_edges, cudaStream_t s)
 {
     if (P->n == 0) return PMH_OK;
     if (n_ptr > 0) {
+        if (!P->slab_info && cudaMalloc(&P->slab_info, sizeof(SlabInfo) * P->n) != cudaSuccess) {
+            cudaGetLastError();
+            P->slab_info = nullptr;
+            return pmh_set_error(PMH_ERR_NOMEM, "slab info allocation failed");
+        }
         PMH_TRY(grow_list(&P->slab_ptr, &P->cap_slab_ptr, n_ptr));
         PMH_TRY(grow_list(&P->slab_edges, &P->cap_slab_edges, n_edges));
         const int blocks = (int)std::min<int64_t>((P->n + 7) / 8, (int64_t)P->ctx->sm_count * 32);
-        slab_fill_kernel<<<blocks, kFillThreads, 0, s>>>(P->xy, P->offsets, P->n, nullptr, P->slab_info,
+        slab_fill_kernel<<<blocks, kFillThreads, 0, s>>>(P->xy, P->offsets, P->n, nullptr, sized, P->slab_info,
                                                          ptr_base, edge_base, P->slab_ptr, P->cap_slab_ptr,
                                                          P->slab_edges, P->cap_slab_edges);
         PMH_LAUNCHED("slab_fill_kernel");
     }
-    if (!P->d_slabs && cudaMalloc(&P->d_slabs, sizeof(SlabPtrs)) != cudaSuccess) {
-        cudaGetLastError();
-        return pmh_set_error(PMH_ERR_NOMEM, "slab pointer allocation failed");
-    }
-    const SlabPtrs v{P->slab_info, P->slab_ptr, P->slab_edges};
-    PMH_CUDA_TRY(cudaMemcpyAsync(P->d_slabs, &v, sizeof(v), cudaMemcpyHostToDevice, s));
+    // (from pinned memory, which the upload's last synchronisation frees)
+    SlabPtrs* v = reinterpret_cast<SlabPtrs*>(P->ctx->h_pinned + 8);
+    *v = SlabPtrs{P->slab_info, P->slab_ptr, P->slab_edges};
+    PMH_CUDA_TRY(cudaMemcpyAsync(P->d_slabs, v, sizeof(*v), cudaMemcpyHostToDevice, s));
     return PMH_OK;
 }
 
@@ -313,7 +320,7 @@ int pmh_launch_slabs_fixed(pmh_ctx ctx, const int2* xy, const int64_t* off, int6
     int64_t* edge_sizes = sizes + (max_polys + 1);
     PMH_TRY(pmh_exclusive_scan_i64(ctx, sizes, sizes, max_polys, s, sums, 2));
     const int blocks = (int)std::min<int64_t>((max_polys + 7) / 8, (int64_t)ctx->sm_count * 16);
-    slab_fill_kernel<<<blocks, kFillThreads, 0, s>>>(xy, off, max_polys, d_n, info, ptr_sizes, edge_sizes,
+    slab_fill_kernel<<<blocks, kFillThreads, 0, s>>>(xy, off, max_polys, d_n, info, info, ptr_sizes, edge_sizes,
                                                      slab_ptr, cap_ptr, slab_edges, cap_edges);
     PMH_LAUNCHED("slab_fill_kernel");
     return PMH_OK;

@@ -146,3 +146,20 @@ def test_graph_on_a_set_reloaded_with_large_rings(B):
     assert launches[0][0] == launches[2][0] == launches[1][0] - 1 == launches[3][0] - 1
     g.close()
     ctx.close()
+
+
+def test_first_slab_index_by_a_reload(B, orc):
+    """A set uploaded without a ring of the slab index's size, reloaded with some, and without again."""
+    sizes = [[200, 250, 150, 200], [500, 100, 80, 120], [200, 250, 150, 200]]
+    ctx = B.Context(0)
+    polys = None
+    for k, s in enumerate(sizes):
+        xy = np.concatenate([_star(n, 9000 + 12000 * i, 30000, 8000, 10 * k + i) for i, n in enumerate(s)])
+        off = np.concatenate([[0], np.cumsum(s)]).astype(np.int64)
+        arrays = torch.from_numpy(xy).to(DEV), torch.from_numpy(off).to(DEV)
+        if polys is None:
+            polys = B.poly_upload(ctx, *arrays)
+        else:
+            B.poly_reload(polys, *arrays)
+        _check(B, ctx, orc, polys, xy, off)
+    ctx.close()
