@@ -84,79 +84,58 @@ __global__ void cell_record_kernel(const int64_t* __restrict__ starts, int K, in
 
 }  // namespace
 
+// what the building of a level works on, sized for the largest: the levels share it, and the build
+// synchronises once at its end
+struct LevelScratch {
+    uint32_t* keys = nullptr;
+    int32_t* vals = nullptr;
+    int64_t* counts = nullptr;
+    int alloc(int64_t points, int64_t cells)
+    {
+        if (cudaMalloc(&keys, sizeof(uint32_t) * points) == cudaSuccess &&
+            cudaMalloc(&vals, sizeof(int32_t) * points) == cudaSuccess &&
+            cudaMalloc(&counts, sizeof(int64_t) * (cells + 1)) == cudaSuccess)
+            return PMH_OK;
+        cudaGetLastError();
+        return pmh_set_error(PMH_ERR_NOMEM, "stream index scratch allocation failed");
+    }
+    void release()
+    {
+        cudaFree(keys);
+        cudaFree(vals);
+        cudaFree(counts);
+    }
+};
+
 // One level: the first M points of every hash's stream on a 2^gbits-square grid.
-// Allocates *first, *beg and *ent; on failure frees what it allocated.
+// Allocates the level's tables (which the caller frees, also after a failure).
 static int build_level(pmh_ctx ctx, const pmh_params* P, cudaStream_t s, int M, int gbits,
-                       uint32_t** first_out, uint32_t** beg_out, uint2** ent_out)
+                       const LevelScratch& w, uint32_t** first, uint32_t** beg, uint2** ent)
 {
     const int shift = 16 - gbits;
     const int64_t n = (int64_t)P->K * M;
     const int64_t n_cells = (int64_t)P->K << (2 * gbits);
     const int64_t rows = 1ll << (2 * gbits), pitch = index_pitch((int)P->K);
-    uint32_t *first = nullptr, *beg = nullptr;
-    uint2* ent = nullptr;
-    if (cudaMalloc(&first, sizeof(uint32_t) * rows * pitch) != cudaSuccess ||
-        cudaMalloc(&beg, sizeof(uint32_t) * (rows + 1) * pitch) != cudaSuccess ||
-        cudaMalloc(&ent, sizeof(uint2) * n) != cudaSuccess) {
+    if (cudaMalloc(first, sizeof(uint32_t) * rows * pitch) != cudaSuccess ||
+        cudaMalloc(beg, sizeof(uint32_t) * (rows + 1) * pitch) != cudaSuccess ||
+        cudaMalloc(ent, sizeof(uint2) * n) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(first);
-        cudaFree(beg);
-        cudaFree(ent);
         return pmh_set_error(PMH_ERR_NOMEM, "stream index allocation failed");
     }
-    uint32_t* keys = nullptr;
-    int32_t* vals = nullptr;
-    int64_t* counts = nullptr;
-    if (cudaMalloc(&keys, sizeof(uint32_t) * n) != cudaSuccess ||
-        cudaMalloc(&vals, sizeof(int32_t) * n) != cudaSuccess ||
-        cudaMalloc(&counts, sizeof(int64_t) * (n_cells + 1)) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(keys);
-        cudaFree(vals);
-        cudaFree(first);
-        cudaFree(beg);
-        cudaFree(ent);
-        return pmh_set_error(PMH_ERR_NOMEM, "stream index scratch allocation failed");
-    }
-    int rc = PMH_OK;
     const int blocks = ctx->sm_count * 16;
-    stream_points_kernel<<<blocks, 256, 0, s>>>(P->seed, (int)P->K, M, shift, gbits, keys, vals);
-    g_pmh_launches.fetch_add(1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) rc = pmh_set_error(PMH_ERR_CUDA, "stream points: %s", cudaGetErrorString(e));
+    stream_points_kernel<<<blocks, 256, 0, s>>>(P->seed, (int)P->K, M, shift, gbits, w.keys, w.vals);
+    PMH_LAUNCHED("stream_points_kernel");
     int key_bits = 2 * gbits;
-    while ((1ll << key_bits) < (int64_t)P->K << (2 * gbits)) ++key_bits;
-    if (rc == PMH_OK) rc = pmh_radix_sort_u32(ctx, keys, vals, n, key_bits, s);
-    if (rc == PMH_OK && cudaMemsetAsync(counts, 0, sizeof(int64_t) * (n_cells + 1), s) != cudaSuccess)
-        rc = pmh_set_error(PMH_ERR_CUDA, "memset failed");
-    if (rc == PMH_OK) {
-        cell_count_kernel<<<blocks, 256, 0, s>>>(keys, n, counts);
-        g_pmh_launches.fetch_add(1);
-        rc = pmh_exclusive_scan_i64(ctx, counts, counts, n_cells, s);
-    }
-    if (rc == PMH_OK) {
-        finish_index_kernel<<<blocks, 256, 0, s>>>(keys, vals, n, P->seed, gbits, ent);
-        g_pmh_launches.fetch_add(1);
-        cell_record_kernel<<<blocks, 256, 0, s>>>(counts, (int)P->K, gbits, ent, beg, first);
-        g_pmh_launches.fetch_add(1);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) rc = pmh_set_error(PMH_ERR_CUDA, "finish: %s", cudaGetErrorString(e));
-    }
-    cudaError_t e2 = cudaStreamSynchronize(s);
-    cudaFree(keys);
-    cudaFree(vals);
-    cudaFree(counts);
-    if (rc == PMH_OK && e2 != cudaSuccess)
-        rc = pmh_set_error(PMH_ERR_CUDA, "stream index build: %s", cudaGetErrorString(e2));
-    if (rc != PMH_OK) {
-        cudaFree(first);
-        cudaFree(beg);
-        cudaFree(ent);
-        return rc;
-    }
-    *first_out = first;
-    *beg_out = beg;
-    *ent_out = ent;
+    while ((1ll << key_bits) < n_cells) ++key_bits;
+    PMH_TRY(pmh_radix_sort_u32(ctx, w.keys, w.vals, n, key_bits, s));
+    PMH_CUDA_TRY(cudaMemsetAsync(w.counts, 0, sizeof(int64_t) * (n_cells + 1), s));
+    cell_count_kernel<<<blocks, 256, 0, s>>>(w.keys, n, w.counts);
+    PMH_LAUNCHED("cell_count_kernel");
+    PMH_TRY(pmh_exclusive_scan_i64(ctx, w.counts, w.counts, n_cells, s));
+    finish_index_kernel<<<blocks, 256, 0, s>>>(w.keys, w.vals, n, P->seed, gbits, *ent);
+    PMH_LAUNCHED("finish_index_kernel");
+    cell_record_kernel<<<blocks, 256, 0, s>>>(w.counts, (int)P->K, gbits, *ent, *beg, *first);
+    PMH_LAUNCHED("cell_record_kernel");
     return PMH_OK;
 }
 
@@ -193,11 +172,23 @@ int pmh_stream_index_get(pmh_ctx ctx, const pmh_params* P, cudaStream_t s, Strea
         free_index(si);
     }
     StreamIndex fresh;
-    int rc = PMH_OK;
+    LevelScratch scratch;
+    const int K = (int)P->K;
+    int64_t points = 0, cells = 0;  // (the finest level that fits; all but the finest always do: K <= 4096)
+    for (int l = 0; l < kIndexLevels; ++l)
+        if (index_level_fits(l, K)) {
+            points = std::max(points, (int64_t)K * index_level_points(l));
+            cells = std::max(cells, (int64_t)K << (2 * index_level_gbits(l)));
+        }
+    int rc = scratch.alloc(points, cells);
     for (int l = 0; l < kIndexLevels && rc == PMH_OK; ++l)
-        if (index_level_fits(l, (int)P->K))  // (all but the finest always do: K <= 4096)
-            rc = build_level(ctx, P, s, index_level_points(l), index_level_gbits(l), &fresh.first[l],
+        if (index_level_fits(l, K))
+            rc = build_level(ctx, P, s, index_level_points(l), index_level_gbits(l), scratch, &fresh.first[l],
                              &fresh.beg[l], &fresh.ent[l]);
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (rc == PMH_OK && e != cudaSuccess)
+        rc = pmh_set_error(PMH_ERR_CUDA, "stream index build: %s", cudaGetErrorString(e));
+    scratch.release();
     if (rc != PMH_OK) {
         free_index(fresh);
         return rc;
