@@ -1,5 +1,7 @@
 """Bucket joins (A4) on synthetic hashes against the bucket definition (the oracle): the one-hashmap
 range join's segments and the joins' edges of tile, row and batch sizes."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -221,3 +223,106 @@ def test_staging_memory(B, orc):
             g[0].close()
         index.close()
         c.close()
+
+
+def rows_of(B, ctx, orc, ph, qh, bands, pick):
+    """lsh_query of all queries, without and with a capacity; the picked rows against the oracle."""
+    K = ph.shape[1]
+    index = B.lsh_build(ctx, on_device(ph), B.make_params(K, bands))
+    rp_ref, cand_ref = orc.candidates(np.ascontiguousarray(qh[pick]), ph, bands, K // bands, T)
+    q, lengths = on_device(qh), None
+    for capacity in (None, "total"):
+        if capacity:
+            capacity = int(rp[-1])
+        row_ptr, cand = B.lsh_query(ctx, index, q, capacity=capacity)
+        rp, cd = row_ptr.cpu().numpy(), cand.cpu().numpy()
+        for i, p in enumerate(pick):
+            assert np.array_equal(cd[rp[p]:rp[p + 1]], cand_ref[rp_ref[i]:rp_ref[i + 1]]), p
+        assert lengths is None or np.array_equal(lengths, np.diff(rp))
+        lengths = np.diff(rp)
+    index.close()
+    return lengths
+
+
+@pytest.mark.parametrize("K,bands,n", [(8, 4, 409_601), (2, 2, 852_100), (4, 2, 1 << 20), (4, 2, (1 << 20) + 1),
+                                       (32, 16, 1 << 20), (32, 16, (1 << 20) + 1), (16, 4, 409_600),
+                                       (16, 4, 409_601)])
+@pytest.mark.parametrize("Q", [5, 200, 800])
+def test_largest_bitmaps(B, ctx, orc, K, bands, n, Q):
+    """Tuples of one or two hashes up to 2^20 ids, longer ones up to 409,600, and the sets just above (merge
+    and open-addressing set); batches that leave SMs a query, give them 512 threads, and reuse their
+    bitmap for another row."""
+    rng = np.random.default_rng(n + K)
+    ph, qh = hashes(rng, n, K, 400 if K // bands <= 2 else 7), hashes(rng, Q, K, 400 if K // bands <= 2 else 7)
+    qh[0] = T
+    qh[1::3] = ph[rng.integers(0, n, len(qh[1::3]))]
+    ph[[0, n - 1, n - 2, n // 2]] = qh[2]  # the first and last bits
+    pick = np.unique(np.concatenate([np.arange(3), rng.integers(0, Q, 4), [Q - 1]]))
+    lengths = rows_of(B, ctx, orc, ph, qh, bands, pick)
+    assert lengths[0] == 0 and lengths[2] >= 4
+
+
+@pytest.mark.parametrize("n", [409_600, 700_000])
+def test_bitmaps_with_threads_by_fit(B, ctx, orc, n):
+    """More queries than two per SM: the block's size follows from how many bitmaps fit an SM."""
+    rng = np.random.default_rng(n)
+    Q = 1200
+    ph, qh = hashes(rng, n, 8, 300), hashes(rng, Q, 8, 300)
+    assert rows_of(B, ctx, orc, ph, qh, 4, rng.choice(Q, 8, replace=False)).sum() > 0
+
+
+def test_set_join_long_rows(B, ctx, orc):
+    """Rows around the small set's 4,096 and the large set's 16,384 distinct ids, beyond them (id-range
+    passes) and past the staging pool, on a set above the bitmap's limit."""
+    rng = np.random.default_rng(9)
+    n, K, bands = 420_000, 48, 16
+    ph = rng.integers(1000, 1 << 20, (n, K)).astype(np.uint32)
+    sizes = [1, 127, 128, 129, 4095, 4096, 4097, 16_383, 16_384, 16_385, 32_768, 40_000, 200_000]
+    qh = rng.integers(1 << 21, 1 << 22, (len(sizes) + 1, K)).astype(np.uint32)
+    for i, size in enumerate(sizes):  # each id in one or two of the query's bands
+        ids = rng.choice(n, size, replace=False)
+        for b in range(2):
+            part = ids if b == 0 else ids[::3]
+            j = (3 * i + b) % bands
+            ph[part, 3 * j:3 * j + 3] = qh[i, 3 * j:3 * j + 3]
+    lengths = rows_of(B, ctx, orc, ph, qh, bands, np.arange(len(qh)))
+    assert lengths[-1] == 0 and lengths[4] <= 4096 < lengths[10] and lengths.max() > 100_000
+    # past the pool: 4,096 ids per query of a batch of long rows
+    many = np.repeat(qh[7:10], 3, axis=0)
+    rows_of(B, ctx, orc, ph, many, bands, np.arange(len(many)))
+
+
+@pytest.mark.parametrize("n", [30_000, 409_601])
+def test_count_then_fill_without_a_capacity(B, ctx, orc, n):
+    """The documented two calls: a count with capacity 0 (nothing staged; the warp join leaves rows to the
+    next join), then the fill, or a second whole call."""
+    rng = np.random.default_rng(n)
+    K, bands, Q = 96, 16, 1100
+    ph, qh = hashes(rng, n, K, 1000), hashes(rng, Q, K, 1000)
+    qh[:400:2] = ph[rng.integers(0, n, 200)]
+    for q, copies in ((1, 8), (3, 9), (5, 300)):  # 128, 144 and 4,800 entries of one row
+        qh[q] = 10_000 + q
+        ph[rng.choice(n, copies, replace=False)] = qh[q]
+    pick = np.concatenate([np.arange(8), rng.choice(Q, 12, replace=False)])
+    rp_ref, cand_ref = orc.candidates(np.ascontiguousarray(qh[pick]), ph, bands, K // bands, T)
+    index = B.lsh_build(ctx, on_device(ph), B.make_params(K, bands))
+    q = on_device(qh)
+    lib = B.load()
+    row_ptr = torch.empty(Q + 1, dtype=torch.int64, device=DEV)
+    total = ctypes.c_int64()
+    call = lambda cand, cap: lib.pmh_lsh_query(ctx.handle, index.handle, q.data_ptr(), Q, row_ptr.data_ptr(), cand, cap,
+                                               ctypes.byref(total), torch.cuda.current_stream().cuda_stream)
+    assert call(None, 0) == B.PMH_ERR_CAPACITY and total.value > 0
+    rp = row_ptr.cpu().numpy()
+    assert rp[-1] == total.value
+    for again in (False, True):
+        cand = torch.full((total.value,), -1, dtype=torch.int32, device=DEV)
+        if again:
+            assert call(cand.data_ptr(), total.value) == 0
+        else:
+            B._check(lib.pmh_lsh_query_fill(ctx.handle, index.handle, q.data_ptr(), Q, row_ptr.data_ptr(),
+                                            cand.data_ptr(), total.value, torch.cuda.current_stream().cuda_stream))
+        cd = cand.cpu().numpy()
+        for i, p in enumerate(pick):
+            assert np.array_equal(cd[rp[p]:rp[p + 1]], cand_ref[rp_ref[i]:rp_ref[i + 1]]), p
+    index.close()
