@@ -431,7 +431,9 @@ def lsh_query(ctx: Context, index: Index, qhashes: torch.Tensor, capacity: int |
     if capacity is None and total.value < cap // 2 and (stream is None or isinstance(stream, torch.cuda.Stream)):
         # do not hold the whole buffer for a short result
         short = torch.empty(max(total.value, 1), dtype=torch.int32, device=dev)
-        if stream is None:
+        if total.value == 0:
+            pass
+        elif stream is None:
             short.copy_(cand[:short.numel()])
         else:
             with torch.cuda.stream(stream):

@@ -564,34 +564,40 @@ join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int bands, i
     }
 }
 
-// fill pass of the staged rows: a block per row copies its pool slice into place
-// (four independent loads per thread in flight)
+// fill pass of the staged rows: a block per row copies its pool slice into place, or, of rows of
+// fewer than kCopyWarpRow ids on average, a warp (four independent loads per thread in
+// flight; rows of a candidate or none leave a block waiting on their three loads)
+constexpr int kCopyWarpRow = 256;
 __global__ void __launch_bounds__(256)
 copy_rows_kernel(JoinStage st, int64_t Q, const int64_t* __restrict__ row_ptr, int32_t* __restrict__ cand,
                  int64_t cap, const int64_t* __restrict__ d_n, int* __restrict__ d_flags)
 {
     if (d_flags && (*d_flags & 7)) return;
-    if (row_ptr[Q] > cap) {
+    const int64_t total = row_ptr[Q];
+    if (total > cap) {
         if (blockIdx.x == 0 && threadIdx.x == 0 && d_flags) atomicOr(d_flags, 8);
         return;
     }
     const int64_t live = d_n ? min(Q, *d_n) : Q;
-    for (int64_t q = blockIdx.x; q < live; q += gridDim.x) {
+    const bool warps = total < live * kCopyWarpRow;
+    const int per = warps ? 32 : (int)blockDim.x, t = (int)threadIdx.x & (per - 1);
+    const int groups = (int)blockDim.x / per;  // rows a block takes at a time
+    for (int64_t q = (int64_t)blockIdx.x * groups + threadIdx.x / per; q < live; q += (int64_t)gridDim.x * groups) {
         const int64_t off = st.where[q];
         if (off < 0) continue;
         const int64_t b = row_ptr[q], len = row_ptr[q + 1] - b;
         const int32_t* src = st.pool + off;
         int32_t* dst = cand + b;
-        for (int64_t i = threadIdx.x; i < len; i += 4 * blockDim.x) {
+        for (int64_t i = t; i < len; i += 4 * per) {
             int32_t v[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int64_t k = i + (int64_t)u * blockDim.x;
+                const int64_t k = i + (int64_t)u * per;
                 v[u] = k < len ? src[k] : 0;
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int64_t k = i + (int64_t)u * blockDim.x;
+                const int64_t k = i + (int64_t)u * per;
                 if (k < len) dst[k] = v[u];
             }
         }
@@ -776,21 +782,24 @@ constexpr int64_t kBitmapMaxIds = 409600;
 constexpr int64_t kBitmapMaxIdsShort = 1 << 20;
 constexpr int kBitmapU = 4;
 
-template <bool kWrite>
-__global__ void __launch_bounds__(1024)
+// kScan: some rows are done already (the warp join's, or staged), so a block looks at as many
+// of its rows at once as it has threads.
+template <bool kWrite, bool kScan>
+__global__ void __launch_bounds__(1024, 2)
 bitmap_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int bands, int rows, uint32_t T,
                    uint64_t lsh_seed, int band_bits, const uint32_t* __restrict__ comp,
                    const int32_t* __restrict__ ids, const uint32_t* __restrict__ dbh,
                    const int64_t* __restrict__ dir, int dsh, int words4 /* 128-id vectors */,
                    int64_t* __restrict__ counts, const int64_t* __restrict__ row_ptr,
-                   int32_t* __restrict__ cand, int64_t cap, JoinStage st, bool deferred,
-                   const int64_t* __restrict__ d_n, int* __restrict__ d_flags)
+                   int32_t* __restrict__ cand, int64_t cap, JoinStage st, const int64_t* __restrict__ d_n,
+                   int* __restrict__ d_flags)
 {
     extern __shared__ uint4 bits[];
     // (32 bits: at most 2^20 ids under 128 bands)
     __shared__ int blo[kMaxBandsPerLane * 32], boff[kMaxBandsPerLane * 32 + 1];
     __shared__ uint32_t bcomp[kMaxBandsPerLane * 32];
     __shared__ int wsum[32];
+    __shared__ unsigned rows_left[kScan ? 32 : 1];  // of the rows looked at together, a bit each: to be joined here
     __shared__ long long stage_off;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const bool failed = d_flags && (*d_flags & 7);
@@ -802,16 +811,50 @@ bitmap_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int b
     // (16-byte tuple loads: the index's rows are aligned when K % 4 == 0, the caller's may not be)
     const bool vec = (K & 3) == 0 && (reinterpret_cast<uintptr_t>(qhashes) & 15) == 0;
     uint32_t* word = reinterpret_cast<uint32_t*>(bits);
-    for (int64_t q = blockIdx.x; q < Q; q += gridDim.x) {
-        if (failed || (d_n && q >= *d_n)) {
-            if (!kWrite && threadIdx.x == 0) {
-                counts[q] = 0;
-                if (st.where) st.where[q] = -1;
+    auto done = [&](int64_t q) { return kScan && (kWrite ? st.where[q] >= 0 : counts[q] >= 0); };
+    auto absent = [&](int64_t q) { return failed || (d_n && q >= *d_n); };
+    auto empty_row = [&](int64_t q) {
+        if (kWrite) return;
+        counts[q] = 0;
+        if (st.where) st.where[q] = -1;
+    };
+    int64_t q = blockIdx.x, c0 = q;  // c0: first of the rows looked at together
+    for (int next = 0;; kScan ? (void)++next : (void)(q += gridDim.x)) {
+        if (!kScan) {
+            if (q >= Q) break;
+            if (absent(q)) {
+                if (threadIdx.x == 0) empty_row(q);
+                continue;
             }
-            continue;
+        } else {
+            if (c0 >= Q) break;
+            if (next == 0) {
+                const int64_t mine = c0 + (int64_t)threadIdx.x * gridDim.x;
+                bool todo = false;
+                if (mine < Q) {
+                    if (absent(mine)) empty_row(mine);
+                    else todo = !done(mine);
+                }
+                const unsigned bal = __ballot_sync(0xffffffffu, todo);
+                if (lane == 0) rows_left[wid] = bal;
+                __syncthreads();
+            }
+            while (next < (int)blockDim.x) {  // (the same for every thread)
+                const unsigned w = rows_left[next >> 5] >> (next & 31);
+                if (w) {
+                    next += __ffs(w) - 1;
+                    break;
+                }
+                next = (next | 31) + 1;
+            }
+            if (next >= (int)blockDim.x) {
+                __syncthreads();  // rows_left is free
+                c0 += (int64_t)blockDim.x * gridDim.x;
+                next = -1;
+                continue;
+            }
+            q = c0 + (int64_t)next * gridDim.x;
         }
-        if (kWrite && st.where && st.where[q] >= 0) continue;  // staged, or the warp join's
-        if (!kWrite && deferred && counts[q] >= 0) continue;   // the warp join's
         const uint32_t* qh = qhashes + q * K;
         // the bands' directory slots, the bitmap cleared meanwhile
         for (int j = threadIdx.x; j < bands; j += blockDim.x) {
@@ -1218,7 +1261,7 @@ static JoinStage stage_view(void* buf, int64_t Q, int64_t pool_ints)
 // 37 KB bitmaps an SM: 331 us with 256 threads, 218 with 512; 32 x 4 bands, 400,000: 122 and 99)
 static int launch_bitmap(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* d_n, int64_t* counts,
                          const int64_t* row_ptr, int32_t* cand, int64_t cap, const JoinStage& st,
-                         bool deferred, int* d_flags, bool write, cudaStream_t s)
+                         bool scan, int* d_flags, bool write, cudaStream_t s)
 {
     const pmh_params& P = X->params;
     const int words4 = (int)((X->n + 127) / 128);
@@ -1227,7 +1270,9 @@ static int launch_bitmap(pmh_index X, const uint32_t* qh, int64_t Q, const int64
     // of 64 x 2 bands, 200,000 polygons: 33 us with 256 threads, 17 with 1,024)
     const int64_t sms = X->ctx->sm_count, fit = (225 * 1024) / ((int64_t)smem + 2048);
     const int threads = fit < 4 || Q <= sms ? 1024 : fit < 8 || Q <= 2 * sms ? 512 : 256;
-    auto fn = write ? bitmap_join_kernel<true> : bitmap_join_kernel<false>;
+    // (scan: some rows are done, marked in st.where or by their count)
+    auto fn = write ? (scan ? bitmap_join_kernel<true, true> : bitmap_join_kernel<true, false>)
+                    : (scan ? bitmap_join_kernel<false, true> : bitmap_join_kernel<false, false>);
     // (the largest bitmap's, not this one's: the attribute is the process's, and a host thread with a
     // small index must not take it from another between its set and its launch)
     PMH_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1237,7 +1282,7 @@ static int launch_bitmap(pmh_index X, const uint32_t* qh, int64_t Q, const int64
     const unsigned blocks = (unsigned)std::min<int64_t>(Q, (int64_t)X->ctx->sm_count * std::max(per_sm, 1));
     fn<<<blocks, threads, smem, s>>>(qh, Q, (int)P.K, (int)P.bands, (int)P.rows, P.T, P.lsh_seed, X->band_bits,
                                      X->sorted_comp, X->sorted_id, X->hashes, X->dir, X->dir_shift, words4,
-                                     counts, row_ptr, cand, cap, st, deferred, d_n, d_flags);
+                                     counts, row_ptr, cand, cap, st, d_n, d_flags);
     PMH_LAUNCHED(write ? "bitmap_join_kernel<fill>" : "bitmap_join_kernel<count>");
     return PMH_OK;
 }
@@ -1265,12 +1310,13 @@ int pmh_launch_query(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* 
         return PMH_OK;
     }
     const JoinStage st = stage_view(stage, Q, pool_ints);
-    // the warp join first where rows are mostly short (tuples of more than four hashes) and the
-    // batch is large enough for its throughput to outweigh a launch (4,096 queries of 16 x 8
-    // bands, 260,000 polygons: 64-77 against 86-91 us a call; 64 queries: 59 against 49); the
-    // fill pass runs it only without a staging pool, and needs `where` to mark its rows
+    // the warp join first where rows are mostly short (tuples of more than four hashes, or few
+    // bands) and the batch is large enough for its throughput to outweigh a launch (4,096 queries
+    // of 16 x 8 bands, 260,000 polygons: 64-77 against 86-91 us a call; 64 queries: 59 against
+    // 49; 30,000 of 4 x 3 bands, 300,000 polygons, a candidate or none: 118 against 371); the fill
+    // pass runs it only without a staging pool, and needs `where` to mark its rows
     const bool staged = st.where && st.pool;
-    const bool warp = P.rows > 4 && Q >= 1024 && (write ? st.where && !staged : true);
+    const bool warp = (P.bands < 16 ? Q >= 256 : P.rows > 4 && Q >= 1024) && (write ? st.where && !staged : true);
     if (write) {
         if (staged) {  // the staged rows: a copy into place
             const unsigned cblocks = (unsigned)std::min<int64_t>(Q, (int64_t)X->ctx->sm_count * 8);
@@ -1292,7 +1338,8 @@ int pmh_launch_query(pmh_index X, const uint32_t* qh, int64_t Q, const int64_t* 
     if (form == JoinForm::kBitmap) {
         // (a pool of the whole capacity holds every row of a total that may be written)
         if (write && staged && pool_ints >= cap) return PMH_OK;
-        return launch_bitmap(X, qh, Q, d_n, counts, row_ptr, cand, cap, sb, warp, d_flags, write, s);
+        return launch_bitmap(X, qh, Q, d_n, counts, row_ptr, cand, cap, sb, write ? sb.where != nullptr : warp, d_flags,
+                             write, s);
     }
     PMH_TRY(launch_join<false>(X, qh, Q, d_n, counts, row_ptr, cand, cap, sb, warp, d_flags, write, s));
     return launch_join<true>(X, qh, Q, d_n, counts, row_ptr, cand, cap, sb, warp, d_flags, write, s);
