@@ -326,3 +326,41 @@ def test_count_then_fill_without_a_capacity(B, ctx, orc, n):
         for i, p in enumerate(pick):
             assert np.array_equal(cd[rp[p]:rp[p + 1]], cand_ref[rp_ref[i]:rp_ref[i + 1]]), p
     index.close()
+
+
+@pytest.mark.parametrize("K,bands,n", [(8, 4, 30_000), (12, 4, 200_000), (4, 2, 600_000)])
+@pytest.mark.parametrize("Q", [255, 256, 5000])
+def test_rows_of_few_bands(B, ctx, orc, K, bands, n, Q):
+    """Batches around the warp join's, most rows of a candidate or none, some of 100 to 10,000 entries (left
+    to the bitmap), and a block whose last rows are such."""
+    rng = np.random.default_rng(n + Q)
+    rows = K // bands
+    ph, qh = hashes(rng, n, K, int(n ** (1 / rows)) * 3), hashes(rng, Q, K, int(n ** (1 / rows)) * 3)
+    long = np.unique(np.concatenate([rng.choice(Q, 9, replace=False), [Q - 1, Q - 2]]))
+    for i, q in enumerate(long):
+        qh[q] = (1 << 22) + 7 * q
+        ph[rng.choice(n, 60 + 1000 * i, replace=False), :rows] = qh[q, :rows]
+    lengths = rows_of(B, ctx, orc, ph, qh, bands, np.concatenate([long, rng.choice(Q, 8, replace=False)]))
+    assert lengths[long].max() > 5000 and np.median(lengths) < 10
+
+
+def test_few_bands_in_the_query_graph(B, ctx):
+    """The captured joins of a batch that takes the warp join, dense and sparse rows: the plain call's rows."""
+    db = synth.star_polygons(3000, 3, n_range=(8, 40), f_range=(1e-4, 2e-1))
+    qs = synth.perturbed_queries(db, 300, 5)
+    P = B.make_params(8, 4, 1 << 22)
+    up = lambda ps: (torch.from_numpy(ps.xy).to(DEV), torch.from_numpy(ps.offsets).to(DEV))
+    h = B.minhash_sign(ctx, B.poly_upload(ctx, *up(db)), P)
+    index = B.lsh_build(ctx, h, P)
+    xy, off = up(qs)
+    row_ptr, cand = B.lsh_query(ctx, index, B.minhash_sign(ctx, B.poly_upload(ctx, xy, off), P))
+    total = cand.numel()
+    assert total > 0
+    for cap in (total, total - 1):
+        g = B.QueryGraph(ctx, index, 400, xy.shape[0] + 9, cap, 8)
+        g.run(xy, off)
+        assert g.status() == (0 if cap == total else 8, total)
+        assert torch.equal(g.row_ptr[:qs.n + 1], row_ptr) and int(g.row_ptr[400]) == total
+        assert cap < total or torch.equal(g.cand, cand)
+        g.close()
+    index.close()
