@@ -655,7 +655,9 @@ refine_pairs_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qo
 //  * a vertex c of B sees the shifted A's edges with min < c.y <= max: slab of c.y - 1;
 //  * an A edge meets B's non-horizontal edges in the slabs from its lowest to its
 //    highest row (a crossing of the shifted edge lies strictly inside B's rows, or just
-//    below B's top vertex), each pair in the first slab that lists both;
+//    below B's top vertex), each pair in the first slab that lists both; or every edge of B
+//    once, if those lists hold more (spiky rings, whose edges are listed in hundreds of slabs:
+//    1,200 pairs of stars of 1,800 to 4,000 vertices 44 ms by the lists, 7.8);
 //  * a horizontal edge of B meets the A edges with min < y <= max: slab of y - 1.
 // The end terms are integers (twice dy (x0 + dx / 2)), the crossings' fp64 terms are
 // added as two integers (multiples of 2^-18, and the remainder's of 2^-56, modulo 2^64):
@@ -931,20 +933,24 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
             const int i = i0 + lane;
             int2 a = make_int2(0, 0), b = make_int2(0, 0);
             int k0 = 0, cntk = 0, q0 = 0;
+            bool all = !B.sp;  // every edge of B, instead of the lists
             if (i < A.n) {
                 a = A.v[i];
                 b = A.vert(i + 1);
                 const int lo = max(min(a.y, b.y), yb0), hi = min(max(a.y, b.y), yb1);
                 if ((a.x != b.x || a.y != b.y) && hi >= lo && max(a.x, b.x) >= B.x0 && min(a.x, b.x) <= B.x1) {
+                    cntk = B.n;
                     if (B.sp) {
                         q0 = slab_div(lo - B.y0, B.magic);
                         const int q1 = min(slab_div(hi - B.y0, B.magic), B.S - 1);
-                        if (q0 <= q1) {
-                            k0 = B.sp[q0];
-                            cntk = B.sp[q1 + 1] - k0;
+                        const int listed = q0 <= q1 ? B.sp[q1 + 1] - B.sp[q0] : 0;
+                        // (long edges of both rings, as of spiky ones: an edge is listed in every slab
+                        // it meets, and its lists exceed the ring)
+                        all = listed > B.n;
+                        if (!all) {
+                            k0 = listed > 0 ? B.sp[q0] : 0;
+                            cntk = listed;
                         }
-                    } else {
-                        cntk = B.n;
                     }
                 }
             }
@@ -955,10 +961,10 @@ refine_big_kernel(const int2* __restrict__ qxy, const int64_t* __restrict__ qoff
                 int j = 0;
                 if (t < cntk) {
                     const int k = k0 + t;
-                    j = B.edge(k);
+                    j = all ? t : B.se[k];
                     const int2 c = B.v[j], d = B.vert(j + 1);
                     bool once = c.y != d.y;
-                    if (B.sp) {
+                    if (!all) {
                         while (k >= B.sp[qs + 1]) ++qs;
                         once = once && qs == max(q0, slab_div(min(c.y, d.y) - B.y0, B.magic));
                     }
