@@ -117,8 +117,8 @@ int pmh_destroy(pmh_ctx ctx);
 /* A0 -- upload polygons (Sec. 3.1 preprocessing: local MBRs).
  * Copies n_polys polygons into library-owned device memory and computes each
  * polygon's half-open bounding box clipped to the domain, twice its signed
- * area (exact int64 shoelace), its signing plan (indexed or walk form, grid
- * level) and the order in which the signing kernels take the polygons.
+ * area (exact int64 shoelace), the edge lists of its large rings and the order in
+ * which the signing kernels take the polygons.
  *   d_xy       int32 [n_vertices][2], interleaved (x, y), device
  *   d_offsets  int64 [n_polys + 1], offsets[0] = 0, offsets[n_polys] =
  *              n_vertices, polygon p = vertices offsets[p] .. offsets[p+1]-1

@@ -775,9 +775,10 @@ warp_join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int ban
 // Which sets: with tuples of one or two hashes (rows of hundreds to thousands) up to
 // 2^20 ids, where one bitmap still fits an SM (4,096 queries of 64 x 2 bands, 520,000
 // and 1,040,000 polygons: 0.73 and 1.37 ms a call against 1.87 and 3.24 with the set);
-// with longer tuples up to 409,600, where four do: the rows that reach the block are
-// then fewer than the blocks an SM needs to hide their latency (16 x 8 bands: 69 against
-// 88 us at 260,000 polygons, 116 against 88 at 520,000).
+// with longer tuples up to 409,600: fewer rows reach the block, and what counts is the bitmaps
+// an SM holds to hide their latency (16 x 8 bands: six at 260,000 polygons 69 us against
+// the set's 88, three at 520,000 116 against 88; the line lies between, at a size of which
+// four fit).
 constexpr int64_t kBitmapMaxIds = 409600;
 constexpr int64_t kBitmapMaxIdsShort = 1 << 20;
 constexpr int kBitmapU = 4;
@@ -1083,7 +1084,7 @@ static size_t dir_len(pmh_index X)
     return (size_t)pmh_dir_len(pmh_dir_cmax(X->params.bands, X->band_bits), X->dir_shift);
 }
 
-// hashes copied in, band keys, (band, key) entries radix-sorted with ids, full keys gathered
+// hashes copied in, (band, key) entries filled from them and radix-sorted with ids, the directory
 static int index_fill(pmh_ctx ctx, pmh_index X, const uint32_t* d_hashes, cudaStream_t s)
 {
     const int64_t n = X->n;

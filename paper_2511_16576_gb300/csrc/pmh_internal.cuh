@@ -379,7 +379,7 @@ int pmh_launch_sign(pmh_ctx ctx, const int2* xy, const int64_t* off, const int4*
                     const StreamIndexView* sidx = nullptr, const uint32_t* masks = nullptr,
                     const int32_t* order_cls = nullptr, int64_t n_indexed = 0,
                     int64_t n_whole_cost = 0);
-// every polygon in one persistent launch (sign_unified.cu): slots list[0 ..
+// every polygon, in persistent launches (sign_unified.cu): slots list[0 ..
 // n_slots) (list nullptr: slot = polygon id), the first n_chunked as (polygon,
 // 32-hash chunk) items, the rest whole; d_n (optional) caps n_slots on the
 // device, d_flags (optional) skips a batch that failed validation; U = points

@@ -25,11 +25,9 @@
 // Theorem 2: E[h] = 1/S_p), which balances polygons whose work differs by
 // orders of magnitude.
 //
-// Which kernel signs which polygon: with the stream index, every polygon is
-// signed by one launch of sign_unified_kernel (sign_unified.cu: indexed or walk
-// form as each polygon's plan says, staged or through its y-slab lists); this
-// file's sign_kernel signs without the stream index, with precomputed coverage
-// masks, and the batches of the captured query pipeline.
+// Which kernel signs which polygon: with the stream index, and in the captured query
+// pipeline, sign_unified.cu's launches sign every polygon; this file's sign_kernel signs
+// without the stream index and with precomputed coverage masks.
 #include <algorithm>
 #include <mutex>
 

@@ -133,9 +133,7 @@ struct SlabEdges {
 // Edges of a polygon staged in shared memory (v[0..n], v[n] = v[0]), binned by
 // the horizontal slabs [y0 + s*2^sh, y0 + (s+1)*2^sh) that their y-range
 // [min y, max y) meets: ids[beg[s] .. beg[s+1]) are the edges of slab s.  Only
-// those edges can straddle a line y = py inside slab s.  Both the
-// warp-cooperative test (lanes split the slab's edges) and the lane-local one
-// (one point per lane) are exact.
+// those edges can straddle a line y = py inside slab s (lanes split them).
 struct StagedEdges {
     const int2* v;
     const uint8_t* ids;
@@ -153,19 +151,6 @@ struct StagedEdges {
             par ^= edge_parity(v[e], v[e + 1], px, py);
         }
         return __popc(__ballot_sync(0xffffffffu, par)) & 1;
-    }
-    template <class W>
-    __device__ __forceinline__ bool lane_inside(int px, int py, W& w) const
-    {
-        const int s = (py - y0) >> sh;
-        const int lo = beg[s], hi = beg[s + 1];
-        w.lane_edges += hi - lo;
-        unsigned par = 0;
-        for (int i = lo; i < hi; ++i) {
-            const int e = ids[i];
-            par ^= edge_parity(v[e], v[e + 1], px, py);
-        }
-        return par;
     }
 };
 

@@ -1,5 +1,7 @@
-// sign_unified.cu -- step A1 (Definition 2, Algorithm 1): one persistent signing
-// launch for polygons of every size, through the stream index.
+// sign_unified.cu -- step A1 (Definition 2, Algorithm 1): persistent signing launches for
+// polygons of every size, through the stream index: one for the rings above the staged size and
+// one for the staged ones (a captured batch: one for both), one before them for few hashes of
+// polygons of large area, and one behind them for the walks past the index.
 //
 // h_k(P) = min{ i : point i of stream k lies in P } is found, per polygon, in
 // the indexed form or in the walk form:
@@ -34,8 +36,8 @@
 // polygons (all K hashes, so that the staging and the mask are paid once per
 // polygon).  A
 // staged polygon met in a chunked slot is signed whole by its chunk 0 (its
-// other chunks return at once), so the captured query pipeline can hand in
-// every polygon as a chunked slot.  Every step is exact, so the result equals
+// other chunks return at once) unless the batch leaves warps idle, so the captured query
+// pipeline can hand in every polygon as a chunked slot.  Every step is exact, so the result equals
 // the definition bit for bit.
 #include <algorithm>
 #include <type_traits>
