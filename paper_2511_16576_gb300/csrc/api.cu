@@ -292,18 +292,12 @@ static int upload_fill(pmh_polys P, const int32_t* xy, const int64_t* offsets, b
     if (e != cudaSuccess) return pmh_set_error(PMH_ERR_CUDA, "upload copy failed: %s", cudaGetErrorString(e));
     // offsets[0] and offsets[n] are checked by the kernel through b/e bounds
     int64_t* sizes = nullptr;
-    SlabInfo* info = P->slab_info;
     if (n_polys > 0) {
-        // (a set without a ring that gets a slab index keeps no info: its sizes go to scratch.
-        // 100,000 polygons: 671 us with an array of its own, 384)
-        const size_t size_bytes = sizeof(int64_t) * (size_t)(2 * (n_polys + 1));
-        PMH_TRY(pmh_scratch(ctx, SCR_MISC, size_bytes + (info ? 0 : sizeof(SlabInfo) * (size_t)n_polys),
-                            (void**)&sizes));
+        PMH_TRY(pmh_scratch(ctx, SCR_MISC, sizeof(int64_t) * (size_t)(2 * (n_polys + 1)), (void**)&sizes));
         int64_t* edge = sizes + n_polys + 1;
-        if (!info) info = reinterpret_cast<SlabInfo*>(edge + n_polys + 1);
         PMH_TRY(pmh_launch_prep(ctx->sm_count, fused ? reinterpret_cast<const int2*>(xy) : P->xy,
                                 fused ? P->xy : nullptr, P->offsets, n_polys, nullptr, n_vertices, P->bbox,
-                                P->area2, SlabSizes{info, sizes, edge}, ctx->d_status, s));
+                                P->area2, SlabSizes{P->slab_info, sizes, edge}, ctx->d_status, s));
         PMH_TRY(pmh_exclusive_scan_i64(ctx, sizes, sizes, n_polys, s, nullptr, 2));  // sizes, edge
         e = cudaMemcpyAsync(ctx->h_pinned + 1, sizes + n_polys, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess)
@@ -327,7 +321,7 @@ static int upload_fill(pmh_polys P, const int32_t* xy, const int64_t* offsets, b
         if ((e = cudaGetLastError()) != cudaSuccess)
             return pmh_set_error(PMH_ERR_CUDA, "feature kernel: %s", cudaGetErrorString(e));
     }
-    PMH_TRY(pmh_build_slabs(P, info, sizes, sizes + n_polys + 1, n_ptr, n_edges, s));
+    PMH_TRY(pmh_build_slabs(P, sizes, sizes + n_polys + 1, n_ptr, n_edges, s));
     return pmh_build_class_order(P, s);
 }
 
@@ -356,18 +350,38 @@ static int upload_common(pmh_ctx ctx, const int32_t* xy, const int64_t* offsets,
     P->device = ctx->device;
     P->n = n_polys;
     P->nv = n_vertices;
+    // every array of a size known now in one allocation (256-byte steps): an upload of a batch of
+    // queries is mostly its allocations, which cost 80 us each where they take a new block of
+    // the driver's (100,000 polygons of 8 to 64 vertices: 679 us with nine allocations, 376;
+    // 100 of 8 to 1,024: 163, 144)
     const size_t np = (size_t)(n_polys > 0 ? n_polys : 1);
-    if (cudaMalloc(&P->xy, sizeof(int2) * (size_t)(n_vertices > 0 ? n_vertices : 1)) != cudaSuccess ||
-        cudaMalloc(&P->offsets, sizeof(int64_t) * (size_t)(n_polys + 1)) != cudaSuccess ||
-        cudaMalloc(&P->bbox, sizeof(int4) * np + sizeof(SlabPtrs)) != cudaSuccess ||
-        cudaMalloc(&P->area2, sizeof(int64_t) * np) != cudaSuccess ||
-        cudaMalloc(&P->feat, sizeof(float2) * np) != cudaSuccess) {
+    size_t bytes = 0;
+    auto place = [&](size_t size) {
+        const size_t at = bytes;
+        bytes += (size + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t at_xy = place(sizeof(int2) * (size_t)(n_vertices > 0 ? n_vertices : 1));
+    const size_t at_off = place(sizeof(int64_t) * (size_t)(n_polys + 1)), at_bbox = place(sizeof(int4) * np);
+    const size_t at_area = place(sizeof(int64_t) * np), at_feat = place(sizeof(float2) * np);
+    const size_t at_info = place(sizeof(SlabInfo) * np), at_slabs = place(sizeof(SlabPtrs));
+    const size_t at_order = place(sizeof(int32_t) * np);
+    if (cudaMalloc(&P->arrays, bytes) != cudaSuccess) {
         cudaGetLastError();
+        P->arrays = nullptr;
         pmh_polys_destroy(P);
         return pmh_set_error(PMH_ERR_NOMEM, "polygon allocation failed (%lld vertices)",
                              (long long)n_vertices);
     }
-    if (n_polys > 0) P->d_slabs = reinterpret_cast<SlabPtrs*>(P->bbox + n_polys);
+    char* base = static_cast<char*>(P->arrays);
+    P->xy = reinterpret_cast<int2*>(base + at_xy);
+    P->offsets = reinterpret_cast<int64_t*>(base + at_off);
+    P->bbox = reinterpret_cast<int4*>(base + at_bbox);
+    P->area2 = reinterpret_cast<int64_t*>(base + at_area);
+    P->feat = reinterpret_cast<float2*>(base + at_feat);
+    P->slab_info = reinterpret_cast<SlabInfo*>(base + at_info);
+    P->d_slabs = reinterpret_cast<SlabPtrs*>(base + at_slabs);
+    P->order_buf = reinterpret_cast<int32_t*>(base + at_order);
     const int rc = upload_fill(P, xy, offsets, host, (cudaStream_t)stream);
     if (rc != PMH_OK) {
         pmh_polys_destroy(P);
@@ -387,12 +401,10 @@ static void free_derived(pmh_polys p, bool all)
     p->order = nullptr;
     p->mask = nullptr;
     p->n_indexed = p->n_whole_cost = 0;
+    p->order_cls = nullptr;
     if (!all) return;
-    void* bufs[] = {p->slab_info, p->slab_ptr, p->slab_edges, p->order_cls};
-    for (void* b : bufs)
-        if (b) cudaFree(b);
-    p->slab_info = nullptr;
-    p->slab_ptr = p->slab_edges = p->order_cls = nullptr;
+    if (p->slab_ptr) cudaFree(p->slab_ptr);
+    p->slab_ptr = p->slab_edges = nullptr;
     p->cap_slab_ptr = p->cap_slab_edges = 0;
 }
 
@@ -410,11 +422,12 @@ extern "C" int pmh_poly_reload(pmh_polys polys, const int32_t* xy, const int64_t
     // keep their buffers while the new lists fit (releasing and taking half a gigabyte was a
     // third of a reload of 400,000 polygons)
     PMH_CUDA_TRY(cudaDeviceSynchronize());
-    if (polys->d_slabs) PMH_CUDA_TRY(cudaMemsetAsync(polys->d_slabs, 0, sizeof(SlabPtrs), s));
+    PMH_CUDA_TRY(cudaMemsetAsync(polys->d_slabs, 0, sizeof(SlabPtrs), s));
     free_derived(polys, false);
     const int rc = upload_fill(polys, xy, offsets, host_memory != 0, s);
     if (rc != PMH_OK) {  // a reload that fails leaves no slab index behind
-        if (polys->d_slabs) cudaMemsetAsync(polys->d_slabs, 0, sizeof(SlabPtrs), s);
+        cudaMemsetAsync(polys->d_slabs, 0, sizeof(SlabPtrs), s);
+        cudaMemsetAsync(polys->slab_info, 0, sizeof(SlabInfo) * polys->n, s);
         cudaDeviceSynchronize();
         free_derived(polys, true);
         polys->max_n = INT32_MAX;  // (unknown)
@@ -460,9 +473,8 @@ extern "C" int pmh_polys_destroy(pmh_polys p)
 {
     if (!p) return PMH_OK;
     cudaSetDevice(p->device);
-    if (p->xy || p->offsets || p->bbox || p->area2) cudaDeviceSynchronize();
-    void* bufs[] = {p->xy, p->offsets, p->bbox, p->area2, p->feat, p->slab_info, p->slab_ptr,
-                    p->slab_edges, p->order, p->order_cls, p->mask};
+    if (p->arrays) cudaDeviceSynchronize();
+    void* bufs[] = {p->arrays, p->slab_ptr, p->order, p->mask};
     for (void* b : bufs)
         if (b) cudaFree(b);
     delete p;

@@ -264,21 +264,22 @@ struct pmh_polys_s {
     pmh_ctx ctx = nullptr;
     int device = 0;
     int64_t n = 0, nv = 0;
+    void* arrays = nullptr;    // one allocation: the arrays below, slab_info, d_slabs and the class order
     int2* xy = nullptr;
     int64_t* offsets = nullptr;
     int4* bbox = nullptr;      // x0, y0, x1, y1 half-open, clipped to the domain
     int64_t* area2 = nullptr;  // twice the signed area
     int32_t max_n = 0;         // largest vertex count
     float2* feat = nullptr;         // [n] log2(area) / 32, log2(n) / 16 (reranker inputs)
-    SlabInfo* slab_info = nullptr;  // [n]; nullptr: no ring of the set ever had a slab index
-    int32_t* slab_ptr = nullptr;    // (kept by a reload while its lists fit)
+    SlabInfo* slab_info = nullptr;  // [n]
+    int32_t* slab_ptr = nullptr;    // (with the edges in one allocation, kept by a reload while its lists fit)
     int32_t* slab_edges = nullptr;
     int64_t cap_slab_ptr = 0, cap_slab_edges = 0;
-    SlabPtrs* d_slabs = nullptr;    // the three above, device-resident behind the boxes (rewritten by a
-                                    // reload)
+    SlabPtrs* d_slabs = nullptr;    // the three above, device-resident (rewritten by a reload)
     int32_t* order = nullptr;       // polygons by expected signing cost, largest first (built
                                     // on the first signing call without the stream index)
-    int32_t* order_cls = nullptr;   // class order: polygons above kChunkMinVerts vertices, then
+    int32_t* order_buf = nullptr;   // [n], the class order's
+    int32_t* order_cls = nullptr;   // order_buf once built: the class order, polygons above kChunkMinVerts vertices, then
                                     // the others above kStagedMaxVerts, each by cost, then the
                                     // staged polygons (Morton order)
     int64_t n_indexed = 0;          // class 0: <= kStagedMaxVerts vertices
@@ -286,9 +287,8 @@ struct pmh_polys_s {
     uint32_t* mask = nullptr;       // [n][16] coverage masks
 };
 
-// the slab lists of P from the sizes that A0 left (`sized`: P->slab_info, or scratch if P has none yet)
-// and their exclusive scans, whose totals the host knows
-int pmh_build_slabs(pmh_polys P, const SlabInfo* sized, const int64_t* ptr_base, const int64_t* edge_base, int64_t n_ptr,
+// the slab lists of P from the exclusive scans of its SlabSizes, whose totals the host knows
+int pmh_build_slabs(pmh_polys P, const int64_t* ptr_base, const int64_t* edge_base, int64_t n_ptr,
                     int64_t n_edges, cudaStream_t s);
 int pmh_launch_slabs_fixed(pmh_ctx ctx, const int2* xy, const int64_t* off, int64_t max_polys,
                            const int64_t* d_n, SlabInfo* info, int64_t* sizes, int64_t* sums,

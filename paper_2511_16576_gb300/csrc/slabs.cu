@@ -54,8 +54,8 @@ __device__ __forceinline__ void for_slab_entries(const int2* __restrict__ xy, in
 }
 
 __global__ void __launch_bounds__(kFillThreads, 8) slab_fill_kernel(const int2* __restrict__ xy, const int64_t* __restrict__ off,
-                                 int64_t n_polys, const int64_t* __restrict__ d_n, const SlabInfo* sized,
-                                 SlabInfo* info, const int64_t* __restrict__ ptr_base, const int64_t* __restrict__ edge_base,
+                                 int64_t n_polys, const int64_t* __restrict__ d_n, SlabInfo* __restrict__ info,
+                                 const int64_t* __restrict__ ptr_base, const int64_t* __restrict__ edge_base,
                                  int32_t* slab_ptr, int64_t cap_ptr, int32_t* __restrict__ slab_edges,
                                  int64_t cap_edges)
 {
@@ -65,26 +65,22 @@ __global__ void __launch_bounds__(kFillThreads, 8) slab_fill_kernel(const int2* 
     if (d_n) n_polys = min(n_polys, *d_n);
     for (int64_t p = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); p < n_polys;
          p += nwarps) {
-        SlabInfo si = sized[p];
+        const SlabInfo si = info[p];
         const int S = si.S, y0 = si.ymin;
-        if (S <= 0) {
-            if (lane == 0 && sized != info) info[p] = si;
-            continue;
-        }
+        if (S <= 0) continue;
         const int64_t b = off[p];
         const int n = (int)(off[p + 1] - b);
         const uint64_t hm = slab_div_magic(si.slab_h);
         const int64_t pb = ptr_base[p], eb = edge_base[p];
         if (ptr_base[p + 1] > cap_ptr || edge_base[p + 1] > cap_edges) {
             // the lists do not fit the fixed buffers: this polygon is tested over all its edges
-            si.S = 0;
-            if (lane == 0) info[p] = si;
+            if (lane == 0) info[p].S = 0;
             continue;
         }
-        si.slab_base = pb;
-        si.edge_base = eb;
-        __syncwarp();  // (sized may be info: every lane has read its entry)
-        if (lane == 0) info[p] = si;
+        if (lane == 0) {
+            info[p].slab_base = pb;
+            info[p].edge_base = eb;
+        }
         int32_t* sp = slab_ptr + pb;
         int32_t* le = slab_edges + eb;
         const bool small = S <= kFillSmemSlabs;
@@ -204,39 +200,39 @@ __global__ void class_key_kernel(const int4* __restrict__ bbox, const int64_t* _
 
 }  // namespace
 
-// room for `need` entries in *buf (a set's lists: exactly as many at first, an eighth more when
-// a reload has to grow them)
-static int grow_list(int32_t** buf, int64_t* cap, int64_t need)
+// room for a set's slab tables and edge lists, in one allocation: exactly as much at first, an
+// eighth more when a reload has to grow them
+static int grow_lists(pmh_polys P, int64_t n_ptr, int64_t n_edges)
 {
-    need = std::max<int64_t>(need, 1);
-    if (*buf && *cap >= need) return PMH_OK;
-    const int64_t want = *buf ? need + need / 8 : need;
-    if (*buf) cudaFree(*buf);
-    *buf = nullptr;
-    *cap = 0;
-    if (cudaMalloc(buf, sizeof(int32_t) * (size_t)want) != cudaSuccess) {
-        cudaGetLastError();
-        *buf = nullptr;
-        return pmh_set_error(PMH_ERR_NOMEM, "slab index allocation failed (%lld entries)", (long long)need);
+    n_edges = std::max<int64_t>(n_edges, 1);
+    if (P->slab_ptr && P->cap_slab_ptr >= n_ptr && P->cap_slab_edges >= n_edges) return PMH_OK;
+    if (P->slab_ptr) {
+        n_ptr = std::max(n_ptr + n_ptr / 8, P->cap_slab_ptr);
+        n_edges = std::max(n_edges + n_edges / 8, P->cap_slab_edges);
+        cudaFree(P->slab_ptr);
     }
-    *cap = want;
+    P->slab_ptr = P->slab_edges = nullptr;
+    P->cap_slab_ptr = P->cap_slab_edges = 0;
+    if (cudaMalloc(&P->slab_ptr, sizeof(int32_t) * (size_t)(n_ptr + n_edges)) != cudaSuccess) {
+        cudaGetLastError();
+        P->slab_ptr = nullptr;
+        return pmh_set_error(PMH_ERR_NOMEM, "slab index allocation failed (%lld entries)",
+                             (long long)(n_ptr + n_edges));
+    }
+    P->slab_edges = P->slab_ptr + n_ptr;
+    P->cap_slab_ptr = n_ptr;
+    P->cap_slab_edges = n_edges;
     return PMH_OK;
 }
 
-int pmh_build_slabs(pmh_polys P, const SlabInfo* sized, const int64_t* ptr_base, const int64_t* edge_base,
-                    int64_t n_ptr, int64_t n_edges, cudaStream_t s)
+int pmh_build_slabs(pmh_polys P, const int64_t* ptr_base, const int64_t* edge_base, int64_t n_ptr,
+                    int64_t n_edges, cudaStream_t s)
 {
     if (P->n == 0) return PMH_OK;
     if (n_ptr > 0) {
-        if (!P->slab_info && cudaMalloc(&P->slab_info, sizeof(SlabInfo) * P->n) != cudaSuccess) {
-            cudaGetLastError();
-            P->slab_info = nullptr;
-            return pmh_set_error(PMH_ERR_NOMEM, "slab info allocation failed");
-        }
-        PMH_TRY(grow_list(&P->slab_ptr, &P->cap_slab_ptr, n_ptr));
-        PMH_TRY(grow_list(&P->slab_edges, &P->cap_slab_edges, n_edges));
+        PMH_TRY(grow_lists(P, n_ptr, n_edges));
         const int blocks = (int)std::min<int64_t>((P->n + 7) / 8, (int64_t)P->ctx->sm_count * 32);
-        slab_fill_kernel<<<blocks, kFillThreads, 0, s>>>(P->xy, P->offsets, P->n, nullptr, sized, P->slab_info,
+        slab_fill_kernel<<<blocks, kFillThreads, 0, s>>>(P->xy, P->offsets, P->n, nullptr, P->slab_info,
                                                          ptr_base, edge_base, P->slab_ptr, P->cap_slab_ptr,
                                                          P->slab_edges, P->cap_slab_edges);
         PMH_LAUNCHED("slab_fill_kernel");
@@ -287,10 +283,7 @@ int pmh_build_class_order(pmh_polys P, cudaStream_t s)
     PMH_TRY(pmh_scratch(ctx, SCR_MISC, 2 * sizeof(unsigned long long) + sizeof(uint32_t) * (size_t)n,
                         (void**)&n_cls));
     uint32_t* keys = reinterpret_cast<uint32_t*>(n_cls + 2);
-    if (!P->order_cls && cudaMalloc(&P->order_cls, sizeof(int32_t) * n) != cudaSuccess) {
-        cudaGetLastError();
-        return pmh_set_error(PMH_ERR_NOMEM, "class order allocation failed");
-    }
+    P->order_cls = P->order_buf;
     PMH_CUDA_TRY(cudaMemsetAsync(n_cls, 0, 2 * sizeof(unsigned long long), s));
     const int blocks = (int)std::min<int64_t>((n + 255) / 256, (int64_t)ctx->sm_count * 4);
     class_key_kernel<<<blocks, 256, 0, s>>>(P->bbox, P->area2, P->offsets, n, keys, P->order_cls, n_cls);
@@ -320,7 +313,7 @@ int pmh_launch_slabs_fixed(pmh_ctx ctx, const int2* xy, const int64_t* off, int6
     int64_t* edge_sizes = sizes + (max_polys + 1);
     PMH_TRY(pmh_exclusive_scan_i64(ctx, sizes, sizes, max_polys, s, sums, 2));
     const int blocks = (int)std::min<int64_t>((max_polys + 7) / 8, (int64_t)ctx->sm_count * 16);
-    slab_fill_kernel<<<blocks, kFillThreads, 0, s>>>(xy, off, max_polys, d_n, info, info, ptr_sizes, edge_sizes,
+    slab_fill_kernel<<<blocks, kFillThreads, 0, s>>>(xy, off, max_polys, d_n, info, ptr_sizes, edge_sizes,
                                                      slab_ptr, cap_ptr, slab_edges, cap_edges);
     PMH_LAUNCHED("slab_fill_kernel");
     return PMH_OK;
