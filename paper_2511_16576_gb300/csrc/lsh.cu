@@ -566,8 +566,10 @@ join_kernel(const uint32_t* __restrict__ qhashes, int64_t Q, int K, int bands, i
 
 // fill pass of the staged rows: a block per row copies its pool slice into place, or, of rows of
 // fewer than kCopyWarpRow ids on average, a warp (four independent loads per thread in
-// flight; rows of a candidate or none leave a block waiting on their three loads)
-constexpr int kCopyWarpRow = 256;
+// flight; rows of a candidate or none leave a block waiting on their three loads, while a warp
+// is long with the longest row of a batch: 4,096 rows of 200 on average and thousands at most 9
+// us by blocks, 28 by warps)
+constexpr int kCopyWarpRow = 16;
 __global__ void __launch_bounds__(256)
 copy_rows_kernel(JoinStage st, int64_t Q, const int64_t* __restrict__ row_ptr, int32_t* __restrict__ cand,
                  int64_t cap, const int64_t* __restrict__ d_n, int* __restrict__ d_flags)
